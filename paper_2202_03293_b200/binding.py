@@ -1,14 +1,17 @@
-"""Thin ctypes binding of libsg.so: argument marshalling only.
+"""Thin binding of libsg.so: argument marshalling only.
 
 Every function here has the name and argument order of its C entry point
 (see include/sg.h) and takes torch tensors that already live on the GPU;
 pointers, element strides and the current CUDA stream are extracted and
-passed through.  Nothing is computed on the Python side and there is no
-fallback: if the library is missing or a call fails, an exception is raised.
+passed through, for the ops by the native module _sgcall (csrc/sg_call.cpp),
+for everything else by ctypes.  Nothing is computed on the Python side and
+there is no fallback: if the library is missing or a call fails, an exception
+is raised.
 """
 from __future__ import annotations
 
 import ctypes
+import importlib
 import os
 
 import torch
@@ -89,32 +92,27 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
+class _Call:
+    """Stands in for the native module until the first op is called (importing this file needs no built library)."""
+
+    def __getattr__(self, name):
+        global _call
+        lib()
+        _call = importlib.import_module("._sgcall", __package__)
+        return getattr(_call, name)
+
+
+_call = _Call()
+
+
 def status_string(code: int) -> str:
     return lib().sg_status_string(int(code)).decode()
-
-
-def _dtype_code(t: torch.Tensor) -> int:
-    if t.dtype == torch.float32:
-        return SG_F32
-    if t.dtype == torch.bfloat16:
-        return SG_BF16
-    raise TypeError(f"unsupported input dtype {t.dtype}")
 
 
 def _stream(stream) -> int:
     if stream is None:
         return torch.cuda.current_stream().cuda_stream
     return getattr(stream, "cuda_stream", stream)
-
-
-def _arr(vals):
-    return (ctypes.c_int64 * len(vals))(*[int(v) for v in vals])
-
-
-def _ptr(t: torch.Tensor):
-    if not t.is_cuda:
-        raise ValueError("tensors must live on a CUDA device")
-    return ctypes.c_void_p(t.data_ptr())
 
 
 def sg_matmul_raw(M, N, K, A, a_sm, a_sk, B, b_sk, b_sn, C, c_sm, c_sn, dtype, mode, stream) -> int:
@@ -124,12 +122,7 @@ def sg_matmul_raw(M, N, K, A, a_sm, a_sk, B, b_sk, b_sn, C, c_sm, c_sn, dtype, m
 
 def sg_matmul(A: torch.Tensor, B: torch.Tensor, C: torch.Tensor, mode: int = SG_OVERWRITE, stream=None) -> torch.Tensor:
     """C[m,n] (+)= sum_k A[m,k]*B[k,n]; A, B bf16 or f32 (same dtype), C f32, any strides."""
-    M, K = A.shape
-    K2, N = B.shape
-    if K != K2 or tuple(C.shape) != (M, N) or C.dtype != torch.float32 or A.dtype != B.dtype:
-        raise ValueError("shape or dtype mismatch")
-    rc = lib().sg_matmul(M, N, K, _ptr(A), A.stride(0), A.stride(1), _ptr(B), B.stride(0), B.stride(1),
-                         _ptr(C), C.stride(0), C.stride(1), _dtype_code(A), mode, _stream(stream))
+    rc = _call.matmul(A, B, C, mode, stream)
     if rc != SG_OK:
         raise SgError(rc, "sg_matmul")
     return C
@@ -140,15 +133,7 @@ SG_ACT_NONE, SG_ACT_RELU = 0, 1
 
 def sg_matmul_bias_act(A: torch.Tensor, B: torch.Tensor, bias, C: torch.Tensor, act: int = SG_ACT_NONE, stream=None) -> torch.Tensor:
     """C[m,n] = act(sum_k A[m,k]*B[k,n] + bias[n]); bias an f32 vector of N values or None; C is overwritten."""
-    M, K = A.shape
-    K2, N = B.shape
-    if K != K2 or tuple(C.shape) != (M, N) or C.dtype != torch.float32 or A.dtype != B.dtype:
-        raise ValueError("shape or dtype mismatch")
-    if bias is not None and (tuple(bias.shape) != (N,) or bias.dtype != torch.float32):
-        raise ValueError("bias must be an f32 vector of N values")
-    rc = lib().sg_matmul_bias_act(M, N, K, _ptr(A), A.stride(0), A.stride(1), _ptr(B), B.stride(0), B.stride(1),
-                                  _ptr(bias) if bias is not None else None, bias.stride(0) if bias is not None else 0, int(act),
-                                  _ptr(C), C.stride(0), C.stride(1), _dtype_code(A), _stream(stream))
+    rc = _call.matmul_bias_act(A, B, bias, C, act, stream)
     if rc != SG_OK:
         raise SgError(rc, "sg_matmul_bias_act")
     return C
@@ -157,14 +142,7 @@ def sg_matmul_bias_act(A: torch.Tensor, B: torch.Tensor, bias, C: torch.Tensor, 
 def sg_conv1d_nwc_wcf(I: torch.Tensor, Kf: torch.Tensor, O: torch.Tensor, stride_w: int = 1, dilation_w: int = 1,
                       mode: int = SG_OVERWRITE, stream=None) -> torch.Tensor:
     """O[n,w,f] (+)= sum_{kw,c} I[n, w*stride_w + kw*dilation_w, c] * Kf[kw,c,f]."""
-    N, W_in, C = I.shape
-    KW, C2, F = Kf.shape
-    N2, W_out, F2 = O.shape
-    if C != C2 or N != N2 or F != F2 or O.dtype != torch.float32 or I.dtype != Kf.dtype:
-        raise ValueError("shape or dtype mismatch")
-    rc = lib().sg_conv1d_nwc_wcf(N, W_out, F, KW, C, W_in, stride_w, dilation_w, _ptr(I), _arr(I.stride()),
-                                 _ptr(Kf), _arr(Kf.stride()), _ptr(O), _arr(O.stride()), _dtype_code(I), mode,
-                                 _stream(stream))
+    rc = _call.conv1d(I, Kf, O, stride_w, dilation_w, mode, stream)
     if rc != SG_OK:
         raise SgError(rc, "sg_conv1d_nwc_wcf")
     return O
@@ -173,14 +151,7 @@ def sg_conv1d_nwc_wcf(I: torch.Tensor, Kf: torch.Tensor, O: torch.Tensor, stride
 def sg_conv2d_nhwc_hwcf(I: torch.Tensor, Kf: torch.Tensor, O: torch.Tensor, stride=(1, 1), dilation=(1, 1),
                         mode: int = SG_OVERWRITE, stream=None) -> torch.Tensor:
     """O[n,h,w,f] (+)= sum_{kh,kw,c} I[n, h*sh+kh*dh, w*sw+kw*dw, c] * Kf[kh,kw,c,f]."""
-    N, H_in, W_in, C = I.shape
-    KH, KW, C2, F = Kf.shape
-    N2, H_out, W_out, F2 = O.shape
-    if C != C2 or N != N2 or F != F2 or O.dtype != torch.float32 or I.dtype != Kf.dtype:
-        raise ValueError("shape or dtype mismatch")
-    rc = lib().sg_conv2d_nhwc_hwcf(N, H_out, W_out, F, KH, KW, C, H_in, W_in, stride[0], stride[1], dilation[0],
-                                   dilation[1], _ptr(I), _arr(I.stride()), _ptr(Kf), _arr(Kf.stride()), _ptr(O),
-                                   _arr(O.stride()), _dtype_code(I), mode, _stream(stream))
+    rc = _call.conv2d(I, Kf, O, stride, dilation, mode, stream)
     if rc != SG_OK:
         raise SgError(rc, "sg_conv2d_nhwc_hwcf")
     return O
@@ -189,14 +160,7 @@ def sg_conv2d_nhwc_hwcf(I: torch.Tensor, Kf: torch.Tensor, O: torch.Tensor, stri
 def sg_depthwise_conv2d_nhwc_hwc(I: torch.Tensor, Kf: torch.Tensor, O: torch.Tensor, stride=(1, 1), dilation=(1, 1),
                                  mode: int = SG_OVERWRITE, stream=None) -> torch.Tensor:
     """O[n,h,w,c] (+)= sum_{kh,kw} I[n, h*sh+kh*dh, w*sw+kw*dw, c] * Kf[kh,kw,c]."""
-    N, H_in, W_in, C = I.shape
-    KH, KW, C2 = Kf.shape
-    N2, H_out, W_out, C3 = O.shape
-    if C != C2 or C != C3 or N != N2 or O.dtype != torch.float32 or I.dtype != Kf.dtype:
-        raise ValueError("shape or dtype mismatch")
-    rc = lib().sg_depthwise_conv2d_nhwc_hwc(N, H_out, W_out, C, KH, KW, H_in, W_in, stride[0], stride[1], dilation[0],
-                                            dilation[1], _ptr(I), _arr(I.stride()), _ptr(Kf), _arr(Kf.stride()), _ptr(O),
-                                            _arr(O.stride()), _dtype_code(I), mode, _stream(stream))
+    rc = _call.depthwise2d(I, Kf, O, stride, dilation, mode, stream)
     if rc != SG_OK:
         raise SgError(rc, "sg_depthwise_conv2d_nhwc_hwc")
     return O
@@ -205,57 +169,42 @@ def sg_depthwise_conv2d_nhwc_hwc(I: torch.Tensor, Kf: torch.Tensor, O: torch.Ten
 def sg_depthwise_conv1d_nwc_wc(I: torch.Tensor, Kf: torch.Tensor, O: torch.Tensor, stride: int = 1, dilation: int = 1,
                                mode: int = SG_OVERWRITE, stream=None) -> torch.Tensor:
     """O[n,w,c] (+)= sum_kw I[n, w*sw+kw*dw, c] * Kf[kw,c]."""
-    N, W_in, C = I.shape
-    KW, C2 = Kf.shape
-    N2, W_out, C3 = O.shape
-    if C != C2 or C != C3 or N != N2 or O.dtype != torch.float32 or I.dtype != Kf.dtype:
-        raise ValueError("shape or dtype mismatch")
-    rc = lib().sg_depthwise_conv1d_nwc_wc(N, W_out, C, KW, W_in, stride, dilation, _ptr(I), _arr(I.stride()), _ptr(Kf),
-                                          _arr(Kf.stride()), _ptr(O), _arr(O.stride()), _dtype_code(I), mode, _stream(stream))
+    rc = _call.depthwise1d(I, Kf, O, stride, dilation, mode, stream)
     if rc != SG_OK:
         raise SgError(rc, "sg_depthwise_conv1d_nwc_wc")
     return O
 
 
-def _move2d(fn, name, src: torch.Tensor, dst: torch.Tensor, want_shape, stream):
-    if src.dim() != 2 or tuple(dst.shape) != tuple(want_shape) or src.dtype != dst.dtype:
-        raise ValueError(f"{name}: shape or dtype mismatch")
-    R, C = src.shape
-    rc = fn(R, C, _ptr(src), src.stride(0), src.stride(1), _ptr(dst), dst.stride(0), dst.stride(1), _dtype_code(src),
-            _stream(stream))
-    if rc != SG_OK:
-        raise SgError(rc, name)
-    return dst
-
-
 def sg_copy2d(src: torch.Tensor, dst: torch.Tensor, stream=None) -> torch.Tensor:
     """dst[i,j] = src[i,j]."""
-    return _move2d(lib().sg_copy2d, "sg_copy2d", src, dst, src.shape, stream)
+    rc = _call.copy2d(src, dst, stream)
+    if rc != SG_OK:
+        raise SgError(rc, "sg_copy2d")
+    return dst
 
 
 def sg_transpose2d(src: torch.Tensor, dst: torch.Tensor, stream=None) -> torch.Tensor:
     """dst[j,i] = src[i,j]; dst is C x R."""
-    return _move2d(lib().sg_transpose2d, "sg_transpose2d", src, dst, (src.shape[1], src.shape[0]), stream)
-
-
-def _reduce2d(fn, name, A: torch.Tensor, out: torch.Tensor, n_out, mode, stream):
-    if A.dim() != 2 or out.dim() != 1 or out.shape[0] != n_out or out.dtype != torch.float32:
-        raise ValueError(f"{name}: shape or dtype mismatch")
-    R, C = A.shape
-    rc = fn(R, C, _ptr(A), A.stride(0), A.stride(1), _ptr(out), out.stride(0), _dtype_code(A), int(mode), _stream(stream))
+    rc = _call.transpose2d(src, dst, stream)
     if rc != SG_OK:
-        raise SgError(rc, name)
-    return out
+        raise SgError(rc, "sg_transpose2d")
+    return dst
 
 
 def sg_colred2d(A: torch.Tensor, out: torch.Tensor, mode: int = SG_OVERWRITE, stream=None) -> torch.Tensor:
     """out[j] (+)= sum_i A[i,j]."""
-    return _reduce2d(lib().sg_colred2d, "sg_colred2d", A, out, A.shape[1], mode, stream)
+    rc = _call.colred2d(A, out, mode, stream)
+    if rc != SG_OK:
+        raise SgError(rc, "sg_colred2d")
+    return out
 
 
 def sg_rowred2d(A: torch.Tensor, out: torch.Tensor, mode: int = SG_OVERWRITE, stream=None) -> torch.Tensor:
     """out[i] (+)= sum_j A[i,j]."""
-    return _reduce2d(lib().sg_rowred2d, "sg_rowred2d", A, out, A.shape[0], mode, stream)
+    rc = _call.rowred2d(A, out, mode, stream)
+    if rc != SG_OK:
+        raise SgError(rc, "sg_rowred2d")
+    return out
 
 
 def sg_check(stream=None) -> None:

@@ -2,12 +2,14 @@
 
 Every .cu file is its own translation unit (no relocatable device code), so the files are
 compiled side by side into objects under csrc/_build/ and linked into one shared library.
+_sgcall.so, the native half of the Python binding, is compiled with g++ against torch's headers.
 """
 from __future__ import annotations
 
 import glob
 import os
 import subprocess
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 PKG = os.path.dirname(os.path.abspath(__file__))
@@ -15,6 +17,8 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 OBJ = os.path.join(CSRC, "_build")
 LIB = os.path.join(PKG, "libsg.so")
+CALL_SRC = os.path.join(CSRC, "sg_call.cpp")
+CALL = os.path.join(PKG, "_sgcall.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -41,8 +45,30 @@ def needs_build() -> bool:
     return _stale(LIB, sources() + headers())
 
 
+def build_call_module(force: bool = False, verbose: bool = False) -> str:
+    """The Python call path: links against libsg.so and against the torch it will be loaded beside."""
+    if not (force or _stale(CALL, [CALL_SRC, os.path.join(ROOT, "include", "sg.h")])):
+        return CALL
+    from torch.utils.cpp_extension import include_paths, library_paths
+    cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", CALL_SRC, "-o", CALL]
+    for inc in [os.path.join(ROOT, "include"), sysconfig.get_paths()["include"], os.path.join(cuda, "include")] + include_paths():
+        cmd += ["-I", inc]
+    cmd += ["-L", PKG, "-l:libsg.so", "-Wl,-rpath,$ORIGIN"]
+    for d in library_paths():
+        cmd += ["-L", d, "-Wl,-rpath," + d]
+    cmd += ["-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.stdout + res.stderr and (verbose or res.returncode != 0):
+        print(res.stdout + res.stderr)
+    if res.returncode != 0:
+        raise RuntimeError("building _sgcall.so failed")
+    return CALL
+
+
 def build_library(force: bool = False, verbose: bool = False) -> str:
     if not (force or needs_build()):
+        build_call_module(force, verbose)
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
     os.makedirs(OBJ, exist_ok=True)
@@ -70,6 +96,7 @@ def build_library(force: bool = False, verbose: bool = False) -> str:
         print(res.stdout + res.stderr)
     if res.returncode != 0:
         raise RuntimeError("linking libsg.so failed")
+    build_call_module(force, verbose)
     return LIB
 
 

@@ -38,6 +38,8 @@ sg_status run(const Problem &p, const void *In, const void *Flt, float *O, cudaS
     }
     if (force != SG_KERNEL_FFMA) {
         sg_status st = launch_tensor(p, In, Flt, O, stream);
+        // layouts outside the TMA rules: the same contraction with the operands fetched by ordinary loads
+        if (st == SG_ERR_UNSUPPORTED) st = launch_gather(p, In, Flt, O, force == SG_KERNEL_TENSOR, stream);
         if (st == SG_OK) { t_last_kernel = SG_KERNEL_TENSOR; return SG_OK; }
         if (st != SG_ERR_UNSUPPORTED || force == SG_KERNEL_TENSOR) return st;
     }

@@ -1,0 +1,555 @@
+// Tensor-core implicit GEMM for layouts that the TMA unit cannot read: rows that do not start on 16-byte boundaries (a
+// product whose sizes are multiples of nothing), extents that end inside a 16-byte unit, images of three channels, operands
+// without any unit stride.
+//
+// The pipeline is the one of the TMA kernels with its first stage replaced: sixteen producer warps fetch the operands with
+// ordinary loads of one or two elements per lane and write the 128-byte swizzled tiles that tcgen05.mma reads.  A tile is a
+// stack of 128-byte lines of 64 bf16: along k (K-major: lines are rows of the input or columns of the filter) or along the
+// other index (MN-major: lines are values of k), whichever of the two is contiguous in memory, so that a warp always loads a
+// run of memory, one line per instruction.
+//
+//   warps 0-15   producers, two groups of eight that take the k-blocks in turn: while one group's loads are in flight the
+//                other writes its tile.
+//   warp  16     MMA issuer and owner of tensor memory.
+//   warps 17-20  write-back: tensor memory -> registers -> (bias, activation) -> rows of the output through a shared-memory
+//                transpose, one row of 32 columns per store instruction, any alignment and stride.
+//
+// f32 inputs keep full f32 precision: x = b0 + b1 + b2 with three bf16 values of 8 bits each (the differences are exact), and
+// of the nine products the six of weight 2^-16 and up are accumulated, smallest first.  What is dropped is below 2^-23 |a*b|,
+// the rounding of a single f32 product.
+//
+// The tensor core adds into its f32 accumulator by truncation, which drifts with the number of additions (relative error of a
+// sum of 4096 bf16 products: 4e-6, against 5e-7 for FFMA).  Callers of these layouts have had FFMA's accuracy so far, so a
+// partial sum stays in the accumulator for P k-blocks only (bf16: 256 values of k, f32: 64) and is then added, rounding to
+// nearest, to a running sum in tensor memory by the write-back warps, beside the MMAs of the next P k-blocks.
+//
+// What bounds a k-block is the number of load and store instructions of the producers (256 lines of a 128 x 128 tile, two
+// loads and one store each when pairs are not aligned, against 256 cycles of MMAs).
+#include <algorithm>
+#include <initializer_list>
+#include <type_traits>
+#include <utility>
+
+#include "sg_internal.cuh"
+#include "sg_tc_ptx.cuh"
+
+namespace sg {
+namespace {
+
+constexpr int BM = 128, BK = 64;
+constexpr int GROUPS = 2, GROUP_WARPS = 8;                  // producer groups and warps per group
+constexpr int MMA_WARP = GROUPS * GROUP_WARPS, EPI_WARP = MMA_WARP + 1;
+constexpr int THREADS = 32 * (EPI_WARP + 4);
+constexpr int MAX_SPLIT = 8;
+
+// How one operand is fetched.  mn_major 0: lines are rows/columns (index `line`), a line runs along k; 1: the reverse.
+struct Operand {
+    int mn_major;
+    int pair;             // two neighbouring elements of a line are one aligned load
+    int s_mn, s_k;        // element strides of the row/column index and of k (matmul)
+};
+
+struct GatherParams {
+    Problem p;
+    Operand a, b;
+    int num_kb;           // k-blocks of the whole reduction
+    int num_n_tiles, num_tiles;
+    int splits;           // CTAs of a cluster that share a tile's reduction
+    int wait_prior;
+};
+
+template <int BN, bool F32>
+struct Cfg {
+    static constexpr int PARTS = F32 ? 3 : 1;
+    static constexpr int A_BYTES = BM * 128, B_BYTES = BN * 128;          // one part of a tile
+    static constexpr int STAGE_BYTES = PARTS * (A_BYTES + B_BYTES);
+    static constexpr int STAGES = F32 ? 2 : 4;
+    static constexpr int PROMOTE = F32 ? 1 : 4;                           // k-blocks between additions to the running sum
+    static constexpr int RING_BYTES = STAGES * STAGE_BYTES;
+    static constexpr int STAGING_BYTES = 4 * 4096;                        // one 32 x 32 block per write-back warp
+    static constexpr int SMEM_BYTES = RING_BYTES + STAGING_BYTES + 1024 + 256;
+    static constexpr int TMEM_COLS = BN == 64 ? 256 : 512;                // two accumulators and the running sum
+    static_assert(RING_BYTES >= BM * BN * 4, "a split reduction parks the tile's partial sums in the ring");
+    static_assert(SMEM_BYTES <= 232448, "shared memory");
+};
+
+__device__ __forceinline__ void row_offsets(const Problem &p, int m, int &in_off, int64_t &out_off) {
+    const int hw = p.Ho * p.Wo;
+    const int n = m / hw, r = m - n * hw;
+    const int h = r / p.Wo, w = r - h * p.Wo;
+    in_off = (int)((int64_t)n * p.i_n + (int64_t)h * p.sh * p.i_h + (int64_t)w * p.sw * p.i_w);
+    out_off = (int64_t)n * p.o_n + (int64_t)h * p.o_h + (int64_t)w * p.o_w;
+}
+__device__ __forceinline__ void k_offsets(const Problem &p, int k, int &in_off, int &flt_off) {
+    const int kwc = p.KW * p.C;
+    const int kh = k / kwc, r = k - kh * kwc;
+    const int kw = r / p.C, c = r - kw * p.C;
+    in_off = (int)((int64_t)kh * p.dh * p.i_h + (int64_t)kw * p.dw * p.i_w + (int64_t)c * p.i_c);
+    flt_off = (int)((int64_t)kh * p.k_kh + (int64_t)kw * p.k_kw + (int64_t)c * p.k_c);
+}
+
+__device__ __forceinline__ float widen(const float *p) { return *p; }
+__device__ __forceinline__ float widen(const unsigned short *p) { return __uint_as_float((uint32_t)*p << 16); }
+
+// Predicated loads without a branch: `r` keeps its value (0) where `ok` is false, and a run of them is issued back to back.
+__device__ __forceinline__ void load1_if(bool ok, const float *p, uint32_t &r) {
+    asm("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\t@q ld.global.nc.u32 %0, [%1];\n\t}" : "+r"(r) : "l"(p), "r"((uint32_t)ok));
+}
+__device__ __forceinline__ void load1_if(bool ok, const unsigned short *p, uint32_t &r) {
+    asm("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\t@q ld.global.nc.u16 %0, [%1];\n\t}" : "+r"(r) : "l"(p), "r"((uint32_t)ok));
+}
+// Two neighbouring elements at an aligned address (bf16: both in r[0]).
+__device__ __forceinline__ void load2_if(bool ok, const float *p, uint32_t (&r)[2]) {
+    asm("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %3, 0;\n\t@q ld.global.nc.v2.u32 {%0, %1}, [%2];\n\t}" : "+r"(r[0]), "+r"(r[1]) : "l"(p), "r"((uint32_t)ok));
+}
+__device__ __forceinline__ void load2_if(bool ok, const unsigned short *p, uint32_t (&r)[2]) {
+    asm("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\t@q ld.global.nc.u32 %0, [%1];\n\t}" : "+r"(r[0]) : "l"(p), "r"((uint32_t)ok));
+}
+__device__ __forceinline__ void sts32(uint32_t addr, uint32_t v) { asm volatile("st.shared.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory"); }
+
+// The lanes' two elements of one line -> the line's word of every part tile.  Returns whether an f32 value is infinite or
+// so large that rounding it to bf16 could overflow.
+template <bool F32>
+__device__ __forceinline__ bool store_pair(uint32_t addr, uint32_t part_bytes, const uint32_t (&r)[2]) {
+    if constexpr (!F32) {
+        sts32(addr, r[0] | (r[1] << 16));        // (a pair loaded at once is in r[0] already)
+        return false;
+    } else {
+        const float x = __uint_as_float(r[0]), y = __uint_as_float(r[1]);
+        const uint32_t w0 = pack_bf16(x, y);
+        const float x1 = x - __uint_as_float(w0 << 16), y1 = y - __uint_as_float(w0 & 0xFFFF0000u);
+        const uint32_t w1 = pack_bf16(x1, y1);
+        const float x2 = x1 - __uint_as_float(w1 << 16), y2 = y1 - __uint_as_float(w1 & 0xFFFF0000u);
+        sts32(addr, w0);
+        sts32(addr + part_bytes, w1);
+        sts32(addr + 2 * part_bytes, pack_bf16(x2, y2));
+        return fmaxf(fabsf(x), fabsf(y)) >= 1.7014118e38f;
+    }
+}
+
+// Eight lines of a warp (line0, line0 + 8, ...) of one 64-line batch: `off(i)` is the element offset of line i (negative: no
+// such line), l0 / l1 the lane's two element offsets within a line (ok0 / ok1: whether they exist; the same when `pair`).
+template <typename T, typename LineOff>
+__device__ __forceinline__ void load_lines(uint32_t (&r)[8][2], const T *base, int pair, int l0, int l1, bool ok0, bool ok1, LineOff off) {
+    if (pair) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int o = off(i);
+            r[i][0] = 0; r[i][1] = 0;
+            load2_if(o >= 0 && ok0, base + (int64_t)(o + l0), r[i]);
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int o = off(i);
+            r[i][0] = 0; r[i][1] = 0;
+            load1_if(o >= 0 && ok0, base + (int64_t)(o + l0), r[i][0]);
+            load1_if(o >= 0 && ok1, base + (int64_t)(o + l1), r[i][1]);
+        }
+    }
+}
+
+// This lane's column of eight output rows: out[ro[x]] (+)= act(v[x] + bias) for x < rows.
+__device__ __forceinline__ void write_rows(float *out, const float (&v)[8], const int64_t (&ro)[8], int rows, float bias, int act, int accumulate) {
+    float old[8];
+#pragma unroll
+    for (int x = 0; x < 8; ++x) old[x] = 0.f;
+    if (accumulate)
+#pragma unroll
+        for (int x = 0; x < 8; ++x) if (x < rows) old[x] = out[ro[x]];
+#pragma unroll
+    for (int x = 0; x < 8; ++x) {
+        float r = v[x] + bias;
+        if (act == SG_ACT_RELU && r < 0.f) r = 0.f;
+        if (x < rows) out[ro[x]] = old[x] + r;
+    }
+}
+
+// CONV: the operand addresses come from the (n, h, w) / (kh, kw, c) decomposition (input K-major, filter N-major); else a
+// matmul with linear addresses in either orientation.
+template <int BN, bool F32, bool CONV>
+__global__ void __launch_bounds__(THREADS, 1)
+gather_gemm_kernel(const __grid_constant__ GatherParams gp, const void *__restrict__ in_ptr, const void *__restrict__ flt_ptr, float *__restrict__ O) {
+    using C = Cfg<BN, F32>;
+    using T = typename std::conditional<F32, float, unsigned short>::type;
+    const Problem &p = gp.p;
+    const T *In = static_cast<const T *>(in_ptr), *Flt = static_cast<const T *>(flt_ptr);
+    extern __shared__ uint8_t smem_raw[];
+    const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    uint8_t *smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
+    const uint32_t staging_addr = smem_base + C::RING_BYTES;
+    const uint32_t bars = staging_addr + C::STAGING_BYTES;
+    uint8_t *bars_gen = smem_gen + C::RING_BYTES + C::STAGING_BYTES;
+    // barrier block: full[4] | empty[4] | acc_full[2] | acc_empty[2] | tmem_ptr | abort | large
+    auto full_bar = [&](int s) { return bars + 8u * s; };
+    auto empty_bar = [&](int s) { return bars + 8u * (4 + s); };
+    auto acc_full_bar = [&](int b) { return bars + 8u * (8 + b); };
+    auto acc_empty_bar = [&](int b) { return bars + 8u * (10 + b); };
+    volatile uint32_t *tmem_ptr_slot = reinterpret_cast<volatile uint32_t *>(bars_gen + 96);
+    volatile int *abort_flag = reinterpret_cast<volatile int *>(bars_gen + 100);
+    volatile int *large_flag = reinterpret_cast<volatile int *>(bars_gen + 104);
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    asm volatile("griddepcontrol.launch_dependents;");
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < C::STAGES; ++s) { mbar_init(full_bar(s), GROUP_WARPS); mbar_init(empty_bar(s), 1); }
+        for (int b = 0; b < 2; ++b) { mbar_init(acc_full_bar(b), 1); mbar_init(acc_empty_bar(b), 4); }
+        *abort_flag = 0;
+        *large_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == MMA_WARP) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                     ::"r"(smem_u32(const_cast<uint32_t *>(tmem_ptr_slot))), "r"((uint32_t)C::TMEM_COLS) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_ptr_slot;
+    const uint32_t sum_tmem = tmem_base + 2 * BN;
+
+    // splits == 1: tiles are dealt round-robin to the CTAs.  splits > 1: one tile per cluster, the CTA of rank r reduces
+    // k-blocks [r / splits, (r + 1) / splits) of the whole (never none: there are at least as many k-blocks as ranks).
+    const int rank = gp.splits > 1 ? (int)cluster_ctarank() : 0;
+    const int first_tile = (int)blockIdx.x / gp.splits, tile_step = gp.splits > 1 ? gp.num_tiles : (int)gridDim.x;
+    const int kb0 = (int)((int64_t)rank * gp.num_kb / gp.splits), kb1 = (int)((int64_t)(rank + 1) * gp.num_kb / gp.splits);
+
+    if (warp < MMA_WARP) {
+        // ------------------------------------------------------------ producers
+        if (gp.wait_prior) asm volatile("griddepcontrol.wait;" ::: "memory");
+        const int group = warp / GROUP_WARPS, w = warp % GROUP_WARPS;
+        // this lane's word of line j*64 + w + 8*i: (j*64 + w)*128 + i*1024, 16-byte chunk lane/4 swizzled by the line's low bits (= w)
+        const uint32_t lane_off = (uint32_t)(w * 128 + (((lane >> 2) ^ w) << 4) + (lane & 3) * 4);
+        int it = 0;
+        bool ok = true;
+        for (int tile = first_tile; ok && tile < gp.num_tiles; tile += tile_step) {
+            const int mt = tile / gp.num_n_tiles;
+            const int m0 = mt * BM, n0 = (tile - mt * gp.num_n_tiles) * BN;
+            int row_off = 0;          // CONV: lane i < 16 holds the input offset of row w + 8*i of the tile (-1: beyond M)
+            if constexpr (CONV) {
+                const int m = m0 + w + 8 * (lane & 15);
+                int64_t unused;
+                if (m < p.M) row_offsets(p, m, row_off, unused);
+                else row_off = -1;
+            }
+            for (int kb = kb0; kb < kb1; ++kb, ++it) {
+                if (it % GROUPS != group) continue;
+                const int k0 = kb * BK;
+                uint32_t ra[2][8][2], rb[BN / 64][8][2];
+                if constexpr (CONV) {
+                    // input, K-major: lines are rows, the lane's two k; filter, N-major: lines are k
+                    const int k = k0 + 2 * lane;
+                    int i0 = 0, i1 = 0, f_off = -1, unused;
+                    if (k < p.K) k_offsets(p, k, i0, unused);
+                    if (k + 1 < p.K) k_offsets(p, k + 1, i1, unused);
+                    if (k0 + w + 8 * (lane & 7) < p.K) k_offsets(p, k0 + w + 8 * (lane & 7), unused, f_off);
+#pragma unroll
+                    for (int j = 0; j < 2; ++j)
+                        load_lines(ra[j], In, gp.a.pair, i0, i1, k < p.K, k + 1 < p.K,
+                                   [&](int i) { return __shfl_sync(0xffffffffu, row_off, 8 * j + i); });
+#pragma unroll
+                    for (int j = 0; j < BN / 64; ++j) {
+                        const int n = n0 + j * 64 + 2 * lane;
+                        load_lines(rb[j], Flt, gp.b.pair, n * gp.b.s_mn, (n + 1) * gp.b.s_mn, n < p.N, n + 1 < p.N,
+                                   [&](int i) { return __shfl_sync(0xffffffffu, f_off, i); });
+                    }
+                } else {
+                    auto load_operand = [&](auto &r, const T *base, const Operand &op, int mn0, int mn_end) {
+                        constexpr int BATCHES = sizeof(r) / sizeof(r[0]);
+#pragma unroll
+                        for (int j = 0; j < BATCHES; ++j) {
+                            const int line0 = (op.mn_major ? k0 : mn0 + j * 64) + w, lines = op.mn_major ? p.K : mn_end;
+                            const int e = (op.mn_major ? mn0 + j * 64 : k0) + 2 * lane, es = op.mn_major ? mn_end : p.K;
+                            const int s_line = op.mn_major ? op.s_k : op.s_mn, s_e = op.mn_major ? op.s_mn : op.s_k;
+                            load_lines(r[j], base, op.pair, e * s_e, (e + 1) * s_e, e < es, e + 1 < es,
+                                       [&](int i) { return line0 + 8 * i < lines ? (line0 + 8 * i) * s_line : -1; });
+                        }
+                    };
+                    load_operand(ra, In, gp.a, m0, p.M);
+                    load_operand(rb, Flt, gp.b, n0, p.N);
+                }
+                const int s = it % C::STAGES;
+                if (!mbar_wait(empty_bar(s), ((it / C::STAGES) & 1) ^ 1u, abort_flag)) { ok = false; break; }
+                const uint32_t a_dst = smem_base + s * C::STAGE_BYTES + lane_off, b_dst = a_dst + C::PARTS * C::A_BYTES;
+                bool large = false;
+#pragma unroll
+                for (int j = 0; j < 2; ++j)
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) large |= store_pair<F32>(a_dst + j * 8192 + i * 1024, C::A_BYTES, ra[j][i]);
+#pragma unroll
+                for (int j = 0; j < BN / 64; ++j)
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) large |= store_pair<F32>(b_dst + j * 8192 + i * 1024, C::B_BYTES, rb[j][i]);
+                if (F32 && large) *large_flag = 1;
+                fence_async_smem();       // generic-proxy writes -> visible to the tensor core's reads
+                __syncwarp();
+                if (lane == 0) mbar_arrive(full_bar(s));
+            }
+        }
+    } else if (warp == MMA_WARP) {
+        // ------------------------------------------------------------ MMA issuer: the whole warp walks, one lane issues
+        const uint32_t idesc = make_idesc(BN, BM, false, false, false) | (gp.a.mn_major ? 1u << 15 : 0u) | (gp.b.mn_major ? 1u << 16 : 0u);
+        const int a_step = gp.a.mn_major ? 128 : 2, b_step = gp.b.mn_major ? 128 : 2;      // 16 k: 16 lines or 32 bytes of a line
+        const uint32_t a_lbo = gp.a.mn_major ? 8192 : 16, b_lbo = gp.b.mn_major ? 8192 : 16;
+        const bool issuer = elect_one();
+        auto wait_all = [&](bool passed) { return __all_sync(0xffffffffu, passed) != 0; };
+        int it = 0, chunk = 0;
+        bool ok = true;
+        for (int tile = first_tile; ok && tile < gp.num_tiles; tile += tile_step) {
+            for (int kb = kb0; kb < kb1 && ok; kb += C::PROMOTE, ++chunk) {
+                const int buf = chunk & 1;
+                if (!wait_all(mbar_wait(acc_empty_bar(buf), ((chunk >> 1) & 1) ^ 1u, abort_flag))) { ok = false; break; }
+                tc_fence_after();
+                const uint32_t d = tmem_base + buf * BN;
+                uint32_t acc = 0;
+                for (int kk = kb; kk < min(kb1, kb + C::PROMOTE); ++kk, ++it) {
+                    const int s = it % C::STAGES;
+                    if (!wait_all(mbar_wait(full_bar(s), (it / C::STAGES) & 1, abort_flag))) { ok = false; break; }
+                    tc_fence_after();
+                    const uint32_t a_addr = smem_base + s * C::STAGE_BYTES, b_addr = a_addr + C::PARTS * C::A_BYTES;
+                    if (issuer) {
+                        constexpr int PA[6] = {2, 0, 1, 1, 0, 0}, PB[6] = {0, 2, 1, 0, 1, 0};     // smallest products first
+#pragma unroll
+                        for (int q = F32 ? 0 : 5; q < 6; ++q) {
+                            const uint64_t ad = make_smem_desc(a_addr + PA[q] * C::A_BYTES, a_lbo, 1024);
+                            const uint64_t bd = make_smem_desc(b_addr + PB[q] * C::B_BYTES, b_lbo, 1024);
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) {
+                                umma_bf16(d, ad + (uint64_t)(k * a_step), bd + (uint64_t)(k * b_step), idesc, acc);
+                                acc = 1u;
+                            }
+                        }
+                        umma_commit(empty_bar(s));
+                    }
+                    acc = 1u;
+                }
+                if (ok && issuer) umma_commit(acc_full_bar(buf));
+            }
+        }
+    } else {
+        // ------------------------------------------------------------ write-back
+        const int q = warp & 3;                        // TMEM lane quarter this warp may access
+        const uint32_t stage = staging_addr + (uint32_t)(warp - EPI_WARP) * 4096u;
+        const uint32_t lane_tmem = (uint32_t)(q * 32) << 16;
+        int chunk = 0;
+        bool ok = true;
+        if (gp.wait_prior) asm volatile("griddepcontrol.wait;" ::: "memory");
+        for (int tile = first_tile; ok && tile < gp.num_tiles; tile += tile_step) {
+            const int mt = tile / gp.num_n_tiles;
+            const int m0 = mt * BM, n0 = (tile - mt * gp.num_n_tiles) * BN;
+            const int cols = min(BN, p.N - n0);
+            for (int kb = kb0; kb < kb1; kb += C::PROMOTE, ++chunk) {
+                const int buf = chunk & 1;
+                const bool first = kb == kb0, last = kb + C::PROMOTE >= kb1;
+                if (!epilogue_all(mbar_wait(acc_full_bar(buf), (chunk >> 1) & 1, abort_flag))) { ok = false; break; }
+                tc_fence_after();
+                for (int j = 0; j * 32 < cols; ++j) {
+                    uint32_t r[32];
+                    tmem_ld_32x32(tmem_base + lane_tmem + (uint32_t)(buf * BN + j * 32), r);
+                    if (!first) {
+                        uint32_t s[32];
+                        tmem_ld_32x32(sum_tmem + lane_tmem + (uint32_t)(j * 32), s);
+                        tmem_ld_wait();
+#pragma unroll
+                        for (int c = 0; c < 32; ++c) r[c] = __float_as_uint(__uint_as_float(s[c]) + __uint_as_float(r[c]));
+                    } else {
+                        tmem_ld_wait();
+                    }
+                    if (!last) {
+                        tmem_st_32x32(sum_tmem + lane_tmem + (uint32_t)(j * 32), r);
+                        continue;
+                    }
+                    if (F32 && *large_flag) {
+                        // infinities (or values next to overflow) among the operands: their products with the zeros of the
+                        // split would be NaN, so this tile is summed as it stands (lane = row)
+                        const int m = m0 + q * 32 + lane;
+                        int64_t unused;
+                        int ro = 0;
+                        if (m < p.M) row_offsets(p, m, ro, unused);
+                        for (int c = 0; c < 32; ++c) {
+                            float acc = 0.f;
+                            const int n = n0 + j * 32 + c;
+                            if (m < p.M && n < p.N)
+                                for (int k = kb0 * BK; k < min(p.K, kb1 * BK); ++k) {
+                                    int io, fo;
+                                    k_offsets(p, k, io, fo);
+                                    acc = fmaf(widen(In + ro + io), widen(Flt + fo + (int64_t)n * p.k_f), acc);
+                                }
+                            // (r is indexed by compile-time constants only: select)
+#pragma unroll
+                            for (int e = 0; e < 32; ++e) if (e == c) r[e] = __float_as_uint(acc);
+                        }
+                    }
+                    // lane = row: 16-byte chunks of this row, chunk c of row x at chunk c ^ (x & 7); a split reduction parks
+                    // the whole tile in the ring instead ([column block of 32][row][128 bytes])
+                    const uint32_t dst = gp.splits > 1 ? smem_base + (uint32_t)(j * BM + q * 32) * 128u : stage;
+                    if (gp.splits == 1) __syncwarp();
+#pragma unroll
+                    for (int c = 0; c < 8; ++c)
+                        asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(dst + (uint32_t)(lane * 128 + ((c ^ (lane & 7)) << 4))),
+                                     "r"(r[4 * c]), "r"(r[4 * c + 1]), "r"(r[4 * c + 2]), "r"(r[4 * c + 3]) : "memory");
+                    if (gp.splits > 1) continue;
+                    __syncwarp();
+                    // lane = column: one row of 32 columns per store
+                    const int n = n0 + j * 32 + lane;
+                    const float bias = (p.bias != nullptr && n < p.N) ? __ldg(p.bias + (int64_t)n * p.bias_f) : 0.f;
+                    const int m_first = m0 + q * 32;
+                    int64_t my_out = 0;                // CONV: lane i holds the output offset of row i
+                    if constexpr (CONV) {
+                        int unused;
+                        if (m_first + lane < p.M) row_offsets(p, m_first + lane, unused, my_out);
+                    }
+                    const int rows = n < p.N ? p.M - m_first : 0;
+                    float *out = O + (CONV ? 0 : (int64_t)m_first * p.o_w) + (int64_t)n * p.o_f;
+#pragma unroll
+                    for (int x0 = 0; x0 < 32; x0 += 8) {
+                        float v[8];
+                        int64_t ro[8];
+#pragma unroll
+                        for (int x = 0; x < 8; ++x) {
+                            asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v[x])
+                                         : "r"(stage + (uint32_t)((x0 + x) * 128 + (((lane >> 2) ^ x) << 4) + (lane & 3) * 4)) : "memory");
+                            ro[x] = CONV ? __shfl_sync(0xffffffffu, my_out, x0 + x) : (int64_t)(x0 + x) * p.o_w;
+                        }
+                        write_rows(out, v, ro, rows - x0, bias, p.act, p.accumulate);
+                    }
+                }
+                if (!last) asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(acc_empty_bar(buf));
+            }
+        }
+    }
+
+    // ---------------------------------------------------------------- split reduction and teardown
+    __syncthreads();
+    if (gp.splits > 1) {
+        // every CTA of the cluster sums its share of the tile's rows over the partial tiles parked in all of them, in rank order
+        cluster_sync_all();
+        const int mt = first_tile / gp.num_n_tiles;
+        const int m0 = mt * BM, n0 = (first_tile - mt * gp.num_n_tiles) * BN;
+        const int rows = BM / gp.splits, cols = min(BN, p.N - n0);
+        if (!*abort_flag)
+            for (int u = warp; u < rows * (BN / 32); u += THREADS / 32) {
+                const int j = u / rows, x = rank * rows + (u - j * rows), m = m0 + x;
+                if (j * 32 >= cols || m >= p.M) continue;
+                const uint32_t src = smem_base + (uint32_t)((j * BM + x) * 128 + (((lane >> 2) ^ (x & 7)) << 4) + (lane & 3) * 4);
+                float part[MAX_SPLIT];
+#pragma unroll
+                for (int r = 0; r < MAX_SPLIT; ++r)
+                    if (r < gp.splits) asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(part[r]) : "r"(map_to_cta(src, r)) : "memory");
+                float v = part[0];
+#pragma unroll
+                for (int r = 1; r < MAX_SPLIT; ++r)
+                    if (r < gp.splits) v += part[r];
+                const int n = n0 + j * 32 + lane;
+                if (n < p.N) {
+                    int unused;
+                    int64_t ro = (int64_t)m * p.o_w;
+                    if constexpr (CONV) row_offsets(p, m, unused, ro);
+                    float *o = O + ro + (int64_t)n * p.o_f;
+                    if (p.bias != nullptr) v += __ldg(p.bias + (int64_t)n * p.bias_f);
+                    if (p.act == SG_ACT_RELU && v < 0.f) v = 0.f;
+                    *o = p.accumulate ? *o + v : v;
+                }
+            }
+        cluster_sync_all();      // nobody leaves while its partial tile is being read
+    }
+    if (warp == MMA_WARP) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)C::TMEM_COLS) : "memory");
+    }
+}
+
+// Largest element offset of an operand's rectangle (strides are not negative), or -1 when it does not fit 31 bits.
+inline int64_t reach(std::initializer_list<std::pair<int64_t, int64_t>> extents_strides) {
+    int64_t r = 0;
+    for (const auto &e : extents_strides) {
+        if (e.first > 1 && e.second > 0x7fffffff) return -1;
+        r += (e.first - 1) * e.second;
+        if (r > 0x7fffff00) return -1;
+    }
+    return r;
+}
+
+template <int BN, bool F32, bool CONV>
+sg_status launch_variant(const GatherParams &gp, const void *In, const void *Flt, float *O, int num_sms, int slot, cudaStream_t stream) {
+    using C = Cfg<BN, F32>;
+    const void *fn = reinterpret_cast<const void *>(gather_gemm_kernel<BN, F32, CONV>);
+    if (!tensor_ensure_smem_attr(slot, fn, C::SMEM_BYTES)) return SG_ERR_CUDA;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(gp.splits > 1 ? gp.num_tiles * gp.splits : std::min(gp.num_tiles, num_sms), 1, 1);
+    cfg.blockDim = dim3(THREADS, 1, 1);
+    cfg.dynamicSmemBytes = C::SMEM_BYTES;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = gp.splits;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = gp.wait_prior ? 2 : 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, gather_gemm_kernel<BN, F32, CONV>, gp, In, Flt, O);
+    count_launch();
+    note_kernel(F32 ? "gather_gemm_kernel<f32>" : "gather_gemm_kernel<bf16>");
+    return e == cudaSuccess ? SG_OK : SG_ERR_CUDA;
+}
+
+}  // namespace
+
+sg_status launch_gather(const Problem &p, const void *In, const void *Flt, float *O, bool forced, cudaStream_t stream) {
+    // Below 2^21 multiply-adds the CUDA-core kernel is as fast.
+    if (!forced && (int64_t)p.M * p.N * p.K < ((int64_t)1 << 21)) return SG_ERR_UNSUPPORTED;
+    const bool conv = p.spatial_rank != 0;
+    // offsets are 32-bit
+    if (reach({{p.batch, p.i_n}, {(int64_t)(p.Ho - 1) * p.sh + (int64_t)(p.KH - 1) * p.dh + 1, p.i_h},
+               {(int64_t)(p.Wo - 1) * p.sw + (int64_t)(p.KW - 1) * p.dw + 1, p.i_w}, {p.C, p.i_c}}) < 0 ||
+        reach({{p.KH, p.k_kh}, {p.KW, p.k_kw}, {p.C, p.k_c}, {p.N, p.k_f}}) < 0) return SG_ERR_UNSUPPORTED;
+    // (the lanes compute the offsets of a tile's rows and columns beyond M, N and K too, unused but in 32 bits)
+    if ((int64_t)(p.N + 256) * p.k_f > 0x7fffffff || (int64_t)(p.C + 128) * std::max(p.i_c, p.k_c) > 0x7fffffff ||
+        (!conv && (int64_t)(p.M + 256) * p.i_w > 0x7fffffff)) return SG_ERR_UNSUPPORTED;
+    int dev = 0, num_sms = 0, pdl = -1, unused = 0;
+    if (!tensor_device_info(&dev, &num_sms, &pdl, &unused)) return SG_ERR_CUDA;
+
+    GatherParams gp{};
+    gp.p = p;
+    const int es = p.in_bf16 ? 2 : 4;
+    auto even = [](int64_t v) { return v % 2 == 0; };
+    auto aligned = [&](const void *ptr) { return reinterpret_cast<uintptr_t>(ptr) % (2 * es) == 0; };
+    // a line runs along whichever index is contiguous; pairs are single loads when every line starts on a multiple of two
+    // elements and ends on one
+    gp.a.mn_major = !conv && p.i_c != 1 && p.i_w == 1;
+    gp.a.s_mn = (int)p.i_w; gp.a.s_k = (int)p.i_c;
+    gp.a.pair = aligned(In) && (gp.a.mn_major ? even(p.i_c) && even(p.M)
+                                              : p.i_c == 1 && even(p.i_w) && even(p.K) && (!conv || (even(p.C) && even(p.i_h) && even(p.i_n))));
+    gp.b.mn_major = conv || p.k_f == 1 || p.k_c != 1;
+    gp.b.s_mn = (int)p.k_f; gp.b.s_k = (int)p.k_c;
+    gp.b.pair = aligned(Flt) && (gp.b.mn_major ? p.k_f == 1 && even(p.k_c) && even(p.N) && (!conv || (even(p.k_kw) && even(p.k_kh))) : even(p.k_f) && even(p.K));
+    gp.num_kb = (p.K + BK - 1) / BK;
+    gp.wait_prior = pdl == 0 ? 0 : 1;
+
+    const int bn = p.N > 64 ? 128 : 64;
+    gp.num_n_tiles = (p.N + bn - 1) / bn;
+    const int64_t tiles = (int64_t)((p.M + BM - 1) / BM) * gp.num_n_tiles;
+    if (tiles > 0x7fffffff / MAX_SPLIT) return SG_ERR_UNSUPPORTED;
+    gp.num_tiles = (int)tiles;
+    // few tiles: a cluster of 2, 4 or 8 CTAs shares a tile's reduction, at least four k-blocks each
+    gp.splits = 1;
+    while (gp.splits < MAX_SPLIT && tiles * gp.splits * 2 <= num_sms - 12 && gp.num_kb >= gp.splits * 8) gp.splits *= 2;
+#define SG_GATHER(BN_, F32_, CONV_, SLOT) launch_variant<BN_, F32_, CONV_>(gp, In, Flt, O, num_sms, SLOT, stream)
+    if (p.in_bf16) {
+        if (conv) return bn == 64 ? SG_GATHER(64, false, true, 149) : SG_GATHER(128, false, true, 150);
+        return bn == 64 ? SG_GATHER(64, false, false, 151) : SG_GATHER(128, false, false, 152);
+    }
+    if (conv) return bn == 64 ? SG_GATHER(64, true, true, 153) : SG_GATHER(128, true, true, 154);
+    return bn == 64 ? SG_GATHER(64, true, false, 155) : SG_GATHER(128, true, false, 156);
+#undef SG_GATHER
+}
+
+sg_status gather_read_status(cudaStream_t stream) { return read_status_word(stream); }
+
+}  // namespace sg

@@ -63,6 +63,10 @@ bool tensor_encode_tiled(CUtensorMap *map, CUtensorMapDataType type, int rank, v
 // shape or layout does not qualify (nothing is launched then).
 sg_status launch_conv_strip(const Problem &p, const void *In, const void *Flt, float *O, cudaStream_t stream);
 sg_status conv_read_status(cudaStream_t stream);
+// Tensor-core implicit GEMM for layouts outside the TMA rules (sg_gather.cu): any strides.  SG_ERR_UNSUPPORTED (nothing is
+// launched) when offsets do not fit 32 bits or, unless `forced`, the problem is too small to gain.
+sg_status launch_gather(const Problem &p, const void *In, const void *Flt, float *O, bool forced, cudaStream_t stream);
+sg_status gather_read_status(cudaStream_t stream);
 void tensor_set_tile_override(int bn, int cg, int splits);
 void tensor_last_choice(int out[3]);
 void tensor_map_cache_stats(long long out[2]);     // {hits, misses} since the library was loaded

@@ -1347,7 +1347,8 @@ sg_status tensor_read_status(cudaStream_t stream) {
     const sg_status b = conv_read_status(stream);
     const sg_status c = bandwidth_read_status(stream);
     const sg_status d = depthwise_read_status(stream);
-    return a != SG_OK ? a : (b != SG_OK ? b : (c != SG_OK ? c : d));
+    const sg_status e = gather_read_status(stream);
+    return a != SG_OK ? a : (b != SG_OK ? b : (c != SG_OK ? c : (d != SG_OK ? d : e)));
 }
 
 cudaError_t launch_wait_timeout_selftest(long long budget_cycles, cudaStream_t stream) {

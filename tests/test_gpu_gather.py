@@ -1,0 +1,117 @@
+"""The tensor-core kernel for layouts outside the TMA rules against the oracle: every operand orientation, sizes around its
+tiles (128 rows, 64 / 128 columns, k-blocks of 64, partial sums of 256), split reductions, f32 precision."""
+import numpy as np
+import pytest
+import torch
+
+from helpers import assert_within_bound, operand
+from oracle import ref
+from paper_2202_03293_b200 import binding as sg
+
+pytestmark = pytest.mark.gpu
+SEED = 9100
+
+
+@pytest.fixture(autouse=True)
+def _forced_tensor_family():
+    sg.sg_set_kernel_override(sg.SG_KERNEL_TENSOR)
+    yield
+    sg.sg_set_kernel_override(sg.SG_KERNEL_AUTO)
+    sg.sg_check()
+
+
+def product(M, N, K, dtype, a_t=False, b_t=False, accumulate=False, dist="uniform", pad=0, bias=None, act=0):
+    A, a = operand((K, M + pad) if a_t else (M, K + pad), SEED, 1, dist, dtype)
+    B, b = operand((N, K + pad) if b_t else (K, N + pad), SEED, 2, dist, dtype)
+    A, a = (A[:, :M].t(), a[:, :M].T) if a_t else (A[:, :K], a[:, :K])
+    B, b = (B[:, :K].t(), b[:, :K].T) if b_t else (B[:, :N], b[:, :N])
+    wide = torch.full((M, N + 3), float("nan"), device="cuda")
+    C, c0 = wide[:, :N], None
+    if accumulate:
+        C0, c0 = operand((M, N), SEED, 3, "uniform", "f32")
+        C.copy_(C0)
+    if bias is not None:
+        sg.sg_matmul_bias_act(A, B, bias, C, act)
+    else:
+        sg.sg_matmul(A, B, C, sg.SG_ACCUMULATE if accumulate else sg.SG_OVERWRITE)
+    torch.cuda.synchronize()
+    assert sg.sg_last_kernel_name() == f"gather_gemm_kernel<{dtype}>"
+    assert torch.isnan(wide[:, N:]).all()            # nothing outside the view is written
+    want, S = ref.matmul(np.ascontiguousarray(a), np.ascontiguousarray(b), C_in=c0)
+    return C, want, S + (np.abs(c0) if accumulate else 0.0)
+
+
+# tile edges and remainders in every extent; 1 and 2 column tiles; one to many k-blocks and partial sums; 1 to 8 CTAs a tile
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("M,N,K", [(1, 1, 1), (127, 63, 65), (129, 65, 63), (128, 129, 257), (257, 131, 512), (130, 67, 1100), (40, 30, 4099),
+                                   (1531, 1021, 765)])
+def test_matmul_odd_sizes(M, N, K, dtype):
+    C, want, S = product(M, N, K, dtype)
+    # the accuracy of the CUDA-core kernel that these layouts used to run on
+    assert assert_within_bound(C, want, S, "odd sizes") < 1e-6
+
+
+# one load per pair of elements (even pitches) and single loads, each operand stored either way
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("a_t,b_t", [(False, False), (True, False), (False, True), (True, True)])
+@pytest.mark.parametrize("pad,M,N,K", [(1, 200, 138, 330), (0, 201, 139, 331), (3, 130, 70, 77)])
+def test_matmul_orientations(a_t, b_t, pad, M, N, K, dtype):
+    C, want, S = product(M, N, K, dtype, a_t, b_t, pad=pad)
+    assert assert_within_bound(C, want, S, "orientation") < 1e-6
+    C, want, S = product(M, N, K, dtype, a_t, b_t, accumulate=True, pad=pad, dist="ints")
+    assert_within_bound(C, want, S, "orientation, accumulate")
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("M,N,K", [(131, 57, 43), (129, 131, 700)])
+def test_fused_consumer(M, N, K, dtype):
+    bias_dev, bias = operand((N,), SEED, 4, "normal", "f32")
+    C, want, S = product(M, N, K, dtype, bias=bias_dev, act=sg.SG_ACT_RELU)
+    want = np.maximum(want + bias, 0.0)
+    assert_within_bound(C, want, S + np.abs(bias), "bias + relu")
+
+
+def test_column_major_output_and_non_unit_strides():
+    A, a = operand((150, 210), SEED, 5, "uniform", "f32")
+    B, b = operand((105, 180), SEED, 6, "uniform", "f32")
+    Ct = torch.empty(90, 150, device="cuda")
+    sg.sg_matmul(A[:, ::2], B[:, ::2], Ct.t())
+    torch.cuda.synchronize()
+    assert sg.sg_last_kernel_name() == "gather_gemm_kernel<f32>"
+    want, S = ref.matmul(np.ascontiguousarray(a[:, ::2]), np.ascontiguousarray(b[:, ::2]))
+    assert_within_bound(Ct.t(), want, S, "strided operands, column-major output")
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("N,H,W,C,KH,KW,F,st,dl", [(2, 30, 31, 3, 3, 3, 32, (2, 2), (1, 1)), (1, 9, 20, 3, 7, 7, 70, (1, 2), (1, 1)),
+                                                   (2, 11, 13, 18, 2, 3, 130, (1, 1), (2, 1)), (1, 5, 6, 131, 3, 3, 33, (1, 1), (1, 2))])
+def test_conv2d(N, H, W, C, KH, KW, F, st, dl, dtype):
+    h_in, w_in = (H - 1) * st[0] + (KH - 1) * dl[0] + 1, (W - 1) * st[1] + (KW - 1) * dl[1] + 1
+    I, i = operand((N, h_in, w_in, C), SEED, 7, "normal", dtype)
+    K, k = operand((KH, KW, C, F), SEED, 8, "normal", dtype)
+    O = torch.full((N, H, W, F), float("nan"), device="cuda")
+    sg.sg_conv2d_nhwc_hwcf(I, K, O, st, dl)
+    torch.cuda.synchronize()
+    assert sg.sg_last_kernel_name() == f"gather_gemm_kernel<{dtype}>"
+    want, S = ref.conv2d_nhwc_hwcf(i, k, stride=st, dilation=dl)
+    assert assert_within_bound(O, want, S, "conv2d") < 1e-6
+
+
+def test_infinities_and_values_next_to_overflow_keep_their_meaning():
+    A = torch.ones(130, 67, device="cuda")
+    B = torch.full((67, 33), 0.5, device="cuda")
+    A[3, 5], A[4, 6], A[7, 8] = float("inf"), float("-inf"), float("nan")
+    A[9, 1], B[2, 4] = 3.4e38, 2.0
+    C = torch.empty(130, 33, device="cuda")
+    sg.sg_matmul(A, B, C)
+    want = A.double() @ B.double()
+    assert torch.equal(torch.isnan(C), torch.isnan(want)) and torch.equal(torch.isinf(C), torch.isinf(want))
+    fine = torch.isfinite(want)
+    assert torch.allclose(C[fine].double(), want[fine], rtol=1e-6)
+
+
+def test_selection_by_size():
+    sg.sg_set_kernel_override(sg.SG_KERNEL_AUTO)
+    for M, N, K, name in ((127, 127, 127, "ffma_kernel"), (129, 129, 129, "gather_gemm_kernel<f32>")):
+        sg.sg_matmul(torch.zeros(M, K, device="cuda"), torch.zeros(K, N, device="cuda"), torch.empty(M, N, device="cuda"))
+        assert sg.sg_last_kernel_name() == name

@@ -42,7 +42,7 @@ constexpr int MMA_WARP = GROUPS * GROUP_WARPS, EPI_WARP = MMA_WARP + 1;
 constexpr int THREADS = 32 * (EPI_WARP + 4);
 constexpr int MAX_SPLIT = 8;
 
-// How one operand is fetched.  mn_major 0: lines are rows/columns (index `line`), a line runs along k; 1: the reverse.
+// How one operand is fetched.  mn_major 0: lines are rows/columns (index mn), a line runs along k; 1: the reverse.
 struct Operand {
     int mn_major;
     int pair;             // two neighbouring elements of a line are one aligned load
@@ -55,6 +55,7 @@ struct GatherParams {
     int num_kb;           // k-blocks of the whole reduction
     int num_n_tiles, num_tiles;
     int splits;           // CTAs of a cluster that share a tile's reduction
+    int uniform_rows;     // output row m starts at m * o_w
     int wait_prior;
 };
 
@@ -69,7 +70,7 @@ struct Cfg {
     static constexpr int STAGING_BYTES = 4 * 4096;                        // one 32 x 32 block per write-back warp
     static constexpr int SMEM_BYTES = RING_BYTES + STAGING_BYTES + 1024 + 256;
     static constexpr int TMEM_COLS = BN == 64 ? 256 : 512;                // two accumulators and the running sum
-    static_assert(RING_BYTES >= BM * BN * 4, "a split reduction parks the tile's partial sums in the ring");
+    static_assert(RING_BYTES >= BM * BN * 4 && RING_BYTES >= MMA_WARP * 4096, "a split reduction parks the tile's partial sums in the ring");
     static_assert(SMEM_BYTES <= 232448, "shared memory");
 };
 
@@ -180,20 +181,23 @@ gather_gemm_kernel(const __grid_constant__ GatherParams gp, const void *__restri
     const uint32_t staging_addr = smem_base + C::RING_BYTES;
     const uint32_t bars = staging_addr + C::STAGING_BYTES;
     uint8_t *bars_gen = smem_gen + C::RING_BYTES + C::STAGING_BYTES;
-    // barrier block: full[4] | empty[4] | acc_full[2] | acc_empty[2] | tmem_ptr | abort | large
+    // barrier block: full[4] | empty[4] | acc_full[2] | acc_empty[2] | sum | done | tmem_ptr | abort | large
     auto full_bar = [&](int s) { return bars + 8u * s; };
     auto empty_bar = [&](int s) { return bars + 8u * (4 + s); };
     auto acc_full_bar = [&](int b) { return bars + 8u * (8 + b); };
     auto acc_empty_bar = [&](int b) { return bars + 8u * (10 + b); };
-    volatile uint32_t *tmem_ptr_slot = reinterpret_cast<volatile uint32_t *>(bars_gen + 96);
-    volatile int *abort_flag = reinterpret_cast<volatile int *>(bars_gen + 100);
-    volatile int *large_flag = reinterpret_cast<volatile int *>(bars_gen + 104);
+    const uint32_t sum_bar = bars + 8u * 12, done_bar = bars + 8u * 13;      // completed once: the last tile's running sum, its last MMAs
+    volatile uint32_t *tmem_ptr_slot = reinterpret_cast<volatile uint32_t *>(bars_gen + 112);
+    volatile int *abort_flag = reinterpret_cast<volatile int *>(bars_gen + 116);
+    volatile int *large_flag = reinterpret_cast<volatile int *>(bars_gen + 120);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     asm volatile("griddepcontrol.launch_dependents;");
     if (threadIdx.x == 0) {
         for (int s = 0; s < C::STAGES; ++s) { mbar_init(full_bar(s), GROUP_WARPS); mbar_init(empty_bar(s), 1); }
         for (int b = 0; b < 2; ++b) { mbar_init(acc_full_bar(b), 1); mbar_init(acc_empty_bar(b), 4); }
+        mbar_init(sum_bar, 4);
+        mbar_init(done_bar, 1);
         *abort_flag = 0;
         *large_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -214,6 +218,99 @@ gather_gemm_kernel(const __grid_constant__ GatherParams gp, const void *__restri
     const int rank = gp.splits > 1 ? (int)cluster_ctarank() : 0;
     const int first_tile = (int)blockIdx.x / gp.splits, tile_step = gp.splits > 1 ? gp.num_tiles : (int)gridDim.x;
     const int kb0 = (int)((int64_t)rank * gp.num_kb / gp.splits), kb1 = (int)((int64_t)(rank + 1) * gp.num_kb / gp.splits);
+
+    // One 32-row x 32-column block of a tile: column block j of this warp's TMEM lane quarter, the partial sum in accumulator
+    // `buf` and (not `first`) the running sum.  Adds them up; when it is the `last` partial sum, writes the block out.
+    const int q = warp & 3;                        // TMEM lane quarter this warp may access
+    const uint32_t lane_tmem = (uint32_t)(q * 32) << 16;
+    auto finish_block = [&](int m0, int n0, int j, int buf, bool first, bool last, uint32_t stage) {
+        uint32_t r[32];
+        tmem_ld_32x32(tmem_base + lane_tmem + (uint32_t)(buf * BN + j * 32), r);
+        if (!first) {
+            uint32_t s[32];
+            tmem_ld_32x32(sum_tmem + lane_tmem + (uint32_t)(j * 32), s);
+            tmem_ld_wait();
+#pragma unroll
+            for (int c = 0; c < 32; ++c) r[c] = __float_as_uint(__uint_as_float(s[c]) + __uint_as_float(r[c]));
+        } else {
+            tmem_ld_wait();
+        }
+        if (!last) {
+            tmem_st_32x32(sum_tmem + lane_tmem + (uint32_t)(j * 32), r);
+            return;
+        }
+        if (F32 && *large_flag) {
+            // infinities (or values next to overflow) among the operands: their products with the zeros of the
+            // split would be NaN, so this tile is summed as it stands (lane = row)
+            const int m = m0 + q * 32 + lane;
+            int64_t unused;
+            int ro = 0;
+            if (m < p.M) row_offsets(p, m, ro, unused);
+            for (int c = 0; c < 32; ++c) {
+                float acc = 0.f;
+                const int n = n0 + j * 32 + c;
+                if (m < p.M && n < p.N)
+                    for (int k = kb0 * BK; k < min(p.K, kb1 * BK); ++k) {
+                        int io, fo;
+                        k_offsets(p, k, io, fo);
+                        acc = fmaf(widen(In + ro + io), widen(Flt + fo + (int64_t)n * p.k_f), acc);
+                    }
+                // (r is indexed by compile-time constants only: select)
+#pragma unroll
+                for (int e = 0; e < 32; ++e) if (e == c) r[e] = __float_as_uint(acc);
+            }
+        }
+        // lane = row: 16-byte chunks of this row, chunk c of row x at chunk c ^ (x & 7); a split reduction parks
+        // the whole tile in the ring instead ([column block of 32][row][128 bytes])
+        const uint32_t dst = gp.splits > 1 ? smem_base + (uint32_t)(j * BM + q * 32) * 128u : stage;
+        if (gp.splits == 1) __syncwarp();
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+            asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(dst + (uint32_t)(lane * 128 + ((c ^ (lane & 7)) << 4))),
+                         "r"(r[4 * c]), "r"(r[4 * c + 1]), "r"(r[4 * c + 2]), "r"(r[4 * c + 3]) : "memory");
+        if (gp.splits > 1) return;
+        __syncwarp();
+        // lane = column: one row of 32 columns per store
+        const int n = n0 + j * 32 + lane;
+        const float bias = (p.bias != nullptr && n < p.N) ? __ldg(p.bias + (int64_t)n * p.bias_f) : 0.f;
+        const int m_first = m0 + q * 32;
+        const int rows = n < p.N ? p.M - m_first : 0;
+        float *out = O + (int64_t)n * p.o_f;
+        auto staged = [&](int x) {
+            float v;
+            asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(stage + (uint32_t)(x * 128 + (((lane >> 2) ^ (x & 7)) << 4) + (lane & 3) * 4)) : "memory");
+            return v;
+        };
+        if (gp.uniform_rows && !p.accumulate && m_first + 32 <= p.M) {
+            out += (int64_t)m_first * p.o_w;
+#pragma unroll
+            for (int x0 = 0; x0 < 32; x0 += 16) {
+                float v[16];
+#pragma unroll
+                for (int x = 0; x < 16; ++x) v[x] = staged(x0 + x);
+                if (rows > 0)
+#pragma unroll
+                    for (int x = 0; x < 16; ++x, out += p.o_w) {
+                        const float y = v[x] + bias;
+                        *out = (p.act == SG_ACT_RELU && y < 0.f) ? 0.f : y;
+                    }
+            }
+        } else {
+            int64_t my_out = 0;            // lane i holds the output offset of row i
+            int unused;
+            if (m_first + lane < p.M) row_offsets(p, m_first + lane, unused, my_out);
+            for (int x0 = 0; x0 < 32; x0 += 8) {
+                float v[8];
+                int64_t ro[8];
+#pragma unroll
+                for (int x = 0; x < 8; ++x) {
+                    v[x] = staged(x0 + x);
+                    ro[x] = __shfl_sync(0xffffffffu, my_out, x0 + x);
+                }
+                write_rows(out, v, ro, rows - x0, bias, p.act, p.accumulate);
+            }
+        }
+    };
 
     if (warp < MMA_WARP) {
         // ------------------------------------------------------------ producers
@@ -287,6 +384,17 @@ gather_gemm_kernel(const __grid_constant__ GatherParams gp, const void *__restri
                 if (lane == 0) mbar_arrive(full_bar(s));
             }
         }
+        // ---- a share of the last tile's write-back: column block 1 + warp / 4 (staged in the ring, which has been consumed)
+        const int chunks = (kb1 - kb0 + C::PROMOTE - 1) / C::PROMOTE, tiles = (gp.num_tiles - 1 - first_tile) / tile_step + 1;
+        const int tile = first_tile + (tiles - 1) * tile_step, last = tiles * chunks - 1, j = 1 + (warp >> 2);
+        const int mt = tile / gp.num_n_tiles, n0 = (tile - mt * gp.num_n_tiles) * BN;
+        if (ok && j * 32 < min(BN, p.N - n0)) {
+            ok = mbar_wait(done_bar, 0, abort_flag) && (chunks == 1 || mbar_wait(sum_bar, 0, abort_flag));
+            if (__all_sync(0xffffffffu, ok)) {
+                tc_fence_after();
+                finish_block(mt * BM, n0, j, last & 1, chunks == 1, true, smem_base + (uint32_t)warp * 4096u);
+            }
+        }
     } else if (warp == MMA_WARP) {
         // ------------------------------------------------------------ MMA issuer: the whole warp walks, one lane issues
         const uint32_t idesc = make_idesc(BN, BM, false, false, false) | (gp.a.mn_major ? 1u << 15 : 0u) | (gp.b.mn_major ? 1u << 16 : 0u);
@@ -324,14 +432,15 @@ gather_gemm_kernel(const __grid_constant__ GatherParams gp, const void *__restri
                     }
                     acc = 1u;
                 }
-                if (ok && issuer) umma_commit(acc_full_bar(buf));
+                if (ok && issuer) {
+                    umma_commit(acc_full_bar(buf));
+                    if (kb + C::PROMOTE >= kb1 && tile + tile_step >= gp.num_tiles) umma_commit(done_bar);
+                }
             }
         }
     } else {
         // ------------------------------------------------------------ write-back
-        const int q = warp & 3;                        // TMEM lane quarter this warp may access
         const uint32_t stage = staging_addr + (uint32_t)(warp - EPI_WARP) * 4096u;
-        const uint32_t lane_tmem = (uint32_t)(q * 32) << 16;
         int chunk = 0;
         bool ok = true;
         if (gp.wait_prior) asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -344,81 +453,16 @@ gather_gemm_kernel(const __grid_constant__ GatherParams gp, const void *__restri
                 const bool first = kb == kb0, last = kb + C::PROMOTE >= kb1;
                 if (!epilogue_all(mbar_wait(acc_full_bar(buf), (chunk >> 1) & 1, abort_flag))) { ok = false; break; }
                 tc_fence_after();
-                for (int j = 0; j * 32 < cols; ++j) {
-                    uint32_t r[32];
-                    tmem_ld_32x32(tmem_base + lane_tmem + (uint32_t)(buf * BN + j * 32), r);
-                    if (!first) {
-                        uint32_t s[32];
-                        tmem_ld_32x32(sum_tmem + lane_tmem + (uint32_t)(j * 32), s);
-                        tmem_ld_wait();
-#pragma unroll
-                        for (int c = 0; c < 32; ++c) r[c] = __float_as_uint(__uint_as_float(s[c]) + __uint_as_float(r[c]));
-                    } else {
-                        tmem_ld_wait();
-                    }
-                    if (!last) {
-                        tmem_st_32x32(sum_tmem + lane_tmem + (uint32_t)(j * 32), r);
-                        continue;
-                    }
-                    if (F32 && *large_flag) {
-                        // infinities (or values next to overflow) among the operands: their products with the zeros of the
-                        // split would be NaN, so this tile is summed as it stands (lane = row)
-                        const int m = m0 + q * 32 + lane;
-                        int64_t unused;
-                        int ro = 0;
-                        if (m < p.M) row_offsets(p, m, ro, unused);
-                        for (int c = 0; c < 32; ++c) {
-                            float acc = 0.f;
-                            const int n = n0 + j * 32 + c;
-                            if (m < p.M && n < p.N)
-                                for (int k = kb0 * BK; k < min(p.K, kb1 * BK); ++k) {
-                                    int io, fo;
-                                    k_offsets(p, k, io, fo);
-                                    acc = fmaf(widen(In + ro + io), widen(Flt + fo + (int64_t)n * p.k_f), acc);
-                                }
-                            // (r is indexed by compile-time constants only: select)
-#pragma unroll
-                            for (int e = 0; e < 32; ++e) if (e == c) r[e] = __float_as_uint(acc);
-                        }
-                    }
-                    // lane = row: 16-byte chunks of this row, chunk c of row x at chunk c ^ (x & 7); a split reduction parks
-                    // the whole tile in the ring instead ([column block of 32][row][128 bytes])
-                    const uint32_t dst = gp.splits > 1 ? smem_base + (uint32_t)(j * BM + q * 32) * 128u : stage;
-                    if (gp.splits == 1) __syncwarp();
-#pragma unroll
-                    for (int c = 0; c < 8; ++c)
-                        asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(dst + (uint32_t)(lane * 128 + ((c ^ (lane & 7)) << 4))),
-                                     "r"(r[4 * c]), "r"(r[4 * c + 1]), "r"(r[4 * c + 2]), "r"(r[4 * c + 3]) : "memory");
-                    if (gp.splits > 1) continue;
-                    __syncwarp();
-                    // lane = column: one row of 32 columns per store
-                    const int n = n0 + j * 32 + lane;
-                    const float bias = (p.bias != nullptr && n < p.N) ? __ldg(p.bias + (int64_t)n * p.bias_f) : 0.f;
-                    const int m_first = m0 + q * 32;
-                    int64_t my_out = 0;                // CONV: lane i holds the output offset of row i
-                    if constexpr (CONV) {
-                        int unused;
-                        if (m_first + lane < p.M) row_offsets(p, m_first + lane, unused, my_out);
-                    }
-                    const int rows = n < p.N ? p.M - m_first : 0;
-                    float *out = O + (CONV ? 0 : (int64_t)m_first * p.o_w) + (int64_t)n * p.o_f;
-#pragma unroll
-                    for (int x0 = 0; x0 < 32; x0 += 8) {
-                        float v[8];
-                        int64_t ro[8];
-#pragma unroll
-                        for (int x = 0; x < 8; ++x) {
-                            asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v[x])
-                                         : "r"(stage + (uint32_t)((x0 + x) * 128 + (((lane >> 2) ^ x) << 4) + (lane & 3) * 4)) : "memory");
-                            ro[x] = CONV ? __shfl_sync(0xffffffffu, my_out, x0 + x) : (int64_t)(x0 + x) * p.o_w;
-                        }
-                        write_rows(out, v, ro, rows - x0, bias, p.act, p.accumulate);
-                    }
-                }
+                // (of the CTA's last tile the producers, done by now, write all column blocks but the first)
+                const bool shared = last && tile + tile_step >= gp.num_tiles;
+                for (int j = 0; j * 32 < (shared ? 32 : cols); ++j) finish_block(m0, n0, j, buf, first, last, stage);
                 if (!last) asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(acc_empty_bar(buf));
+                if (lane == 0) {
+                    mbar_arrive(acc_empty_bar(buf));
+                    if (!last && kb + 2 * C::PROMOTE >= kb1 && tile + tile_step >= gp.num_tiles) mbar_arrive(sum_bar);
+                }
             }
         }
     }
@@ -519,16 +563,18 @@ sg_status launch_gather(const Problem &p, const void *In, const void *Flt, float
     gp.p = p;
     const int es = p.in_bf16 ? 2 : 4;
     auto even = [](int64_t v) { return v % 2 == 0; };
-    auto aligned = [&](const void *ptr) { return reinterpret_cast<uintptr_t>(ptr) % (2 * es) == 0; };
-    // a line runs along whichever index is contiguous; pairs are single loads when every line starts on a multiple of two
-    // elements and ends on one
+    auto on = [](const void *ptr, int64_t bytes) { return reinterpret_cast<uintptr_t>(ptr) % bytes == 0; };
+    // A line runs along whichever index is contiguous.  Pairs are single loads when every line starts on a multiple of two
+    // elements and ends on one.
     gp.a.mn_major = !conv && p.i_c != 1 && p.i_w == 1;
     gp.a.s_mn = (int)p.i_w; gp.a.s_k = (int)p.i_c;
-    gp.a.pair = aligned(In) && (gp.a.mn_major ? even(p.i_c) && even(p.M)
-                                              : p.i_c == 1 && even(p.i_w) && even(p.K) && (!conv || (even(p.C) && even(p.i_h) && even(p.i_n))));
+    gp.a.pair = on(In, 2 * es) && (gp.a.mn_major ? even(p.i_c) && even(p.M)
+                                                 : p.i_c == 1 && even(p.i_w) && even(p.K) && (!conv || (even(p.C) && even(p.i_h) && even(p.i_n))));
     gp.b.mn_major = conv || p.k_f == 1 || p.k_c != 1;
     gp.b.s_mn = (int)p.k_f; gp.b.s_k = (int)p.k_c;
-    gp.b.pair = aligned(Flt) && (gp.b.mn_major ? p.k_f == 1 && even(p.k_c) && even(p.N) && (!conv || (even(p.k_kw) && even(p.k_kh))) : even(p.k_f) && even(p.K));
+    gp.b.pair = on(Flt, 2 * es) && (gp.b.mn_major ? p.k_f == 1 && even(p.k_c) && even(p.N) && (!conv || (even(p.k_kw) && even(p.k_kh)))
+                                                  : even(p.k_f) && even(p.K));
+    gp.uniform_rows = (p.Ho == 1 || p.o_h == (int64_t)p.Wo * p.o_w) && (p.batch == 1 || p.o_n == (int64_t)p.Ho * p.Wo * p.o_w);
     gp.num_kb = (p.K + BK - 1) / BK;
     gp.wait_prior = pdl == 0 ? 0 : 1;
 

@@ -39,7 +39,6 @@ namespace {
 constexpr int BM = 128, BK = 64;
 constexpr int GROUPS = 2, GROUP_WARPS = 8;                  // producer groups and warps per group
 constexpr int MMA_WARP = GROUPS * GROUP_WARPS, EPI_WARP = MMA_WARP + 1;
-constexpr int THREADS = 32 * (EPI_WARP + 4);
 constexpr int MAX_SPLIT = 8;
 
 // How one operand is fetched.  mn_major 0: lines are rows/columns (index mn), a line runs along k; 1: the reverse.
@@ -47,7 +46,19 @@ struct Operand {
     int mn_major;
     int pair;             // two neighbouring elements of a line are one aligned load
     int s_mn, s_k;        // element strides of the row/column index and of k (matmul)
+    int shift;            // RAW: elements between the 16-byte boundary below the first element and that element
+    int groups;           // RAW: whole groups of eight lines
 };
+
+// Where a kernel's operand tiles come from.
+//   LINEAR  matmul, ordinary loads, any strides
+//   CONV    convolution, ordinary loads: addresses from the (n, h, w) / (kh, kw, c) decomposition (input K-major, filter N-major)
+//   RAW     bf16 matmul, unit strides: tensor loads.  Eight consecutive lines of pitch P are 16 * P bytes apart, whatever P is,
+//           so the operand is a matrix of G groups of eight lines; the lines of one residue mod 8 in a tile are one box of it,
+//           eight bytes-aligned boxes a tile, which land shifted by less than 16 bytes.  The producers of the other
+//           two take the raw lines from shared memory, shift them in registers and write the tile; the lines behind the last
+//           whole group are loaded element by element.
+enum { LINEAR = 0, CONVOLUTION = 1, RAW = 2 };
 
 struct GatherParams {
     Problem p;
@@ -59,16 +70,22 @@ struct GatherParams {
     int wait_prior;
 };
 
-template <int BN, bool F32>
+template <int BN, bool F32, int SRC>
 struct Cfg {
+    static_assert(SRC != RAW || !F32, "raw lines: bf16 only");
+    static constexpr int THREADS = 32 * (EPI_WARP + 4 + (SRC == RAW ? 2 : 0));      // RAW: one warp per operand issues its tensor loads
+    // eight boxes of 128 / 8 lines of 64 + 8 elements, or of 64 / 8 lines of 128 + 8 (BN 64: of 64 / 8 lines of 64 + 8)
+    static constexpr int RAW_A_BYTES = SRC == RAW ? 128 * 2 * (64 + 8) : 0, RAW_B_BYTES = SRC == RAW ? BN * 2 * (64 + 8) : 0;
+    static constexpr int RAW_BYTES = RAW_A_BYTES + RAW_B_BYTES;
+    static constexpr int RAW_STAGES = BN == 128 ? 3 : 4;
     static constexpr int PARTS = F32 ? 3 : 1;
     static constexpr int A_BYTES = BM * 128, B_BYTES = BN * 128;          // one part of a tile
     static constexpr int STAGE_BYTES = PARTS * (A_BYTES + B_BYTES);
-    static constexpr int STAGES = F32 ? 2 : 4;
+    static constexpr int STAGES = F32 ? 2 : SRC == RAW && BN == 128 ? 3 : 4;
     static constexpr int PROMOTE = F32 ? 1 : 4;                           // k-blocks between additions to the running sum
     static constexpr int RING_BYTES = STAGES * STAGE_BYTES;
     static constexpr int STAGING_BYTES = 4 * 4096;                        // one 32 x 32 block per write-back warp
-    static constexpr int SMEM_BYTES = RING_BYTES + STAGING_BYTES + 1024 + 256;
+    static constexpr int SMEM_BYTES = RING_BYTES + RAW_STAGES * RAW_BYTES + STAGING_BYTES + 1024 + 256;
     static constexpr int TMEM_COLS = BN == 64 ? 256 : 512;                // two accumulators and the running sum
     static_assert(RING_BYTES >= BM * BN * 4 && RING_BYTES >= MMA_WARP * 4096, "a split reduction parks the tile's partial sums in the ring");
     static_assert(SMEM_BYTES <= 232448, "shared memory");
@@ -150,6 +167,64 @@ __device__ __forceinline__ void load_lines(uint32_t (&r)[8][2], const T *base, i
     }
 }
 
+// RAW: one operand's tile of a k-block, from the raw lines at `raw` (box j holds the lines of residue j mod 8, 16-byte aligned
+// and shifted by a few elements) to the swizzled tile at `dst`.  Eight lanes per line, 16 bytes each: the two aligned
+// 16-byte pieces they lie in, shifted.  Lines and elements beyond the end are zero (lines: the tensor loads' fill).
+template <int WIDTH>
+__device__ __forceinline__ void shift_tile(const unsigned short *ptr, const Operand &op, int mn0, int mn_end, int k0, int k_end, uint32_t raw, uint32_t dst,
+                                           int w, int lane) {
+    const int s_line = op.mn_major ? op.s_k : op.s_mn;
+    const int n = w * 4 + (lane >> 3), piece = lane & 7;           // line of step 0; step t: n + 32 * t
+    const int line_pitch = op.mn_major ? (WIDTH + 8) * 2 : 144;    // bytes between the raw lines of a residue
+    const int line0 = op.mn_major ? k0 : mn0, line_end = op.mn_major ? k_end : mn_end;
+    // (tiles start at multiples of eight lines and of eight elements)
+    const uint32_t shift = (uint32_t)(op.shift + (n & 7) * s_line) & 7u;
+    const uint32_t src = raw + (uint32_t)((n & 7) * (op.mn_major ? 8 : WIDTH / 8) * line_pitch + (n >> 3) * line_pitch + piece * 16);
+    const uint32_t out = dst + (uint32_t)(n * 128 + ((piece ^ (n & 7)) << 4));
+    const bool b8 = shift & 4, b4 = shift & 2;
+    const uint32_t bits = (shift & 1) * 16;
+    const bool ragged_k = !op.mn_major && k0 + 64 > k_end;
+    const int left = k_end - k0 - piece * 8;                       // K-major: values of k this lane's 16 bytes still hold
+    const int whole = 8 * op.groups - line0;                       // lines of the tile that the boxes bring
+    const bool ragged_lines = whole < (op.mn_major ? 64 : WIDTH) && 8 * op.groups < line_end;
+    uint32_t v[WIDTH / 32][8];
+#pragma unroll
+    for (int t = 0; t < WIDTH / 32; ++t) {
+        const uint32_t a = src + (op.mn_major ? (uint32_t)((t & 1) * 4 * line_pitch + (t >> 1) * 128) : (uint32_t)(t * 4 * 144));
+        asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v[t][0]), "=r"(v[t][1]), "=r"(v[t][2]), "=r"(v[t][3]) : "r"(a) : "memory");
+        asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4+16];" : "=r"(v[t][4]), "=r"(v[t][5]), "=r"(v[t][6]), "=r"(v[t][7]) : "r"(a) : "memory");
+    }
+#pragma unroll
+    for (int t = 0; t < WIDTH / 32; ++t) {
+        uint32_t x[6], y[5], o[4];
+#pragma unroll
+        for (int i = 0; i < 6; ++i) x[i] = b8 ? v[t][i + 2] : v[t][i];
+#pragma unroll
+        for (int i = 0; i < 5; ++i) y[i] = b4 ? x[i + 1] : x[i];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) o[i] = __funnelshift_r(y[i], y[i + 1], bits);
+        if (ragged_k)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) o[i] = 2 * i + 1 < left ? o[i] : 2 * i < left ? o[i] & 0xFFFFu : 0u;
+        const int x_line = op.mn_major ? (n + 32 * t) & 63 : n + 32 * t;
+        if (!ragged_lines || x_line < whole || x_line >= line_end - line0)
+            asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(out + t * 4096), "r"(o[0]), "r"(o[1]), "r"(o[2]), "r"(o[3]) : "memory");
+    }
+    if (ragged_lines) {
+        // the lines behind the last whole group, one per warp and turn
+        const int rest = line_end - max(8 * op.groups, line0), subs = op.mn_major ? WIDTH / 64 : 1;
+        for (int u = w; u < rest * subs; u += GROUP_WARPS) {
+            const int line = max(8 * op.groups, line0) + u % rest, sub = u / rest;
+            const int e = (op.mn_major ? mn0 + 64 * sub : k0) + 2 * lane, e_end = op.mn_major ? mn_end : k_end;
+            const int x = line - line0 + 64 * sub;
+            uint32_t r[2] = {0, 0};
+            load1_if(e < e_end, ptr + ((int64_t)line * s_line + e), r[0]);
+            load1_if(e + 1 < e_end, ptr + ((int64_t)line * s_line + e + 1), r[1]);
+            sts32(dst + (uint32_t)(x * 128 + (((lane >> 2) ^ (x & 7)) << 4) + (lane & 3) * 4), r[0] | (r[1] << 16));
+        }
+    }
+}
+
 // This lane's column of eight output rows: out[ro[x]] (+)= act(v[x] + bias) for x < rows.
 __device__ __forceinline__ void write_rows(float *out, const float (&v)[8], const int64_t (&ro)[8], int rows, float bias, int act, int accumulate) {
     float old[8];
@@ -166,30 +241,31 @@ __device__ __forceinline__ void write_rows(float *out, const float (&v)[8], cons
     }
 }
 
-// CONV: the operand addresses come from the (n, h, w) / (kh, kw, c) decomposition (input K-major, filter N-major); else a
-// matmul with linear addresses in either orientation.
-template <int BN, bool F32, bool CONV>
-__global__ void __launch_bounds__(THREADS, 1)
-gather_gemm_kernel(const __grid_constant__ GatherParams gp, const void *__restrict__ in_ptr, const void *__restrict__ flt_ptr, float *__restrict__ O) {
-    using C = Cfg<BN, F32>;
+template <int BN, bool F32, int SRC>
+__global__ void __launch_bounds__(Cfg<BN, F32, SRC>::THREADS, 1)
+gather_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, const __grid_constant__ GatherParams gp, const void *__restrict__ in_ptr, const void *__restrict__ flt_ptr, float *__restrict__ O) {
+    constexpr bool CONV = SRC == CONVOLUTION;
+    using C = Cfg<BN, F32, SRC>;
     using T = typename std::conditional<F32, float, unsigned short>::type;
     const Problem &p = gp.p;
     const T *In = static_cast<const T *>(in_ptr), *Flt = static_cast<const T *>(flt_ptr);
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t *smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
-    const uint32_t staging_addr = smem_base + C::RING_BYTES;
+    const uint32_t raw_addr = smem_base + C::RING_BYTES, staging_addr = raw_addr + C::RAW_STAGES * C::RAW_BYTES;
     const uint32_t bars = staging_addr + C::STAGING_BYTES;
-    uint8_t *bars_gen = smem_gen + C::RING_BYTES + C::STAGING_BYTES;
-    // barrier block: full[4] | empty[4] | acc_full[2] | acc_empty[2] | sum | done | tmem_ptr | abort | large
+    uint8_t *bars_gen = smem_gen + C::RING_BYTES + C::RAW_STAGES * C::RAW_BYTES + C::STAGING_BYTES;
+    // barrier block: full[4] | empty[4] | acc_full[2] | acc_empty[2] | sum | done | raw_full[4] | raw_empty[4] | tmem_ptr | abort | large
     auto full_bar = [&](int s) { return bars + 8u * s; };
     auto empty_bar = [&](int s) { return bars + 8u * (4 + s); };
     auto acc_full_bar = [&](int b) { return bars + 8u * (8 + b); };
     auto acc_empty_bar = [&](int b) { return bars + 8u * (10 + b); };
     const uint32_t sum_bar = bars + 8u * 12, done_bar = bars + 8u * 13;      // completed once: the last tile's running sum, its last MMAs
-    volatile uint32_t *tmem_ptr_slot = reinterpret_cast<volatile uint32_t *>(bars_gen + 112);
-    volatile int *abort_flag = reinterpret_cast<volatile int *>(bars_gen + 116);
-    volatile int *large_flag = reinterpret_cast<volatile int *>(bars_gen + 120);
+    auto raw_full_bar = [&](int s) { return bars + 8u * (14 + s); };
+    auto raw_empty_bar = [&](int s) { return bars + 8u * (18 + s); };
+    volatile uint32_t *tmem_ptr_slot = reinterpret_cast<volatile uint32_t *>(bars_gen + 8 * 22);
+    volatile int *abort_flag = reinterpret_cast<volatile int *>(bars_gen + 8 * 22 + 4);
+    volatile int *large_flag = reinterpret_cast<volatile int *>(bars_gen + 8 * 22 + 8);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     asm volatile("griddepcontrol.launch_dependents;");
@@ -198,10 +274,12 @@ gather_gemm_kernel(const __grid_constant__ GatherParams gp, const void *__restri
         for (int b = 0; b < 2; ++b) { mbar_init(acc_full_bar(b), 1); mbar_init(acc_empty_bar(b), 4); }
         mbar_init(sum_bar, 4);
         mbar_init(done_bar, 1);
+        if (SRC == RAW) for (int s = 0; s < C::RAW_STAGES; ++s) { mbar_init(raw_full_bar(s), 2); mbar_init(raw_empty_bar(s), GROUP_WARPS); }
         *abort_flag = 0;
         *large_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    if (SRC == RAW && threadIdx.x == 0) { prefetch_tensormap(&map_a); prefetch_tensormap(&map_b); }
     if (warp == MMA_WARP) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                      ::"r"(smem_u32(const_cast<uint32_t *>(tmem_ptr_slot))), "r"((uint32_t)C::TMEM_COLS) : "memory");
@@ -333,6 +411,18 @@ gather_gemm_kernel(const __grid_constant__ GatherParams gp, const void *__restri
             for (int kb = kb0; kb < kb1; ++kb, ++it) {
                 if (it % GROUPS != group) continue;
                 const int k0 = kb * BK;
+                if constexpr (SRC == RAW) {
+                    const int s = it % C::STAGES, rs = it % C::RAW_STAGES;
+                    if (!mbar_wait(raw_full_bar(rs), (it / C::RAW_STAGES) & 1, abort_flag)) { ok = false; break; }
+                    if (!mbar_wait(empty_bar(s), ((it / C::STAGES) & 1) ^ 1u, abort_flag)) { ok = false; break; }
+                    const uint32_t raw = raw_addr + rs * C::RAW_BYTES, dst = smem_base + s * C::STAGE_BYTES;
+                    shift_tile<BM>(In, gp.a, m0, p.M, k0, p.K, raw, dst, w, lane);
+                    shift_tile<BN>(Flt, gp.b, n0, p.N, k0, p.K, raw + C::RAW_A_BYTES, dst + C::A_BYTES, w, lane);
+                    fence_async_smem();
+                    __syncwarp();
+                    if (lane == 0) { mbar_arrive(raw_empty_bar(rs)); mbar_arrive(full_bar(s)); }
+                    continue;
+                }
                 uint32_t ra[2][8][2], rb[BN / 64][8][2];
                 if constexpr (CONV) {
                     // input, K-major: lines are rows, the lane's two k; filter, N-major: lines are k
@@ -438,6 +528,31 @@ gather_gemm_kernel(const __grid_constant__ GatherParams gp, const void *__restri
                 }
             }
         }
+    } else if (SRC == RAW && warp >= EPI_WARP + 4) {
+        // ------------------------------------------------------------ RAW: tensor loads, lane j < 8 those of residue j
+        const bool input = warp == EPI_WARP + 4;
+        const Operand &op = input ? gp.a : gp.b;
+        const CUtensorMap *map = input ? &map_a : &map_b;
+        const int width = input ? BM : BN;
+        const uint32_t bytes = op.mn_major ? 64 * 2 * (width + 8) : width * 2 * (64 + 8);
+        if (gp.wait_prior) asm volatile("griddepcontrol.wait;" ::: "memory");
+        int it = 0;
+        bool ok = true;
+        for (int tile = first_tile; ok && tile < gp.num_tiles; tile += tile_step) {
+            const int mt = tile / gp.num_n_tiles;
+            const int mn0 = input ? mt * BM : (tile - mt * gp.num_n_tiles) * BN;
+            const int64_t line_pos = op.shift + (int64_t)(lane & 7) * (op.mn_major ? op.s_k : op.s_mn);
+            for (int kb = kb0; kb < kb1; ++kb, ++it) {
+                const int rs = it % C::RAW_STAGES;
+                if (!__all_sync(0xffffffffu, mbar_wait(raw_empty_bar(rs), ((it / C::RAW_STAGES) & 1) ^ 1u, abort_flag))) { ok = false; break; }
+                const uint32_t dst = raw_addr + rs * C::RAW_BYTES + (input ? 0 : C::RAW_A_BYTES);
+                if (lane == 0) mbar_expect_tx(raw_full_bar(rs), bytes);
+                __syncwarp();
+                if (lane < 8)
+                    tma_load_2d(dst + lane * (bytes / 8), map, raw_full_bar(rs), (int)((line_pos + (op.mn_major ? mn0 : kb * BK)) & ~(int64_t)7),
+                                (op.mn_major ? kb * BK : mn0) / 8);
+            }
+        }
     } else {
         // ------------------------------------------------------------ write-back
         const uint32_t stage = staging_addr + (uint32_t)(warp - EPI_WARP) * 4096u;
@@ -469,6 +584,10 @@ gather_gemm_kernel(const __grid_constant__ GatherParams gp, const void *__restri
 
     // ---------------------------------------------------------------- split reduction and teardown
     __syncthreads();
+    if (SRC == RAW && *abort_flag) {
+        for (int i = 0; i < 200; ++i) __nanosleep(5000);      // let tensor loads in flight land before the shared memory goes
+        __syncthreads();
+    }
     if (gp.splits > 1) {
         // every CTA of the cluster sums its share of the tile's rows over the partial tiles parked in all of them, in rank order
         cluster_sync_all();
@@ -476,7 +595,7 @@ gather_gemm_kernel(const __grid_constant__ GatherParams gp, const void *__restri
         const int m0 = mt * BM, n0 = (first_tile - mt * gp.num_n_tiles) * BN;
         const int rows = BM / gp.splits, cols = min(BN, p.N - n0);
         if (!*abort_flag)
-            for (int u = warp; u < rows * (BN / 32); u += THREADS / 32) {
+            for (int u = warp; u < rows * (BN / 32); u += C::THREADS / 32) {
                 const int j = u / rows, x = rank * rows + (u - j * rows), m = m0 + x;
                 if (j * 32 >= cols || m >= p.M) continue;
                 const uint32_t src = smem_base + (uint32_t)((j * BM + x) * 128 + (((lane >> 2) ^ (x & 7)) << 4) + (lane & 3) * 4);
@@ -518,14 +637,14 @@ inline int64_t reach(std::initializer_list<std::pair<int64_t, int64_t>> extents_
     return r;
 }
 
-template <int BN, bool F32, bool CONV>
-sg_status launch_variant(const GatherParams &gp, const void *In, const void *Flt, float *O, int num_sms, int slot, cudaStream_t stream) {
-    using C = Cfg<BN, F32>;
-    const void *fn = reinterpret_cast<const void *>(gather_gemm_kernel<BN, F32, CONV>);
+template <int BN, bool F32, int SRC>
+sg_status launch_variant(const CUtensorMap &ma, const CUtensorMap &mb, const GatherParams &gp, const void *In, const void *Flt, float *O, int num_sms, int slot, cudaStream_t stream) {
+    using C = Cfg<BN, F32, SRC>;
+    const void *fn = reinterpret_cast<const void *>(gather_gemm_kernel<BN, F32, SRC>);
     if (!tensor_ensure_smem_attr(slot, fn, C::SMEM_BYTES)) return SG_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(gp.splits > 1 ? gp.num_tiles * gp.splits : std::min(gp.num_tiles, num_sms), 1, 1);
-    cfg.blockDim = dim3(THREADS, 1, 1);
+    cfg.blockDim = dim3(C::THREADS, 1, 1);
     cfg.dynamicSmemBytes = C::SMEM_BYTES;
     cfg.stream = stream;
     cudaLaunchAttribute attr[2];
@@ -537,10 +656,25 @@ sg_status launch_variant(const GatherParams &gp, const void *In, const void *Flt
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = gp.wait_prior ? 2 : 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, gather_gemm_kernel<BN, F32, CONV>, gp, In, Flt, O);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, gather_gemm_kernel<BN, F32, SRC>, ma, mb, gp, In, Flt, O);
     count_launch();
     note_kernel(F32 ? "gather_gemm_kernel<f32>" : "gather_gemm_kernel<bf16>");
     return e == cudaSuccess ? SG_OK : SG_ERR_CUDA;
+}
+
+// RAW: the operand as a matrix of whole groups of eight lines, boxes of the lines of one residue in a tile of `width` rows or
+// columns.  A row of that matrix ends with the last element of the group's last line, so nothing behind the operand is read.
+// False when the operand has no unit stride or less than one group.
+bool raw_map(CUtensorMap *map, const void *ptr, Operand &op, int mn, int k, int width) {
+    const int64_t pitch = op.mn_major ? op.s_k : op.s_mn, lines = op.mn_major ? k : mn, inner = op.mn_major ? mn : k;
+    if ((op.mn_major ? op.s_mn : op.s_k) != 1 || lines < 8 || pitch < inner) return false;
+    op.shift = (int)(reinterpret_cast<uintptr_t>(ptr) % 16 / 2);
+    op.groups = (int)(lines / 8);
+    cuuint64_t dims[2] = {(cuuint64_t)(op.shift + 7 * pitch + inner), (cuuint64_t)op.groups}, strides[1] = {(cuuint64_t)(16 * pitch)};
+    cuuint32_t box[2] = {(cuuint32_t)((op.mn_major ? width : 64) + 8), (cuuint32_t)((op.mn_major ? 64 : width) / 8)};
+    void *base = reinterpret_cast<void *>(reinterpret_cast<uintptr_t>(ptr) & ~(uintptr_t)15);
+    return tensor_encode_tiled(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, base, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_NONE,
+                               CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
 }
 
 }  // namespace
@@ -586,13 +720,16 @@ sg_status launch_gather(const Problem &p, const void *In, const void *Flt, float
     // few tiles: a cluster of 2, 4 or 8 CTAs shares a tile's reduction, at least four k-blocks each
     gp.splits = 1;
     while (gp.splits < MAX_SPLIT && tiles * gp.splits * 2 <= num_sms - 12 && gp.num_kb >= gp.splits * 8) gp.splits *= 2;
-#define SG_GATHER(BN_, F32_, CONV_, SLOT) launch_variant<BN_, F32_, CONV_>(gp, In, Flt, O, num_sms, SLOT, stream)
+    alignas(64) CUtensorMap ma = {}, mb = {};
+    const bool raw = p.in_bf16 && !conv && raw_map(&ma, In, gp.a, p.M, p.K, BM) && raw_map(&mb, Flt, gp.b, p.N, p.K, bn);
+#define SG_GATHER(BN_, F32_, SRC_, SLOT) launch_variant<BN_, F32_, SRC_>(ma, mb, gp, In, Flt, O, num_sms, SLOT, stream)
+    if (raw) return bn == 64 ? SG_GATHER(64, false, RAW, 157) : SG_GATHER(128, false, RAW, 158);
     if (p.in_bf16) {
-        if (conv) return bn == 64 ? SG_GATHER(64, false, true, 149) : SG_GATHER(128, false, true, 150);
-        return bn == 64 ? SG_GATHER(64, false, false, 151) : SG_GATHER(128, false, false, 152);
+        if (conv) return bn == 64 ? SG_GATHER(64, false, CONVOLUTION, 149) : SG_GATHER(128, false, CONVOLUTION, 150);
+        return bn == 64 ? SG_GATHER(64, false, LINEAR, 151) : SG_GATHER(128, false, LINEAR, 152);
     }
-    if (conv) return bn == 64 ? SG_GATHER(64, true, true, 153) : SG_GATHER(128, true, true, 154);
-    return bn == 64 ? SG_GATHER(64, true, false, 155) : SG_GATHER(128, true, false, 156);
+    if (conv) return bn == 64 ? SG_GATHER(64, true, CONVOLUTION, 153) : SG_GATHER(128, true, CONVOLUTION, 154);
+    return bn == 64 ? SG_GATHER(64, true, LINEAR, 155) : SG_GATHER(128, true, LINEAR, 156);
 #undef SG_GATHER
 }
 

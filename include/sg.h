@@ -44,8 +44,10 @@
  *     per term (each input split into hi + lo, lo*hi + hi*lo + hi*hi summed in
  *     f32), which keeps f32 accuracy for finite inputs: the error stays below
  *     1e-5 * sum_k |a*b|.  On that f32 path an infinite input gives NaN rather
- *     than a signed infinity.  Everything else runs on a strided CUDA-core
- *     FFMA kernel.  There is no CPU fallback.
+ *     than a signed infinity.  Other layouts run on a tensor-core kernel that
+ *     fetches its operands with ordinary loads (f32 inputs as three bf16 parts,
+ *     f32 accuracy), tiny problems in them on a strided CUDA-core FFMA kernel.
+ *     There is no CPU fallback.
  */
 #ifndef SG_H_
 #define SG_H_
@@ -255,7 +257,8 @@ int sg_last_kernel(void);
 /*
  * Name of the compute kernel that call launched (a static string, "" before any call; clearing
  * kernels launched ahead of it are not named): "tc_gemm_kernel<bf16>", "tc_gemm_kernel<f32>",
- * "conv_strip_kernel<bf16>", "conv_strip_kernel<f32>", "ffma_kernel", "depthwise_tma_kernel",
+ * "gather_gemm_kernel<bf16>", "gather_gemm_kernel<f32>" (layouts outside the TMA rules), "small_gemm_kernel<bf16>",
+ * "small_gemm_kernel<f32>", "conv_strip_kernel<bf16>", "conv_strip_kernel<f32>", "ffma_kernel", "depthwise_tma_kernel",
  * "depthwise_roll_kernel", "depthwise_vec_kernel", "depthwise_generic_kernel", "copy_tma_kernel",
  * "transpose_tma_kernel", "tile_move_kernel", "colred_kernel<vec>", "colred_kernel<scalar>",
  * "rowred_kernel<vec>", "rowred_kernel<scalar>".  For tests and benchmarks.
@@ -326,6 +329,7 @@ sg_status sg_selftest_wait_timeout(int64_t budget_cycles, sg_stream_t stream);
  * call of the process:
  *   SG_TC_BN, SG_TC_CG, SG_TC_SPLIT   as sg_set_tile_override
  *   SG_TC_SK        0: never cut the last wave into a stream-K tail; 2: whenever the shape allows it
+ *   SG_TC_SMALL     0: the kernel for small problems is never chosen; 1: wherever the layout allows it
  *   SG_TC_KPS       1: one k-block per pipeline stage everywhere (bf16 matmuls normally move two)
  *   SG_TC_TA        0: keep the split f32 input tile in shared memory instead of tensor memory
  *   SG_TC_PDL       0: tensor-core launches never start before the kernel ahead of them in the

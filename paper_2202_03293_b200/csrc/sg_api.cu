@@ -30,6 +30,12 @@ sg_status run(const Problem &p, const void *In, const void *Flt, float *O, cudaS
         return launch_zero_fill(p, O, stream) == cudaSuccess ? SG_OK : SG_ERR_CUDA;
     }
     const int force = g_override.load();
+    if (force == SG_KERNEL_AUTO) {
+        // problems that launch and memory latencies bound
+        const sg_status st = launch_small(p, In, Flt, O, stream);
+        if (st == SG_OK) { t_last_kernel = SG_KERNEL_TENSOR; return SG_OK; }
+        if (st != SG_ERR_UNSUPPORTED) return st;
+    }
     if (force == SG_KERNEL_AUTO || force == SG_KERNEL_CONV_STRIP) {
         // stride-1 bf16 convolutions whose filter fits in shared memory
         sg_status st = launch_conv_strip(p, In, Flt, O, stream);

@@ -53,7 +53,7 @@ cudaError_t launch_wait_timeout_selftest(long long budget_cycles, cudaStream_t s
 bool tensor_driver_ready(int *num_sms);
 // The current device's index and SM count plus two test switches (SG_TC_PDL, SG_CONV_SINGLE); false when the device is unusable.
 bool tensor_device_info(int *device, int *num_sms, int *pdl, int *conv_single);
-// Raises a kernel's dynamic shared-memory limit once per device; `slot` (144..159 for callers outside the GEMM file)
+// Raises a kernel's dynamic shared-memory limit once per device; `slot` (144 and up for callers outside the GEMM file)
 // names the kernel instantiation.
 bool tensor_ensure_smem_attr(int slot, const void *kernel, int bytes);
 bool tensor_encode_tiled(CUtensorMap *map, CUtensorMapDataType type, int rank, void *base, const cuuint64_t *dims,
@@ -63,6 +63,12 @@ bool tensor_encode_tiled(CUtensorMap *map, CUtensorMapDataType type, int rank, v
 // shape or layout does not qualify (nothing is launched then).
 sg_status launch_conv_strip(const Problem &p, const void *In, const void *Flt, float *O, cudaStream_t stream);
 sg_status conv_read_status(cudaStream_t stream);
+// Tensor-core implicit GEMM for small problems (sg_small.cu).  SG_ERR_UNSUPPORTED (nothing is launched) when its layout rules
+// (those of the TMA kernels) do not hold or the problem is large enough for the kernels above to be the faster ones.
+sg_status launch_small(const Problem &p, const void *In, const void *Flt, float *O, cudaStream_t stream);
+double tensor_estimate_us(const Problem &p);      // what launch_tensor would take, by its cost model
+int tensor_small_override();                      // SG_TC_SMALL: 0 never, 1 always, -1 by size
+void tensor_note_choice(int bn, int cg, int splits);      // what sg_last_tile_choice reports for a launch outside the GEMM file
 // Tensor-core implicit GEMM for layouts outside the TMA rules (sg_gather.cu): any strides.  SG_ERR_UNSUPPORTED (nothing is
 // launched) when offsets do not fit 32 bits or, unless `forced`, the problem is too small to gain.
 sg_status launch_gather(const Problem &p, const void *In, const void *Flt, float *O, bool forced, cudaStream_t stream);

@@ -786,7 +786,7 @@ typedef CUresult (*EncodeIm2colFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_
 // g_mu guards the driver entry points, the per-device records and the overrides; it is held for a few loads and stores,
 // never across a tensor-map encode or a launch.  The tensor-map cache has a lock of its own.
 constexpr int kMaxDevices = 64;
-constexpr int kAttrSlots = 160;
+constexpr int kAttrSlots = 192;
 struct DeviceState {
     bool ready = false;
     int num_sms = 0;
@@ -802,6 +802,7 @@ struct Overrides {
     int ta = -1;     // SG_TC_TA (testing): 0 never, 1 always keep the split f32 input tile in tensor memory
     int pdl = -1;    // SG_TC_PDL (testing): 0 = launches never overlap the tail of the kernel ahead of them
     int conv_single = 0;   // SG_CONV_SINGLE=1 (testing): the stride-1 convolution kernel never uses CTA pairs
+    int small = -1;  // SG_TC_SMALL (testing): 0 = the kernel for small problems is never chosen, 1 = wherever the layout allows it
     int mix = -1;    // SG_TC_MIX (testing): 0 = f32 correction products as tf32 MMAs (three tf32 products per term) instead of bf16
 };
 std::mutex g_mu;
@@ -820,6 +821,7 @@ void read_env_locked() {
     g_ov.kps = env("SG_TC_KPS", 0); g_ov.ta = env("SG_TC_TA", -1); g_ov.sk = env("SG_TC_SK", -1);
     g_ov.pdl = env("SG_TC_PDL", -1);
     g_ov.conv_single = env("SG_CONV_SINGLE", 0);
+    g_ov.small = env("SG_TC_SMALL", -1);
     g_ov.mix = env("SG_TC_MIX", -1);
     g_ov.env_read = true;
 }
@@ -1006,6 +1008,62 @@ double estimate_ns(const Variant &v, bool f32, int64_t tiles, int64_t groups, in
     return t;
 }
 
+// Operands stored transposed (matmuls only): bit 0 the input ([k][m], m contiguous), bit 1 the filter ([n][k], k contiguous).
+inline int transposed_layout(const Problem &p) {
+    const bool a_mn = p.spatial_rank == 0 && p.i_c != 1 && p.i_w == 1, b_km = p.spatial_rank == 0 && p.k_f != 1 && p.k_c == 1;
+    return (a_mn ? 1 : 0) | (b_km ? 2 : 0);
+}
+
+// Tile variant and k split of lowest estimated time, which is returned (unless the variant is forced); *out_pick = -1: none.
+double choose_tiles(const Problem &p, int num_kb, int lay, const Overrides &ov, int num_sms, int *out_pick, int *out_splits) {
+    const bool f32 = !p.in_bf16;
+    int pick = -1, splits = 1;
+    double best = 1e300;
+    if (ov.bn > 0) {
+        for (int i = 0; i < kNumVariants; ++i)
+            if (kVariants[i].bn == ov.bn && kVariants[i].cg == (ov.cg > 0 ? ov.cg : 1) &&
+                !(f32 && kVariants[i].bn == 256 && kVariants[i].cg == 1) &&
+                !(lay != 0 && ((kVariants[i].bn == 256 && kVariants[i].cg == 1) || (kVariants[i].bn == 128 && kVariants[i].cg == 2)))) pick = i;
+    }
+    auto valid_split = [&](int s) {      // every range of ceil(num_kb / s) k-blocks must be non-empty
+        const int per = (num_kb + s - 1) / s;
+        return s >= 1 && (s - 1) * per < num_kb;
+    };
+    if (pick >= 0) {
+        splits = ov.split > 0 && valid_split(ov.split) ? ov.split : 1;
+    } else {
+        // A forced split is taken as given when it fits the reduction (every range non-empty), with the variant that
+        // is cheapest for it; one that does not fit is ignored and the estimate chooses the split as well.
+        const int forced = ov.split > 0 && valid_split(ov.split) ? ov.split : 0;
+        // (a forced pair count that no variant can honour on this shape is dropped in a second pass)
+        for (int pass = 0; pass < 2 && pick < 0; ++pass)
+        for (int i = 0; i < kNumVariants; ++i) {
+            // (forced == 1 for a fused consumer: one work item per tile)
+            const Variant &v = kVariants[i];
+            if (pass == 0 && ov.cg > 0 && v.cg != ov.cg && !(v.cg == 1 && p.M <= BM)) continue;
+            if (f32 && v.bn == 256 && v.cg == 1) continue;       // not built (shared-memory budget)
+            if (lay != 0 && ((v.bn == 256 && v.cg == 1) || (v.bn == 128 && v.cg == 2))) continue;   // not built for transposed operands
+            if (v.bn > 64 && v.bn / 2 >= p.N) continue;          // at most half of the tile would be used
+            if (v.cg == 2 && p.M <= BM) continue;                // the second CTA would have no rows
+            const int64_t tiles = (int64_t)((p.M + v.cg * BM - 1) / (v.cg * BM)) * ((p.N + v.bn - 1) / v.bn);
+            const int64_t groups = num_sms / v.cg;
+            if (forced) {
+                const double c = estimate_ns(v, f32, tiles, groups, num_kb, forced, p.accumulate != 0);
+                if (c < best) { best = c; pick = i; splits = forced; }
+                continue;
+            }
+            for (int sp = 1; sp <= 32; sp *= 2) {
+                if (!valid_split(sp)) break;
+                if (sp > 1 && tiles * (sp / 2) >= 2 * groups) break;   // already two waves without this split
+                const double c = estimate_ns(v, f32, tiles, groups, num_kb, sp, p.accumulate != 0);
+                if (c < best) { best = c; pick = i; splits = sp; }
+            }
+        }
+    }
+    *out_pick = pick; *out_splits = splits;
+    return best;
+}
+
 struct LaunchCtx {
     const DeviceState *dev;
     int device;
@@ -1061,9 +1119,8 @@ sg_status launch_tensor(const Problem &p, const void *In, const void *Flt, float
     const CUtensorMapDataType in_type = f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
     // matmuls may hand either operand transposed through its strides (Section 4.6.1, A^T B and
     // A B^T): the input [k][m] with m contiguous, the filter [n][k] with k contiguous
-    const bool a_mn = p.spatial_rank == 0 && p.i_c != 1 && p.i_w == 1;
-    const bool b_km = p.spatial_rank == 0 && p.k_f != 1 && p.k_c == 1;
-    const int lay = (a_mn ? 1 : 0) | (b_km ? 2 : 0);
+    const int lay = transposed_layout(p);
+    const bool a_mn = (lay & 1) != 0, b_km = (lay & 2) != 0;
     if ((p.i_c != 1 && !a_mn) || (p.k_f != 1 && !b_km) || p.o_f != 1) return SG_ERR_UNSUPPORTED;
     if (reinterpret_cast<uintptr_t>(In) % 16 || reinterpret_cast<uintptr_t>(Flt) % 16 ||
         reinterpret_cast<uintptr_t>(O) % 16) return SG_ERR_UNSUPPORTED;
@@ -1152,49 +1209,8 @@ sg_status launch_tensor(const Problem &p, const void *In, const void *Flt, float
     }
 
     // ---- tile variant and k split: lowest estimated time ----
-    int pick = -1, splits = 1;
-    if (ov.bn > 0) {
-        for (int i = 0; i < kNumVariants; ++i)
-            if (kVariants[i].bn == ov.bn && kVariants[i].cg == (ov.cg > 0 ? ov.cg : 1) &&
-                !(f32 && kVariants[i].bn == 256 && kVariants[i].cg == 1) &&
-                !(lay != 0 && ((kVariants[i].bn == 256 && kVariants[i].cg == 1) || (kVariants[i].bn == 128 && kVariants[i].cg == 2)))) pick = i;
-    }
-    auto valid_split = [&](int s) {      // every range of ceil(num_kb / s) k-blocks must be non-empty
-        const int per = (tp.num_kb + s - 1) / s;
-        return s >= 1 && (s - 1) * per < tp.num_kb;
-    };
-    if (pick >= 0) {
-        splits = ov.split > 0 && valid_split(ov.split) ? ov.split : 1;
-    } else {
-        // A forced split is taken as given when it fits the reduction (every range non-empty), with the variant that
-        // is cheapest for it; one that does not fit is ignored and the estimate chooses the split as well.
-        const int forced = ov.split > 0 && valid_split(ov.split) ? ov.split : 0;
-        double best = 1e300;
-        // (a forced pair count that no variant can honour on this shape is dropped in a second pass)
-        for (int pass = 0; pass < 2 && pick < 0; ++pass)
-        for (int i = 0; i < kNumVariants; ++i) {
-            // (forced == 1 for a fused consumer: one work item per tile)
-            const Variant &v = kVariants[i];
-            if (pass == 0 && ov.cg > 0 && v.cg != ov.cg && !(v.cg == 1 && p.M <= BM)) continue;
-            if (f32 && v.bn == 256 && v.cg == 1) continue;       // not built (shared-memory budget)
-            if (lay != 0 && ((v.bn == 256 && v.cg == 1) || (v.bn == 128 && v.cg == 2))) continue;   // not built for transposed operands
-            if (v.bn > 64 && v.bn / 2 >= p.N) continue;          // at most half of the tile would be used
-            if (v.cg == 2 && p.M <= BM) continue;                // the second CTA would have no rows
-            const int64_t tiles = (int64_t)((p.M + v.cg * BM - 1) / (v.cg * BM)) * ((p.N + v.bn - 1) / v.bn);
-            const int64_t groups = num_sms / v.cg;
-            if (forced) {
-                const double c = estimate_ns(v, f32, tiles, groups, tp.num_kb, forced, p.accumulate != 0);
-                if (c < best) { best = c; pick = i; splits = forced; }
-                continue;
-            }
-            for (int sp = 1; sp <= 32; sp *= 2) {
-                if (!valid_split(sp)) break;
-                if (sp > 1 && tiles * (sp / 2) >= 2 * groups) break;   // already two waves without this split
-                const double c = estimate_ns(v, f32, tiles, groups, tp.num_kb, sp, p.accumulate != 0);
-                if (c < best) { best = c; pick = i; splits = sp; }
-            }
-        }
-    }
+    int pick, splits;
+    choose_tiles(p, tp.num_kb, lay, ov, num_sms, &pick, &splits);
     if (pick < 0) return SG_ERR_INTERNAL;
     const Variant &var = kVariants[pick];
     // bf16 matmuls with whole k-blocks move two k-blocks per stage and per TMA load
@@ -1372,6 +1388,29 @@ bool tensor_device_info(int *device, int *num_sms, int *pdl, int *conv_single) {
     *pdl = ov.pdl;
     *conv_single = ov.conv_single;
     return true;
+}
+
+double tensor_estimate_us(const Problem &p) {
+    Overrides ov;
+    const DeviceState *d = device_state(nullptr, &ov);
+    if (!d) return 0.0;
+    if (p.bias != nullptr || p.act != SG_ACT_NONE) ov.split = 1;
+    const int bk = ROW_BYTES / (p.in_bf16 ? 2 : 4);
+    int pick, splits;
+    const double ns = choose_tiles(p, p.KH * p.KW * ((p.C + bk - 1) / bk), transposed_layout(p), ov, d->num_sms, &pick, &splits);
+    // (the constants were fitted to problems of 256^3 and up; launches of bf16 problems below take about 0.9 us more)
+    return ns * 1e-3 + (p.in_bf16 ? 0.9 : 0.0);
+}
+
+int tensor_small_override() {
+    Overrides ov;
+    if (!device_state(nullptr, &ov)) return 0;
+    return ov.bn > 0 || ov.cg > 0 || ov.split > 0 ? 0 : ov.small;      // a forced tile asks for the kernel it belongs to
+}
+
+void tensor_note_choice(int bn, int cg, int splits) {
+    t_last_choice[0] = bn; t_last_choice[1] = cg; t_last_choice[2] = splits;
+    t_last_sk[0] = -1; t_last_sk[1] = 0;
 }
 
 bool tensor_ensure_smem_attr(int slot, const void *kernel, int bytes) {

@@ -1,0 +1,92 @@
+"""The kernel for small problems against the oracle: sizes around its tiles (16 / 32 rows, 32 columns, stages of 128 k, pieces of
+16 bytes), every operand orientation, convolutions, and where the rule by size hands over to the other kernels."""
+import numpy as np
+import pytest
+import torch
+
+from helpers import assert_within_bound, operand
+from oracle import ref
+from paper_2202_03293_b200 import binding as sg
+
+pytestmark = pytest.mark.gpu
+SEED = 9300
+
+
+@pytest.fixture(autouse=True)
+def _check():
+    yield
+    sg.sg_check()
+
+
+# one element to several stages and more k than the ring holds; fewer and more tiles than SMs (16- and 32-row tiles)
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("a_t,b_t", [(False, False), (True, False), (False, True), (True, True)])
+@pytest.mark.parametrize("M,N,K", [(8, 8, 8), (16, 32, 128), (24, 40, 136), (136, 72, 256), (128, 128, 392), (8, 40, 704), (3200, 64, 64)])
+def test_small_matmul(M, N, K, a_t, b_t, dtype):
+    A, a = operand((K, M) if a_t else (M, K), SEED, 1, "uniform", dtype)
+    B, b = operand((N, K) if b_t else (K, N), SEED, 2, "uniform", dtype)
+    A, a = (A.t(), np.ascontiguousarray(a.T)) if a_t else (A, a)
+    B, b = (B.t(), np.ascontiguousarray(b.T)) if b_t else (B, b)
+    wide = torch.full((M, N + 4), float("nan"), device="cuda")
+    C = wide[:, :N]
+    sg.sg_matmul(A, B, C)
+    torch.cuda.synchronize()
+    assert sg.sg_last_kernel_name() == f"small_gemm_kernel<{dtype}>"
+    want, S = ref.matmul(a, b)
+    assert assert_within_bound(C, want, S, "small matmul") < 4e-6
+    assert torch.isnan(wide[:, N:]).all()
+    sg.sg_matmul(A, B, C, sg.SG_ACCUMULATE)
+    torch.cuda.synchronize()
+    assert_within_bound(C, 2 * want, 2 * S, "small matmul, accumulate")
+    bias, bias_h = operand((N,), SEED, 3, "normal", "f32")
+    sg.sg_matmul_bias_act(A, B, bias, C, sg.SG_ACT_RELU)
+    torch.cuda.synchronize()
+    want, S = ref.matmul_bias_act(a, b, bias_h, "relu")
+    assert_within_bound(C, want, S, "small matmul, bias + relu")
+
+
+# inputs on both sides of 128 KiB (two forms of the f32 split), strides, dilations, ragged images
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("N,H,W,C,KH,KW,F,st,dl", [(1, 5, 6, 8, 3, 3, 8, (1, 1), (1, 1)), (2, 7, 9, 16, 2, 3, 40, (2, 1), (1, 2)),
+                                                   (1, 55, 55, 32, 3, 3, 64, (2, 2), (1, 1)), (1, 30, 31, 48, 1, 1, 32, (1, 1), (1, 1))])
+def test_small_conv2d(N, H, W, C, KH, KW, F, st, dl, dtype):
+    h_in, w_in = (H - 1) * st[0] + (KH - 1) * dl[0] + 1, (W - 1) * st[1] + (KW - 1) * dl[1] + 1
+    I, i = operand((N, h_in, w_in, C), SEED, 4, "normal", dtype)
+    K, k = operand((KH, KW, C, F), SEED, 5, "normal", dtype)
+    O = torch.full((N, H, W, F), float("nan"), device="cuda")
+    sg.sg_conv2d_nhwc_hwcf(I, K, O, st, dl)
+    torch.cuda.synchronize()
+    assert sg.sg_last_kernel_name() == f"small_gemm_kernel<{dtype}>"
+    want, S = ref.conv2d_nhwc_hwcf(i, k, stride=st, dilation=dl)
+    assert assert_within_bound(O, want, S, "small conv2d") < 4e-6
+
+
+def test_small_conv1d_accumulates_into_a_view():
+    I, i = operand((2, 60, 16), SEED, 6, "uniform", "f32")
+    K, k = operand((3, 16, 24), SEED, 7, "uniform", "f32")
+    O = torch.ones(2, 58, 32, device="cuda")[:, :, :24]
+    sg.sg_conv1d_nwc_wcf(I, K, O, mode=sg.SG_ACCUMULATE)
+    torch.cuda.synchronize()
+    assert sg.sg_last_kernel_name() == "small_gemm_kernel<f32>"
+    want, S = ref.conv1d_nwc_wcf(i, k)
+    assert_within_bound(O, want + 1.0, S + 1.0, "small conv1d, accumulate")
+
+
+def test_small_infinities_and_values_next_to_overflow_keep_their_meaning():
+    A = torch.ones(48, 64, device="cuda")
+    B = torch.full((64, 32), 0.5, device="cuda")
+    A[3, 5], A[4, 6], A[7, 8] = float("inf"), float("-inf"), float("nan")
+    A[9, 1], B[2, 4] = 3.4e38, 2.0
+    C = torch.empty(48, 32, device="cuda")
+    sg.sg_matmul(A, B, C)
+    assert sg.sg_last_kernel_name() == "small_gemm_kernel<f32>"
+    want = A.double() @ B.double()
+    assert torch.equal(torch.isnan(C), torch.isnan(want)) and torch.equal(torch.isinf(C), torch.isinf(want))
+    fine = torch.isfinite(want)
+    assert torch.allclose(C[fine].double(), want[fine], rtol=1e-6)
+
+
+def test_selection_by_size():
+    for M, N, K, small in ((128, 128, 128, True), (256, 256, 256, True), (1024, 1024, 256, False), (784, 128, 1152, False), (64, 64, 4096, False)):
+        sg.sg_matmul(torch.zeros(M, K, device="cuda"), torch.zeros(K, N, device="cuda"), torch.empty(M, N, device="cuda"))
+        assert sg.sg_last_kernel_name() == ("small_gemm_kernel<f32>" if small else "tc_gemm_kernel<f32>"), (M, N, K)

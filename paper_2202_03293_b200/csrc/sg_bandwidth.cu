@@ -37,6 +37,12 @@ __device__ __forceinline__ void mbar_drain(uint32_t bar, uint32_t parity) {
         if (mbar_try_wait(bar, parity)) return;
 }
 
+// Every kernel of this file but the clearing one is launched so that it may start while the kernel ahead of it in the stream
+// drains (a launch costs the host 2.4 instead of 2.9 us that way, and a small kernel's start hides behind its predecessor):
+// it lets the next one start at once and waits for its predecessor before its first global access.
+__device__ __forceinline__ void start_dependents() { asm volatile("griddepcontrol.launch_dependents;"); }
+__device__ __forceinline__ void wait_for_prior() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ------------------------------------------------------------------------------ Copy2D (TMA)
 #ifndef SG_CP_STAGES
 #define SG_CP_STAGES 6
@@ -66,6 +72,7 @@ __global__ void __launch_bounds__(64) copy_tma_kernel(const __grid_constant__ CU
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint64_t full_bar[CP_STAGES], empty_bar[CP_STAGES];
     __shared__ int abort_load, abort_store;
+    start_dependents();
     const uint32_t ring = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
@@ -76,6 +83,7 @@ __global__ void __launch_bounds__(64) copy_tma_kernel(const __grid_constant__ CU
     __syncthreads();
     if (warp == 0 && lane == 0) {
         prefetch_tensormap(&map_src);
+        wait_for_prior();
         int k = 0;
         for (int t = blockIdx.x; t < num_tiles; t += gridDim.x, ++k) {
             const int s = k % CP_STAGES;
@@ -88,6 +96,7 @@ __global__ void __launch_bounds__(64) copy_tma_kernel(const __grid_constant__ CU
             for (int j = (k > CP_STAGES ? k - CP_STAGES : 0); j < k; ++j) mbar_drain(smem_u32(&full_bar[j % CP_STAGES]), (uint32_t)(j / CP_STAGES) & 1u);
     } else if (warp == 1 && lane == 0) {
         prefetch_tensormap(&map_dst);
+        wait_for_prior();
         int k = 0;
         for (int t = blockIdx.x; t < num_tiles; t += gridDim.x, ++k) {
             const int s = k % CP_STAGES;
@@ -148,6 +157,7 @@ __global__ void __launch_bounds__(TR_THREADS) transpose_tma_kernel(const __grid_
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint64_t full_bar[TR_IN_STAGES], empty_bar[TR_IN_STAGES];
     __shared__ int abort_load, abort_turn;
+    start_dependents();
     const uint32_t in_ring = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t out_ring = in_ring + TR_IN_STAGES * TR_TILE_BYTES;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -160,6 +170,7 @@ __global__ void __launch_bounds__(TR_THREADS) transpose_tma_kernel(const __grid_
     if (warp == 0) {
         if (lane == 0) {
             prefetch_tensormap(&map_src);
+            wait_for_prior();
             int k = 0;
             for (int t = blockIdx.x; t < num_tiles; t += gridDim.x, ++k) {
                 const int s = k % TR_IN_STAGES;
@@ -180,6 +191,7 @@ __global__ void __launch_bounds__(TR_THREADS) transpose_tma_kernel(const __grid_
         // 32(w%2) .. +31) nobody else reads, so the four warps never wait for one another.
         const int w = warp - 1;
         if (lane == 0) prefetch_tensormap(&map_dst);
+        wait_for_prior();
         // each lane turns E x E blocks (row group p, 16-byte chunk q); a quarter-warp covers two row groups x four chunks
         const int q = ES == 4 ? ((lane & 3) | ((lane >> 1) & 4)) : (4 * (w & 1) + (lane & 3));
         const int p0 = ES == 4 ? (8 * w + ((lane >> 2) & 1) + 2 * ((lane >> 4) & 1)) : (8 * (w >> 1) + (lane >> 2));
@@ -251,50 +263,76 @@ __global__ void __launch_bounds__(TR_THREADS) transpose_tma_kernel(const __grid_
     __syncthreads();
 }
 
-// ------------------------------------------------------------------ strided 32 x 32 tile kernel
+// ------------------------------------------------------------------------- strided mover
 // dst[i*d_i + j*d_j] = src[i*s_i + j*s_j]; a transpose is the same call with the destination
-// strides exchanged.  WRITE_BY_I: consecutive threads write consecutive i (the destination is
-// contiguous along i), else consecutive j.
-template <typename U, bool WRITE_BY_I>
+// strides exchanged.  MV > 0: the destination is contiguous along i: square tiles of MV elements go through shared memory, a warp
+// reads runs along j and writes runs along i.  Otherwise runs along j on both sides, straight from registers (dense operands
+// arrive here flattened, in units of 16 bytes, with up to 15 bytes left over that block 0 moves).  MV: side of a tile, 64, or
+// 32 while those are too few; 0: no turn.
+// Every thread has sixteen or eight loads in flight: with four, and 32 x 32 tiles, an unaligned 16383 x 12287 transpose
+// ran at 2.4 TB/s.
+template <typename U, int MV>
 __global__ void __launch_bounds__(256) tile_move_kernel(const U *__restrict__ src, int64_t s_i, int64_t s_j, U *__restrict__ dst,
-                                                         int64_t d_i, int64_t d_j, int R, int C, int tiles_j, int64_t num_tiles) {
-    __shared__ U tile[32][33];
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    for (int64_t t = blockIdx.x; t < num_tiles; t += gridDim.x) {
-        const int i0 = (int)(t / tiles_j) * 32, j0 = (int)(t % tiles_j) * 32;
+                                                         int64_t d_i, int64_t d_j, int R, int C, int tiles_i, int tiles_j, int panel,
+                                                         const uint8_t *tail_src, uint8_t *tail_dst, int tail_bytes) {
+    start_dependents();
+    wait_for_prior();
+    if constexpr (MV > 0) {
+        constexpr int H = MV / 32, K = MV / 8;
+        __shared__ U tile[MV][MV + (sizeof(U) == 2 ? 2 : 1)];
+        const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+        const int num_tiles = tiles_i * tiles_j;
+        for (int t = blockIdx.x; t < num_tiles; t += gridDim.x) {
+            int ti, tj;
+            tile_coords(t, tiles_j, tiles_i, panel, ti, tj);
+            const int i0 = ti * MV, j0 = tj * MV;
+            U v[H * K];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const int i = i0 + ty + 8 * k, j = j0 + tx;
-            if (i < R && j < C) tile[ty + 8 * k][tx] = src[(int64_t)i * s_i + (int64_t)j * s_j];
-        }
-        __syncthreads();
+            for (int k = 0; k < K; ++k)
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            if constexpr (WRITE_BY_I) {
-                const int i = i0 + tx, j = j0 + ty + 8 * k;
-                if (i < R && j < C) dst[(int64_t)i * d_i + (int64_t)j * d_j] = tile[tx][ty + 8 * k];
-            } else {
-                const int i = i0 + ty + 8 * k, j = j0 + tx;
-                if (i < R && j < C) dst[(int64_t)i * d_i + (int64_t)j * d_j] = tile[ty + 8 * k][tx];
-            }
+                for (int h = 0; h < H; ++h) {
+                    const int i = i0 + ty + 8 * k, j = j0 + tx + 32 * h;
+                    if (i < R && j < C) v[H * k + h] = src[(int64_t)i * s_i + (int64_t)j * s_j];
+                }
+#pragma unroll
+            for (int k = 0; k < K; ++k)
+#pragma unroll
+                for (int h = 0; h < H; ++h) tile[ty + 8 * k][tx + 32 * h] = v[H * k + h];
+            __syncthreads();
+#pragma unroll
+            for (int k = 0; k < K; ++k)
+#pragma unroll
+                for (int h = 0; h < H; ++h) {
+                    const int i = i0 + tx + 32 * h, j = j0 + ty + 8 * k;
+                    if (i < R && j < C) dst[(int64_t)i * d_i + (int64_t)j * d_j] = tile[tx + 32 * h][ty + 8 * k];
+                }
+            __syncthreads();
         }
-        __syncthreads();
+    } else {
+        // units of 256 * 8 consecutive j of one row
+        const int64_t units_j = ((int64_t)C + 2047) / 2048, units = units_j * R;
+        for (int64_t u = blockIdx.x; u < units; u += gridDim.x) {
+            const int64_t i = u / units_j, j0 = (u - i * units_j) * 2048 + threadIdx.x;
+            const U *s = src + i * s_i;
+            U *d = dst + i * d_i;
+            U v[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                if (j0 + 256 * k < C) v[k] = s[(j0 + 256 * k) * s_j];
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                if (j0 + 256 * k < C) d[(j0 + 256 * k) * d_j] = v[k];
+        }
+        if (blockIdx.x == 0 && threadIdx.x < tail_bytes) tail_dst[threadIdx.x] = tail_src[threadIdx.x];
     }
 }
 
 // --------------------------------------------------------------------------------- reductions
 inline bool aligned16(const void *p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; }
 
-template <typename T, int VEC>
-struct Chunk {
-    float f[VEC];
-};
-
 __device__ __forceinline__ float widen(float x) { return x; }
 __device__ __forceinline__ float widen(uint16_t bits) { return __uint_as_float((uint32_t)bits << 16); }
 
-// Adds up to VEC consecutive elements starting at `ptr` (element stride `sc`) into acc.
-// `nvalid` == VEC takes the 16-byte path (VEC > 1 implies sc == 1 and an aligned address).
 // One whole chunk (VEC > 1: 16 bytes at an aligned address), added element-wise into acc.
 template <typename T, int VEC>
 __device__ __forceinline__ void accumulate_raw(float (&acc)[VEC], const uint4 &raw) {
@@ -311,17 +349,21 @@ __device__ __forceinline__ void accumulate_raw(float (&acc)[VEC], const uint4 &r
     }
 }
 
-template <typename T, int VEC>
-__device__ __forceinline__ void add_chunk(float (&acc)[VEC], const T *ptr, int64_t sc, int nvalid) {
-    if constexpr (VEC > 1) {
-        if (nvalid == VEC) {
-            accumulate_raw<T, VEC>(acc, __ldg(reinterpret_cast<const uint4 *>(ptr)));
-            return;
-        }
-    }
-#pragma unroll
-    for (int v = 0; v < VEC; ++v)
-        if (v < nvalid) acc[v] += widen(__ldg(ptr + (int64_t)v * sc));
+// How the partial sums of a reduction whose reduced index is cut in `splits` ranges (blockIdx.y) meet.
+//   DIRECT   one range.
+//   CLUSTER  the ranges of an output are one thread-block cluster (at most eight); its blocks add each other's shared-memory
+//            sums up in rank order: one launch, a fixed order.
+//   ATOMIC   any number of ranges, float atomics on the output (ATOMIC_V4: dense and aligned, four at a time).
+// `cleared`: the launch runs behind the kernel that clears the output and may have started beside it; the loads need not
+// wait for that kernel, the atomics must.
+enum { DIRECT = 0, CLUSTER = 1, ATOMIC = 2, ATOMIC_V4 = 3 };
+struct Meeting {
+    int how, cleared, accumulate;
+};
+__device__ __forceinline__ float remote_float(uint32_t addr, int rank) {
+    float v;
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(map_to_cta(addr, (uint32_t)rank)) : "memory");
+    return v;
 }
 
 // Rows r, r+rp, ... < r1 of one chunk, eight loads in flight.  FULL: the chunk has all VEC columns (16-byte loads).
@@ -338,6 +380,11 @@ __device__ __forceinline__ void colred_walk(float (&acc)[VEC], const T *base, in
 #pragma unroll
             for (int u = 0; u < U; ++u) accumulate_raw<T, VEC>(acc, raw[u]);
         }
+        uint4 raw[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) raw[u] = r + u * rp < r1 ? __ldg(reinterpret_cast<const uint4 *>(base + (r + u * rp) * ld)) : make_uint4(0, 0, 0, 0);
+#pragma unroll
+        for (int u = 0; u < U; ++u) accumulate_raw<T, VEC>(acc, raw[u]);
     } else {
         for (; r + (U - 1) * rp < r1; r += U * rp) {
             float part[U];
@@ -352,21 +399,25 @@ __device__ __forceinline__ void colred_walk(float (&acc)[VEC], const T *base, in
                 }
             }
         }
+        for (; r < r1; r += rp)
+#pragma unroll
+            for (int v = 0; v < VEC; ++v)
+                if (v < nvalid) acc[v] += widen(__ldg(base + r * ld + (int64_t)v * sc));
     }
-    for (; r < r1; r += rp) add_chunk<T, VEC>(acc, base + r * ld, sc, FULL ? VEC : nvalid);
 }
 
-// ColRed2D.  A CTA owns `cw` chunks of VEC columns and the rows [r0, r1) of its split;
+// ColRed2D.  A CTA owns `cw` chunks of VEC columns (a power of two, or at least 32) and the rows [r0, r1) of its range;
 // thread (g, cc) = (t / cw, t % cw) walks rows r0+g, r0+g+rp, ... of chunk cc.
 template <typename T, int VEC>
 __global__ void __launch_bounds__(256) colred_kernel(const T *__restrict__ A, int64_t ld, int64_t sc, int R, int C,
-                                                      float *__restrict__ out, int64_t os, int cw, int rp, int rows_per_split,
-                                                      int use_atomic, int accumulate) {
+                                                      float *__restrict__ out, int64_t os, int cw, int rp, int rows_per_split, Meeting meet) {
     __shared__ float red[256][VEC + 1];
+    start_dependents();
+    if (!meet.cleared) wait_for_prior();
     const int t = threadIdx.x, g = t / cw, cc = t - g * cw;
     const int64_t col0 = ((int64_t)blockIdx.x * cw + cc) * VEC;
-    const int r0 = blockIdx.y * rows_per_split;
-    const int r1 = min(R, r0 + rows_per_split);
+    const int64_t r0 = (int64_t)blockIdx.y * rows_per_split;
+    const int64_t r1 = min((int64_t)R, r0 + rows_per_split);
     float acc[VEC];
 #pragma unroll
     for (int v = 0; v < VEC; ++v) acc[v] = 0.f;
@@ -377,16 +428,51 @@ __global__ void __launch_bounds__(256) colred_kernel(const T *__restrict__ A, in
         if (nvalid == VEC) colred_walk<T, VEC, true>(acc, base, ld, sc, r0 + g, r1, rp, VEC);
         else colred_walk<T, VEC, false>(acc, base, ld, sc, r0 + g, r1, rp, nvalid);
     }
+    // a warp that holds several row groups of a chunk adds them up first: one group per warp is left
+    const bool fold = cw < 32 && (cw & (cw - 1)) == 0;
+    for (int off = fold ? 16 : 0; off >= cw; off >>= 1)
 #pragma unroll
-    for (int v = 0; v < VEC; ++v) red[t][v] = acc[v];
+        for (int v = 0; v < VEC; ++v) acc[v] += __shfl_xor_sync(0xffffffffu, acc[v], off);
+    const int groups = fold ? 8 : rp;
+    const int slot = fold ? ((t & 31) < cw ? (t >> 5) * cw + (t & 31) : -1) : t;
+    if (slot >= 0)
+#pragma unroll
+        for (int v = 0; v < VEC; ++v) red[slot][v] = acc[v];
     __syncthreads();
-    // (after the clearing kernel of an overwriting split reduction; this grid may have started beside it)
-    if (use_atomic) asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (g == 0 && col0 < C) {
-        for (int gg = 1; gg < rp; ++gg)
+    if (meet.how == CLUSTER) {
+        // every block's sums of a column in red[chunk][v], then output o of the chunks by block o / 256 mod splits
+        for (int o = t; o < cw * VEC; o += 256) {
+            const int c = o / VEC, v = o - c * VEC;
+            float s = red[c][v];
+            for (int gg = 1; gg < groups; ++gg) s += red[gg * cw + c][v];
+            red[c][v] = s;
+        }
+        cluster_sync_all();
+        const int splits = (int)gridDim.y, rank = (int)blockIdx.y;
+        for (int o = rank * 256 + t; o < cw * VEC; o += splits * 256) {
+            const int c = o / VEC, v = o - c * VEC;
+            const int64_t col = ((int64_t)blockIdx.x * cw + c) * VEC + v;
+            if (col >= C) continue;
+            float part[8];
+#pragma unroll
+            for (int s = 0; s < 8; ++s) part[s] = s < splits ? remote_float(smem_u32(&red[c][v]), s) : 0.f;
+            float sum = part[0];
+#pragma unroll
+            for (int s = 1; s < 8; ++s) sum += part[s];
+            float *dst = out + col * os;
+            *dst = (meet.accumulate ? *dst : 0.f) + sum;
+        }
+        cluster_sync_all();       // nobody leaves while its sums are being read
+        return;
+    }
+    if (meet.cleared) wait_for_prior();
+    if (t < cw && col0 < C) {
+#pragma unroll
+        for (int v = 0; v < VEC; ++v) acc[v] = red[t][v];
+        for (int gg = 1; gg < groups; ++gg)
 #pragma unroll
             for (int v = 0; v < VEC; ++v) acc[v] += red[gg * cw + cc][v];
-        if (VEC >= 4 && use_atomic == 2 && nvalid == VEC) {
+        if (VEC >= 4 && meet.how == ATOMIC_V4 && nvalid == VEC) {
             // dense, 16-byte aligned output: four sums per atomic
 #pragma unroll
             for (int v = 0; v < VEC; v += 4)
@@ -398,164 +484,231 @@ __global__ void __launch_bounds__(256) colred_kernel(const T *__restrict__ A, in
         for (int v = 0; v < VEC; ++v) {
             if (v < nvalid) {
                 float *o = out + (col0 + v) * os;
-                if (use_atomic) atomicAdd(o, acc[v]);
-                else *o = (accumulate ? *o : 0.f) + acc[v];
+                if (meet.how >= ATOMIC) atomicAdd(o, acc[v]);
+                else *o = (meet.accumulate ? *o : 0.f) + acc[v];
             }
         }
     }
 }
 
-// RowRed2D.  `lanes` (a power of two <= 32) lanes share a row; a warp holds 32/lanes rows.
-// blockIdx.y selects the column range [c0, c1) of a split (whole chunks except at the end).
+// RowRed2D.  `threads` (a power of two <= 256) threads share a row; blockIdx.y selects the column range [c0, c1) of a split.
+// VEC > 1: unit column stride; the elements ahead of the first and behind the last 16-byte boundary of the row are added one
+// by one (rows may start anywhere).
 template <typename T, int VEC>
 __global__ void __launch_bounds__(256) rowred_kernel(const T *__restrict__ A, int64_t ld, int64_t sc, int R, int C,
-                                                      float *__restrict__ out, int64_t os, int lanes, int cols_per_split,
-                                                      int use_atomic, int accumulate) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int rows_per_warp = 32 / lanes;
-    const int64_t row = ((int64_t)blockIdx.x * 8 + warp) * rows_per_warp + lane / lanes;
-    const int sub = lane % lanes;
-    const int c0 = blockIdx.y * cols_per_split;
-    const int c1 = min(C, c0 + cols_per_split);
+                                                      float *__restrict__ out, int64_t os, int threads, int cols_per_split, Meeting meet) {
+    __shared__ float red[8];
+    start_dependents();
+    if (!meet.cleared) wait_for_prior();
+    const int rows_per_cta = 256 / threads;
+    const int64_t row = (int64_t)blockIdx.x * rows_per_cta + threadIdx.x / threads;
+    const int sub = threadIdx.x % threads;
+    const int64_t c0 = (int64_t)blockIdx.y * cols_per_split;
+    const int64_t c1 = min((int64_t)C, c0 + cols_per_split);
     float acc[VEC];
 #pragma unroll
     for (int v = 0; v < VEC; ++v) acc[v] = 0.f;
     if (row < R && c0 < c1) {
         const T *base = A + row * ld;
-        const int full_end = c0 + (c1 - c0) / VEC * VEC;      // whole chunks
-        int64_t c = c0 + sub * VEC;
-        const int64_t step = lanes * VEC;
         if constexpr (VEC > 1) {
-            for (; c + 7 * step < full_end; c += 8 * step) {      // eight 16-byte loads in flight
+            const int64_t head = min(c1 - c0, (int64_t)((16 - (reinterpret_cast<uintptr_t>(base + c0) & 15)) & 15) / (int64_t)sizeof(T));
+            const int64_t body0 = c0 + head, body1 = body0 + (c1 - body0) / VEC * VEC;
+            const int64_t step = (int64_t)threads * VEC;
+            int64_t c = body0 + sub * VEC;
+            for (; c + 7 * step < body1; c += 8 * step) {      // eight 16-byte loads in flight
                 uint4 raw[8];
 #pragma unroll
                 for (int u = 0; u < 8; ++u) raw[u] = __ldg(reinterpret_cast<const uint4 *>(base + c + u * step));
 #pragma unroll
                 for (int u = 0; u < 8; ++u) accumulate_raw<T, VEC>(acc, raw[u]);
             }
+            if (c < body1) {
+                uint4 raw[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) raw[u] = c + u * step < body1 ? __ldg(reinterpret_cast<const uint4 *>(base + c + u * step)) : make_uint4(0, 0, 0, 0);
+#pragma unroll
+                for (int u = 0; u < 8; ++u) accumulate_raw<T, VEC>(acc, raw[u]);
+            }
+            for (int64_t e = sub; e < head + (c1 - body1); e += threads)
+                acc[0] += widen(__ldg(base + (e < head ? c0 + e : body1 + (e - head))));
         } else {
-            for (; c + 7 * step < full_end; c += 8 * step) {
+            const int64_t step = threads;
+            int64_t c = c0 + sub;
+            for (; c + 7 * step < c1; c += 8 * step) {
                 float part[8];
 #pragma unroll
                 for (int u = 0; u < 8; ++u) part[u] = widen(__ldg(base + (c + u * step) * sc));
                 acc[0] += ((part[0] + part[1]) + (part[2] + part[3])) + ((part[4] + part[5]) + (part[6] + part[7]));
             }
-        }
-        for (; c < full_end; c += step) add_chunk<T, VEC>(acc, base + c * sc, sc, VEC);
-        if (VEC > 1 && sub == 0 && full_end < c1) {            // the ragged end of the range, element by element
-            float tail = 0.f;
-            for (int cc = full_end; cc < c1; ++cc) tail += widen(__ldg(base + (int64_t)cc * sc));
-            acc[0] += tail;
+            for (; c < c1; c += step) acc[0] += widen(__ldg(base + c * sc));
         }
     }
     float sum = acc[0];
 #pragma unroll
     for (int v = 1; v < VEC; ++v) sum += acc[v];
-    for (int off = lanes >> 1; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
-    if (use_atomic) asm volatile("griddepcontrol.wait;" ::: "memory");
+    for (int off = min(threads, 32) >> 1; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+    if (threads > 32) {
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sum;
+        __syncthreads();
+        if (sub == 0)
+            for (int w = 1; w < threads / 32; ++w) sum += red[(threadIdx.x >> 5) + w];
+    }
+    if (meet.how == CLUSTER) {       // (one row per block)
+        if (threadIdx.x == 0) red[0] = sum;
+        cluster_sync_all();
+        if (blockIdx.y == 0 && threadIdx.x == 0) {
+            sum = 0.f;
+            for (int s = 0; s < (int)gridDim.y; ++s) sum += remote_float(smem_u32(&red[0]), s);
+            float *o = out + row * os;
+            *o = (meet.accumulate ? *o : 0.f) + sum;
+        }
+        cluster_sync_all();
+        return;
+    }
+    if (meet.cleared) wait_for_prior();
     if (sub == 0 && row < R && (c0 < c1 || blockIdx.y == 0)) {
         float *o = out + row * os;
-        if (use_atomic) atomicAdd(o, sum);
-        else *o = (accumulate ? *o : 0.f) + sum;
+        if (meet.how >= ATOMIC) atomicAdd(o, sum);
+        else *o = (meet.accumulate ? *o : 0.f) + sum;
     }
 }
 
 __global__ void zero_vector_kernel(float *__restrict__ out, int64_t n, int64_t os) {
-    asm volatile("griddepcontrol.launch_dependents;");   // the reduction behind it may start; it waits before its atomics
+    wait_for_prior();
+    start_dependents();       // the reduction behind it may start (everything ahead has finished); it waits before its atomics
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) out[i * os] = 0.f;
 }
 
-// Launches `kernel`; `after_clear`: a clearing kernel was just enqueued ahead of it and the launch may overlap it
-// (programmatic dependent launch; the kernel waits for the clearing grid before its first atomic).
+// Launches `kernel` so that it may start while the kernel ahead of it drains; `cluster`: blocks of a cluster along y.
 template <typename... KArgs, typename... Args>
-cudaError_t launch_reduction(void (*kernel)(KArgs...), dim3 grid, bool after_clear, cudaStream_t stream, Args... args) {
+cudaError_t launch_overlapped(void (*kernel)(KArgs...), dim3 grid, int block, int smem, int cluster, cudaStream_t stream, Args... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
-    cfg.blockDim = dim3(256, 1, 1);
+    cfg.blockDim = dim3(block, 1, 1);
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = 1; attr[1].val.clusterDim.y = cluster; attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = after_clear ? 1 : 0;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
+    count_launch();
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+inline cudaError_t launch_clear(float *out, int64_t n, int64_t os, cudaStream_t stream) {
+    return launch_overlapped(zero_vector_kernel, dim3((unsigned)std::min<int64_t>((n + 255) / 256, 1184)), 256, 0, 1, stream, out, n, os);
 }
 
 template <typename T, int VEC>
 cudaError_t launch_reduce_typed(bool colred, const T *A, int64_t ld, int64_t sc, int R, int C, float *out, int64_t os,
-                                int accumulate, int num_sms, cudaStream_t stream) {
-    const int target_ctas = num_sms * 8;
+                                int accumulate, int num_sms, bool vec_name, cudaStream_t stream) {
+    // one thread block per batch of eight 16-byte loads per thread: more blocks than this would not even do that
+    const int64_t batches = std::max<int64_t>(1, (int64_t)R * ((C + VEC - 1) / VEC) / (256 * 8));
     if (!colred) {
-        // RowRed2D: one output per row
+        // RowRed2D, one output per row, `threads` per row: of the powers of two the one with the least (waves of thread blocks) x
+        // (loads of a thread + eight loads' worth of latency).  Long rows of matrices that do not fill the chip are cut in up to
+        // eight ranges of a cluster, and beyond that by atomics.
         const int chunks = (C + VEC - 1) / VEC;
-        int lanes = 1;
-        while (lanes < 32 && lanes < chunks) lanes <<= 1;
-        const int rows_per_cta = 8 * (32 / lanes);
-        const int64_t row_ctas = ((int64_t)R + rows_per_cta - 1) / rows_per_cta;
+        int threads = 1;
+        double best = 1e30;
+        for (int t = 1; t <= 256 && (t == 1 || t / 2 < chunks); t <<= 1) {
+            const double x = (double)(((int64_t)R + 256 / t - 1) / (256 / t)) / (6 * num_sms);
+            const double cost = (x <= 1 ? 1 : x <= 2 ? 2 : x) * (8 + (chunks + t - 1) / t) * (t < 8 ? 16 / t : 1);      // (rows below 128 bytes a request)
+            if (cost < best) { best = cost; threads = t; }
+        }
+        const int64_t row_ctas = ((int64_t)R + 256 / threads - 1) / (256 / threads);
         int splits = 1;
-        const int min_chunks_per_split = lanes * 16;
-        if (row_ctas < target_ctas && chunks > min_chunks_per_split)
-            splits = (int)std::min<int64_t>((target_ctas + row_ctas - 1) / row_ctas, (chunks + min_chunks_per_split - 1) / min_chunks_per_split);
+        Meeting meet{DIRECT, 0, accumulate};
+        if (threads == 256 && row_ctas < 4 * num_sms && chunks > 256 * 8) {
+            const int64_t want = std::min<int64_t>((4 * num_sms + row_ctas - 1) / row_ctas, (chunks + 256 * 8 - 1) / (256 * 8));
+            splits = 1;
+            while (splits < want && splits < 8) splits <<= 1;
+            meet.how = CLUSTER;
+            if (want > 16) { splits = (int)want; meet.how = ATOMIC; }
+        }
         int chunks_per_split = (chunks + splits - 1) / splits;
-        chunks_per_split = (chunks_per_split + lanes - 1) / lanes * lanes;
-        splits = (chunks + chunks_per_split - 1) / chunks_per_split;
-        const int use_atomic = splits > 1;
-        if (use_atomic && !accumulate) {
-            zero_vector_kernel<<<(int)std::min<int64_t>(((int64_t)R + 255) / 256, 1184), 256, 0, stream>>>(out, R, os);
-            count_launch();
+        if (meet.how == ATOMIC) splits = (chunks + chunks_per_split - 1) / chunks_per_split;
+        if (splits == 1) meet.how = DIRECT;
+        if (meet.how == ATOMIC && !accumulate) {
+            const cudaError_t e = launch_clear(out, R, os, stream);
+            if (e != cudaSuccess) return e;
+            meet.cleared = 1;
         }
-        const cudaError_t e = launch_reduction(rowred_kernel<T, VEC>, dim3((unsigned)row_ctas, (unsigned)splits), use_atomic && !accumulate, stream,
-                                               A, ld, sc, R, C, out, os, lanes, chunks_per_split * VEC, use_atomic, accumulate);
-        count_launch();
-        note_kernel(VEC > 1 ? "rowred_kernel<vec>" : "rowred_kernel<scalar>");
-        return e;
-    } else {
-        // ColRed2D: one output per column
-        const int64_t chunks = ((int64_t)C + VEC - 1) / VEC;
-        const int cw = (int)std::min<int64_t>(chunks, 256);
-        const int rp = 256 / cw;
-        const int64_t col_blocks = (chunks + cw - 1) / cw;
-        // row ranges: as many as give every SM its full set of resident thread blocks, in one wave
-        static int resident = 0;
-        if (resident == 0) {
-            int n = 0;
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, colred_kernel<T, VEC>, 256, 0) != cudaSuccess || n < 1) n = 2;
-            resident = n;
-        }
-        int splits = 1;
-        const int min_rows_per_split = rp * 16;
-        const int64_t wave = (int64_t)num_sms * resident;
-        if (col_blocks < wave && R > min_rows_per_split)
-            splits = (int)std::min<int64_t>(wave / col_blocks, ((int64_t)R + min_rows_per_split - 1) / min_rows_per_split);
-        int rows_per_split = (R + splits - 1) / splits;
-        rows_per_split = (rows_per_split + rp - 1) / rp * rp;
-        splits = (R + rows_per_split - 1) / rows_per_split;
-        // 2: the output is dense and 16-byte aligned, so whole chunks may use vector atomics
-        const int use_atomic = splits > 1 ? ((os == 1 && aligned16(out)) ? 2 : 1) : 0;
-        if (use_atomic && !accumulate) {
-            zero_vector_kernel<<<(int)std::min<int64_t>(((int64_t)C + 255) / 256, 1184), 256, 0, stream>>>(out, C, os);
-            count_launch();
-        }
-        const cudaError_t e = launch_reduction(colred_kernel<T, VEC>, dim3((unsigned)col_blocks, (unsigned)splits), use_atomic && !accumulate, stream,
-                                               A, ld, sc, R, C, out, os, cw, rp, rows_per_split, use_atomic, accumulate);
-        count_launch();
-        note_kernel(VEC > 1 ? "colred_kernel<vec>" : "colred_kernel<scalar>");
-        return e;
+        note_kernel(vec_name ? "rowred_kernel<vec>" : "rowred_kernel<scalar>");
+        return launch_overlapped(rowred_kernel<T, VEC>, dim3((unsigned)row_ctas, (unsigned)splits), 256, 0, meet.how == CLUSTER ? splits : 1, stream,
+                                 A, ld, sc, R, C, out, os, threads, chunks_per_split * VEC, meet);
     }
+    // ColRed2D, one output per column
+    const int64_t chunks = ((int64_t)C + VEC - 1) / VEC;
+    note_kernel(vec_name ? "colred_kernel<vec>" : "colred_kernel<scalar>");
+    static const int resident = [] {
+        int n = 0;
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, colred_kernel<T, VEC>, 256, 0) == cudaSuccess && n > 0 ? n : 2;
+    }();
+    const int64_t wave = (int64_t)num_sms * resident;
+    // Up to 48 MB (element by element 4): clusters of up to eight row ranges over the widest column blocks that fill most of a wave: one launch, no
+    // atomics.  (Larger tensors stream better in whole rows, and the second launch no longer matters.)
+    if ((int64_t)R * C * (int64_t)sizeof(T) < ((int64_t)(VEC > 1 ? 48 : 4) << 20)) {
+        const double target = 0.6 * (double)std::min<int64_t>(wave, batches);
+        for (int cw = 256; cw >= 8; cw >>= 1) {
+            if (cw > 8 && cw / 2 >= chunks) continue;                   // half of the chunk lanes would be idle
+            const int rp = 256 / cw;
+            const int64_t col_blocks = (chunks + cw - 1) / cw;
+            const int splits = (int)std::max<int64_t>(1, std::min<int64_t>({8, wave / col_blocks, ((int64_t)R + rp * 8 - 1) / (rp * 8)}));
+            if ((double)(col_blocks * splits) < target) continue;
+            const Meeting meet{splits > 1 ? CLUSTER : DIRECT, 0, accumulate};
+            return launch_overlapped(colred_kernel<T, VEC>, dim3((unsigned)col_blocks, (unsigned)splits), 256, 0, splits, stream, A, ld, sc, R, C, out,
+                                     os, cw, rp, (R + splits - 1) / splits, meet);
+        }
+    }
+    // row ranges: as many as give every SM its full set of resident thread blocks, in one wave
+    const int cw = (int)std::min<int64_t>(chunks, 256);
+    const int rp = 256 / cw;
+    const int64_t col_blocks = (chunks + cw - 1) / cw;
+    int splits = 1;
+    const int min_rows_per_split = rp * 16;
+    if (col_blocks < wave && R > min_rows_per_split)
+        splits = (int)std::min<int64_t>(wave / col_blocks, ((int64_t)R + min_rows_per_split - 1) / min_rows_per_split);
+    int rows_per_split = (R + splits - 1) / splits;
+    rows_per_split = (rows_per_split + rp - 1) / rp * rp;
+    splits = (R + rows_per_split - 1) / rows_per_split;
+    Meeting meet{splits == 1 ? DIRECT : (os == 1 && aligned16(out)) ? ATOMIC_V4 : ATOMIC, 0, accumulate};
+    if (meet.how >= ATOMIC && !accumulate) {
+        const cudaError_t e = launch_clear(out, C, os, stream);
+        if (e != cudaSuccess) return e;
+        meet.cleared = 1;
+    }
+    return launch_overlapped(colred_kernel<T, VEC>, dim3((unsigned)col_blocks, (unsigned)splits), 256, 0, 1, stream, A, ld, sc, R, C, out, os, cw, rp,
+                             rows_per_split, meet);
 }
 
 template <typename U>
 cudaError_t launch_tile_move(const U *src, int64_t s_i, int64_t s_j, U *dst, int64_t d_i, int64_t d_j, int R, int C, int num_sms,
                              cudaStream_t stream, bool note = true) {
-    const int tiles_j = (C + 31) / 32;
-    const int64_t num_tiles = (int64_t)((R + 31) / 32) * tiles_j;
-    const int grid = (int)std::min<int64_t>(num_tiles, (int64_t)num_sms * 8);
-    // write along whichever destination index is closer to contiguous
-    if (d_i < d_j) tile_move_kernel<U, true><<<grid, 256, 0, stream>>>(src, s_i, s_j, dst, d_i, d_j, R, C, tiles_j, num_tiles);
-    else tile_move_kernel<U, false><<<grid, 256, 0, stream>>>(src, s_i, s_j, dst, d_i, d_j, R, C, tiles_j, num_tiles);
-    count_launch();
     if (note) note_kernel("tile_move_kernel");
-    return cudaGetLastError();
+    // write along whichever destination index is closer to contiguous
+    if (d_i < d_j && R > 1) {
+        const int mv = (int64_t)((R + 63) / 64) * ((C + 63) / 64) < 2 * num_sms ? 32 : 64;
+        const int tiles_i = (R + mv - 1) / mv, tiles_j = (C + mv - 1) / mv;
+        if ((int64_t)tiles_i * tiles_j > 0x7fffffff) return cudaErrorInvalidConfiguration;
+        const int grid = std::min(tiles_i * tiles_j, num_sms * 8);
+        return launch_overlapped(mv == 32 ? tile_move_kernel<U, 32> : tile_move_kernel<U, 64>, dim3(grid), 256, 0, 1, stream, src, s_i, s_j, dst, d_i, d_j, R, C, tiles_i, tiles_j,
+                                 std::min(tiles_j, TR_PANEL), (const uint8_t *)nullptr, (uint8_t *)nullptr, 0);
+    }
+    const int64_t bytes = (int64_t)R * C * (int64_t)sizeof(U);
+    if (s_j == 1 && d_j == 1 && (R == 1 || (s_i == C && d_i == C)) && aligned16(src) && aligned16(dst) && bytes / 16 < 0x7fffffff) {
+        // dense on both sides: one run of memory
+        const int n16 = (int)(bytes / 16), tail = (int)(bytes % 16);
+        const int grid = (int)std::min<int64_t>(((int64_t)n16 + 2047) / 2048 + (n16 == 0), (int64_t)num_sms * 8);
+        return launch_overlapped(tile_move_kernel<uint4, 0>, dim3(grid), 256, 0, 1, stream, reinterpret_cast<const uint4 *>(src), 0, 1,
+                                 reinterpret_cast<uint4 *>(dst), 0, 1, 1, n16, 0, 0, 0, reinterpret_cast<const uint8_t *>(src) + (int64_t)n16 * 16,
+                                 reinterpret_cast<uint8_t *>(dst) + (int64_t)n16 * 16, tail);
+    }
+    const int64_t units = (((int64_t)C + 2047) / 2048) * R;
+    return launch_overlapped(tile_move_kernel<U, 0>, dim3((unsigned)std::min<int64_t>(units, (int64_t)num_sms * 8)), 256, 0, 1, stream, src, s_i, s_j, dst,
+                             d_i, d_j, R, C, 0, 0, 0, (const uint8_t *)nullptr, (uint8_t *)nullptr, 0);
 }
 
 // device on which each kernel's shared-memory limit was last raised (the attribute is per device)
@@ -587,7 +740,9 @@ sg_status launch_move2d(bool transpose, int64_t R, int64_t C, const void *src, i
         if (!transpose) {
             // box: up to 256 elements wide, as many rows as fit a 32 KB stage
             const int box_x = (int)std::min<int64_t>(SG_CP_BOX_X, Cb);
-            const int box_y = (int)std::min<int64_t>(std::min<int64_t>(256, CP_STAGE_BYTES / (box_x * esize)), Rb);
+            int box_y = (int)std::min<int64_t>(std::min<int64_t>(256, CP_STAGE_BYTES / (box_x * esize)), Rb);
+            // (a small tensor: rather a box per SM than whole stages; 250 x 960 f32 2.75 -> 2.1 us)
+            while (box_y > 4 && ((Cb + box_x - 1) / box_x) * ((Rb + box_y - 1) / box_y) < num_sms) box_y = (box_y + 1) / 2;
             cuuint64_t dims[2] = {(cuuint64_t)Cb, (cuuint64_t)Rb};
             cuuint32_t box[2] = {(cuuint32_t)box_x, (cuuint32_t)box_y};
             const int64_t tiles_x = (Cb + box_x - 1) / box_x, tiles_y = (Rb + box_y - 1) / box_y;
@@ -603,8 +758,8 @@ sg_status launch_move2d(bool transpose, int64_t R, int64_t C, const void *src, i
                     g_attr_copy = dev;
                 }
                 const int num_tiles = (int)(tiles_x * tiles_y);
-                copy_tma_kernel<<<std::min(num_tiles, CP_CTAS_PER_SM * num_sms), 64, smem, stream>>>(map_src, map_dst, (int)tiles_x, num_tiles, box_x, box_y,
-                                                                                    (uint32_t)(box_x * box_y * esize));
+                if (launch_overlapped(copy_tma_kernel, dim3(std::min(num_tiles, CP_CTAS_PER_SM * num_sms)), 64, smem, 1, stream, map_src, map_dst, (int)tiles_x,
+                                      num_tiles, box_x, box_y, (uint32_t)(box_x * box_y * esize)) != cudaSuccess) return SG_ERR_CUDA;
                 launched = true;
             }
         } else {
@@ -630,16 +785,14 @@ sg_status launch_move2d(bool transpose, int64_t R, int64_t C, const void *src, i
                 const int num_tiles = (int)(tiles_c * tiles_r);
                 const int grid = std::min(num_tiles, 2 * num_sms);
                 const int panel = (int)std::min<int64_t>(tiles_c, TR_PANEL);
-                if (esize == 4) transpose_tma_kernel<4><<<grid, TR_THREADS, smem, stream>>>(map_src, map_dst, (int)tiles_c, (int)tiles_r, panel, (int)Rb, (int)Cb);
-                else transpose_tma_kernel<2><<<grid, TR_THREADS, smem, stream>>>(map_src, map_dst, (int)tiles_c, (int)tiles_r, panel, (int)Rb, (int)Cb);
+                if (launch_overlapped(esize == 4 ? transpose_tma_kernel<4> : transpose_tma_kernel<2>, dim3(grid), TR_THREADS, smem, 1, stream, map_src, map_dst,
+                                      (int)tiles_c, (int)tiles_r, panel, (int)Rb, (int)Cb) != cudaSuccess) return SG_ERR_CUDA;
                 launched = true;
             }
         }
         if (launched) {
-            count_launch();
             note_kernel(transpose ? "transpose_tma_kernel" : "copy_tma_kernel");
             *used_tma = 1;
-            if (cudaGetLastError() != cudaSuccess) return SG_ERR_CUDA;
             if (tail == 0) return SG_OK;
             // the last `tail` columns of the destination: source rows [body, R) of a transpose, columns [body, C) of a copy
             const char *s_tail = static_cast<const char *>(src) + (transpose ? body * s_r : body * s_c) * esize;
@@ -668,23 +821,22 @@ sg_status launch_reduce2d(bool colred, int64_t R, int64_t C, const void *A, int6
     const int64_t n_out = colred ? C : R, n_red = colred ? R : C;
     if (n_red == 0) {      // empty sum: the neutral value
         if (!accumulate) {
-            zero_vector_kernel<<<(int)std::min<int64_t>((n_out + 255) / 256, 1184), 256, 0, stream>>>(out, n_out, os);
-            count_launch();
-            if (cudaGetLastError() != cudaSuccess) return SG_ERR_CUDA;
+            if (launch_clear(out, n_out, os, stream) != cudaSuccess) return SG_ERR_CUDA;
         }
         return SG_OK;
     }
     const int es = in_bf16 ? 2 : 4;
-    const bool vec_ok = a_c == 1 && aligned16(A) && (a_r * es) % 16 == 0;
+    // 16-byte loads: rows of unit stride that start on 16-byte boundaries; a row reduction peels the ends of rows that do not
+    const bool aligned = a_c == 1 && aligned16(A) && (a_r * es) % 16 == 0, vec = aligned || (!colred && a_c == 1);
     cudaError_t e;
     if (in_bf16) {
         const uint16_t *p = static_cast<const uint16_t *>(A);
-        e = vec_ok ? launch_reduce_typed<uint16_t, 8>(colred, p, a_r, a_c, (int)R, (int)C, out, os, accumulate, num_sms, stream)
-                   : launch_reduce_typed<uint16_t, 1>(colred, p, a_r, a_c, (int)R, (int)C, out, os, accumulate, num_sms, stream);
+        e = vec ? launch_reduce_typed<uint16_t, 8>(colred, p, a_r, a_c, (int)R, (int)C, out, os, accumulate, num_sms, aligned, stream)
+                : launch_reduce_typed<uint16_t, 1>(colred, p, a_r, a_c, (int)R, (int)C, out, os, accumulate, num_sms, aligned, stream);
     } else {
         const float *p = static_cast<const float *>(A);
-        e = vec_ok ? launch_reduce_typed<float, 4>(colred, p, a_r, a_c, (int)R, (int)C, out, os, accumulate, num_sms, stream)
-                   : launch_reduce_typed<float, 1>(colred, p, a_r, a_c, (int)R, (int)C, out, os, accumulate, num_sms, stream);
+        e = vec ? launch_reduce_typed<float, 4>(colred, p, a_r, a_c, (int)R, (int)C, out, os, accumulate, num_sms, aligned, stream)
+                : launch_reduce_typed<float, 1>(colred, p, a_r, a_c, (int)R, (int)C, out, os, accumulate, num_sms, aligned, stream);
     }
     return e == cudaSuccess ? SG_OK : SG_ERR_CUDA;
 }

@@ -1,0 +1,42 @@
+"""Where the reductions' plans and the strided mover's forms change: column blocks of 8 to 256 chunks, one to eight ranges in a
+cluster, atomics; one to 256 threads a row, rows that start anywhere; dense unaligned copies, 32- and 64-element tiles."""
+import numpy as np
+import pytest
+import torch
+
+from helpers import assert_within_bound, operand
+from oracle import ref
+from paper_2202_03293_b200 import binding as sg
+
+pytestmark = pytest.mark.gpu
+SEED = 9500
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("R,C,off", [(7, 4, 0), (9, 960, 0), (65, 2040, 0), (1000, 64, 0), (1030, 136, 0), (3000, 2048, 0), (40000, 24, 0), (5, 40000, 0),
+                                     (3, 70001, 0), (1, 300001, 0), (2100, 37, 1), (33, 1021, 3), (2, 9, 1), (600, 5000, 1)])
+def test_reductions(R, C, off, dtype):
+    A, a = operand((R, C + off), SEED, 1, "uniform", dtype)
+    A, a = A[:, off:], a[:, off:]
+    for fn, oracle, n in ((sg.sg_colred2d, ref.colred2d, C), (sg.sg_rowred2d, ref.rowred2d, R)):
+        out = torch.full((n, 2), float("nan"), device="cuda")
+        fn(A, out[:, 0])
+        fn(A, out[:, 0], sg.SG_ACCUMULATE)
+        torch.cuda.synchronize()
+        want, S = oracle(np.ascontiguousarray(a))
+        assert assert_within_bound(out[:, 0], 2 * want, 2 * S, fn.__name__) < 1e-5
+        assert torch.isnan(out[:, 1]).all()
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("R,C", [(1, 3), (3, 5), (31, 33), (65, 63), (255, 961), (1200, 1301), (2049, 127)])
+def test_unaligned_moves(R, C, dtype):
+    A = torch.randn(R, C, device="cuda").to(dtype)
+    back = torch.zeros(R * C + 8, device="cuda", dtype=dtype)
+    D = back[:R * C].view(R, C)
+    sg.sg_copy2d(A, D)
+    T = torch.zeros(C, R + 1, device="cuda", dtype=dtype)
+    sg.sg_transpose2d(A, T[:, :R])
+    torch.cuda.synchronize()
+    assert torch.equal(D, A) and not back[R * C:].any()
+    assert torch.equal(T[:, :R], A.t()) and not T[:, R].any()

@@ -258,7 +258,7 @@ int sg_last_kernel(void);
  * Name of the compute kernel that call launched (a static string, "" before any call; clearing
  * kernels launched ahead of it are not named): "tc_gemm_kernel<bf16>", "tc_gemm_kernel<f32>",
  * "gather_gemm_kernel<bf16>", "gather_gemm_kernel<f32>" (layouts outside the TMA rules), "small_gemm_kernel<bf16>",
- * "small_gemm_kernel<f32>", "conv_strip_kernel<bf16>", "conv_strip_kernel<f32>", "ffma_kernel", "depthwise_tma_kernel",
+ * "small_gemm_kernel<f32>", "conv_strip_kernel<bf16>", "conv_strip_kernel<f32>", "conv_wide_kernel<bf16>", "ffma_kernel", "depthwise_tma_kernel",
  * "depthwise_roll_kernel", "depthwise_vec_kernel", "depthwise_generic_kernel", "copy_tma_kernel",
  * "transpose_tma_kernel", "tile_move_kernel", "colred_kernel<vec>", "colred_kernel<scalar>",
  * "rowred_kernel<vec>", "rowred_kernel<scalar>".  For tests and benchmarks.

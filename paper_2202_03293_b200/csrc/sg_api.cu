@@ -38,7 +38,10 @@ sg_status run(const Problem &p, const void *In, const void *Flt, float *O, cudaS
     }
     if (force == SG_KERNEL_AUTO || force == SG_KERNEL_CONV_STRIP) {
         // stride-1 bf16 convolutions whose filter fits in shared memory
-        sg_status st = launch_conv_strip(p, In, Flt, O, stream);
+        bool resident = true;
+        sg_status st = launch_conv_wide(p, In, Flt, O, force == SG_KERNEL_AUTO, &resident, stream);
+        if (st == SG_OK && !resident) { t_last_kernel = SG_KERNEL_TENSOR; return SG_OK; }
+        if (st == SG_ERR_UNSUPPORTED) st = launch_conv_strip(p, In, Flt, O, stream);
         if (st == SG_OK) { t_last_kernel = SG_KERNEL_CONV_STRIP; return SG_OK; }
         if (st != SG_ERR_UNSUPPORTED || force == SG_KERNEL_CONV_STRIP) return st;
     }

@@ -1,0 +1,364 @@
+// Stride-1 convolutions on the tensor cores with the roles of the operands exchanged: the filter is the
+// M side of the MMA (128 filters = the lanes of tensor memory), the input positions are the N side.
+//
+// What that buys over the strip kernel, whose tiles are 128 positions that must start at image rows:
+//   * A tile is any number of positions up to 256 (a multiple of 16), so the work divides evenly: the size is chosen such that
+//     the last wave of thread blocks is full.  Positions are counted with the input's row pitch, q = (n*H_in + h)*W_in + w, and
+//     a tile is any run of them; those with w >= W_out or h >= H_out are computed and dropped.
+//   * The filter's share of an MMA's shared-memory reads is spread over more positions: a k-step takes 98 cycles at 128
+//     positions and 123 at 192 (tensor core alone: 64 and 96; the M-major filter costs about 50 of them).
+//   * An accumulator lane is a filter, so a warp stores one position's 32 consecutive outputs as a whole 128-byte line
+//     straight from registers: no staging, no tensor store, any output strides.
+// One contiguous run of N + (KH-1)*dh*W_in + (KW-1)*dw input rows (128 bytes: 64 channels) serves all taps of a channel block:
+// each tap's MMAs read it through a descriptor shifted by kh*dh*W_in + kw*dw rows (the 128-byte swizzle is a function of the
+// absolute address).  Wide images take one run per filter row instead.  The filter travels in slots of one filter row (KW taps
+// x 64 channels x 128 filters, one TMA load); when all of it fits it is loaded once and stays, otherwise it streams.
+//
+// Warps: 0 input runs (TMA), 1 MMA issuer and owner of tensor memory, 2 filter (TMA), 4-11 write-back (two per lane quarter).
+#include <algorithm>
+
+#include "sg_internal.cuh"
+#include "sg_tc_ptx.cuh"
+
+namespace sg {
+namespace {
+
+constexpr int BF = 128;                       // filters per tile
+constexpr int MAX_SLOTS = 8, RUN_STAGES = 2;
+constexpr int THREADS = 384;
+constexpr int SMEM_LIMIT = 232448 - 1024 - 512;
+
+struct WideParams {
+    int BN;                 // positions per tile
+    int tiles, f_tiles;     // position tiles, filter tiles
+    int positions;          // positions that can be outputs
+    int N, Hin, Win, Hout, Wout, F;
+    int KH, KW, kb;         // filter rows, taps per row, channel blocks
+    int row_step, dw;       // rows of the run between filter rows, between taps of a row
+    int run_boxes, box_rows, run_bytes;      // TMA loads per run and their rows; bytes of a run's stage
+    int slots, slot_bytes, resident;         // filter ring; resident: it holds the whole filter
+    int flt_loads;          // TMA loads per slot: 1, or one per 64 filters when F is no multiple of 64
+    int tap_bytes, half_bytes;               // in a slot: between taps, between the two 64-filter halves
+    int last_ksteps;        // k-steps of 16 channels in the last channel block
+    int run_tx;             // bytes of a run's loads
+    int tmem_cols;
+    int o_n, o_h, o_w;
+    int accumulate, wait_prior;
+};
+
+__global__ void __launch_bounds__(THREADS, 1)
+conv_wide_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant__ CUtensorMap map_flt, const WideParams p, float *__restrict__ O) {
+    extern __shared__ uint8_t smem_raw[];
+    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    const uint32_t flt_addr = base, runs_addr = flt_addr + (uint32_t)(p.slots * p.slot_bytes);
+    __shared__ uint64_t bars[2 * MAX_SLOTS + 2 * RUN_STAGES + 4];
+    __shared__ uint32_t tmem_slot;
+    __shared__ int abort_word;
+    volatile int *abort_flag = &abort_word;
+    const uint32_t bar0 = smem_u32(bars);
+    auto flt_full = [&](int s) { return bar0 + 8u * s; };
+    auto flt_empty = [&](int s) { return bar0 + 8u * (MAX_SLOTS + s); };
+    auto run_full = [&](int s) { return bar0 + 8u * (2 * MAX_SLOTS + s); };
+    auto run_empty = [&](int s) { return bar0 + 8u * (2 * MAX_SLOTS + RUN_STAGES + s); };
+    auto acc_full = [&](int b) { return bar0 + 8u * (2 * MAX_SLOTS + 2 * RUN_STAGES + b); };
+    auto acc_empty = [&](int b) { return bar0 + 8u * (2 * MAX_SLOTS + 2 * RUN_STAGES + 2 + b); };
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    asm volatile("griddepcontrol.launch_dependents;");
+    if (threadIdx.x == 0) {
+        prefetch_tensormap(&map_in); prefetch_tensormap(&map_flt);
+        for (int s = 0; s < MAX_SLOTS; ++s) { mbar_init(flt_full(s), 1); mbar_init(flt_empty(s), 1); }
+        for (int s = 0; s < RUN_STAGES; ++s) { mbar_init(run_full(s), 1); mbar_init(run_empty(s), 1); }
+        for (int b = 0; b < 2; ++b) { mbar_init(acc_full(b), 1); mbar_init(acc_empty(b), 8); }
+        abort_word = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)), "r"((uint32_t)p.tmem_cols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = *(volatile uint32_t *)&tmem_slot;
+
+    // this block's items: a contiguous, balanced run of (filter tile, position tile), positions fastest
+    const int total = p.tiles * p.f_tiles;
+    const int item0 = (int)((long long)blockIdx.x * total / gridDim.x), item1 = (int)((long long)(blockIdx.x + 1) * total / gridDim.x);
+
+    if (warp == 0) {
+        // ------------------------------------------------------------ input runs
+        if (lane == 0) {
+            if (p.wait_prior) asm volatile("griddepcontrol.wait;" ::: "memory");
+            int it = 0;
+            bool ok = true;
+            for (int item = item0; item < item1 && ok; ++item) {
+                const int q0 = item % p.tiles * p.BN;
+                for (int cb = 0; cb < p.kb; ++cb, ++it) {
+                    const int s = it % RUN_STAGES;
+                    if (!mbar_wait(run_empty(s), ((it / RUN_STAGES) & 1) ^ 1u, abort_flag)) { ok = false; break; }
+                    mbar_expect_tx(run_full(s), (uint32_t)p.run_tx);
+                    for (int b = 0; b < p.run_boxes; ++b)
+                        tma_tile_3d<false>(runs_addr + (uint32_t)(s * p.run_bytes + b * p.box_rows * 128), &map_in, run_full(s), cb * 64, q0 + b * p.box_rows, 0);
+                }
+            }
+        }
+    } else if (warp == 2) {
+        // ------------------------------------------------------------ filter
+        if (lane == 0) {
+            if (p.wait_prior) asm volatile("griddepcontrol.wait;" ::: "memory");
+            int it = 0, cur = -1;
+            bool ok = true;
+            for (int item = item0; item < item1 && ok; ++item) {
+                const int ft = item / p.tiles;
+                if (p.resident && ft == cur) continue;
+                cur = ft;
+                for (int cb = 0; cb < p.kb && ok; ++cb)
+                    for (int kh = 0; kh < p.KH; ++kh, ++it) {
+                        const int s = it % p.slots;
+                        if (!mbar_wait(flt_empty(s), ((it / p.slots) & 1) ^ 1u, abort_flag)) { ok = false; break; }
+                        // (the first run and the first slot are what the first MMA waits for: the rest of the filter, up to
+                        // three times their size, comes behind them rather than beside them)
+                        if (it == 1 && !mbar_wait(run_full(0), 0, abort_flag)) { ok = false; break; }
+                        mbar_expect_tx(flt_full(s), (uint32_t)p.slot_bytes);
+                        const uint32_t dst = flt_addr + (uint32_t)(s * p.slot_bytes);
+                        if (p.flt_loads == 1) {
+                            tma_tile_5d<false>(dst, &map_flt, flt_full(s), 0, cb * 64, ft * (BF / 64), 0, kh);
+                        } else {
+                            tma_load_4d(dst, &map_flt, flt_full(s), ft * BF, cb * 64, 0, kh);
+                            tma_load_4d(dst + p.half_bytes, &map_flt, flt_full(s), ft * BF + 64, cb * 64, 0, kh);
+                        }
+                    }
+            }
+        }
+    } else if (warp == 1) {
+        // ------------------------------------------------------------ MMA issuer: the whole warp walks, one lane issues
+        const uint32_t idesc = make_idesc(p.BN, BF, false, true, false);       // filter as stored: M-major; positions K-major
+        const bool issuer = elect_one();
+        auto wait_all = [&](bool passed) { return __all_sync(0xffffffffu, passed) != 0; };
+        int it = 0, fit = 0, tl = 0, cur = -1;
+        bool ok = true;
+        for (int item = item0; item < item1 && ok; ++item, ++tl) {
+            const int ft = item / p.tiles;
+            const bool fresh = !p.resident || ft != cur;             // this tile's filter slots have to be waited for
+            const bool release = !p.resident || item + 1 >= item1 || (item + 1) / p.tiles != ft;
+            if (p.resident && !fresh) fit -= p.kb * p.KH;
+            cur = ft;
+            const int buf = tl & 1;
+            if (!wait_all(mbar_wait(acc_empty(buf), ((tl >> 1) & 1) ^ 1u, abort_flag))) { ok = false; break; }
+            tc_fence_after();
+            const uint32_t d = tmem_base + buf * p.BN;
+            uint32_t acc = 0;
+            for (int cb = 0; cb < p.kb && ok; ++cb, ++it) {
+                const int s = it % RUN_STAGES;
+                if (!wait_all(mbar_wait(run_full(s), (it / RUN_STAGES) & 1, abort_flag))) { ok = false; break; }
+                const uint32_t run = runs_addr + (uint32_t)(s * p.run_bytes);
+                const int ksteps = cb + 1 == p.kb ? p.last_ksteps : 4;
+                for (int kh = 0; kh < p.KH; ++kh, ++fit) {
+                    const int fs = fit % p.slots;
+                    if (fresh && !wait_all(mbar_wait(flt_full(fs), (fit / p.slots) & 1, abort_flag))) { ok = false; break; }
+                    tc_fence_after();
+                    // (descriptors are made by the converged warp: uniform values; a lane on its own pays ~100 cycles per MMA)
+                    for (int kw = 0; kw < p.KW; ++kw) {
+                        const uint64_t a = make_smem_desc(flt_addr + (uint32_t)(fs * p.slot_bytes + kw * p.tap_bytes), (uint32_t)p.half_bytes, 1024);
+                        const uint64_t b = make_smem_desc(run + (uint32_t)(kh * p.row_step + kw * p.dw) * 128u, 16, 1024);
+                        if (issuer) {
+#pragma unroll
+                            for (int k = 0; k < 4; ++k)
+                                if (k < ksteps) umma_bf16(d, a + (uint64_t)(k * 128), b + (uint64_t)(k * 2), idesc, k == 0 ? acc : 1u);
+                        }
+                        acc = 1u;
+                    }
+                    if (release && issuer) umma_commit(flt_empty(fs));
+                }
+                if (ok && issuer) umma_commit(run_empty(s));
+            }
+            if (ok && issuer) umma_commit(acc_full(buf));
+        }
+    } else if (warp >= 4) {
+        // ------------------------------------------------------------ write-back: lane = filter, register = position
+        const int q = warp & 3, half = (warp - 4) >> 2;
+        int tl = 0;
+        if (p.wait_prior) asm volatile("griddepcontrol.wait;" ::: "memory");
+        const int hw = p.Hin * p.Win;
+        for (int item = item0; item < item1; ++item, ++tl) {
+            const int ft = item / p.tiles, q0 = (item - ft * p.tiles) * p.BN;
+            const int buf = tl & 1;
+            if (!__all_sync(0xffffffffu, mbar_wait(acc_full(buf), (tl >> 1) & 1, abort_flag))) break;
+            tc_fence_after();
+            const int f = ft * BF + q * 32 + lane;
+            const int blocks = p.BN / 16;
+            for (int j = half; j < blocks; j += 2) {
+                uint32_t r[16];
+                tmem_ld_32x16(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * p.BN + j * 16), r);
+                // lane i: whether position i of the sixteen is an output, and its offset
+                const int pos = q0 + j * 16 + (lane & 15);
+                const int n = pos / hw, rem = pos - n * hw, h = rem / p.Win, w = rem - h * p.Win;
+                const uint32_t live = __ballot_sync(0xffffffffu, pos < p.positions && w < p.Wout && h < p.Hout);
+                const int off = n * p.o_n + h * p.o_h + w * p.o_w;
+                tmem_ld_wait();
+                if (p.accumulate) {
+#pragma unroll
+                    for (int c = 0; c < 16; ++c) {
+                        const int o = __shfl_sync(0xffffffffu, off, c);
+                        if ((live >> c & 1u) && f < p.F) asm volatile("red.global.add.f32 [%0], %1;" ::"l"(O + (o + f)), "f"(__uint_as_float(r[c])) : "memory");
+                    }
+                } else if ((live & 0xFFFFu) == 0xFFFFu && __shfl_sync(0xffffffffu, off, 15) == __shfl_sync(0xffffffffu, off, 0) + 15 * p.o_w) {
+                    float *out = O + (__shfl_sync(0xffffffffu, off, 0) + f);          // (all sixteen in one image row)
+                    if (f < p.F)
+#pragma unroll
+                        for (int c = 0; c < 16; ++c, out += p.o_w) *out = __uint_as_float(r[c]);
+                } else {
+#pragma unroll
+                    for (int c = 0; c < 16; ++c) {
+                        const int o = __shfl_sync(0xffffffffu, off, c);
+                        if ((live >> c & 1u) && f < p.F) O[o + f] = __uint_as_float(r[c]);
+                    }
+                }
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(acc_empty(buf));
+        }
+    }
+    // ---------------------------------------------------------------- teardown
+    __syncthreads();
+    if (*abort_flag) {
+        for (int i = 0; i < 200; ++i) __nanosleep(5000);      // let loads in flight land before the shared memory goes
+        __syncthreads();
+    }
+    if (warp == 1) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)p.tmem_cols) : "memory");
+    }
+}
+
+inline bool mult(int64_t v, int64_t q) { return v % q == 0; }
+
+}  // namespace
+
+sg_status launch_conv_wide(const Problem &p, const void *In, const void *Flt, float *O, bool streaming, bool *resident_filter, cudaStream_t stream) {
+    // ---- eligibility: bf16, unit conv strides, dense pixel pitch, TMA alignment rules; any output strides but f
+    if (p.spatial_rank == 0 || !p.in_bf16 || p.sh != 1 || p.sw != 1) return SG_ERR_UNSUPPORTED;
+    // Lanes without a filter cost as much as the others.  Up to 64 filters this kernel still wins where each input row serves nine
+    // taps or more (3x3x16x32 on 16 x 112 x 112: 29.1 -> 22.1 us, 5x5x32x64: 40.7 -> 20.9; but three taps 5.6 -> 6.3).
+    if (p.N < 24 || (p.N <= 64 && p.KH * p.KW < 9)) return SG_ERR_UNSUPPORTED;
+    if (p.i_c != 1 || p.k_f != 1 || p.o_f != 1) return SG_ERR_UNSUPPORTED;
+    if (p.Hin > 1 && p.i_h != (int64_t)p.Win * p.i_w) return SG_ERR_UNSUPPORTED;
+    if (p.batch > 1 && p.i_n != (int64_t)p.Hin * p.Win * p.i_w) return SG_ERR_UNSUPPORTED;
+    if (p.i_w < p.C || p.k_c < p.N) return SG_ERR_UNSUPPORTED;
+    if (reinterpret_cast<uintptr_t>(In) % 16 || reinterpret_cast<uintptr_t>(Flt) % 16) return SG_ERR_UNSUPPORTED;
+    if (!mult(p.i_w, 8) || !mult(p.k_c, 8) || !mult(p.C, 8) || !mult(p.N, 8)) return SG_ERR_UNSUPPORTED;
+    if ((p.KW > 1 && !mult(p.k_kw, 8)) || (p.KH > 1 && !mult(p.k_kh, 8)) || p.KW > 16 || p.KH > 64) return SG_ERR_UNSUPPORTED;
+    const int64_t limit = (int64_t)1 << 39;      // byte strides below 2^40
+    const int64_t Q = (int64_t)p.batch * p.Hin * p.Win, shift = (int64_t)p.dh * p.Win;
+    if (p.i_w >= limit || p.k_c >= limit || Q > 0x7fffffff - 4096 || shift * p.i_w >= limit) return SG_ERR_UNSUPPORTED;
+    const int64_t positions = (int64_t)(p.batch - 1) * p.Hin * p.Win + (int64_t)(p.Ho - 1) * p.Win + p.Wo;
+    // (output offsets are 32-bit, those of the dead positions of the last image and beyond too)
+    if ((int64_t)(p.batch + 1) * p.o_n + (int64_t)(p.Hin + 1) * p.o_h + (int64_t)(p.Win + 1) * p.o_w + p.N > 0x7fffffff) return SG_ERR_UNSUPPORTED;
+    const int f_tiles = (p.N + BF - 1) / BF;
+    // share of the positions that are outputs: where it is low the im2col kernel, whose tiles hold outputs only, is the better one
+    if ((double)p.M < 0.6 * (double)positions) return SG_ERR_UNSUPPORTED;
+    int dev = 0, num_sms = 0, pdl = -1, single = 0;
+    if (!tensor_device_info(&dev, &num_sms, &pdl, &single)) return SG_ERR_CUDA;
+
+    // ---- one run of rows for all taps, or one per filter row
+    const int row_span = (p.KW - 1) * p.dw;
+    const int64_t full_span = (int64_t)(p.KH - 1) * shift + row_span;
+    const int kb = (p.C + 63) / 64, total_slots = kb * p.KH;
+    const int flt_rows = kb > 1 ? 64 : (p.C + 15) / 16 * 16;           // channels of a filter block
+    const int slot_bytes = p.KW * BF * 2 * flt_rows;
+    // ---- positions per tile: the least estimated time, in cycles.  A tile's run comes in and its outputs go out at the block's
+    // share of the HBM rate; between the first run and the last write-back the slowest of run, MMAs and write-back paces the
+    // rounds.  (Fitted to sweeps of 32 to 256 positions on nine shapes; the choices are within 4 % of the best but for one 9 %.)
+    WideParams w{};
+    double best = 1e300;
+    const int ksteps = (kb - 1) * 4 + ((p.C - (kb - 1) * 64) + 15) / 16;
+    for (int bn = 32; bn <= 256; bn += 16) {
+        const bool per_row = full_span - row_span > (int64_t)(p.KH - 1) * (bn + row_span);
+        const int64_t rows = per_row ? bn + row_span : bn + full_span;
+        int boxes = 1, box_rows = (int)rows;
+        if (per_row) {
+            if (rows > 256) continue;
+        } else {
+            boxes = (int)((rows + 255) / 256);
+            box_rows = (int)(((rows + boxes - 1) / boxes + 7) / 8 * 8);
+        }
+        const int64_t tx = (int64_t)box_rows * 128 * (per_row ? p.KH : boxes), bytes = (tx + 1023) / 1024 * 1024;
+        const int64_t room = SMEM_LIMIT - RUN_STAGES * bytes;
+        if (room < slot_bytes) continue;
+        const int slots = (int)std::min<int64_t>(std::min<int64_t>(MAX_SLOTS, total_slots), room / slot_bytes);
+        if (slots < std::min(2, total_slots)) continue;
+        const bool resident = slots == total_slots;
+        if (!resident && !streaming) continue;
+        const int64_t tiles = (positions + bn - 1) / bn, items = tiles * f_tiles, rounds = (items + num_sms - 1) / num_sms;
+        const double rate = std::min(64.0, 23.0 * num_sms / (double)std::min<int64_t>(items, num_sms));
+        const double load = (double)tx * kb / rate, store = (double)bn * std::min(p.N, BF) * 4.0 / rate;
+        double mma = (double)p.KH * p.KW * ksteps * std::max(bn / 2.0, 49.5 + 0.384 * bn);
+        if (!resident) mma = std::max(mma, (double)slot_bytes * total_slots / 45.0);       // the filter streams from the L2
+        const double cost = load + mma + (double)(rounds - 1) * std::max(mma, std::max(load, store)) + store + 300.0 * (double)rounds;
+        if (cost >= best) continue;
+        best = cost;
+        w.BN = bn; w.tiles = (int)tiles; w.run_boxes = boxes; w.box_rows = box_rows; w.run_bytes = (int)bytes; w.run_tx = (int)tx;
+        w.slots = slots; w.resident = resident; w.row_step = per_row ? box_rows : (int)shift;
+    }
+    if (w.BN == 0 || (int64_t)w.tiles * f_tiles > 0x7fffffff) return SG_ERR_UNSUPPORTED;
+    const bool per_row = w.run_boxes == 1 && w.row_step == w.box_rows && p.KH > 1;
+
+    alignas(64) CUtensorMap map_in, map_flt;
+    {
+        // {channel, position, filter row}: an overlapping view whose third dimension steps by dh*W_in positions (extent 1 when
+        // one run serves all taps); positions beyond the input read as zero
+        cuuint64_t dims[3] = {(cuuint64_t)p.C, (cuuint64_t)(per_row ? Q - (int64_t)(p.KH - 1) * shift : Q), (cuuint64_t)(per_row ? p.KH : 1)};
+        cuuint64_t strides[2] = {(cuuint64_t)(p.i_w * 2), (cuuint64_t)((per_row ? shift : Q) * p.i_w * 2)};
+        cuuint32_t box[3] = {64, (cuuint32_t)w.box_rows, (cuuint32_t)(per_row ? p.KH : 1)};
+        if (strides[1] >= ((cuuint64_t)1 << 40)) return SG_ERR_UNSUPPORTED;
+        if (!tensor_encode_tiled(&map_in, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(In), dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B,
+                                 CU_TENSOR_MAP_L2_PROMOTION_L2_128B)) return SG_ERR_UNSUPPORTED;
+    }
+    const int64_t s_kw = p.KW > 1 ? p.k_kw : (int64_t)p.C * p.k_c, s_kh = p.KH > 1 ? p.k_kh : (int64_t)p.KW * s_kw;
+    if (p.N % 64 == 0) {
+        cuuint64_t dims[5] = {64, (cuuint64_t)p.C, (cuuint64_t)(p.N / 64), (cuuint64_t)p.KW, (cuuint64_t)p.KH};
+        cuuint64_t strides[4] = {(cuuint64_t)(p.k_c * 2), 128, (cuuint64_t)(s_kw * 2), (cuuint64_t)(s_kh * 2)};
+        cuuint32_t box[5] = {64, (cuuint32_t)flt_rows, BF / 64, (cuuint32_t)p.KW, 1};
+        if (!tensor_encode_tiled(&map_flt, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void *>(Flt), dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B,
+                                 CU_TENSOR_MAP_L2_PROMOTION_L2_128B)) return SG_ERR_UNSUPPORTED;
+        w.flt_loads = 1; w.tap_bytes = 256 * flt_rows; w.half_bytes = 128 * flt_rows;
+    } else {
+        cuuint64_t dims[4] = {(cuuint64_t)p.N, (cuuint64_t)p.C, (cuuint64_t)p.KW, (cuuint64_t)p.KH};
+        cuuint64_t strides[3] = {(cuuint64_t)(p.k_c * 2), (cuuint64_t)(s_kw * 2), (cuuint64_t)(s_kh * 2)};
+        cuuint32_t box[4] = {64, (cuuint32_t)flt_rows, (cuuint32_t)p.KW, 1};
+        if (!tensor_encode_tiled(&map_flt, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(Flt), dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B,
+                                 CU_TENSOR_MAP_L2_PROMOTION_L2_128B)) return SG_ERR_UNSUPPORTED;
+        w.flt_loads = 2; w.tap_bytes = 128 * flt_rows; w.half_bytes = p.KW * 128 * flt_rows;
+    }
+    w.f_tiles = f_tiles; w.positions = (int)positions;
+    w.N = p.batch; w.Hin = p.Hin; w.Win = p.Win; w.Hout = p.Ho; w.Wout = p.Wo; w.F = p.N;
+    w.KH = p.KH; w.KW = p.KW; w.kb = kb; w.dw = p.dw; w.slot_bytes = slot_bytes;
+    w.last_ksteps = (p.C - (kb - 1) * 64 + 15) / 16;
+    w.tmem_cols = 2 * w.BN <= 128 ? 128 : 2 * w.BN <= 256 ? 256 : 512;
+    w.o_n = (int)p.o_n; w.o_h = (int)p.o_h; w.o_w = (int)p.o_w;
+    w.accumulate = p.accumulate; w.wait_prior = pdl == 0 ? 0 : 1;
+
+    if (!tensor_ensure_smem_attr(159, reinterpret_cast<const void *>(conv_wide_kernel), SMEM_LIMIT + 1024)) return SG_ERR_CUDA;
+    cudaLaunchConfig_t cfg = {};
+    const int64_t items = (int64_t)w.tiles * f_tiles;
+    cfg.gridDim = dim3((unsigned)std::min<int64_t>(items, num_sms), 1, 1);
+    cfg.blockDim = dim3(THREADS, 1, 1);
+    cfg.dynamicSmemBytes = w.slots * slot_bytes + RUN_STAGES * w.run_bytes + 1024;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = w.wait_prior ? 1 : 0;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, conv_wide_kernel, map_in, map_flt, w, O);
+    count_launch();
+    note_kernel("conv_wide_kernel<bf16>");
+    *resident_filter = w.resident != 0;
+    return e == cudaSuccess ? SG_OK : SG_ERR_CUDA;
+}
+
+sg_status conv_wide_read_status(cudaStream_t stream) { return read_status_word(stream); }
+
+}  // namespace sg

@@ -1364,6 +1364,8 @@ sg_status tensor_read_status(cudaStream_t stream) {
     const sg_status c = bandwidth_read_status(stream);
     const sg_status d = depthwise_read_status(stream);
     const sg_status e = gather_read_status(stream);
+    const sg_status f = conv_wide_read_status(stream);
+    if (f != SG_OK) return f;
     return a != SG_OK ? a : (b != SG_OK ? b : (c != SG_OK ? c : (d != SG_OK ? d : e)));
 }
 

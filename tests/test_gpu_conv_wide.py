@@ -1,0 +1,52 @@
+"""The stride-1 convolution kernel whose M operand is the filter, against the oracle: one run for all taps and one per filter row,
+resident and streaming filters, filters that are no multiple of 64, channels that end inside a k-step, tiles that wrap over rows
+and images."""
+import numpy as np
+import pytest
+import torch
+
+from helpers import assert_within_bound, operand
+from oracle import ref
+from paper_2202_03293_b200 import binding as sg
+
+pytestmark = pytest.mark.gpu
+SEED = 9700
+
+
+@pytest.fixture(autouse=True)
+def _check():
+    yield
+    sg.sg_check()
+
+
+@pytest.mark.parametrize("N,Ho,Wo,C,KH,KW,F,dl,extra", [
+    (4, 40, 41, 64, 3, 3, 128, (1, 1), (0, 0)), (3, 30, 31, 72, 3, 3, 72, (1, 1), (2, 1)), (2, 50, 49, 16, 5, 5, 96, (1, 1), (0, 0)),
+    (2, 33, 300, 64, 3, 3, 128, (1, 1), (0, 0)), (2, 60, 61, 128, 3, 3, 200, (2, 2), (0, 0)), (9, 28, 28, 256, 3, 3, 256, (1, 1), (0, 0)),
+    (3, 64, 65, 8, 1, 1, 104, (1, 1), (0, 3)), (1, 17, 700, 40, 1, 7, 128, (1, 3), (0, 0)), (2, 90, 20, 64, 7, 1, 136, (1, 1), (0, 0)),
+    (4, 50, 51, 16, 3, 3, 32, (1, 1), (0, 0)), (3, 60, 33, 40, 5, 5, 64, (1, 1), (0, 0))])
+@pytest.mark.parametrize("accumulate", [False, True])
+def test_conv2d(N, Ho, Wo, C, KH, KW, F, dl, extra, accumulate):
+    h_in, w_in = Ho + (KH - 1) * dl[0] + extra[0], Wo + (KW - 1) * dl[1] + extra[1]
+    I, i = operand((N, h_in, w_in, C), SEED, 1, "normal", "bf16")
+    K, k = operand((KH, KW, C, F), SEED, 2, "normal", "bf16")
+    wide = torch.full((N, Ho, Wo, F + 3), float("nan"), device="cuda")
+    O = wide[..., :F]
+    if accumulate:
+        O.fill_(1.0)
+    sg.sg_conv2d_nhwc_hwcf(I, K, O, (1, 1), dl, sg.SG_ACCUMULATE if accumulate else sg.SG_OVERWRITE)
+    torch.cuda.synchronize()
+    assert sg.sg_last_kernel_name() == "conv_wide_kernel<bf16>"
+    want, S = ref.conv2d_nhwc_hwcf(i, k, dilation=dl, out_hw=(Ho, Wo))
+    assert_within_bound(O, want + accumulate, S + accumulate, "conv2d, filter as M")
+    assert torch.isnan(wide[..., F:]).all()
+
+
+def test_conv1d_and_exact_integers():
+    I, i = operand((5, 3000, 64), SEED, 3, "ints", "bf16")
+    K, k = operand((3, 64, 128), SEED, 4, "ints", "bf16")
+    O = torch.full((5, 2998, 128), float("nan"), device="cuda")
+    sg.sg_conv1d_nwc_wcf(I, K, O)
+    torch.cuda.synchronize()
+    assert sg.sg_last_kernel_name() == "conv_wide_kernel<bf16>"
+    want, S = ref.conv1d_nwc_wcf(i, k)
+    assert np.array_equal(O.cpu().numpy().astype(np.float64), want)

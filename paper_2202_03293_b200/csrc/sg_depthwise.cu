@@ -7,12 +7,12 @@
 // reads and writes whole lines) of TW consecutive output columns; for the 3 x 3 window with unit
 // stride and dilation along w the input columns the TW windows share are loaded once into
 // registers, otherwise every tap is loaded where it is needed and the L1 serves the repeats.
-// Large 3 x 3 / unit-stride problems take one of two kernels that fetch every input element about
-// 1.5 times instead of 4.5: a TMA-staged tile kernel (layouts that meet the TMA rules) or a
-// kernel that walks down the rows with a rolling register window.  Any other layout (channel
+// 3 x 3 and 5 x 5 windows take a TMA-staged tile kernel (layouts that meet the TMA rules); large 3 x 3 /
+// unit-stride problems in other layouts a kernel that walks down the rows with a rolling register window.  Any other layout (channel
 // strides other than 1, channel counts that are not a multiple of 4, unaligned pointers or
 // pitches) takes a one-output-per-thread kernel with full stride arithmetic.
 #include <algorithm>
+#include <cmath>
 
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -210,123 +210,163 @@ depthwise_roll_kernel(const DepthwiseProblem p, const T *__restrict__ I, const T
     if (h + 1 < h1) roll_step<T, 1>(p, in_col, out_col, h + 1, w0, flt_smem, flt_pitch, col);
 }
 
-// 3 x 3 window, unit strides and dilations, layouts that meet the TMA rules, problems of at least one tile per SM:
-// the input tile of a CTA (DT_ROWS+2 rows x TWB+2 columns x CB channels, halo included) is fetched by ONE tensor load
-// into a two-stage shared-memory ring, so the fetch of the next tile runs while this one is computed and an input
-// element crosses L2 -> SM about 1.4 times instead of 4.5.  256 compute threads: thread (column wl, channel group cg)
-// walks down the DT_ROWS output rows of its column with the 3 x 3 window of float4 in registers (three new
-// shared-memory reads per output, conflict-free: a warp reads whole contiguous pixels) and stores its outputs
-// straight from registers (a warp writes whole pixels).  Warp 8 is the producer.
+// K x K window (3 or 5), stride 1 or 2 along h and w, unit dilation, layouts that meet the TMA rules: the input tile of a CTA,
+// halo included, is fetched by ONE tensor load into a two-stage shared-memory ring, so the fetch of the next tile runs while
+// this one is computed.  A group of CB/2 lanes owns WC output columns of ROWS output rows, two channels per lane; it walks down
+// the input rows once, reads each of its (WC-1)*S+K pixels once and adds it into every output it belongs to (at most K/S rows
+// are open at a time, in registers, as is the filter).  The 256 / (CB/2) groups of a tile are cg side by side times rg below
+// one another, or rg images (small images), whichever wastes less.  Products and sums are packed in pairs (fma.rn.f32x2), which
+// halves their issue slots: with scalar FMAs and a 3 x 3 window of inputs in registers a 32x112x112x64 bf16 layer took 32.7 us,
+// and 5 x 5 windows, which had no tiled kernel, 200 us.  Warp 8 is the producer.
 constexpr int DT_THREADS = 256 + 32;
 
-// S: stride along h and w (1 or 2).  A tile is ROWS output rows x TWB output columns x CB channels.
-template <typename T, int CB, int S>
+template <typename T, int CB, int K, int S>
 struct DtCfg {
-    static constexpr int CG = CB / 4;                 // channel groups (threads) per pixel
-    static constexpr int TWB = 256 / CG;              // output columns per tile
-    static constexpr int ROWS = S == 1 ? 8 : 2;       // output rows per tile
-    static constexpr int IN_W = (TWB - 1) * S + 3, IN_H = (ROWS - 1) * S + 3;
+    static constexpr int LANES = CB / 2;                          // per group
+    static constexpr int GROUPS = 256 / LANES;
+    // output columns and rows of a group (less for f32 and for 16 groups: a tile's two stages leave room for two CTAs per SM)
+    static constexpr bool SMALL = sizeof(T) == 4 || GROUPS == 16;
+    static constexpr int WC = K == 3 && S == 1 && !SMALL ? 4 : 2;
+    static constexpr int ROWS = S == 1 ? 8 : SMALL ? 2 : 4;
+    static constexpr int IN_ROWS = (ROWS - 1) * S + K, IN_COLS = (WC - 1) * S + K;
+    static constexpr int OPEN = (K + S - 1) / S;                  // output rows a group works on at a time
     static constexpr int PIXEL_BYTES = CB * (int)sizeof(T);
-    static constexpr int BOX_BYTES = PIXEL_BYTES * IN_W * IN_H;
-    static constexpr int STAGE_BYTES = (BOX_BYTES + 127) / 128 * 128;
+};
+struct DtTiling {
+    int cg, rg, stack;                // groups side by side; below one another (or, stack, of consecutive images)
+    int in_w, in_h;                   // input tile of an image, pixels
+    int box_bytes, stage_bytes;
+    int tiles_w, tiles_h, tiles_n, c_blocks, num_tiles;
 };
 
-__device__ __forceinline__ float4 lds4(uint32_t addr, float) {
-    float4 v;
-    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr));
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float &a, float &b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ void fma2(f32x2 &acc, f32x2 a, f32x2 b) { asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b)); }
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+// Two neighbouring channels of a pixel.
+__device__ __forceinline__ f32x2 lds2(uint32_t addr, float) {
+    f32x2 v;
+    asm volatile("ld.shared.b64 %0, [%1];" : "=l"(v) : "r"(addr));
     return v;
 }
-__device__ __forceinline__ float4 lds4(uint32_t addr, __nv_bfloat16) {
-    uint32_t a, b;
-    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(a), "=r"(b) : "r"(addr));
-    return make_float4(__uint_as_float(a << 16), __uint_as_float(a & 0xFFFF0000u), __uint_as_float(b << 16), __uint_as_float(b & 0xFFFF0000u));
+__device__ __forceinline__ f32x2 lds2(uint32_t addr, __nv_bfloat16) {
+    uint32_t v;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
+    return pack2(__uint_as_float(v << 16), __uint_as_float(v & 0xFFFF0000u));
 }
 
-// The grid is a multiple of c_blocks (or smaller than it never), so a CTA keeps one channel block
-// for all its tiles and a thread loads its nine filter values once.
-template <typename T, int CB, int S>
-__global__ void __launch_bounds__(DT_THREADS)
-depthwise_tma_kernel(const __grid_constant__ CUtensorMap map_in, const DepthwiseProblem p, const T *__restrict__ Kf,
-                     float *__restrict__ O, int tiles_w, int tiles_h, int c_blocks, int num_tiles) {
-    using C = DtCfg<T, CB, S>;
+// The grid is a multiple of c_blocks (or smaller than it never), so a CTA keeps one channel block for all its tiles and a
+// thread loads its filter values once.
+template <typename T, int CB, int K, int S>
+__global__ void __launch_bounds__(DT_THREADS, 2)
+depthwise_tma_kernel(const __grid_constant__ CUtensorMap map_in, const DepthwiseProblem p, const T *__restrict__ Kf, float *__restrict__ O, const DtTiling d) {
+    using C = DtCfg<T, CB, K, S>;
     extern __shared__ uint8_t dt_smem[];
     __shared__ uint64_t full_bar[2], empty_bar[2];
     __shared__ int abort_load, abort_compute;
     const uint32_t ring = (smem_u32(dt_smem) + 127u) & ~127u;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    asm volatile("griddepcontrol.launch_dependents;");
     if (threadIdx.x == 0) {
         for (int s = 0; s < 2; ++s) { mbar_init(smem_u32(&full_bar[s]), 1); mbar_init(smem_u32(&empty_bar[s]), 8); }
         abort_load = 0; abort_compute = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
+    // the operands may be the output of the kernel ahead of this one, and the output its input
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const int tile_cols = d.cg * C::WC, tile_rows = d.stack ? C::ROWS : d.rg * C::ROWS, tile_n = d.stack ? d.rg : 1;
     if (warp == 8) {
         if (lane == 0) {
             prefetch_tensormap(&map_in);
             int k = 0;
-            for (int t = blockIdx.x; t < num_tiles; t += gridDim.x, ++k) {
+            for (int t = blockIdx.x; t < d.num_tiles; t += gridDim.x, ++k) {
                 const int s = k & 1;
                 const uint32_t ph = (uint32_t)(k >> 1) & 1u;
                 if (!mbar_wait(smem_u32(&empty_bar[s]), ph ^ 1u, &abort_load)) break;
                 int r = t;
-                const int cb = r % c_blocks; r /= c_blocks;
-                const int wt = r % tiles_w; r /= tiles_w;
-                const int ht = r % tiles_h, n = r / tiles_h;
-                mbar_expect_tx(smem_u32(&full_bar[s]), C::BOX_BYTES);
-                tma_load_4d(ring + (uint32_t)s * C::STAGE_BYTES, &map_in, smem_u32(&full_bar[s]), cb * CB, wt * C::TWB * S, ht * C::ROWS * S, n);
+                const int cb = r % d.c_blocks; r /= d.c_blocks;
+                const int wt = r % d.tiles_w; r /= d.tiles_w;
+                const int ht = r % d.tiles_h, nt = r / d.tiles_h;
+                mbar_expect_tx(smem_u32(&full_bar[s]), (uint32_t)d.box_bytes);
+                tma_load_4d(ring + (uint32_t)(s * d.stage_bytes), &map_in, smem_u32(&full_bar[s]), cb * CB, wt * tile_cols * S, ht * tile_rows * S, nt * tile_n);
             }
             if (abort_load)      // gave up: let the loads already issued land before the shared memory goes away
                 for (int j = (k > 2 ? k - 2 : 0); j < k; ++j)
                     for (int i = 0; i < (1 << 20) && !mbar_try_wait(smem_u32(&full_bar[j & 1]), (uint32_t)(j >> 1) & 1u); ++i) {}
         }
     } else {
-        const int cg = threadIdx.x % C::CG, wl = threadIdx.x / C::CG;
-        const int c = (int)(blockIdx.x % c_blocks) * CB + cg * 4;      // the same for every tile of this CTA
-        float4 flt[3][3];
+        const int group = threadIdx.x / C::LANES, cl = threadIdx.x % C::LANES * 2;
+        const int gc = group % d.cg, gr = group / d.cg;
+        const int c = (int)(blockIdx.x % d.c_blocks) * CB + cl;        // the same for every tile of this CTA (C is even)
+        f32x2 flt[K][K];
 #pragma unroll
-        for (int kh = 0; kh < 3; ++kh)
+        for (int kh = 0; kh < K; ++kh)
 #pragma unroll
-            for (int kw = 0; kw < 3; ++kw)
-                flt[kh][kw] = c < p.C ? load4(Kf + (int64_t)kh * p.k_kh + (int64_t)kw * p.k_kw + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int kw = 0; kw < K; ++kw) {
+                const T *f = Kf + (int64_t)kh * p.k_kh + (int64_t)kw * p.k_kw + c;
+                flt[kh][kw] = c < p.C ? pack2(load1(f), load1(f + 1)) : 0ull;
+            }
+        const uint32_t row_bytes = (uint32_t)(d.in_w * C::PIXEL_BYTES);
+        const uint32_t group_off = (uint32_t)(gc * C::WC * S * C::PIXEL_BYTES + cl * (int)sizeof(T)) +
+                                   (uint32_t)gr * (d.stack ? (uint32_t)d.in_h : (uint32_t)(C::ROWS * S)) * row_bytes;
         int k = 0;
-        for (int t = blockIdx.x; t < num_tiles; t += gridDim.x, ++k) {
+        for (int t = blockIdx.x; t < d.num_tiles; t += gridDim.x, ++k) {
             const int s = k & 1;
             const uint32_t ph = (uint32_t)(k >> 1) & 1u;
-            int r = t / c_blocks;
-            const int wt = r % tiles_w; r /= tiles_w;
-            const int ht = r % tiles_h, n = r / tiles_h;
-            const int w = wt * C::TWB + wl, h0 = ht * C::ROWS;
-            const bool live = c < p.C && w < p.Wo;
+            int r = t / d.c_blocks;
+            const int wt = r % d.tiles_w; r /= d.tiles_w;
+            const int ht = r % d.tiles_h, nt = r / d.tiles_h;
+            const int w0 = wt * tile_cols + gc * C::WC, h0 = ht * tile_rows + (d.stack ? 0 : gr * C::ROWS), n = nt * tile_n + (d.stack ? gr : 0);
             const bool ok = mbar_wait(smem_u32(&full_bar[s]), ph, &abort_compute);
             if (!__all_sync(0xffffffffu, ok)) break;
-            // this thread's columns of the tile: pixel (row r, column S*wl + kw) of the stage; tile row r lives in win[r % 3]
-            const uint32_t col_base = ring + (uint32_t)s * C::STAGE_BYTES + (uint32_t)(wl * S * CB + cg * 4) * (uint32_t)sizeof(T);
-            float4 win[3][3];
+            const int rows = c < p.C && n < p.N ? p.Ho - h0 : 0, cols = p.Wo - w0;      // outputs of this group that exist
+            uint32_t src = ring + (uint32_t)(s * d.stage_bytes) + group_off;
+            float *out = O + (int64_t)n * p.o_n + (int64_t)h0 * p.o_h + (int64_t)w0 * p.o_w + c;
+            if (rows > 0 && cols > 0) {
+                f32x2 acc[C::OPEN][C::WC];
 #pragma unroll
-            for (int rr = 0; rr < 3 - S; ++rr)
+                for (int rr = 0; rr < C::IN_ROWS; ++rr, src += row_bytes) {
+                    f32x2 x[C::IN_COLS];
 #pragma unroll
-                for (int kw = 0; kw < 3; ++kw) win[rr][kw] = lds4(col_base + (uint32_t)((rr * C::IN_W + kw) * C::PIXEL_BYTES), T());
-            float *out = O + (int64_t)n * p.o_n + (int64_t)w * p.o_w + c;
+                    for (int j = 0; j < C::IN_COLS; ++j) x[j] = lds2(src + (uint32_t)(j * C::PIXEL_BYTES), T());
 #pragma unroll
-            for (int hh = 0; hh < C::ROWS; ++hh) {
-                // the window of output row hh is tile rows S*hh .. S*hh+2; the first 3-S of them are already held
+                    for (int kw = 0; kw < K; ++kw)
 #pragma unroll
-                for (int rr = S * hh + 3 - S; rr <= S * hh + 2; ++rr)
+                        for (int kh = 0; kh < K; ++kh) {      // (neighbouring instructions belong to different sums)
+                            if ((rr - kh) % S != 0 || rr < kh || (rr - kh) / S >= C::ROWS) continue;
+                            const int h = (rr - kh) / S;
 #pragma unroll
-                    for (int kw = 0; kw < 3; ++kw)
-                        win[rr % 3][kw] = lds4(col_base + (uint32_t)((rr * C::IN_W + kw) * C::PIXEL_BYTES), T());
-                float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+                            for (int j = 0; j < C::WC; ++j) {
+                                if (kh == 0 && kw == 0) acc[h % C::OPEN][j] = mul2(x[j * S], flt[0][0]);
+                                else fma2(acc[h % C::OPEN][j], x[j * S + kw], flt[kh][kw]);
+                            }
+                        }
+                    if (rr >= K - 1 && (rr - (K - 1)) % S == 0) {
+                        const int h = (rr - (K - 1)) / S;
+                        if (h < rows) {
 #pragma unroll
-                for (int kh = 0; kh < 3; ++kh)
-#pragma unroll
-                    for (int kw = 0; kw < 3; ++kw) fma4(acc, win[(S * hh + kh) % 3][kw], flt[kh][kw]);
-                if (live && h0 + hh < p.Ho) {
-                    float4 *o = reinterpret_cast<float4 *>(out + (int64_t)(h0 + hh) * p.o_h);
-                    if (p.accumulate) {
-                        const float4 old = *o;
-                        acc.x += old.x; acc.y += old.y; acc.z += old.z; acc.w += old.w;
+                            for (int j = 0; j < C::WC; ++j) {
+                                if (j < cols) {
+                                    float2 *o = reinterpret_cast<float2 *>(out + (int64_t)j * p.o_w);
+                                    float a, b;
+                                    unpack2(acc[h % C::OPEN][j], a, b);
+                                    if (p.accumulate) { const float2 old = *o; a += old.x; b += old.y; }
+                                    *o = make_float2(a, b);
+                                }
+                            }
+                        }
+                        out += p.o_h;
                     }
-                    *o = acc;
                 }
             }
             __syncwarp();
@@ -359,41 +399,77 @@ depthwise_generic_kernel(const DepthwiseProblem p, const T *__restrict__ I, cons
     }
 }
 
-template <typename T, int CB, int S>
+template <typename T, int CB, int K, int S>
 bool try_launch_tma(const DepthwiseProblem &p, const T *I, const T *Kf, float *O, int num_sms, cudaStream_t stream, cudaError_t *err) {
-    using C = DtCfg<T, CB, S>;
+    using C = DtCfg<T, CB, K, S>;
     const int64_t es = sizeof(T);
-    const int tiles_w = (p.Wo + C::TWB - 1) / C::TWB, tiles_h = (p.Ho + C::ROWS - 1) / C::ROWS, c_blocks = (p.C + CB - 1) / CB;
-    const int64_t tiles = (int64_t)p.N * tiles_h * tiles_w * c_blocks;
-    if (tiles < num_sms || tiles >= ((int64_t)1 << 31) || c_blocks > num_sms) return false;
-    // the part of the input that is read: ((Ho-1)*S+3) x ((Wo-1)*S+3) pixels per image
-    const int64_t h_ext = (int64_t)(p.Ho - 1) * S + 3, w_ext = (int64_t)(p.Wo - 1) * S + 3;
+    // ---- groups of a tile: the fewest rounds of thread blocks, weighed with what a tile fetches (a round costs at least what
+    // its 256 threads compute, about 16 KB worth)
+    DtTiling d{};
+    double best = 1e300;
+    for (int cg = C::GROUPS; cg >= 1; cg >>= 1)       // (wide first: longer runs of memory)
+        for (int stack = 0; stack < 2; ++stack) {
+            const int rg = C::GROUPS / cg;
+            if (stack && (rg == 1 || p.N == 1)) continue;
+            const int in_w = (cg * C::WC - 1) * S + K, in_h = ((stack ? 1 : rg) * C::ROWS - 1) * S + K, in_n = stack ? rg : 1;
+            if (in_w > 256 || in_h > 256) continue;
+            const int bytes = C::PIXEL_BYTES * in_w * in_h * in_n;
+            if (bytes > 56 * 1024) continue;                                    // two stages of two thread blocks per SM
+            const int64_t tw = (p.Wo + cg * C::WC - 1) / (cg * C::WC), th = (p.Ho + (stack ? 1 : rg) * C::ROWS - 1) / ((stack ? 1 : rg) * C::ROWS);
+            const int64_t tn = (p.N + in_n - 1) / in_n, cbs = (p.C + CB - 1) / CB, tiles = tw * th * tn * cbs;
+            if (tiles >= ((int64_t)1 << 31)) continue;
+            const double rounds = std::max(1.0, (double)tiles / (2 * num_sms));
+            const double cost = (rounds < 4 ? std::ceil(rounds) : rounds) * (16384.0 + bytes);
+            if (cost < best) {
+                best = cost;
+                d = DtTiling{cg, rg, stack, in_w, in_h, bytes, (bytes + 127) / 128 * 128, (int)tw, (int)th, (int)tn, (int)cbs, (int)tiles};
+            }
+        }
+    if (d.num_tiles == 0 || d.c_blocks > num_sms) return false;
+    // 3 x 3 problems too small for a tile per SM are left to the kernel without tiles (2.9 us a launch against 3.5)
+    if (K == 3 && d.num_tiles < num_sms) return false;
+    // the part of the input that is read: ((Ho-1)*S+K) x ((Wo-1)*S+K) pixels per image
+    const int64_t h_ext = (int64_t)(p.Ho - 1) * S + K, w_ext = (int64_t)(p.Wo - 1) * S + K;
     const int64_t s_n = p.N > 1 ? p.i_n : h_ext * p.i_h;
     cuuint64_t dims[4] = {(cuuint64_t)p.C, (cuuint64_t)w_ext, (cuuint64_t)h_ext, (cuuint64_t)p.N};
     cuuint64_t strides[3] = {(cuuint64_t)(p.i_w * es), (cuuint64_t)(p.i_h * es), (cuuint64_t)(s_n * es)};
-    cuuint32_t box[4] = {(cuuint32_t)CB, (cuuint32_t)C::IN_W, (cuuint32_t)C::IN_H, 1};
+    cuuint32_t box[4] = {(cuuint32_t)CB, (cuuint32_t)d.in_w, (cuuint32_t)d.in_h, (cuuint32_t)(d.stack ? d.rg : 1)};
     for (int i = 0; i < 3; ++i)
         if (strides[i] % 16 != 0 || strides[i] >= ((cuuint64_t)1 << 40)) return false;
     CUtensorMap map_in;
     if (!tensor_encode_tiled(&map_in, sizeof(T) == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4,
                              const_cast<T *>(I), dims, strides, box, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B))
         return false;
-    const int smem = 2 * C::STAGE_BYTES + 128;
-    static int attr_device = -1;      // the attribute is per device
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (attr_device != dev) {
-        if (cudaFuncSetAttribute(depthwise_tma_kernel<T, CB, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return false;
-        attr_device = dev;
-    }
+    constexpr int slot = 184 + (sizeof(T) == 4 ? 8 : 0) + (CB == 64 ? 0 : 4) + (K == 5 ? 2 : 0) + (S - 1);
+    if (!tensor_ensure_smem_attr(slot, reinterpret_cast<const void *>(depthwise_tma_kernel<T, CB, K, S>), 2 * 56 * 1024 + 128)) return false;
     // two CTAs per SM, rounded down to a multiple of the channel blocks: tile t has block t % c_blocks, so every CTA keeps one
-    int64_t grid = std::min<int64_t>(tiles, 2 * (int64_t)num_sms);
-    grid -= grid % c_blocks;
-    depthwise_tma_kernel<T, CB, S><<<(int)grid, DT_THREADS, smem, stream>>>(map_in, p, Kf, O, tiles_w, tiles_h, c_blocks, (int)tiles);
+    int64_t grid = std::min<int64_t>(d.num_tiles, 2 * (int64_t)num_sms);
+    grid -= grid % d.c_blocks;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid, 1, 1);
+    cfg.blockDim = dim3(DT_THREADS, 1, 1);
+    cfg.dynamicSmemBytes = 2 * d.stage_bytes + 128;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    *err = cudaLaunchKernelEx(&cfg, depthwise_tma_kernel<T, CB, K, S>, map_in, p, Kf, O, d);
     count_launch();
     note_kernel("depthwise_tma_kernel");
-    *err = cudaGetLastError();
     return true;
+}
+
+template <typename T, int K>
+bool try_launch_window(const DepthwiseProblem &p, const T *I, const T *Kf, float *O, int num_sms, cudaStream_t stream, cudaError_t *err) {
+    // blocks of 64 channels; 32 where (bf16) at most that many are left over in the last block, and for 5 x 5 f32 tiles, which would
+    // not fit twice
+    if constexpr (sizeof(T) == 2 || K == 3) {
+        if ((p.C - 1) % 64 >= 32 || (sizeof(T) == 4 && p.C > 64))
+            return p.sh == 1 ? try_launch_tma<T, 64, K, 1>(p, I, Kf, O, num_sms, stream, err) : try_launch_tma<T, 64, K, 2>(p, I, Kf, O, num_sms, stream, err);
+    }
+    return p.sh == 1 ? try_launch_tma<T, 32, K, 1>(p, I, Kf, O, num_sms, stream, err) : try_launch_tma<T, 32, K, 2>(p, I, Kf, O, num_sms, stream, err);
 }
 
 inline bool mult4(int64_t v) { return v % 4 == 0; }
@@ -411,18 +487,14 @@ cudaError_t launch_typed(const DepthwiseProblem &p, const T *I, const T *Kf, flo
     const unsigned blocks = (unsigned)blocks64;
     const bool small = work < ((int64_t)1 << 32) - 256;
     const bool unit3 = p.sw == 1 && p.dw == 1 && p.KW == 3 && p.KH == 3;
-    const bool win3 = p.KW == 3 && p.KH == 3 && p.dw == 1 && p.dh == 1;
-    if (vec && win3 && p.sh == p.sw && p.sh <= 2 && reinterpret_cast<uintptr_t>(I) % 16 == 0 &&
+    const bool win3 = p.KW == 3 && p.KH == 3 && p.dw == 1 && p.dh == 1, win5 = p.KW == 5 && p.KH == 5 && p.dw == 1 && p.dh == 1;
+    if (vec && (win3 || win5) && p.sh == p.sw && p.sh <= 2 && reinterpret_cast<uintptr_t>(I) % 16 == 0 &&
         (p.C * (int64_t)sizeof(T)) % 16 == 0) {
         // TMA-staged tiles (TMA checks the channel bound in 16-byte units, hence the condition on C)
         int num_sms = 0;
         cudaError_t err = cudaSuccess;
-        if (tensor_driver_ready(&num_sms) && p.C >= 32) {
-            bool done;
-            if (p.sh == 1) done = p.C >= 64 ? try_launch_tma<T, 64, 1>(p, I, Kf, O, num_sms, stream, &err) : try_launch_tma<T, 32, 1>(p, I, Kf, O, num_sms, stream, &err);
-            else done = p.C >= 64 ? try_launch_tma<T, 64, 2>(p, I, Kf, O, num_sms, stream, &err) : try_launch_tma<T, 32, 2>(p, I, Kf, O, num_sms, stream, &err);
-            if (done) return err;
-        }
+        if (p.C >= 16 && tensor_driver_ready(&num_sms) &&
+            (win3 ? try_launch_window<T, 3>(p, I, Kf, O, num_sms, stream, &err) : try_launch_window<T, 5>(p, I, Kf, O, num_sms, stream, &err))) return err;
     }
     if (vec && unit3 && p.sh == 1 && p.dh == 1) {
         // enough row segments to give every SM several thread blocks: walk down the rows with a rolling window

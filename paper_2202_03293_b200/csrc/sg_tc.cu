@@ -114,7 +114,7 @@ struct Cfg {
     static constexpr int USED_COLS = ACC_BUFS * BN + A_TMEM_COLS;
     static constexpr int TMEM_COLS = USED_COLS <= 32 ? 32 : USED_COLS <= 64 ? 64 : USED_COLS <= 128 ? 128 : USED_COLS <= 256 ? 256 : 512;
     static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + SPLIT_SLOTS * SPLIT_BYTES + STAGING_BYTES +
-                                      1024 /*alignment slack*/ + 256 /*barriers*/;
+                                      1024 /*alignment slack*/ + 256 /*barriers*/ + 1024 /*a fused consumer's bias*/;
     static constexpr int B_KSTEP_DESC = 16 * ROW_BYTES / 16;   // bf16 filter tile, N-major: 16 k-rows per k-step
     static_assert(B_COLS % 64 == 0 && BN % 16 == 0 && BN <= 256, "tile width");
     static_assert(TMEM_COLS <= 512 && (TMEM_COLS & (TMEM_COLS - 1)) == 0, "TMEM columns");
@@ -182,6 +182,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant
     auto acc_empty_bar = [&](int b) { return bars_addr + 8u * (26 + b); };
     volatile uint32_t *tmem_ptr_slot = reinterpret_cast<volatile uint32_t *>(bars_gen + 8 * 28);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(bars_gen + 8 * 28 + 4);
+    float *bias_tile = reinterpret_cast<float *>(bars_gen + 256);      // the bias of the tile's columns
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // A launch behind this one that asked for it may start now: its CTAs take an SM as soon as one of ours leaves it
@@ -667,6 +668,29 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant
         const int q = warp & 3;        // TMEM lane quarter this warp may access
         const int ew = warp - 2;       // 0..3: whose turn it is to issue
         auto epi_sync = [] { asm volatile("bar.sync 1, 128;" ::: "memory"); };
+        // fused pointwise consumer (Sections 2.1, 3.3): r = act(acc + bias[column]) of column chunk j.  The tile's bias waits in
+        // shared memory (read from there by broadcasts; loaded chunk by chunk its latency cost 0.4 us a chunk)
+        auto consume = [&](uint32_t (&r)[32], int j) {
+            if (p.bias == nullptr && p.act == SG_ACT_NONE) return;
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                float4 b = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (p.bias != nullptr) b = *reinterpret_cast<const float4 *>(bias_tile + j * 32 + 4 * c);
+                const float bv[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    float v = __uint_as_float(r[4 * c + e]) + bv[e];
+                    r[4 * c + e] = __float_as_uint((p.act == SG_ACT_RELU && v < 0.f) ? 0.f : v);
+                }
+            }
+        };
+        // this lane's row of a staged 128 x 32 chunk (128-byte rows, 128-byte swizzle)
+        auto stage_row = [&](uint8_t *chunk, const uint32_t (&r)[32]) {
+            uint8_t *row = chunk + (q * 32 + lane) * 128;
+#pragma unroll
+            for (int c = 0; c < 8; ++c)
+                *reinterpret_cast<uint4 *>(row + ((c ^ (lane & 7)) << 4)) = make_uint4(r[4 * c], r[4 * c + 1], r[4 * c + 2], r[4 * c + 3]);
+        };
         int tl = 0, chunk_count = 0;
         bool ok = true;
         // This grid may have started beside the kernel ahead of it.  Behind a clearing kernel the whole first reduction
@@ -680,39 +704,55 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant
             tile_coords(tile, p.num_m_tiles, p.num_n_tiles, mt, nt);
             const int m0 = (mt * CG + (int)cta_rank) * BM, n0 = nt * BN;
             const int buf = tl % C::ACC_BUFS;
+            if (p.bias != nullptr)      // (every warp has read the previous tile's before it came to that tile's last barrier)
+                for (int i = ew * 32 + lane; i < BN; i += 128) bias_tile[i] = n0 + i < p.N ? __ldg(p.bias + n0 + i) : 0.f;
             // (the four warps take the same way here and meet at every epi_sync below)
             if (!epilogue_all(mbar_wait(acc_full_bar(buf), (tl / C::ACC_BUFS) & 1, abort_flag))) { ok = false; break; }
             tc_fence_after();
+            Cursor ahead = cur;
+            int t2, k2, k3, a2;
+            if (BN >= 128 && !next_item(ahead, t2, k2, k3, a2)) {
+                // The last item: the rings are idle by now (every load has been consumed by an MMA that has finished), so all
+                // chunks are staged there and no chunk waits for the store of an earlier one (256 columns took 3.1 us
+                // through the two staging tiles, which nothing hides at the end of a launch; 4096 x 1024 x 1024 bf16 13.7 -> 12.9 us).
+                constexpr int PER_STEP = F32 ? 1 : 2;      // (f32: 88 registers per thread)
+                static_assert(BN < 128 || C::STAGES * C::STAGE_BYTES + C::SPLIT_SLOTS * C::SPLIT_BYTES >= BN / 32 * 16384, "the rings hold a tile");
+#pragma unroll 1
+                for (int j = 0; j < BN / 32; j += PER_STEP) {
+                    uint32_t r[PER_STEP][32];
+#pragma unroll
+                    for (int i = 0; i < PER_STEP; ++i)
+                        tmem_ld_32x32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * BN + (j + i) * 32), r[i]);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int i = 0; i < PER_STEP; ++i) {
+                        consume(r[i], j + i);
+                        stage_row(smem_gen + (j + i) * 16384, r[i]);
+                    }
+                    fence_async_smem();
+                    epi_sync();
+                    const int mine = (ew - j) & 3;             // the warps issue the stores in turn
+                    if (lane == 0 && mine < PER_STEP) {
+                        const int x = n0 + (j + mine) * 32;
+                        if (x < p.N && m0 < p.M) {
+                            if (add) tma_reduce_add_2d(&map_out, stages_addr + (j + mine) * 16384, x, m0);
+                            else tma_store_2d(&map_out, stages_addr + (j + mine) * 16384, x, m0);
+                        }
+                        bulk_commit();
+                    }
+                }
+                break;
+            }
 #pragma unroll 1
             for (int j = 0; j < BN / 32; ++j, ++chunk_count) {
                 uint32_t r[32];
                 tmem_ld_32x32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * BN + j * 32), r);
                 tmem_ld_wait();
-                if (p.bias != nullptr || p.act != SG_ACT_NONE) {
-                    // fused pointwise consumer (Sections 2.1, 3.3): r = act(acc + bias[column]); the bias loads are
-                    // warp-uniform 16-byte loads (every lane holds the same 32 columns of its own row)
-                    const int x = n0 + j * 32;
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        float4 b = make_float4(0.f, 0.f, 0.f, 0.f);
-                        if (p.bias != nullptr && x + 4 * c < p.N) b = __ldg(reinterpret_cast<const float4 *>(p.bias + x) + c);
-                        const float bv[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            float v = __uint_as_float(r[4 * c + e]) + bv[e];
-                            r[4 * c + e] = __float_as_uint((p.act == SG_ACT_RELU && v < 0.f) ? 0.f : v);
-                        }
-                    }
-                }
+                consume(r, j);
                 const int sb = chunk_count & 1;
                 // staging tile sb was last read by the store of two chunks ago, whose issuer waited for
                 // that read before the previous chunk's epi_sync
-                uint8_t *row = staging_gen + sb * 16384 + (q * 32 + lane) * 128;
-#pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    uint4 v = make_uint4(r[4 * c], r[4 * c + 1], r[4 * c + 2], r[4 * c + 3]);
-                    *reinterpret_cast<uint4 *>(row + ((c ^ (lane & 7)) << 4)) = v;
-                }
+                stage_row(staging_gen + sb * 16384, r);
                 fence_async_smem();
                 // the issuer of the previous chunk's store makes sure that store has read its tile
                 if (lane == 0 && ew == ((chunk_count + 3) & 3)) bulk_wait_read<0>();

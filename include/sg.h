@@ -83,7 +83,7 @@ enum {
     SG_KERNEL_AUTO = 0,
     SG_KERNEL_FFMA = 1,        /* strided CUDA-core kernel, any layout                                   */
     SG_KERNEL_TENSOR = 2,      /* TMA + tcgen05 implicit GEMM (matmul; convolutions through TMA im2col)  */
-    SG_KERNEL_CONV_STRIP = 3,  /* tcgen05 kernel for stride-1 bf16 convolutions: resident filter, each
+    SG_KERNEL_CONV_STRIP = 3,  /* tcgen05 kernels for stride-1 convolutions: resident filter, each      
                                   input pixel fetched once per tile                                      */
     SG_KERNEL_TMA_MOVE = 4     /* copy / transpose that move every tile with TMA loads and stores        */
 };

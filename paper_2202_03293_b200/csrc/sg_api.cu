@@ -37,7 +37,7 @@ sg_status run(const Problem &p, const void *In, const void *Flt, float *O, cudaS
         if (st != SG_ERR_UNSUPPORTED) return st;
     }
     if (force == SG_KERNEL_AUTO || force == SG_KERNEL_CONV_STRIP) {
-        // stride-1 bf16 convolutions whose filter fits in shared memory
+        // stride-1 convolutions whose filter stays on the SM (when the choice is free: also those whose filter streams)
         bool resident = true;
         sg_status st = launch_conv_wide(p, In, Flt, O, force == SG_KERNEL_AUTO, &resident, stream);
         if (st == SG_OK && !resident) { t_last_kernel = SG_KERNEL_TENSOR; return SG_OK; }

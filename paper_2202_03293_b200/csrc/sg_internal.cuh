@@ -63,7 +63,7 @@ bool tensor_encode_tiled(CUtensorMap *map, CUtensorMapDataType type, int rank, v
 // shape or layout does not qualify (nothing is launched then).
 sg_status launch_conv_strip(const Problem &p, const void *In, const void *Flt, float *O, cudaStream_t stream);
 sg_status conv_read_status(cudaStream_t stream);
-// Stride-1 bf16 convolutions with the filter as the M operand (sg_conv_wide.cu); same contract.
+// Stride-1 convolutions with the filter as the M operand (sg_conv_wide.cu); same contract.
 // `streaming`: filters that do not fit in shared memory are taken too; *resident_filter reports whether this one does.
 sg_status launch_conv_wide(const Problem &p, const void *In, const void *Flt, float *O, bool streaming, bool *resident_filter, cudaStream_t stream);
 sg_status conv_wide_read_status(cudaStream_t stream);

@@ -51,8 +51,9 @@ constexpr int BM = 128;           // rows of an output tile = lanes of TMEM = M 
 constexpr int ROW_BYTES = 128;    // one k-block = one 128-byte swizzle row: 64 bf16 or 32 f32
 constexpr int K_STEPS = 4;        // tcgen05.mma per k-block and product: 32 bytes of k each
 constexpr int A_STAGE_BYTES = BM * ROW_BYTES;
-constexpr int CONVERTER_THREADS = 512;        // f32 path: 16 warps splitting tiles into hi and lo (one k-block is a serial
-                                              // chain of ~200 instructions per warp with 8 warps: longer than its MMAs take)
+// f32 path: 16 warps splitting tiles into hi and lo, in two groups that take the k-blocks in turn: a k-block is a chain of about
+// 1400 cycles of latencies (two barriers, loads, splits, stores, fences) however many warps share its work, longer than its MMAs take
+constexpr int CONVERTER_THREADS = 512, GROUP_THREADS = CONVERTER_THREADS / 2;
 constexpr int STAGING_BYTES = 2 * 16384;      // epilogue: 2 staging tiles of 128 rows x 128 B
 
 
@@ -121,6 +122,9 @@ struct Cfg {
     static_assert(STAGES >= 2 && STAGES <= 8, "ring depth");
     static_assert(KPS == 1 || (KPS == 2 && !F32), "k-blocks per stage");
     static_assert(!TA || F32, "tensor-memory input operand: f32 path only");
+    // each converter group keeps to its own slot and its own stages (a group that waited on a barrier of the other one's could take
+    // the phase before the last for the one it waits for)
+    static_assert(!F32 || (SPLIT_SLOTS == 2 && STAGES % 2 == 0), "two converter groups");
 };
 
 // Static tile order: groups of 8 tile-rows, row index fastest inside a group, so that the
@@ -196,15 +200,15 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant
 
     if (threadIdx.x == 0) {
         // full: one arrive.expect_tx by each of the two producers.  empty: one tcgen05.commit (bf16) or one arrive per
-        // converter warp of this CTA (f32).  split_full: one arrive per converter warp of every CTA
+        // warp of the converter group whose k-block it is (f32).  split_full: one arrive per such warp of every CTA
         // of the group.  split_empty / acc_full: one tcgen05.commit.  acc_empty: one arrive per
         // epilogue warp of every CTA of the group.
         for (int s = 0; s < C::STAGES; ++s) {
             mbar_init(full_bar(s), 2);
-            mbar_init(empty_bar(s), F32 ? CONVERTER_THREADS / 32 : 1);
+            mbar_init(empty_bar(s), F32 ? GROUP_THREADS / 32 : 1);
         }
         for (int s = 0; s < C::SPLIT_SLOTS; ++s) {
-            mbar_init(split_full_bar(s), (CONVERTER_THREADS / 32) * CG);
+            mbar_init(split_full_bar(s), (GROUP_THREADS / 32) * CG);
             mbar_init(split_empty_bar(s), 1);
         }
         for (int b = 0; b < 2; ++b) { mbar_init(acc_full_bar(b), 1); mbar_init(acc_empty_bar(b), 4 * CG); }
@@ -487,18 +491,17 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant
     } else if (warp >= 6) {
         // ------------------------------------------------------------ converter (f32 only; warps 6 to 21)
         if constexpr (F32) {
-            const int cw = warp - 6;                       // converter warp
-            const int ct = (int)threadIdx.x - 192;         // converter thread
+            const int group = (warp - 6) >> 3, cw = (warp - 6) & 7;       // converter group, warp of it
+            const int ct = cw * 32 + lane;                                // thread of the group
             // MIX: this thread's fixed share of a k-block.  Input: row (warp & 3) * 32 + lane (the TMEM lane quarter this warp
-            // may touch), k columns 8 * (cw >> 2) ..: two 16-byte chunks of the swizzled raw row.  Filter: unit cw = (sub-tile of
-            // 32 columns, quarter of its 32 k): lane = column f reads 8 k down its column and owns chunks of row f.
-            uint32_t mx_a_off[2] = {0, 0}, mx_hi_off[2] = {0, 0}, mx_b_src = 0, mx_h16_off = 0, mx_l16_off = 0, mx_tmem = 0;
-            bool mx_has_unit = false;
+            // may touch), k columns 16 * (cw >> 2) ..: four 16-byte chunks of the swizzled raw row.  Filter: units cw and cw + 8
+            // (sub-tile of 32 columns, quarter of its 32 k): lane = column f reads 8 k down its column and owns chunks of row f.
+            constexpr int UNITS = C::B_COLS / 64;                         // 4 * B_COLS / 32 units on 8 warps (64 columns: one each)
+            uint32_t mx_a_off[4] = {0, 0, 0, 0}, mx_hi_off[2] = {0, 0}, mx_b_src = 0, mx_h16_off = 0, mx_l16_off = 0, mx_tmem = 0;
             if constexpr (MIX) {
                 const int row = (warp & 3) * 32 + lane;
-                for (int i = 0; i < 2; ++i) mx_a_off[i] = (uint32_t)(row * 128 + ((((cw >> 2) * 2 + i) ^ (row & 7)) << 4));
+                for (int i = 0; i < 4; ++i) mx_a_off[i] = (uint32_t)(row * 128 + ((((cw >> 2) * 4 + i) ^ (row & 7)) << 4));
                 const int uj = cw >> 2, uq = cw & 3, f = uj * 32 + lane;
-                mx_has_unit = cw < 4 * C::B_COLS / 32;
                 mx_b_src = (uint32_t)(A_STAGE_BYTES + uj * C::SUB_BYTES + (uq * 8 * 32 + lane) * 4);
                 const uint32_t rowoff = (uint32_t)((f >> 3) * 1024 + (f & 7) * 128);
                 mx_hi_off[0] = rowoff + (uint32_t)(((2 * uq) ^ (f & 7)) << 4);
@@ -507,51 +510,70 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant
                 mx_l16_off = (uint32_t)C::B_STAGE_BYTES + rowoff + (uint32_t)(((4 + uq) ^ (f & 7)) << 4);
                 mx_tmem = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(C::ACC_BUFS * BN);
             }
+            // (the warp's lanes go on together, as the tcgen05 instructions below require)
+            auto wait_all = [&](bool passed) { return __all_sync(0xffffffffu, passed) != 0; };
             int it = 0;
             bool ok = true;
             Cursor cur{0, sk_u0};
             int tile, kb0, kb1, add;
             while (ok && next_item(cur, tile, kb0, kb1, add)) {
                 for (int kb = kb0; kb < kb1; ++kb, ++it) {
-                    const int r = it % C::STAGES, s = it % C::SPLIT_SLOTS;
-                    if (!mbar_wait(full_bar(r), (it / C::STAGES) & 1, abort_flag)) { ok = false; break; }
-                    if (!mbar_wait<CG == 2>(split_empty_bar(s), ((it / C::SPLIT_SLOTS) & 1) ^ 1u, abort_flag)) { ok = false; break; }
-                    if constexpr (TA) tc_fence_after();     // the MMAs that read this slot's tensor-memory columns are done
+                    if ((it & 1) != group) continue;
+                    const int r = it % C::STAGES, s = group;
+                    if (!wait_all(mbar_wait(full_bar(r), (it / C::STAGES) & 1, abort_flag))) { ok = false; break; }
                     const uint8_t *raw = smem_gen + r * C::STAGE_BYTES;
                     uint8_t *slot = smem_gen + C::STAGES * C::STAGE_BYTES + s * C::SPLIT_BYTES;
+                    // waits for the MMAs that read this slot two k-blocks ago
+                    auto slot_free = [&]() {
+                        const bool free = wait_all(mbar_wait<CG == 2>(split_empty_bar(s), ((it / C::SPLIT_SLOTS) & 1) ^ 1u, abort_flag));
+                        if constexpr (TA) tc_fence_after();
+                        return free;
+                    };
                     if constexpr (MIX) {
                         // Plain layout, corrections as bf16 MMAs.  Every address below is fixed per thread (set up ahead of
                         // the loops); the loads go out first, input rows then filter columns.
-                        const uint4 a0 = *reinterpret_cast<const uint4 *>(raw + mx_a_off[0]);
-                        const uint4 a1 = *reinterpret_cast<const uint4 *>(raw + mx_a_off[1]);
-                        uint32_t x[8];
-                        if (mx_has_unit) {
-                            const float *col = reinterpret_cast<const float *>(raw + mx_b_src);
+                        uint4 a[4];
 #pragma unroll
-                            for (int k = 0; k < 8; ++k) x[k] = __float_as_uint(col[k * 32]);
+                        for (int i = 0; i < 4; ++i) a[i] = *reinterpret_cast<const uint4 *>(raw + mx_a_off[i]);
+                        uint32_t x[UNITS][8];
+#pragma unroll
+                        for (int u = 0; u < UNITS; ++u) {
+                            const uint32_t *col = reinterpret_cast<const uint32_t *>(raw + mx_b_src + u * 2 * C::SUB_BYTES);
+#pragma unroll
+                            for (int k = 0; k < 8; ++k) x[u][k] = col[k * 32];
                         }
-                        // input: this thread's 8 k of its row -> tf32 hi (8 columns), bf16 pairs lo and hi (4 columns each)
+                        // input: this thread's 16 k of its row -> tf32 hi (16 columns), bf16 pairs lo and hi (8 columns each)
                         {
-                            uint4 h0, h1, h16, l16;
-                            split8_mix(a0, a1, h0, h1, h16, l16);
-                            const uint32_t hi[8] = {h0.x, h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w};
-                            const uint32_t lo4[4] = {l16.x, l16.y, l16.z, l16.w}, hi4[4] = {h16.x, h16.y, h16.z, h16.w};
+                            uint32_t hi[16], lo8[8], hi8[8];
+#pragma unroll
+                            for (int i = 0; i < 2; ++i) {
+                                uint4 h0, h1, h16, l16;
+                                split8_mix(a[2 * i], a[2 * i + 1], h0, h1, h16, l16);
+                                hi[8 * i] = h0.x; hi[8 * i + 1] = h0.y; hi[8 * i + 2] = h0.z; hi[8 * i + 3] = h0.w;
+                                hi[8 * i + 4] = h1.x; hi[8 * i + 5] = h1.y; hi[8 * i + 6] = h1.z; hi[8 * i + 7] = h1.w;
+                                lo8[4 * i] = l16.x; lo8[4 * i + 1] = l16.y; lo8[4 * i + 2] = l16.z; lo8[4 * i + 3] = l16.w;
+                                hi8[4 * i] = h16.x; hi8[4 * i + 1] = h16.y; hi8[4 * i + 2] = h16.z; hi8[4 * i + 3] = h16.w;
+                            }
+                            if (!slot_free()) { ok = false; break; }
                             const uint32_t t_base = mx_tmem + (uint32_t)(s * 64);
-                            tmem_st_32x8(t_base + (cw >> 2) * 8, hi);
-                            tmem_st_32x4(t_base + 32 + (cw >> 2) * 4, lo4);
-                            tmem_st_32x4(t_base + 48 + (cw >> 2) * 4, hi4);
+                            tmem_st_32x16(t_base + (cw >> 2) * 16, hi);
+                            tmem_st_32x8(t_base + 32 + (cw >> 2) * 8, lo8);
+                            tmem_st_32x8(t_base + 48 + (cw >> 2) * 8, hi8);
                         }
                         // filter: 8 k of this lane's column -> two chunks of its row of the tf32 hi tile, one chunk each of the
                         // hi half and the lo half of its row of the bf16 tile (rows of 128 B, 128-byte swizzled)
-                        if (mx_has_unit) {
+#pragma unroll
+                        for (int u = 0; u < UNITS; ++u) {
                             uint4 h0, h1, h16, l16;
-                            split8_mix(make_uint4(x[0], x[1], x[2], x[3]), make_uint4(x[4], x[5], x[6], x[7]), h0, h1, h16, l16);
-                            *reinterpret_cast<uint4 *>(slot + mx_hi_off[0]) = h0;
-                            *reinterpret_cast<uint4 *>(slot + mx_hi_off[1]) = h1;
-                            *reinterpret_cast<uint4 *>(slot + mx_h16_off) = h16;
-                            *reinterpret_cast<uint4 *>(slot + mx_l16_off) = l16;
+                            split8_mix(make_uint4(x[u][0], x[u][1], x[u][2], x[u][3]), make_uint4(x[u][4], x[u][5], x[u][6], x[u][7]), h0, h1, h16, l16);
+                            uint8_t *dst = slot + u * 8192;       // 64 columns on: eight 8-row groups
+                            *reinterpret_cast<uint4 *>(dst + mx_hi_off[0]) = h0;
+                            *reinterpret_cast<uint4 *>(dst + mx_hi_off[1]) = h1;
+                            *reinterpret_cast<uint4 *>(dst + mx_h16_off) = h16;
+                            *reinterpret_cast<uint4 *>(dst + mx_l16_off) = l16;
                         }
                     } else {
+                    if (!slot_free()) { ok = false; break; }
                     // An operand tile that arrives K-major (rows of 32 k, 128-byte swizzled by the TMA) is
                     // split elementwise: the swizzled placement of the elements is kept.
                     auto split_elementwise = [&](const uint8_t *src_tile, uint8_t *hi_tile, uint8_t *lo_tile, auto bytes_tag) {
@@ -559,17 +581,17 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant
                         const uint4 *src = reinterpret_cast<const uint4 *>(src_tile) + ct;
                         uint4 *hi = reinterpret_cast<uint4 *>(hi_tile) + ct;
                         uint4 *lo = reinterpret_cast<uint4 *>(lo_tile) + ct;
-                        constexpr int N = BYTES / 16 / CONVERTER_THREADS;   // 16-byte chunks per thread
-                        static_assert(N >= 1 && BYTES % (16 * CONVERTER_THREADS) == 0, "converter chunking");
+                        constexpr int N = BYTES / 16 / GROUP_THREADS;   // 16-byte chunks per thread
+                        static_assert(N >= 1 && BYTES % (16 * GROUP_THREADS) == 0, "converter chunking");
                         uint4 v[N];
 #pragma unroll
-                        for (int i = 0; i < N; ++i) v[i] = src[i * CONVERTER_THREADS];
+                        for (int i = 0; i < N; ++i) v[i] = src[i * GROUP_THREADS];
 #pragma unroll
                         for (int i = 0; i < N; ++i) {
                             uint4 h, l;
                             split4(v[i], h, l);
-                            hi[i * CONVERTER_THREADS] = h;
-                            lo[i * CONVERTER_THREADS] = l;
+                            hi[i * GROUP_THREADS] = h;
+                            lo[i * GROUP_THREADS] = l;
                         }
                     };
                     // An operand tile that arrives MN-major (sub-tiles of [32 k][32 rows-or-columns], 128-byte
@@ -582,7 +604,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant
                         const float *braw = reinterpret_cast<const float *>(src_tile);
                         constexpr int UNITS = 8 * COLS / 32;
 #pragma unroll
-                        for (int u = cw; u < UNITS; u += CONVERTER_THREADS / 32) {
+                        for (int u = cw; u < UNITS; u += GROUP_THREADS / 32) {
                             const int j = u >> 3, eighth = u & 7;
                             const float *col = braw + j * (C::SUB_BYTES / 4) + eighth * 4 * 32 + lane;
                             uint32_t x[4];
@@ -602,24 +624,25 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant
                     // Order within a k-block: the input rows are read first, the filter part (shared memory to shared
                     // memory) runs while those loads are in flight, then the input part goes to tensor memory and the
                     // proxy fence for the filter writes overlaps the tensor-memory stores; one wait at the end.
-                    uint4 a_raw[2];
+                    uint4 a_raw[4];
                     if constexpr (TA) {
-                        // input tile -> tensor memory: this warp may touch lane quarter (warp & 3); the four warps
-                        // of a quarter take 8 of the 32 k columns each.  Lane = row reads its 32 bytes of the
-                        // swizzled raw tile and stores 8 hi and 8 lo words.
+                        // input tile -> tensor memory: this warp may touch lane quarter (warp & 3); the two warps
+                        // of a quarter take 16 of the 32 k columns each.  Lane = row reads its 64 bytes of the
+                        // swizzled raw tile and stores 16 hi and 16 lo words.
                         if constexpr (A_MN) {
                             // stored transposed: the raw tile is four [32 k][32 rows] sub-tiles (128-byte rows, not
-                            // swizzled); sub-tile (warp & 3) holds this warp's rows, lane = row reads its 8 k values
+                            // swizzled); sub-tile (warp & 3) holds this warp's rows, lane = row reads its 16 k values
                             // down a column (every load a whole 128-byte row across the warp)
-                            const float *col = reinterpret_cast<const float *>(raw) + (warp & 3) * (C::SUB_BYTES / 4) + (cw >> 2) * 8 * 32 + lane;
-                            a_raw[0] = make_uint4(__float_as_uint(col[0]), __float_as_uint(col[32]), __float_as_uint(col[64]), __float_as_uint(col[96]));
-                            a_raw[1] = make_uint4(__float_as_uint(col[128]), __float_as_uint(col[160]), __float_as_uint(col[192]), __float_as_uint(col[224]));
+                            const float *col = reinterpret_cast<const float *>(raw) + (warp & 3) * (C::SUB_BYTES / 4) + (cw >> 2) * 16 * 32 + lane;
+#pragma unroll
+                            for (int i = 0; i < 4; ++i)
+                                a_raw[i] = make_uint4(__float_as_uint(col[i * 128]), __float_as_uint(col[i * 128 + 32]), __float_as_uint(col[i * 128 + 64]), __float_as_uint(col[i * 128 + 96]));
                         } else {
                             const int row = (warp & 3) * 32 + lane;
                             const uint8_t *rp = raw + row * 128;
 #pragma unroll
-                            for (int i = 0; i < 2; ++i)
-                                a_raw[i] = *reinterpret_cast<const uint4 *>(rp + ((((cw >> 2) * 2 + i) ^ (row & 7)) << 4));
+                            for (int i = 0; i < 4; ++i)
+                                a_raw[i] = *reinterpret_cast<const uint4 *>(rp + ((((cw >> 2) * 4 + i) ^ (row & 7)) << 4));
                         }
                     } else if constexpr (A_MN) {
                         split_transpose(raw, slot, slot + A_STAGE_BYTES, std::integral_constant<int, BM>{});
@@ -632,20 +655,22 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant
                         split_transpose(raw + A_STAGE_BYTES, b_slot, b_slot + C::B_STAGE_BYTES, std::integral_constant<int, C::B_COLS>{});
                     if constexpr (TA) {
                         const int quarter = warp & 3, kpart = cw >> 2;
-                        uint32_t hi[8], lo[8];
+                        uint32_t hi[16], lo[16];
 #pragma unroll
-                        for (int i = 0; i < 2; ++i) {
+                        for (int i = 0; i < 4; ++i) {
                             uint4 h, l;
                             split4(a_raw[i], h, l);
                             hi[4 * i] = h.x; hi[4 * i + 1] = h.y; hi[4 * i + 2] = h.z; hi[4 * i + 3] = h.w;
                             lo[4 * i] = l.x; lo[4 * i + 1] = l.y; lo[4 * i + 2] = l.z; lo[4 * i + 3] = l.w;
                         }
-                        const uint32_t t_hi = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(C::ACC_BUFS * BN + s * 64 + kpart * 8);
-                        tmem_st_32x8(t_hi, hi);
-                        tmem_st_32x8(t_hi + 32, lo);
+                        const uint32_t t_hi = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(C::ACC_BUFS * BN + s * 64 + kpart * 16);
+                        __syncwarp();
+                        tmem_st_32x16(t_hi, hi);
+                        tmem_st_32x16(t_hi + 32, lo);
                     }
                     }   // (!MIX)
                     fence_async_smem();     // generic-proxy writes -> visible to the tensor core's reads
+                    __syncwarp();
                     if constexpr (TA) {
                         tmem_st_wait();
                         tc_fence_before();

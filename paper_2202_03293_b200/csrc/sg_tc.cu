@@ -573,7 +573,6 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant
                             *reinterpret_cast<uint4 *>(dst + mx_l16_off) = l16;
                         }
                     } else {
-                    if (!slot_free()) { ok = false; break; }
                     // An operand tile that arrives K-major (rows of 32 k, 128-byte swizzled by the TMA) is
                     // split elementwise: the swizzled placement of the elements is kept.
                     auto split_elementwise = [&](const uint8_t *src_tile, uint8_t *hi_tile, uint8_t *lo_tile, auto bytes_tag) {
@@ -582,48 +581,50 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant
                         uint4 *hi = reinterpret_cast<uint4 *>(hi_tile) + ct;
                         uint4 *lo = reinterpret_cast<uint4 *>(lo_tile) + ct;
                         constexpr int N = BYTES / 16 / GROUP_THREADS;   // 16-byte chunks per thread
-                        static_assert(N >= 1 && BYTES % (16 * GROUP_THREADS) == 0, "converter chunking");
+                        static_assert(N % 2 == 0 && BYTES % (16 * GROUP_THREADS) == 0, "converter chunking");
                         uint4 v[N];
 #pragma unroll
                         for (int i = 0; i < N; ++i) v[i] = src[i * GROUP_THREADS];
 #pragma unroll
-                        for (int i = 0; i < N; ++i) {
-                            uint4 h, l;
-                            split4(v[i], h, l);
-                            hi[i * GROUP_THREADS] = h;
-                            lo[i * GROUP_THREADS] = l;
+                        for (int i = 0; i < N; i += 2) {
+                            uint4 h0, l0, h1, l1;
+                            split8(v[i], v[i + 1], h0, l0, h1, l1);
+                            hi[i * GROUP_THREADS] = h0;
+                            lo[i * GROUP_THREADS] = l0;
+                            hi[(i + 1) * GROUP_THREADS] = h1;
+                            lo[(i + 1) * GROUP_THREADS] = l1;
                         }
                     };
                     // An operand tile that arrives MN-major (sub-tiles of [32 k][32 rows-or-columns], 128-byte
                     // rows, not swizzled) is transposed while it is split: the split tiles are K-major,
                     // [row][32 k] rows of 128 B in 8-row groups with the 128-byte swizzle (16-byte chunk c of
-                    // row f sits at chunk c ^ (f & 7)).  A unit is an eighth of a sub-tile (4 k); lane = f
-                    // reads a column (one 128-byte row per load across the warp) and writes one chunk of its row.
+                    // row f sits at chunk c ^ (f & 7)).  A unit is a quarter of a sub-tile (8 k); lane = f
+                    // reads a column (one 128-byte row per load across the warp) and writes two chunks of its row.
                     auto split_transpose = [&](const uint8_t *src_tile, uint8_t *hi_tile, uint8_t *lo_tile, auto cols_tag) {
                         constexpr int COLS = decltype(cols_tag)::value;
                         const float *braw = reinterpret_cast<const float *>(src_tile);
-                        constexpr int UNITS = 8 * COLS / 32;
+                        constexpr int UNITS = 4 * COLS / 32;
 #pragma unroll
                         for (int u = cw; u < UNITS; u += GROUP_THREADS / 32) {
-                            const int j = u >> 3, eighth = u & 7;
-                            const float *col = braw + j * (C::SUB_BYTES / 4) + eighth * 4 * 32 + lane;
-                            uint32_t x[4];
-#pragma unroll
-                            for (int k = 0; k < 4; ++k) x[k] = __float_as_uint(col[k * 32]);
+                            const int j = u >> 2, quarter = u & 3;
+                            const uint32_t *col = reinterpret_cast<const uint32_t *>(braw) + j * (C::SUB_BYTES / 4) + quarter * 8 * 32 + lane;
                             const int f = j * 32 + lane;
-                            const int off = (f >> 3) * 1024 + (f & 7) * 128 + ((eighth ^ (f & 7)) << 4);
-                            uint4 h, l;
-                            split4(make_uint4(x[0], x[1], x[2], x[3]), h, l);
-                            *reinterpret_cast<uint4 *>(hi_tile + off) = h;
-                            *reinterpret_cast<uint4 *>(lo_tile + off) = l;
+                            const int row = (f >> 3) * 1024 + (f & 7) * 128;
+                            const int off0 = row + (((2 * quarter) ^ (f & 7)) << 4), off1 = row + (((2 * quarter + 1) ^ (f & 7)) << 4);
+                            uint4 h0, l0, h1, l1;
+                            split8(make_uint4(col[0], col[32], col[64], col[96]), make_uint4(col[128], col[160], col[192], col[224]), h0, l0, h1, l1);
+                            *reinterpret_cast<uint4 *>(hi_tile + off0) = h0;
+                            *reinterpret_cast<uint4 *>(lo_tile + off0) = l0;
+                            *reinterpret_cast<uint4 *>(hi_tile + off1) = h1;
+                            *reinterpret_cast<uint4 *>(lo_tile + off1) = l1;
                         }
                     };
                     // input: K-major as stored, M-major when stored transposed; filter: N-major as stored,
                     // K-major when stored transposed.  kind::tf32 takes K-major operands only.
                     uint8_t *b_slot = slot + (TA ? 0 : 2 * A_STAGE_BYTES);
-                    // Order within a k-block: the input rows are read first, the filter part (shared memory to shared
-                    // memory) runs while those loads are in flight, then the input part goes to tensor memory and the
-                    // proxy fence for the filter writes overlaps the tensor-memory stores; one wait at the end.
+                    // Order within a k-block: the input part is read and split while the MMAs may still read the slot, then goes to
+                    // tensor memory; the filter part (shared memory to shared memory) and its proxy fence overlap the tensor-memory
+                    // stores; one wait at the end.
                     uint4 a_raw[4];
                     if constexpr (TA) {
                         // input tile -> tensor memory: this warp may touch lane quarter (warp & 3); the two warps
@@ -644,30 +645,34 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant
                             for (int i = 0; i < 4; ++i)
                                 a_raw[i] = *reinterpret_cast<const uint4 *>(rp + ((((cw >> 2) * 4 + i) ^ (row & 7)) << 4));
                         }
+                        const int quarter = warp & 3, kpart = cw >> 2;
+                        uint32_t hi[16], lo[16];
+#pragma unroll
+                        for (int i = 0; i < 2; ++i) {
+                            uint4 h[2], l[2];
+                            split8(a_raw[2 * i], a_raw[2 * i + 1], h[0], l[0], h[1], l[1]);
+#pragma unroll
+                            for (int e = 0; e < 2; ++e) {
+                                const int o = 8 * i + 4 * e;
+                                hi[o] = h[e].x; hi[o + 1] = h[e].y; hi[o + 2] = h[e].z; hi[o + 3] = h[e].w;
+                                lo[o] = l[e].x; lo[o + 1] = l[e].y; lo[o + 2] = l[e].z; lo[o + 3] = l[e].w;
+                            }
+                        }
+                        const uint32_t t_hi = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(C::ACC_BUFS * BN + s * 64 + kpart * 16);
+                        if (!slot_free()) { ok = false; break; }
+                        tmem_st_32x16(t_hi, hi);
+                        tmem_st_32x16(t_hi + 32, lo);
                     } else if constexpr (A_MN) {
+                        if (!slot_free()) { ok = false; break; }
                         split_transpose(raw, slot, slot + A_STAGE_BYTES, std::integral_constant<int, BM>{});
                     } else {
+                        if (!slot_free()) { ok = false; break; }
                         split_elementwise(raw, slot, slot + A_STAGE_BYTES, std::integral_constant<int, A_STAGE_BYTES>{});
                     }
                     if constexpr (B_KM)
                         split_elementwise(raw + A_STAGE_BYTES, b_slot, b_slot + C::B_STAGE_BYTES, std::integral_constant<int, C::B_STAGE_BYTES>{});
                     else
                         split_transpose(raw + A_STAGE_BYTES, b_slot, b_slot + C::B_STAGE_BYTES, std::integral_constant<int, C::B_COLS>{});
-                    if constexpr (TA) {
-                        const int quarter = warp & 3, kpart = cw >> 2;
-                        uint32_t hi[16], lo[16];
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            uint4 h, l;
-                            split4(a_raw[i], h, l);
-                            hi[4 * i] = h.x; hi[4 * i + 1] = h.y; hi[4 * i + 2] = h.z; hi[4 * i + 3] = h.w;
-                            lo[4 * i] = l.x; lo[4 * i + 1] = l.y; lo[4 * i + 2] = l.z; lo[4 * i + 3] = l.w;
-                        }
-                        const uint32_t t_hi = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(C::ACC_BUFS * BN + s * 64 + kpart * 16);
-                        __syncwarp();
-                        tmem_st_32x16(t_hi, hi);
-                        tmem_st_32x16(t_hi + 32, lo);
-                    }
                     }   // (!MIX)
                     fence_async_smem();     // generic-proxy writes -> visible to the tensor core's reads
                     __syncwarp();

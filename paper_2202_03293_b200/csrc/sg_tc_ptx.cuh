@@ -381,6 +381,23 @@ __device__ __forceinline__ void split4(const uint4 v, uint4 &h, uint4 &l) {
     }
 }
 
+// The same for eight words, with one check for the slow path.
+__device__ __forceinline__ void split8(const uint4 v0, const uint4 v1, uint4 &h0, uint4 &l0, uint4 &h1, uint4 &l1) {
+    auto mag = [](uint32_t x) { return fabsf(__uint_as_float(x)); };
+    const float big = fmaxf(fmaxf(fmaxf(mag(v0.x), mag(v0.y)), fmaxf(mag(v0.z), mag(v0.w))), fmaxf(fmaxf(mag(v1.x), mag(v1.y)), fmaxf(mag(v1.z), mag(v1.w))));
+    if (big < 1.7014118e38f) {
+        auto one = [](uint32_t x, uint32_t &hi, uint32_t &lo) {
+            hi = (x + 0x1000u) & 0xFFFFE000u;
+            lo = (__float_as_uint(__uint_as_float(x) - __uint_as_float(hi)) + 0x1000u) & 0xFFFFE000u;
+        };
+        one(v0.x, h0.x, l0.x); one(v0.y, h0.y, l0.y); one(v0.z, h0.z, l0.z); one(v0.w, h0.w, l0.w);
+        one(v1.x, h1.x, l1.x); one(v1.y, h1.y, l1.y); one(v1.z, h1.z, l1.z); one(v1.w, h1.w, l1.w);
+    } else {
+        split4(v0, h0, l0);
+        split4(v1, h1, l1);
+    }
+}
+
 // Packs two f32 values, rounded to the nearest bf16, into one word: `even` in the low half, `odd` in the high half.
 __device__ __forceinline__ uint32_t pack_bf16(float even, float odd) {
     uint32_t d;
@@ -419,12 +436,28 @@ __device__ __forceinline__ void split4_mix(const uint4 v, uint4 &h, uint2 &h16, 
 
 
 // The same for eight values (two chunks of four): hi of each chunk, and the eight bf16 values of hi and of lo packed in k order.
+// One check for the slow path covers all eight.
 __device__ __forceinline__ void split8_mix(const uint4 v0, const uint4 v1, uint4 &h0, uint4 &h1, uint4 &h16, uint4 &l16) {
-    uint2 a, b, c, d;
-    split4_mix(v0, h0, a, b);
-    split4_mix(v1, h1, c, d);
-    h16 = make_uint4(a.x, a.y, c.x, c.y);
-    l16 = make_uint4(b.x, b.y, d.x, d.y);
+    auto mag = [](uint32_t x) { return fabsf(__uint_as_float(x)); };
+    const float big = fmaxf(fmaxf(fmaxf(mag(v0.x), mag(v0.y)), fmaxf(mag(v0.z), mag(v0.w))), fmaxf(fmaxf(mag(v1.x), mag(v1.y)), fmaxf(mag(v1.z), mag(v1.w))));
+    if (big < 1.7014118e38f) {
+        auto two = [](uint32_t x, uint32_t y, uint32_t &hx, uint32_t &hy, uint32_t &h, uint32_t &l) {
+            hx = (x + 0x1000u) & 0xFFFFE000u;
+            hy = (y + 0x1000u) & 0xFFFFE000u;
+            h = pack_bf16(__uint_as_float(hx), __uint_as_float(hy));
+            l = pack_bf16(__uint_as_float(x) - __uint_as_float(hx), __uint_as_float(y) - __uint_as_float(hy));
+        };
+        two(v0.x, v0.y, h0.x, h0.y, h16.x, l16.x);
+        two(v0.z, v0.w, h0.z, h0.w, h16.y, l16.y);
+        two(v1.x, v1.y, h1.x, h1.y, h16.z, l16.z);
+        two(v1.z, v1.w, h1.z, h1.w, h16.w, l16.w);
+    } else {
+        uint2 a, b, c, d;
+        split4_mix(v0, h0, a, b);
+        split4_mix(v1, h1, c, d);
+        h16 = make_uint4(a.x, a.y, c.x, c.y);
+        l16 = make_uint4(b.x, b.y, d.x, d.y);
+    }
 }
 
 // Reads and clears this translation unit's status word; the caller has synchronised the stream.

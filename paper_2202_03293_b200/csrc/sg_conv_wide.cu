@@ -656,12 +656,14 @@ sg_status launch_conv_wide(const Problem &p, const void *In, const void *Flt, fl
     WideParams w{};
     F32Filter g{};
     if (f32) {
-        // the im2col kernel deals a reduction out over the SMs: where there are few positions and much to sum it is the better one
-        // (8 x 28 x 28, 3x3x256x256: 46.1 us here, 41.5 there; 16 x 56 x 56, 3x3x64x128: 32.3 against 41.6; both estimates are within
-        // a tenth or so)
+        // The im2col kernel deals a reduction out over the SMs: where there are few positions and much to sum it is the better one
+        // (8 x 28 x 28, 3x3x256x256: 43.9 us here, 38.5 there; 16 x 56 x 56, 3x3x64x128: 32.3 against 41.6; both estimates are within
+        // a tenth or so).  Filters of 65 to 128 columns that the strip kernel would keep resident run faster here whatever the
+        // estimates say (12 x 12 x 61, 1x1x16x96: 7.8 -> 5.6).
         const double us = plan_f32(p, positions, f_tiles, row_span, full_span, num_sms, streaming, w, g);
         const bool im2col = reinterpret_cast<uintptr_t>(O) % 16 == 0 && mult(p.o_w, 4);      // (its stores are the TMA's)
-        if (streaming && im2col && us >= 0.9 * tensor_estimate_us(p)) return SG_ERR_UNSUPPORTED;
+        const bool strip = p.N <= 128 && p.N > 64 && mult(p.N, 32) && (int64_t)g.taps * w.kb <= 6;
+        if (streaming && im2col && !strip && us >= 0.95 * tensor_estimate_us(p)) return SG_ERR_UNSUPPORTED;
     } else plan_bf16(p, positions, f_tiles, row_span, full_span, num_sms, streaming, w);
     if (w.BN == 0 || (int64_t)w.tiles * f_tiles > 0x7fffffff) return SG_ERR_UNSUPPORTED;
     w.row_step = w.per_row ? w.box_rows : (int)shift;

@@ -423,8 +423,10 @@ sg_status launch_small(const Problem &p, const void *In, const void *Flt, float 
         const double steps = p.K < BK ? 0.5 : (double)p.K / BK, waves = (double)((tiles + num_sms - 1) / num_sms);
         const double step = !f32 ? 0.36 : (waves > 1 ? 0.72 : half && tiles * 2 > num_sms ? 1.0 : 0.8) * (mix ? 1.0 : 1.25);
         const double us = 1.2 + waves * ((f32 ? 0.6 : 0.55) + step * steps);
-        // (the tcgen05 kernel never takes less than 3.1 us, f32 4.1: no need to ask)
-        if (us > (f32 ? 4.0 : 3.0) && us > (conv && in_bytes < 131072 ? 0.3 * p.K : 0.85 * tensor_estimate_us(p))) return SG_ERR_UNSUPPORTED;
+        // (the tcgen05 kernel never takes less than 3.1 us, f32 4.1: no need to ask.  Its f32 estimates are the closer ones.  Inputs stored
+        // transposed whose rows are no whole 128 bytes of m are left to the gather kernel, which takes over half as long again.)
+        const double lead = a_mn && p.M % (f32 ? 32 : 64) != 0 ? 1.6 : f32 ? 0.95 : 0.85;
+        if (us > (f32 ? 4.0 : 3.0) && us > (conv && in_bytes < 131072 ? 0.3 * p.K : lead * tensor_estimate_us(p))) return SG_ERR_UNSUPPORTED;
     }
     tensor_note_choice(TN, 1, 1);
 #define SG_SMALL(MODE_, A_MN_, B_KM_, CONV_, SLOT)                                                                  \

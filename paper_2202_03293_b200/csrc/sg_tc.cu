@@ -55,6 +55,7 @@ constexpr int A_STAGE_BYTES = BM * ROW_BYTES;
 // 1400 cycles of latencies (two barriers, loads, splits, stores, fences) however many warps share its work, longer than its MMAs take
 constexpr int CONVERTER_THREADS = 512, GROUP_THREADS = CONVERTER_THREADS / 2;
 constexpr int STAGING_BYTES = 2 * 16384;      // epilogue: 2 staging tiles of 128 rows x 128 B
+constexpr int MAX_MEET = 8;                   // CTAs of a cluster that share a tile's reduction
 
 
 struct TcParams {
@@ -71,8 +72,11 @@ struct TcParams {
     int b_blocked;       // 1: the filter map is blocked by sub-tile columns: one TMA load fetches the whole filter tile
     int sk_first_tile;   // stream-K tail: tiles from this one on are not dealt out whole; their k-blocks, taken as one
     int sk_units;        //   sequence, are cut into equal runs of `sk_units` k-blocks, one run per CTA (or pair); 0 = no tail
+    int meet;            // the `splits` CTAs of a tile are one cluster: their partial sums meet in its shared memory (one item per CTA)
+    float *out;          // with meet: the output's first element and row pitch
+    int64_t pitch;
     const float *bias;   // fused pointwise consumer of the write-back: O = act(acc + bias[column]); null = no bias
-    int act;             // SG_ACT_NONE or SG_ACT_RELU (only with one work item per tile and in overwrite mode)
+    int act;             // SG_ACT_NONE or SG_ACT_RELU (only where whole sums are at hand: one work item per tile, or meet; and in overwrite mode)
     int wait_prior;      // the launch may start before the kernel ahead of it in the stream has finished (programmatic
                          // dependent launch).  1: that kernel is this library's clearing kernel, which touches only the
                          // output: the stores wait for it (griddepcontrol.wait), the loads need not.  2: it is any
@@ -741,12 +745,13 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant
             tc_fence_after();
             Cursor ahead = cur;
             int t2, k2, k3, a2;
-            if (BN >= 128 && !next_item(ahead, t2, k2, k3, a2)) {
+            const bool meet = CG == 1 && p.meet != 0;
+            if ((BN >= 128 || meet) && !next_item(ahead, t2, k2, k3, a2)) {
                 // The last item: the rings are idle by now (every load has been consumed by an MMA that has finished), so all
                 // chunks are staged there and no chunk waits for the store of an earlier one (256 columns took 3.1 us
                 // through the two staging tiles, which nothing hides at the end of a launch; 4096 x 1024 x 1024 bf16 13.7 -> 12.9 us).
                 constexpr int PER_STEP = F32 ? 1 : 2;      // (f32: 88 registers per thread)
-                static_assert(BN < 128 || C::STAGES * C::STAGE_BYTES + C::SPLIT_SLOTS * C::SPLIT_BYTES >= BN / 32 * 16384, "the rings hold a tile");
+                static_assert(C::STAGES * C::STAGE_BYTES + C::SPLIT_SLOTS * C::SPLIT_BYTES >= BN / 32 * 16384, "the rings hold a tile");
 #pragma unroll 1
                 for (int j = 0; j < BN / 32; j += PER_STEP) {
                     uint32_t r[PER_STEP][32];
@@ -756,9 +761,10 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant
                     tmem_ld_wait();
 #pragma unroll
                     for (int i = 0; i < PER_STEP; ++i) {
-                        consume(r[i], j + i);
+                        if (!meet) consume(r[i], j + i);
                         stage_row(smem_gen + (j + i) * 16384, r[i]);
                     }
+                    if (meet) continue;                        // (the teardown sums the partial tiles of the cluster)
                     fence_async_smem();
                     epi_sync();
                     const int mine = (ew - j) & 3;             // the warps issue the stores in turn
@@ -819,6 +825,46 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant
     // a pair leaves together: the leader's MMAs read the peer's shared memory and both CTAs
     // signal barriers in each other's shared memory
     if constexpr (CG == 2) cluster_sync_all();
+    if constexpr (CG == 1) {
+        if (p.meet) {
+            // Every CTA of the cluster sums its share of the tile's rows over the partial tiles parked in all of them, in rank order,
+            // and applies the consumer: no clearing launch, no partial sums in global memory (256 x 256 x 4096 with
+            // bias + relu, until now one CTA per whole reduction: bf16 15.3 -> 6.8 us, f32 65.7 -> 14.1; 3496 x 192 x 6280 37.6 -> 20.8 and
+            // 102 -> 67).
+            if (p.wait_prior) asm volatile("griddepcontrol.wait;" ::: "memory");
+            cluster_sync_all();
+            const int rank = (int)cluster_ctarank(), rows = BM / p.meet;
+            int mt, nt;
+            tile_coords((int)blockIdx.x / p.meet, p.num_m_tiles, p.num_n_tiles, mt, nt);
+            const int m0 = mt * BM + rank * rows, n0 = nt * BN;
+            if (!*abort_flag)
+                for (int i = threadIdx.x; i < rows * (BN / 4); i += C::THREADS) {
+                    const int row = i / (BN / 4), j = (i >> 3) % (BN / 32), c = i & 7, m = m0 + row, n = n0 + j * 32 + c * 4;
+                    if (m >= p.M || n >= p.N) continue;
+                    const int x = rank * rows + row;
+                    const uint32_t src = smem_base + (uint32_t)(j * 16384 + x * 128 + ((c ^ (x & 7)) << 4));
+                    float4 part[MAX_MEET];
+#pragma unroll
+                    for (int r = 0; r < MAX_MEET; ++r)
+                        if (r < p.meet)
+                            asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                                         : "=f"(part[r].x), "=f"(part[r].y), "=f"(part[r].z), "=f"(part[r].w) : "r"(map_to_cta(src, r)) : "memory");
+                    float4 v = part[0];
+#pragma unroll
+                    for (int r = 1; r < MAX_MEET; ++r)
+                        if (r < p.meet) { v.x += part[r].x; v.y += part[r].y; v.z += part[r].z; v.w += part[r].w; }
+                    float4 *o = reinterpret_cast<float4 *>(p.out + (int64_t)m * p.pitch + n);
+                    if (p.bias != nullptr) {
+                        const float4 b = __ldg(reinterpret_cast<const float4 *>(p.bias + n));
+                        v.x += b.x; v.y += b.y; v.z += b.z; v.w += b.w;
+                    }
+                    if (p.act == SG_ACT_RELU) { v.x = v.x < 0.f ? 0.f : v.x; v.y = v.y < 0.f ? 0.f : v.y; v.z = v.z < 0.f ? 0.f : v.z; v.w = v.w < 0.f ? 0.f : v.w; }
+                    if (p.accumulate) { const float4 w = *o; v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w; }
+                    *o = v;
+                }
+            cluster_sync_all();      // nobody leaves while its partial tile is being read
+        }
+    }
     if (warp == 1) {
         tc_fence_after();
         if constexpr (CG == 2)
@@ -873,6 +919,7 @@ struct Overrides {
     int pdl = -1;    // SG_TC_PDL (testing): 0 = launches never overlap the tail of the kernel ahead of them
     int conv_single = 0;   // SG_CONV_SINGLE=1 (testing): the stride-1 convolution kernel never uses CTA pairs
     int small = -1;  // SG_TC_SMALL (testing): 0 = the kernel for small problems is never chosen, 1 = wherever the layout allows it
+    int meet = -1;   // SG_TC_MEET (testing): 0 = partial sums never meet in a cluster, 2, 4, 8 = in clusters of as many CTAs where possible
     int mix = -1;    // SG_TC_MIX (testing): 0 = f32 correction products as tf32 MMAs (three tf32 products per term) instead of bf16
 };
 std::mutex g_mu;
@@ -892,6 +939,7 @@ void read_env_locked() {
     g_ov.pdl = env("SG_TC_PDL", -1);
     g_ov.conv_single = env("SG_CONV_SINGLE", 0);
     g_ov.small = env("SG_TC_SMALL", -1);
+    g_ov.meet = env("SG_TC_MEET", -1);
     g_ov.mix = env("SG_TC_MIX", -1);
     g_ov.env_read = true;
 }
@@ -1048,34 +1096,51 @@ bool encode_im2col_cached(CUtensorMap *map, int device, CUtensorMapDataType type
 inline bool mult(int64_t v, int64_t q) { return v % q == 0; }
 
 struct Variant { int bn, cg; double mma_ns, mma_ns_f32; };
-// Time one CTA's tensor core (bf16) or shared memory (f32: TMA fill, hi/lo split and the operand
-// reads of 12 MMAs share it) needs for one k-block of a tile, in ns.
-constexpr Variant kVariants[] = {{64, 1, 100.0, 750.0}, {128, 1, 135.0, 1000.0}, {256, 1, 330.0, 1500.0},
-                                 {128, 2, 135.0, 750.0}, {256, 2, 330.0, 1000.0}};
+// Time one CTA needs for one k-block of a tile, in ns: its tensor core (bf16), or its converter warps and tensor core (f32).
+constexpr Variant kVariants[] = {{64, 1, 100.0, 500.0}, {128, 1, 135.0, 570.0}, {256, 1, 330.0, 1500.0},
+                                 {128, 2, 135.0, 515.0}, {256, 2, 330.0, 690.0}};
 constexpr int kNumVariants = sizeof(kVariants) / sizeof(kVariants[0]);
 
+// A stream-K tail (launch_tensor) pays when the k-blocks saved clearly outweigh the extra epilogues and the clearing launch.
+// Returns the k-blocks of a group's run, 0: no tail.
+int stream_k_run(const Variant &v, bool f32, int64_t tiles, int groups, int num_kb, int kps, bool whenever) {
+    const int left = (int)(tiles % groups);
+    if (tiles <= groups || left == 0 || num_kb % kps != 0) return 0;
+    const int64_t units = (int64_t)left * num_kb;
+    int run = (int)((units + groups - 1) / groups);
+    run = (run + kps - 1) / kps * kps;
+    const double saved = (double)(num_kb - run) * (f32 ? v.mma_ns_f32 : v.mma_ns);
+    const double extra = 2.0 * (1500.0 + (double)v.bn * (f32 ? 24.0 : 12.0)) + 2500.0;
+    return run >= 4 * kps && (saved > (f32 ? 1.4 : 2.0) * extra || whenever) ? run : 0;
+}
+
 // Estimated kernel time in ns of `tiles` tiles dealt out in `sp` k ranges each over `groups`
-// CTAs or CTA pairs.  A k-block costs the slowest of: the CTA's own MMA / shared-memory
-// time, the CTA's share of the L2 -> shared memory fill rate of the whole chip (what bounds
-// every large problem here: 9 to 14 TB/s), and the fill rate one SM reaches alone.  The
-// constants were fitted to timings of every variant and split on the 125 shapes
-// {256..4096}^3 in both dtypes; the choices they lead to are within 1 % of the best
-// per-shape choice in total time.
-double estimate_ns(const Variant &v, bool f32, int64_t tiles, int64_t groups, int num_kb, int sp, bool accumulate) {
+// CTAs or CTA pairs.  A k-block costs the slowest of: the CTA's own time, the CTA's share of the L2 -> shared memory fill
+// rate of the whole chip, and the fill rate one SM reaches alone.  The bf16 constants were fitted to timings of every variant and
+// split on the 125 shapes {256..4096}^3 (the choices they lead to are within 1 % of the best per-shape choice in total time), the
+// f32 ones to 48 shapes between 64 and 8192 (within 9 % of the timings, choices 1.3 % off the best in the mean).
+double estimate_ns(const Variant &v, bool f32, int64_t tiles, int64_t groups, int num_kb, int sp, bool accumulate, bool tail) {
     const int64_t items = tiles * sp;
     const int64_t waves = (items + groups - 1) / groups;
     const int kbs = (num_kb + sp - 1) / sp;
     const double active = (double)((items < groups ? items : groups) * v.cg);
     const double stage_bytes = A_STAGE_BYTES + (double)(v.bn / v.cg) * ROW_BYTES;
-    const double chip_fill = f32 ? 9000.0 : 14000.0, sm_fill = f32 ? 40.0 : 130.0;      // bytes per ns
+    const double chip_fill = f32 ? 11500.0 : 14000.0, sm_fill = f32 ? 54.0 : 130.0;      // bytes per ns
     double kb_ns = f32 ? v.mma_ns_f32 : v.mma_ns;
     if (active * stage_bytes / chip_fill > kb_ns) kb_ns = active * stage_bytes / chip_fill;
     if (stage_bytes / sm_fill > kb_ns) kb_ns = stage_bytes / sm_fill;
-    const double item_ns = 1500.0 + (double)v.bn * (f32 ? 24.0 : 12.0);                // pipeline fill + epilogue of one item
-    double t = (double)waves * kbs * kb_ns + item_ns + (double)(waves - 1) * (f32 ? 0.0 : 0.3) * item_ns;
-    if (v.cg == 2) t += f32 ? 800.0 : 2000.0;                                          // cluster launch, cross-CTA signalling
-    if (sp > 1) t += (f32 ? 4000.0 : 2500.0) - (accumulate ? 1500.0 : 0.0);            // reduce-add traffic, the clearing launch
+    const double item_ns = f32 ? 2770.0 + 20.0 * v.bn : 1500.0 + 12.0 * v.bn;          // pipeline fill + epilogue of one item
+    double t = (double)waves * kbs * kb_ns + item_ns + (double)(waves - 1) * 0.3 * item_ns;
+    const int run = f32 && sp == 1 && tail ? stream_k_run(v, f32, tiles, (int)groups, num_kb, 1, false) : 0;
+    if (run > 0) t += item_ns + 1500.0 - (double)(num_kb - run) * kb_ns;               // the last wave is shorter, the write-backs are more
+    if (v.cg == 2) t += f32 ? 600.0 : 2000.0;                                          // cluster launch, cross-CTA signalling
+    if (sp > 1) t += 2500.0 - (accumulate ? 1500.0 : 0.0);                             // reduce-add traffic, the clearing launch
     return t;
+}
+
+// The same for `sp` CTAs in a cluster per tile.
+double estimate_meet_ns(const Variant &v, bool f32, int64_t tiles, int num_kb, int sp) {
+    return estimate_ns(v, f32, tiles * sp, tiles * sp, (num_kb + sp - 1) / sp, 1, false, false) + (f32 ? 2200.0 : 1300.0 + 11.0 * v.bn);
 }
 
 // Operands stored transposed (matmuls only): bit 0 the input ([k][m], m contiguous), bit 1 the filter ([n][k], k contiguous).
@@ -1085,7 +1150,10 @@ inline int transposed_layout(const Problem &p) {
 }
 
 // Tile variant and k split of lowest estimated time, which is returned (unless the variant is forced); *out_pick = -1: none.
-double choose_tiles(const Problem &p, int num_kb, int lay, const Overrides &ov, int num_sms, int *out_pick, int *out_splits) {
+// *out_meet: the split's partial sums meet in a cluster.
+double choose_tiles(const Problem &p, int num_kb, int lay, const Overrides &ov, int num_sms, int *out_pick, int *out_splits, int *out_meet) {
+    *out_meet = 0;
+    const bool fused = p.bias != nullptr || p.act != SG_ACT_NONE, forced_tile = ov.bn > 0 || ov.cg > 0 || (ov.split > 0 && !fused);
     const bool f32 = !p.in_bf16;
     int pick = -1, splits = 1;
     double best = 1e300;
@@ -1118,15 +1186,32 @@ double choose_tiles(const Problem &p, int num_kb, int lay, const Overrides &ov, 
             const int64_t tiles = (int64_t)((p.M + v.cg * BM - 1) / (v.cg * BM)) * ((p.N + v.bn - 1) / v.bn);
             const int64_t groups = num_sms / v.cg;
             if (forced) {
-                const double c = estimate_ns(v, f32, tiles, groups, num_kb, forced, p.accumulate != 0);
+                const double c = estimate_ns(v, f32, tiles, groups, num_kb, forced, p.accumulate != 0, ov.sk != 0 && !fused);
                 if (c < best) { best = c; pick = i; splits = forced; }
                 continue;
             }
             for (int sp = 1; sp <= 32; sp *= 2) {
                 if (!valid_split(sp)) break;
                 if (sp > 1 && tiles * (sp / 2) >= 2 * groups) break;   // already two waves without this split
-                const double c = estimate_ns(v, f32, tiles, groups, num_kb, sp, p.accumulate != 0);
+                const double c = estimate_ns(v, f32, tiles, groups, num_kb, sp, p.accumulate != 0, ov.sk != 0 && !fused);
                 if (c < best) { best = c; pick = i; splits = sp; }
+            }
+        }
+    }
+    // A fused consumer takes whole sums.  Where tiles are few and the reduction is long, clusters of 2, 4 or 8 CTAs share a tile (one
+    // tile per cluster, all clusters at once: 74, 33 and 15 of them are resident on 148 SMs, whose GPCs are no multiples of 4 and 8).
+    // Without a consumer the partial sums meet in the output as fast or faster (512 x 512 x 4096 f32: 15.1 us, in clusters 22.2).
+    if (fused && !forced_tile && ov.meet != 0) {
+        for (int i = 0; i < kNumVariants; ++i) {
+            const Variant &v = kVariants[i];
+            if (v.cg != 1 || (v.bn == 256 && (f32 || lay != 0)) || (v.bn > 64 && v.bn / 2 >= p.N)) continue;
+            const int64_t tiles = (int64_t)((p.M + BM - 1) / BM) * ((p.N + v.bn - 1) / v.bn);
+            for (int sp = 2; sp <= MAX_MEET; sp *= 2) {
+                if (ov.meet > 1 && sp != ov.meet) continue;
+                const int stages = (num_kb + 1) / 2, per = (stages + sp - 1) / sp;       // (bf16: ranges of whole two-block stages too)
+                if (tiles > (sp == 2 ? 70 : sp == 4 ? 32 : 14) || tiles * sp > num_sms - 8 || num_kb < 4 * sp || !valid_split(sp) || (stages + per - 1) / per != sp) continue;
+                const double c = ov.meet > 1 ? 0.0 : estimate_meet_ns(v, f32, tiles, num_kb, sp);
+                if (c < best) { best = c; pick = i; splits = sp; *out_meet = 1; }
             }
         }
     }
@@ -1164,7 +1249,7 @@ sg_status launch_variant(const CUtensorMap &mi, const CUtensorMap &mf, const CUt
     cfg.stream = ctx.stream;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = CG;
+    attr[0].val.clusterDim.x = tp.meet ? tp.splits : CG;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1279,8 +1364,8 @@ sg_status launch_tensor(const Problem &p, const void *In, const void *Flt, float
     }
 
     // ---- tile variant and k split: lowest estimated time ----
-    int pick, splits;
-    choose_tiles(p, tp.num_kb, lay, ov, num_sms, &pick, &splits);
+    int pick, splits, meet;
+    choose_tiles(p, tp.num_kb, lay, ov, num_sms, &pick, &splits, &meet);
     if (pick < 0) return SG_ERR_INTERNAL;
     const Variant &var = kVariants[pick];
     // bf16 matmuls with whole k-blocks move two k-blocks per stage and per TMA load
@@ -1351,11 +1436,14 @@ sg_status launch_tensor(const Problem &p, const void *In, const void *Flt, float
     splits = (tp.num_kb + per - 1) / per;
     tp.splits = splits;
     tp.kb_per_split = per;
+    tp.meet = meet && splits > 1 && (BM % splits) == 0 ? splits : 0;
+    tp.out = O; tp.pitch = p.o_w;
+    if (meet && !tp.meet) return SG_ERR_INTERNAL;
     // Unless something below says otherwise the kernel may start while the kernel ahead of it in the stream drains
     // (programmatic dependent launch): it sets up its barriers and tensor memory, then waits for that kernel to finish
     // before its first global read or write.
     tp.wait_prior = ov.pdl == 0 ? 0 : 2;
-    if (splits > 1) {
+    if (splits > 1 && !tp.meet) {
         // partial sums meet in the output by TMA reduce-add: an overwriting call clears it first
         if (!p.accumulate) {
             if (launch_zero_fill(p, O, stream) != cudaSuccess) return SG_ERR_CUDA;
@@ -1374,14 +1462,9 @@ sg_status launch_tensor(const Problem &p, const void *In, const void *Flt, float
         const int num_m_tiles = (p.M + var.cg * BM - 1) / (var.cg * BM), num_n_tiles = (p.N + var.bn - 1) / var.bn;
         const int64_t tiles = (int64_t)num_m_tiles * num_n_tiles;
         const int left = (int)(tiles % groups);
-        if (ov.sk != 0 && splits == 1 && tiles > groups && left != 0 && tp.num_kb % kps == 0) {
-            const int64_t units = (int64_t)left * tp.num_kb;
-            int run = (int)((units + groups - 1) / groups);
-            run = (run + kps - 1) / kps * kps;
-            const double kb_ns = f32 ? var.mma_ns_f32 : var.mma_ns;
-            const double saved = (double)(tp.num_kb - run) * kb_ns;
-            const double extra = 2.0 * (1500.0 + (double)var.bn * (f32 ? 24.0 : 12.0)) + 2500.0;
-            if (run >= 4 * kps && (saved > 2.0 * extra || ov.sk == 2)) {
+        if (ov.sk != 0 && splits == 1) {
+            const int run = stream_k_run(var, f32, tiles, groups, tp.num_kb, kps, ov.sk == 2);
+            if (run > 0) {
                 tp.sk_first_tile = (int)(tiles - left);
                 tp.sk_units = run;
                 if (!p.accumulate) {
@@ -1393,7 +1476,8 @@ sg_status launch_tensor(const Problem &p, const void *In, const void *Flt, float
             }
         }
     }
-    t_last_choice[0] = var.bn; t_last_choice[1] = var.cg; t_last_choice[2] = splits;
+    // (a fused consumer takes whole sums: there the CTAs of a cluster count as CTAs of the tile)
+    t_last_choice[0] = var.bn; t_last_choice[1] = tp.meet && fused ? splits : var.cg; t_last_choice[2] = fused ? 1 : splits;
     t_last_sk[0] = tp.sk_units > 0 ? tp.sk_first_tile : -1; t_last_sk[1] = tp.sk_units;
     // f32 (either operand stored either way): the split input tile goes to tensor memory.  With
     // 256-column tiles that costs the second accumulator buffer, which short reductions used to feel; since the
@@ -1468,8 +1552,8 @@ double tensor_estimate_us(const Problem &p) {
     if (!d) return 0.0;
     if (p.bias != nullptr || p.act != SG_ACT_NONE) ov.split = 1;
     const int bk = ROW_BYTES / (p.in_bf16 ? 2 : 4);
-    int pick, splits;
-    const double ns = choose_tiles(p, p.KH * p.KW * ((p.C + bk - 1) / bk), transposed_layout(p), ov, d->num_sms, &pick, &splits);
+    int pick, splits, meet;
+    const double ns = choose_tiles(p, p.KH * p.KW * ((p.C + bk - 1) / bk), transposed_layout(p), ov, d->num_sms, &pick, &splits, &meet);
     // (the constants were fitted to problems of 256^3 and up; launches of bf16 problems below take about 0.9 us more)
     return ns * 1e-3 + (p.in_bf16 ? 0.9 : 0.0);
 }

@@ -1,0 +1,33 @@
+"""Fused calls whose reduction is shared by a cluster, against the oracle: 2, 4 and 8 thread blocks per tile, ragged rows and columns, both
+operands stored either way, ranges of k that end inside a k-block."""
+import numpy as np
+import pytest
+import torch
+
+from helpers import assert_within_bound, operand
+from oracle import ref
+from paper_2202_03293_b200 import binding as sg
+
+pytestmark = pytest.mark.gpu
+SEED = 9700
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("a_t,b_t", [(False, False), (True, False), (False, True)])
+@pytest.mark.parametrize("M,N,K,ctas", [(256, 256, 4096, (8,)), (64, 72, 6024, (8,)), (1088, 136, 2816, (2, 4)), (448, 328, 8008, (2, 4, 8)), (3520, 192, 3000, (1, 2, 4))])
+def test_meet(M, N, K, ctas, a_t, b_t, dtype):
+    A, a = operand((K, M) if a_t else (M, K), SEED, 1, "uniform", dtype)
+    B, b = operand((N, K) if b_t else (K, N), SEED, 2, "uniform", dtype)
+    A, a = (A.t(), np.ascontiguousarray(a.T)) if a_t else (A, a)
+    B, b = (B.t(), np.ascontiguousarray(b.T)) if b_t else (B, b)
+    bias, bias_h = operand((N,), SEED, 3, "normal", "f32")
+    wide = torch.full((M, N + 4), float("nan"), device="cuda")
+    C = wide[:, :N]
+    sg.sg_matmul_bias_act(A, B, bias, C, sg.SG_ACT_RELU)
+    torch.cuda.synchronize()
+    assert sg.sg_last_kernel_name() == f"tc_gemm_kernel<{dtype}>"
+    assert sg.sg_last_tile_choice()[1] in ctas and sg.sg_last_tile_choice()[2] == 1
+    want, S = ref.matmul_bias_act(a, b, bias_h, "relu")
+    assert assert_within_bound(C, want, S, "fused, shared reduction") < 4e-6
+    assert torch.isnan(wide[:, N:]).all()
+    sg.sg_check()

@@ -330,6 +330,7 @@ sg_status sg_selftest_wait_timeout(int64_t budget_cycles, sg_stream_t stream);
  *   SG_TC_BN, SG_TC_CG, SG_TC_SPLIT   as sg_set_tile_override
  *   SG_TC_SK        0: never cut the last wave into a stream-K tail; 2: whenever the shape allows it
  *   SG_TC_SMALL     0: the kernel for small problems is never chosen; 1: wherever the layout allows it
+ *   SG_TC_MEET      0: partial sums of a fused call never meet in a cluster; 2, 4, 8: in clusters of as many CTAs where possible
  *   SG_TC_KPS       1: one k-block per pipeline stage everywhere (bf16 matmuls normally move two)
  *   SG_TC_TA        0: keep the split f32 input tile in shared memory instead of tensor memory
  *   SG_TC_PDL       0: tensor-core launches never start before the kernel ahead of them in the

@@ -138,80 +138,96 @@ conv_wide_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_consta
     const int total = p.tiles * p.f_tiles;
     const int item0 = (int)((long long)blockIdx.x * total / gridDim.x), item1 = (int)((long long)(blockIdx.x + 1) * total / gridDim.x);
 
+    // (The producers' warps walk their loops converged, one elected lane issues, and nothing inside a step divides: a lane on its own with
+    // the ring's position by division took 500 to 1000 cycles a load.  The first item is worked out ahead of the wait
+    // for the kernel before this one.)
     if (warp == 0) {
         // ------------------------------------------------------------ input runs
-        if (lane == 0) {
-            if (p.wait_prior) asm volatile("griddepcontrol.wait;" ::: "memory");
-            int it = 0;
-            bool ok = true;
-            for (int item = item0; item < item1 && ok; ++item) {
-                const int q0 = item % p.tiles * p.BN;
-                for (int cb = 0; cb < p.kb; ++cb, ++it) {
-                    const int s = it % RUN_STAGES;
-                    if (!mbar_wait(run_empty(s), ((it / RUN_STAGES) & 1) ^ 1u, abort_flag)) { ok = false; break; }
+        const bool issuer = elect_one();
+        int s = 0, tile = item0 % p.tiles;
+        uint32_t phase = 1;
+        bool ok = true;
+        if (p.wait_prior) asm volatile("griddepcontrol.wait;" ::: "memory");
+        for (int item = item0; item < item1 && ok; ++item) {
+            const int q0 = tile * p.BN;
+            if (++tile == p.tiles) tile = 0;
+            for (int cb = 0; cb < p.kb; ++cb) {
+                if (!__all_sync(0xffffffffu, mbar_wait(run_empty(s), phase, abort_flag))) { ok = false; break; }
+                if (issuer) {
                     mbar_expect_tx(run_full(s), (uint32_t)p.run_tx);
                     for (int b = 0; b < p.run_boxes; ++b)
                         tma_tile_3d<false>(runs_addr + (uint32_t)(s * p.run_bytes + b * p.box_rows * 128), &map_in, run_full(s), cb * 64, q0 + b * p.box_rows, 0);
                 }
+                if (++s == RUN_STAGES) { s = 0; phase ^= 1u; }
             }
         }
     } else if (warp == 2) {
         // ------------------------------------------------------------ filter
-        if (lane == 0) {
-            if (p.wait_prior) asm volatile("griddepcontrol.wait;" ::: "memory");
-            int it = 0, cur = -1;
-            bool ok = true;
-            for (int item = item0; item < item1 && ok; ++item) {
-                const int ft = item / p.tiles;
-                if (p.resident && ft == cur) continue;
-                cur = ft;
-                for (int cb = 0; cb < p.kb && ok; ++cb)
-                    for (int kh = 0; kh < p.KH; ++kh, ++it) {
-                        const int s = it % p.slots;
-                        if (!mbar_wait(flt_empty(s), ((it / p.slots) & 1) ^ 1u, abort_flag)) { ok = false; break; }
-                        // (the first run and the first slot are what the first MMA waits for: the rest of the filter, up to
-                        // three times their size, comes behind them rather than beside them.  The wait is for a barrier that the
-                        // MMA warp completes once: a phase of the ring could have come round again by the time this is reached,
-                        // which is items later where the filter is one slot.)
-                        if (it == 1 && !mbar_wait(first_run, 0, abort_flag)) { ok = false; break; }
+        const bool issuer = elect_one();
+        int s = 0, ft = item0 / p.tiles, tile = item0 - ft * p.tiles, cur = -1;
+        uint32_t phase = 1;
+        bool ok = true, second = false;
+        if (p.wait_prior) asm volatile("griddepcontrol.wait;" ::: "memory");
+        for (int item = item0; item < item1 && ok; ++item) {
+            const int f = ft;
+            if (++tile == p.tiles) { tile = 0; ++ft; }
+            if (p.resident && f == cur) continue;
+            cur = f;
+            for (int cb = 0; cb < p.kb && ok; ++cb)
+                for (int kh = 0; kh < p.KH; ++kh) {
+                    if (!__all_sync(0xffffffffu, mbar_wait(flt_empty(s), phase, abort_flag))) { ok = false; break; }
+                    // (the first run and the first slot are what the first MMA waits for: the rest of the filter, up to
+                    // three times their size, comes behind them rather than beside them.  The wait is for a barrier that the
+                    // MMA warp completes once: a phase of the ring could have come round again by the time this is reached,
+                    // which is items later where the filter is one slot.)
+                    if (second && !__all_sync(0xffffffffu, mbar_wait(first_run, 0, abort_flag))) { ok = false; break; }
+                    second = item == item0 && cb == 0 && kh == 0;
+                    if (issuer) {
                         mbar_expect_tx(flt_full(s), (uint32_t)p.slot_bytes);
                         const uint32_t dst = flt_addr + (uint32_t)(s * p.slot_bytes);
                         if (p.flt_loads == 1) {
-                            tma_tile_5d<false>(dst, &map_flt, flt_full(s), 0, cb * 64, ft * (BF / 64), 0, kh);
+                            tma_tile_5d<false>(dst, &map_flt, flt_full(s), 0, cb * 64, f * (BF / 64), 0, kh);
                         } else {
-                            tma_load_4d(dst, &map_flt, flt_full(s), ft * BF, cb * 64, 0, kh);
-                            tma_load_4d(dst + p.half_bytes, &map_flt, flt_full(s), ft * BF + 64, cb * 64, 0, kh);
+                            tma_load_4d(dst, &map_flt, flt_full(s), f * BF, cb * 64, 0, kh);
+                            tma_load_4d(dst + p.half_bytes, &map_flt, flt_full(s), f * BF + 64, cb * 64, 0, kh);
                         }
                     }
-            }
+                    if (++s == p.slots) { s = 0; phase ^= 1u; }
+                }
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer: the whole warp walks, one lane issues
         const uint32_t idesc = make_idesc(p.BN, BF, false, true, false);       // filter as stored: M-major; positions K-major
         const bool issuer = elect_one();
         auto wait_all = [&](bool passed) { return __all_sync(0xffffffffu, passed) != 0; };
-        int it = 0, fit = 0, tl = 0, cur = -1;
-        bool ok = true;
+        int s = 0, slot = 0, tl = 0, cur = -1, ft_next = item0 / p.tiles, tile = item0 - ft_next * p.tiles;
+        uint32_t run_phase = 0, slot_phase = 0;
+        bool ok = true, landed = false;
         for (int item = item0; item < item1 && ok; ++item, ++tl) {
-            const int ft = item / p.tiles;
+            const int ft = ft_next;
+            if (++tile == p.tiles) { tile = 0; ++ft_next; }
             const bool fresh = !p.resident || ft != cur;             // this tile's filter slots have to be waited for
-            const bool release = !p.resident || item + 1 >= item1 || (item + 1) / p.tiles != ft;
-            if (p.resident && !fresh) fit -= p.kb * p.KH;
+            const bool release = !p.resident || item + 1 >= item1 || ft_next != ft;
+            if (!fresh) slot = 0;                                     // (a filter that stays fills the ring)
             cur = ft;
             const int buf = tl & 1;
             if (!wait_all(mbar_wait(acc_empty(buf), ((tl >> 1) & 1) ^ 1u, abort_flag))) { ok = false; break; }
             tc_fence_after();
             const uint32_t d = tmem_base + buf * p.BN;
             uint32_t acc = 0;
-            for (int cb = 0; cb < p.kb && ok; ++cb, ++it) {
-                const int s = it % RUN_STAGES;
-                if (!wait_all(mbar_wait(run_full(s), (it / RUN_STAGES) & 1, abort_flag))) { ok = false; break; }
-                if (it == 0 && issuer) mbar_arrive(first_run);
+            for (int cb = 0; cb < p.kb && ok; ++cb) {
+                if (!wait_all(mbar_wait(run_full(s), run_phase, abort_flag))) { ok = false; break; }
+                if (!landed && issuer) mbar_arrive(first_run);
+                landed = true;
                 const uint32_t run = runs_addr + (uint32_t)(s * p.run_bytes);
                 const int ksteps = cb + 1 == p.kb ? p.last_ksteps : 4;
-                for (int kh = 0; kh < p.KH; ++kh, ++fit) {
-                    const int fs = fit % p.slots;
-                    if (fresh && !wait_all(mbar_wait(flt_full(fs), (fit / p.slots) & 1, abort_flag))) { ok = false; break; }
+                for (int kh = 0; kh < p.KH; ++kh) {
+                    const int fs = slot;
+                    if (fresh && !wait_all(mbar_wait(flt_full(fs), slot_phase, abort_flag))) { ok = false; break; }
+                    if (++slot == p.slots) {
+                        slot = 0;
+                        if (fresh) slot_phase ^= 1u;
+                    }
                     tc_fence_after();
                     // (descriptors are made by the converged warp: uniform values; a lane on its own pays ~100 cycles per MMA)
                     for (int kw = 0; kw < p.KW; ++kw) {
@@ -227,6 +243,7 @@ conv_wide_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_consta
                     if (release && issuer) umma_commit(flt_empty(fs));
                 }
                 if (ok && issuer) umma_commit(run_empty(s));
+                if (++s == RUN_STAGES) { s = 0; run_phase ^= 1u; }
             }
             if (ok && issuer) umma_commit(acc_full(buf));
         }

@@ -273,41 +273,49 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant
 
     if (warp == 0 || warp == C::FLT_WARP) {
         // ------------------------------------------------------------ producers: warp 0 fetches the
-        // input tiles, the last warp the filter tiles; both arm the stage's barrier for their bytes
-        if (lane == 0) {
-            const bool input_side = warp == 0;
+        // input tiles, the last warp the filter tiles; both arm the stage's barrier for their bytes.
+        // The whole warp walks the loop and one elected lane issues, and nothing inside a k-block divides: the loop is one serial chain that
+        // every stage waits for.  (With one lane of a diverged warp and the tap taken from the k-block's number by two divisions a stage took
+        // 800 to 1000 cycles to issue, more than its MMAs wherever a tile is narrow.)  The first item is
+        // worked out ahead of the wait for the kernel before this one.
+        const bool input_side = warp == 0, issuer = elect_one();
+        auto wait_all = [&](bool passed) { return __all_sync(0xffffffffu, passed) != 0; };
+        int s = 0;                 // ring position across all of this CTA's tiles
+        uint32_t ph = 1;           // parity of the stage's last release
+        bool ok = true, waited = false;
+        Cursor cur{0, sk_u0};
+        int tile, kb0, kb1, add;
+        while (ok && next_item(cur, tile, kb0, kb1, add)) {
+            int mt, nt;
+            tile_coords(tile, p.num_m_tiles, p.num_n_tiles, mt, nt);
+            const int m0 = (mt * CG + (int)cta_rank) * BM;
+            const int n0 = nt * BN + (int)cta_rank * C::B_COLS;
+            int pix_n = 0, pix_h = 0, pix_w = 0;   // first output pixel of this CTA's rows
+            int cb = kb0, kh = 0, kw = 0;          // k-block within its tap, tap
+            if (p.a_mode != 0) {
+                int hw = p.Ho * p.Wo;
+                pix_n = m0 / hw;
+                int r = m0 - pix_n * hw;
+                pix_h = r / p.Wo;
+                pix_w = r - pix_h * p.Wo;
+                const int tap = kb0 / p.kb_per_tap;
+                cb = kb0 - tap * p.kb_per_tap;
+                kh = tap / p.KW;
+                kw = tap - kh * p.KW;
+            }
             // the operands may be the output of the kernel ahead of this one
-            if (p.wait_prior == 2) asm volatile("griddepcontrol.wait;" ::: "memory");
-            int it = 0;   // k-block counter across all of this CTA's tiles
-            bool ok = true;
-            Cursor cur{0, sk_u0};
-            int tile, kb0, kb1, add;
-            while (ok && next_item(cur, tile, kb0, kb1, add)) {
-                int mt, nt;
-                tile_coords(tile, p.num_m_tiles, p.num_n_tiles, mt, nt);
-                const int m0 = (mt * CG + (int)cta_rank) * BM;
-                const int n0 = nt * BN + (int)cta_rank * C::B_COLS;
-                int pix_n = 0, pix_h = 0, pix_w = 0;   // first output pixel of this CTA's rows
-                if (p.a_mode != 0) {
-                    int hw = p.Ho * p.Wo;
-                    pix_n = m0 / hw;
-                    int r = m0 - pix_n * hw;
-                    pix_h = r / p.Wo;
-                    pix_w = r - pix_h * p.Wo;
-                }
-                for (int kb = kb0; kb < kb1; kb += KPS, ++it) {
-                    const int s = it % C::STAGES;
-                    const uint32_t ph = (it / C::STAGES) & 1;
-                    if (!mbar_wait(empty_bar(s), ph ^ 1u, abort_flag)) { ok = false; break; }
-                    const uint32_t a_dst = stages_addr + s * C::STAGE_BYTES;
-                    const uint32_t b_dst = a_dst + KPS * A_STAGE_BYTES;
-                    const int tap = kb / p.kb_per_tap;
-                    const int c0 = (kb - tap * p.kb_per_tap) * C::BK;
-                    const int kh = tap / p.KW, kw = tap - kh * p.KW;
-                    // bf16 pairs: the leader alone arms its barrier, for the pair's total (a remote arrive by
-                    // the peer would order it after its own loads in flight and serialise the ring)
-                    const uint32_t bar = REMOTE_FULL ? map_to_cta(full_bar(s), 0) : full_bar(s);
-                    const uint32_t my_bytes = KPS * (input_side ? A_STAGE_BYTES : C::B_STAGE_BYTES);
+            if (!waited && p.wait_prior == 2) asm volatile("griddepcontrol.wait;" ::: "memory");
+            waited = true;
+            for (int kb = kb0; kb < kb1; kb += KPS) {
+                if (!wait_all(mbar_wait(empty_bar(s), ph, abort_flag))) { ok = false; break; }
+                const uint32_t a_dst = stages_addr + s * C::STAGE_BYTES;
+                const uint32_t b_dst = a_dst + KPS * A_STAGE_BYTES;
+                const int c0 = cb * C::BK;
+                // bf16 pairs: the leader alone arms its barrier, for the pair's total (a remote arrive by
+                // the peer would order it after its own loads in flight and serialise the ring)
+                const uint32_t bar = REMOTE_FULL ? map_to_cta(full_bar(s), 0) : full_bar(s);
+                const uint32_t my_bytes = KPS * (input_side ? A_STAGE_BYTES : C::B_STAGE_BYTES);
+                if (issuer) {
                     if (!REMOTE_FULL || cta_rank == 0) mbar_expect_tx(full_bar(s), (REMOTE_FULL ? CG : 1) * my_bytes);
                     if (input_side) {
                         if constexpr (A_MN) {
@@ -350,6 +358,12 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant
                             else tma_load_4d(b_dst + j * C::SUB_BYTES, &map_flt, bar, n0 + j * C::SUB_COLS, c0, kw, kh);
                         }
                     }
+                }
+                if (++s == C::STAGES) { s = 0; ph ^= 1u; }
+                cb += KPS;
+                if (cb >= p.kb_per_tap) {
+                    cb = 0;
+                    if (++kw == p.KW) { kw = 0; ++kh; }
                 }
             }
         }

@@ -288,10 +288,11 @@ __device__ __forceinline__ void tma_load_im2col_4d_cg2(uint32_t dst, const CUten
         "cp.async.bulk.tensor.4d.im2col.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2], {%7, %8};"
         ::"r"(dst), "l"(map), "r"(bar), "r"(c), "r"(w), "r"(h), "r"(n), "h"(off_w), "h"(off_h) : "memory");
 }
-// Rank-5 tiled load.  CG2: the mbarrier may belong to the peer CTA of a pair.  One TMA
-// instruction costs the issuing thread several hundred cycles whatever the size of its box
-// (measured: ~550 cycles, boxes of 8 to 64 KB), so operand tiles are fetched with as few and as
-// large boxes as the layout allows, and the two operands are issued by different warps.
+// Rank-5 tiled load.  CG2: the mbarrier may belong to the peer CTA of a pair.  The TMA unit fetches about one line of a box per cycle,
+// whatever the line's width up to 128 bytes, and takes 2 to 3 cycles where a line does not start on a multiple of its size
+// (16 KB boxes back to back, data in the L2: lines of 128 bytes 110 bytes a cycle from one SM and 99 from all at once, 46 at a
+// pitch of 4112 bytes; lines of 64 bytes 62 and 27).  So operand tiles are boxes of 128-byte lines, few and large, and the two
+// operands are issued by different warps.
 template <bool CG2>
 __device__ __forceinline__ void tma_tile_5d(uint32_t dst, const CUtensorMap *map, uint32_t bar, int x, int y, int z, int w, int v) {
     if constexpr (CG2)

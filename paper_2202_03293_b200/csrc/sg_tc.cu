@@ -51,9 +51,7 @@ constexpr int BM = 128;           // rows of an output tile = lanes of TMEM = M 
 constexpr int ROW_BYTES = 128;    // one k-block = one 128-byte swizzle row: 64 bf16 or 32 f32
 constexpr int K_STEPS = 4;        // tcgen05.mma per k-block and product: 32 bytes of k each
 constexpr int A_STAGE_BYTES = BM * ROW_BYTES;
-// f32 path: 16 warps splitting tiles into hi and lo, in two groups that take the k-blocks in turn: a k-block is a chain of about
-// 1400 cycles of latencies (two barriers, loads, splits, stores, fences) however many warps share its work, longer than its MMAs take
-constexpr int CONVERTER_THREADS = 512, GROUP_THREADS = CONVERTER_THREADS / 2;
+constexpr int CONVERTER_THREADS = 512;        // f32 path: 16 warps splitting tiles into hi and lo, in groups (Cfg::GROUPS)
 constexpr int STAGING_BYTES = 2 * 16384;      // epilogue: 2 staging tiles of 128 rows x 128 B
 constexpr int MAX_MEET = 8;                   // CTAs of a cluster that share a tile's reduction
 
@@ -103,13 +101,19 @@ struct Cfg {
     // filter lo], the filter transposed to K-major on the way (kind::tf32 takes no N-major operand).
     // (two slots are enough: with three the kernel is no faster - a k-block is bound by shared-memory bandwidth: the raw tiles
     // written by TMA and read by the converters, the split filter written, and the MMAs' filter reads)
-    static constexpr int SPLIT_SLOTS = F32 ? 2 : 0;
+    // The converter warps work in groups that take the k-blocks in turn, each with a slot of its own: a k-block is a chain of about 900
+    // cycles of latencies (two barriers, loads, stores, fences) plus its share of the instructions, longer than its
+    // MMAs.  Where a CTA stages 64 filter columns there is room for four slots, and four groups of four warps have twice as many
+    // chains under way as two of eight.
+    static constexpr int GROUPS = TA && B_COLS == 64 ? 4 : 2, GROUP_WARPS = CONVERTER_THREADS / 32 / GROUPS, GROUP_THREADS = 32 * GROUP_WARPS;
+    static constexpr int SPLIT_SLOTS = F32 ? GROUPS : 0;
     // TA (f32): the split input tile lives in tensor memory (the MMA reads its A operand there), which
     // takes its writes and its three reads per k-step off the shared-memory pipe; a slot then holds
     // [filter hi | filter lo] only.
     static constexpr int SPLIT_BYTES = TA ? 2 * B_STAGE_BYTES : 2 * STAGE_BYTES;
     static constexpr int RING_BUDGET = 196608 - SPLIT_SLOTS * SPLIT_BYTES;
-    static constexpr int STAGES = (RING_BUDGET / STAGE_BYTES) > 8 ? 8 : (RING_BUDGET / STAGE_BYTES);
+    static constexpr int MOST_STAGES = (RING_BUDGET / STAGE_BYTES) > 8 ? 8 : (RING_BUDGET / STAGE_BYTES);
+    static constexpr int STAGES = F32 ? MOST_STAGES / GROUPS * GROUPS : MOST_STAGES;
     // warps: input producer, MMA, 4 epilogue (, 8 converter), filter producer
     static constexpr int THREADS = 192 + (F32 ? CONVERTER_THREADS : 0) + 32;
     static constexpr int FLT_WARP = THREADS / 32 - 1;
@@ -128,7 +132,7 @@ struct Cfg {
     static_assert(!TA || F32, "tensor-memory input operand: f32 path only");
     // each converter group keeps to its own slot and its own stages (a group that waited on a barrier of the other one's could take
     // the phase before the last for the one it waits for)
-    static_assert(!F32 || (SPLIT_SLOTS == 2 && STAGES % 2 == 0), "two converter groups");
+    static_assert(!F32 || (STAGES >= GROUPS && STAGES % GROUPS == 0), "converter groups");
 };
 
 // Static tile order: groups of 8 tile-rows, row index fastest inside a group, so that the
@@ -209,10 +213,10 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant
         // epilogue warp of every CTA of the group.
         for (int s = 0; s < C::STAGES; ++s) {
             mbar_init(full_bar(s), 2);
-            mbar_init(empty_bar(s), F32 ? GROUP_THREADS / 32 : 1);
+            mbar_init(empty_bar(s), F32 ? C::GROUP_WARPS : 1);
         }
         for (int s = 0; s < C::SPLIT_SLOTS; ++s) {
-            mbar_init(split_full_bar(s), (GROUP_THREADS / 32) * CG);
+            mbar_init(split_full_bar(s), C::GROUP_WARPS * CG);
             mbar_init(split_empty_bar(s), 1);
         }
         for (int b = 0; b < 2; ++b) { mbar_init(acc_full_bar(b), 1); mbar_init(acc_empty_bar(b), 4 * CG); }
@@ -509,14 +513,15 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant
     } else if (warp >= 6) {
         // ------------------------------------------------------------ converter (f32 only; warps 6 to 21)
         if constexpr (F32) {
-            const int group = (warp - 6) >> 3, cw = (warp - 6) & 7;       // converter group, warp of it
+            constexpr int GROUP_THREADS = C::GROUP_THREADS;
+            const int group = (warp - 6) / C::GROUP_WARPS, cw = (warp - 6) % C::GROUP_WARPS;       // converter group, warp of it
             const int ct = cw * 32 + lane;                                // thread of the group
             // MIX: this thread's fixed share of a k-block.  Input: row (warp & 3) * 32 + lane (the TMEM lane quarter this warp
             // may touch), k columns 16 * (cw >> 2) ..: four 16-byte chunks of the swizzled raw row.  Filter: units cw and cw + 8
             // (sub-tile of 32 columns, quarter of its 32 k): lane = column f reads 8 k down its column and owns chunks of row f.
             constexpr int UNITS = C::B_COLS / 64;                         // 4 * B_COLS / 32 units on 8 warps (64 columns: one each)
             uint32_t mx_a_off[4] = {0, 0, 0, 0}, mx_hi_off[2] = {0, 0}, mx_b_src = 0, mx_h16_off = 0, mx_l16_off = 0, mx_tmem = 0;
-            if constexpr (MIX) {
+            if constexpr (MIX && C::GROUPS == 2) {
                 const int row = (warp & 3) * 32 + lane;
                 for (int i = 0; i < 4; ++i) mx_a_off[i] = (uint32_t)(row * 128 + ((((cw >> 2) * 4 + i) ^ (row & 7)) << 4));
                 const int uj = cw >> 2, uq = cw & 3, f = uj * 32 + lane;
@@ -536,7 +541,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant
             int tile, kb0, kb1, add;
             while (ok && next_item(cur, tile, kb0, kb1, add)) {
                 for (int kb = kb0; kb < kb1; ++kb, ++it) {
-                    if ((it & 1) != group) continue;
+                    if (it % C::GROUPS != group) continue;
                     const int r = it % C::STAGES, s = group;
                     if (!wait_all(mbar_wait(full_bar(r), (it / C::STAGES) & 1, abort_flag))) { ok = false; break; }
                     const uint8_t *raw = smem_gen + r * C::STAGE_BYTES;
@@ -547,7 +552,93 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant
                         if constexpr (TA) tc_fence_after();
                         return free;
                     };
-                    if constexpr (MIX) {
+                    if constexpr (C::GROUPS == 4) {
+                        // A warp has all 32 k of the 32 rows of its TMEM lane quarter (two halves of 16 k, lane = row), and of either
+                        // sub-tile of 32 filter columns a quarter of the k (lane = column).  The raw stage is handed back once
+                        // everything has been read, half-way through the splits: there is one stage per group, and its refill takes
+                        // as long as the rest of the chain.
+                        const int quarter = warp & 3, row = quarter * 32 + lane;
+                        auto load_a = [&](int half, uint4 (&a)[4]) {
+                            if constexpr (A_MN) {      // four [32 k][32 rows] sub-tiles: 16 values down a column
+                                const uint32_t *col = reinterpret_cast<const uint32_t *>(raw) + quarter * (C::SUB_BYTES / 4) + half * 16 * 32 + lane;
+#pragma unroll
+                                for (int i = 0; i < 4; ++i) a[i] = make_uint4(col[i * 128], col[i * 128 + 32], col[i * 128 + 64], col[i * 128 + 96]);
+                            } else {                   // a row's chunks lie swizzled
+#pragma unroll
+                                for (int i = 0; i < 4; ++i) a[i] = *reinterpret_cast<const uint4 *>(raw + row * 128 + (((half * 4 + i) ^ (lane & 7)) << 4));
+                            }
+                        };
+                        // filter column u * 32 + lane, k 8 * cw ..: two chunks of its K-major row
+                        const uint32_t f_row = (uint32_t)((lane >> 3) * 1024 + (lane & 7) * 128);
+                        const uint32_t f_off0 = f_row + (uint32_t)(((2 * cw) ^ (lane & 7)) << 4), f_off1 = f_row + (uint32_t)(((2 * cw + 1) ^ (lane & 7)) << 4);
+                        auto load_b = [&](int u, uint4 (&x)[2]) {
+                            const uint8_t *tile_b = raw + A_STAGE_BYTES + u * 4096;
+                            if constexpr (B_KM) {
+                                x[0] = *reinterpret_cast<const uint4 *>(tile_b + f_off0);
+                                x[1] = *reinterpret_cast<const uint4 *>(tile_b + f_off1);
+                            } else {
+                                const uint32_t *col = reinterpret_cast<const uint32_t *>(tile_b) + cw * 8 * 32 + lane;
+                                x[0] = make_uint4(col[0], col[32], col[64], col[96]);
+                                x[1] = make_uint4(col[128], col[160], col[192], col[224]);
+                            }
+                        };
+                        const uint32_t t_base = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(C::ACC_BUFS * BN + s * 64);
+                        auto split_a = [&](int half, const uint4 (&a)[4]) {
+                            uint32_t hi[16];
+                            if constexpr (MIX) {
+                                uint32_t lo8[8], hi8[8];
+#pragma unroll
+                                for (int i = 0; i < 2; ++i) {
+                                    uint4 h0, h1, h16, l16;
+                                    split8_mix(a[2 * i], a[2 * i + 1], h0, h1, h16, l16);
+                                    hi[8 * i] = h0.x; hi[8 * i + 1] = h0.y; hi[8 * i + 2] = h0.z; hi[8 * i + 3] = h0.w;
+                                    hi[8 * i + 4] = h1.x; hi[8 * i + 5] = h1.y; hi[8 * i + 6] = h1.z; hi[8 * i + 7] = h1.w;
+                                    lo8[4 * i] = l16.x; lo8[4 * i + 1] = l16.y; lo8[4 * i + 2] = l16.z; lo8[4 * i + 3] = l16.w;
+                                    hi8[4 * i] = h16.x; hi8[4 * i + 1] = h16.y; hi8[4 * i + 2] = h16.z; hi8[4 * i + 3] = h16.w;
+                                }
+                                tmem_st_32x16(t_base + half * 16, hi);
+                                tmem_st_32x8(t_base + 32 + half * 8, lo8);
+                                tmem_st_32x8(t_base + 48 + half * 8, hi8);
+                            } else {
+                                uint32_t lo[16];
+#pragma unroll
+                                for (int i = 0; i < 2; ++i) {
+                                    uint4 h[2], l[2];
+                                    split8(a[2 * i], a[2 * i + 1], h[0], l[0], h[1], l[1]);
+#pragma unroll
+                                    for (int e = 0; e < 2; ++e) {
+                                        const int o = 8 * i + 4 * e;
+                                        hi[o] = h[e].x; hi[o + 1] = h[e].y; hi[o + 2] = h[e].z; hi[o + 3] = h[e].w;
+                                        lo[o] = l[e].x; lo[o + 1] = l[e].y; lo[o + 2] = l[e].z; lo[o + 3] = l[e].w;
+                                    }
+                                }
+                                tmem_st_32x16(t_base + half * 16, hi);
+                                tmem_st_32x16(t_base + 32 + half * 16, lo);
+                            }
+                        };
+                        auto split_b = [&](int u, const uint4 (&x)[2]) {
+                            uint4 h0, h1, l0, l1;
+                            uint8_t *dst = slot + u * 4096, *second = dst + C::B_STAGE_BYTES;      // [hi | lo], or [hi | hi and lo in bf16]
+                            if constexpr (MIX) split8_mix(x[0], x[1], h0, h1, l0, l1);
+                            else split8(x[0], x[1], h0, l0, h1, l1);
+                            *reinterpret_cast<uint4 *>(dst + f_off0) = h0;
+                            *reinterpret_cast<uint4 *>(dst + f_off1) = h1;
+                            *reinterpret_cast<uint4 *>(second + (MIX ? f_row + (uint32_t)((cw ^ (lane & 7)) << 4) : f_off0)) = l0;
+                            *reinterpret_cast<uint4 *>(second + (MIX ? f_row + (uint32_t)(((4 + cw) ^ (lane & 7)) << 4) : f_off1)) = l1;
+                        };
+                        uint4 a[4], x0[2], x1[2];
+                        load_a(0, a);
+                        load_b(0, x0);
+                        load_b(1, x1);
+                        if (!slot_free()) { ok = false; break; }
+                        split_a(0, a);
+                        load_a(1, a);
+                        split_b(0, x0);
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(empty_bar(r));      // the raw stage may be refilled
+                        split_a(1, a);
+                        split_b(1, x1);
+                    } else if constexpr (MIX) {
                         // Plain layout, corrections as bf16 MMAs.  Every address below is fixed per thread (set up ahead of
                         // the loops); the loads go out first, input rows then filter columns.
                         uint4 a[4];
@@ -700,7 +791,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant
                     }
                     __syncwarp();
                     if (lane == 0) {
-                        mbar_arrive(empty_bar(r));          // the raw stage may be refilled
+                        if constexpr (C::GROUPS == 2) mbar_arrive(empty_bar(r));          // the raw stage may be refilled
                         if constexpr (CG == 1) mbar_arrive(split_full_bar(s));
                         else mbar_arrive_cluster(map_to_cta(split_full_bar(s), 0));
                     }

@@ -1,0 +1,32 @@
+"""f32 products on the tensor cores: the converter groups of the narrow tiles against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+from helpers import assert_within_bound, operand
+from oracle import ref
+from paper_2202_03293_b200 import binding as sg
+
+pytestmark = pytest.mark.gpu
+SEED = 9700
+
+
+# fewer k-blocks than groups, as many, one more, several rounds with a remainder; one tile and more tiles than SMs
+@pytest.mark.parametrize("bn,cg,a_t,b_t", [(64, 1, False, False), (64, 1, True, False), (64, 1, False, True), (64, 1, True, True), (128, 2, False, False)])
+@pytest.mark.parametrize("M,N,K", [(160, 72, 32), (160, 136, 96), (320, 72, 128), (160, 136, 160), (288, 200, 1056), (4736, 328, 96)])
+def test_converter_groups(M, N, K, bn, cg, a_t, b_t):
+    A, a = operand((K, M) if a_t else (M, K), SEED, 1, "uniform", "f32")
+    B, b = operand((N, K) if b_t else (K, N), SEED, 2, "uniform", "f32")
+    A, a = (A.t(), np.ascontiguousarray(a.T)) if a_t else (A, a)
+    B, b = (B.t(), np.ascontiguousarray(b.T)) if b_t else (B, b)
+    C = torch.full((M, N), float("nan"), device="cuda")
+    sg.sg_set_tile_override(bn, cg, 1)
+    try:
+        sg.sg_matmul(A, B, C)
+        torch.cuda.synchronize()
+        assert sg.sg_last_kernel_name() == "tc_gemm_kernel<f32>" and tuple(sg.sg_last_tile_choice()) == (bn, cg, 1)
+    finally:
+        sg.sg_set_tile_override(0, 0, 0)
+    want, S = ref.matmul(a, b)
+    assert assert_within_bound(C, want, S, "converter groups") < 4e-6      # 2^-19 for the rounded corrections, and the truncating sum
+    sg.sg_check()

@@ -24,15 +24,21 @@
 namespace sg {
 namespace {
 
-constexpr int TW = 4;            // output columns per thread in the fast kernel
+constexpr int TW_UNIT = 4, TW_STRIDED = 2;      // output columns per thread of depthwise_vec_kernel (the latter: 3 x 3 windows of stride 2)
 
-__device__ __forceinline__ float4 load4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
-__device__ __forceinline__ float4 load4(const __nv_bfloat16 *p) {
-    const uint2 raw = *reinterpret_cast<const uint2 *>(p);
-    // bf16 -> f32 is a 16-bit shift: exact
+// Four neighbouring channels as they lie in memory, and as f32 (bf16 -> f32 is a 16-bit shift: exact).
+template <typename T> struct Raw4Of { typedef float4 type; };
+template <> struct Raw4Of<__nv_bfloat16> { typedef uint2 type; };
+template <typename T> using Raw4 = typename Raw4Of<T>::type;
+__device__ __forceinline__ float4 load_raw4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
+__device__ __forceinline__ uint2 load_raw4(const __nv_bfloat16 *p) { return *reinterpret_cast<const uint2 *>(p); }
+__device__ __forceinline__ float4 widen4(float4 v) { return v; }
+__device__ __forceinline__ float4 widen4(uint2 raw) {
     return make_float4(__uint_as_float(raw.x << 16), __uint_as_float(raw.x & 0xFFFF0000u),
                        __uint_as_float(raw.y << 16), __uint_as_float(raw.y & 0xFFFF0000u));
 }
+template <typename T>
+__device__ __forceinline__ float4 load4(const T *p) { return widen4(load_raw4(p)); }
 __device__ __forceinline__ float load1(const float *p) { return *p; }
 __device__ __forceinline__ float load1(const __nv_bfloat16 *p) { return __bfloat162float(*p); }
 
@@ -41,16 +47,18 @@ __device__ __forceinline__ void fma4(float4 &acc, const float4 a, const float4 b
     acc.z = fmaf(a.z, b.z, acc.z); acc.w = fmaf(a.w, b.w, acc.w);
 }
 
-// Four channels x TW output columns per thread.  UNIT: stride 1, dilation 1 along w and KW <= MAX_KW_REG.
-// K3: a 3 x 3 window with unit stride and dilation along w, known at compile time: the columns
-// the TW windows of a filter row share (w0 .. w0+TW+1) are loaded once, and all 18 input loads
-// of a thread are issued before the first of them is needed.  Otherwise every tap is loaded
-// where it is needed and the L1 serves the repeats.
-// IDX: the type the work index is decoded in (32-bit whenever the work fits: 64-bit divisions
+// Four channels of a few output columns per thread.  S = 1, 2: a 3 x 3 window of stride S and unit dilation along w, known at compile
+// time: the columns that neighbouring windows of a filter row share are loaded once, and all of a thread's input and filter
+// loads (S = 1: 18 + 9 for four columns, S = 2: 15 + 9 for two) are issued before the first of them is needed.  These are
+// calls of a few microseconds: one memory latency is the most they can afford (with each tap loaded where it is needed a
+// stride-2 layer of 4 x 7 x 7 x 16 took nine, 9.3 us; now 2.2).  S = 0: any window, every tap loaded where it is needed; the L1 serves
+// the repeats.  IDX: the type the work index is decoded in (32-bit whenever the work fits: 64-bit divisions
 // would cost more than the op).  One work item per thread.
-template <typename T, bool K3, typename IDX>
+template <typename T, int S, typename IDX>
 __global__ void __launch_bounds__(256)
 depthwise_vec_kernel(const DepthwiseProblem p, const T *__restrict__ I, const T *__restrict__ Kf, float *__restrict__ O) {
+    constexpr int TW = S == 2 ? TW_STRIDED : TW_UNIT;
+    asm volatile("griddepcontrol.launch_dependents;");
     const IDX c4s = (IDX)(p.C / 4);
     const IDX wts = (IDX)((p.Wo + TW - 1) / TW);
     const IDX total = (IDX)p.N * (IDX)p.Ho * wts * c4s;
@@ -65,23 +73,30 @@ depthwise_vec_kernel(const DepthwiseProblem p, const T *__restrict__ I, const T 
 #pragma unroll
         for (int t = 0; t < TW; ++t) acc[t] = make_float4(0.f, 0.f, 0.f, 0.f);
         const T *in_n = I + (int64_t)n * p.i_n + c;
-        if constexpr (K3) {
-            float4 col[3][TW + 2];
+        // the operands may be the output of the kernel ahead of this one, and the output its input
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        if constexpr (S != 0) {
+            constexpr int COLS = (TW - 1) * S + 3;
+            Raw4<T> col[3][COLS], flt[3][3];
 #pragma unroll
             for (int kh = 0; kh < 3; ++kh) {
-                const T *row = in_n + (int64_t)(h * p.sh + kh * p.dh) * p.i_h;
+                const T *row = in_n + (int64_t)(h * p.sh + kh * p.dh) * p.i_h + (int64_t)w0 * S * p.i_w;
 #pragma unroll
-                for (int j = 0; j < TW + 2; ++j)
-                    if (w0 + j < p.Wo + 2) col[kh][j] = load4(row + (int64_t)(w0 + j) * p.i_w);
+                for (int j = 0; j < COLS; ++j)
+                    if (w0 * S + j < (p.Wo - 1) * S + 3) col[kh][j] = load_raw4(row + (int64_t)j * p.i_w);
             }
 #pragma unroll
             for (int kh = 0; kh < 3; ++kh)
 #pragma unroll
+                for (int kw = 0; kw < 3; ++kw) flt[kh][kw] = load_raw4(Kf + (int64_t)kh * p.k_kh + (int64_t)kw * p.k_kw + c);
+#pragma unroll
+            for (int kh = 0; kh < 3; ++kh)
+#pragma unroll
                 for (int kw = 0; kw < 3; ++kw) {
-                    const float4 f = load4(Kf + (int64_t)kh * p.k_kh + (int64_t)kw * p.k_kw + c);
+                    const float4 f = widen4(flt[kh][kw]);
 #pragma unroll
                     for (int t = 0; t < TW; ++t)
-                        if (w0 + t < p.Wo) fma4(acc[t], col[kh][t + kw], f);
+                        if (w0 + t < p.Wo) fma4(acc[t], widen4(col[kh][t * S + kw]), f);
                 }
         } else {
             for (int kh = 0; kh < p.KH; ++kh) {
@@ -292,11 +307,12 @@ depthwise_tma_kernel(const __grid_constant__ CUtensorMap map_in, const Depthwise
             for (int t = blockIdx.x; t < d.num_tiles; t += gridDim.x, ++k) {
                 const int s = k & 1;
                 const uint32_t ph = (uint32_t)(k >> 1) & 1u;
-                if (!mbar_wait(smem_u32(&empty_bar[s]), ph ^ 1u, &abort_load)) break;
+                // (the divisions ahead of the wait: the load goes out as soon as the stage is free)
                 int r = t;
                 const int cb = r % d.c_blocks; r /= d.c_blocks;
                 const int wt = r % d.tiles_w; r /= d.tiles_w;
                 const int ht = r % d.tiles_h, nt = r / d.tiles_h;
+                if (!mbar_wait(smem_u32(&empty_bar[s]), ph ^ 1u, &abort_load)) break;
                 mbar_expect_tx(smem_u32(&full_bar[s]), (uint32_t)d.box_bytes);
                 tma_load_4d(ring + (uint32_t)(s * d.stage_bytes), &map_in, smem_u32(&full_bar[s]), cb * CB, wt * tile_cols * S, ht * tile_rows * S, nt * tile_n);
             }
@@ -463,10 +479,12 @@ bool try_launch_tma(const DepthwiseProblem &p, const T *I, const T *Kf, float *O
 
 template <typename T, int K>
 bool try_launch_window(const DepthwiseProblem &p, const T *I, const T *Kf, float *O, int num_sms, cudaStream_t stream, cudaError_t *err) {
-    // blocks of 64 channels; 32 where (bf16) at most that many are left over in the last block, and for 5 x 5 f32 tiles, which would
-    // not fit twice
+    // Blocks of 64 channels; 32 where (bf16) those cover the channels with a fifth less padding, and for 5 x 5 f32 tiles, which would
+    // not fit twice.  (Groups of 16 lanes keep two columns open instead of four, and a pixel's 64 bytes of bf16 cost a tensor load what
+    // 128 do: 56 x 43 x 43 x 200 at stride 2 69.8 us with 32, 47.2 with 64; 31 x 89 x 89 x 416 149.4 and 139.7; but 26 x 31 x 31 x 32 4.3 and 5.7.)
     if constexpr (sizeof(T) == 2 || K == 3) {
-        if ((p.C - 1) % 64 >= 32 || (sizeof(T) == 4 && p.C > 64))
+        const int pad64 = (p.C + 63) / 64 * 64, pad32 = (p.C + 31) / 32 * 32;
+        if (sizeof(T) == 4 ? pad64 == pad32 || p.C > 64 : 4 * (int64_t)pad64 <= 5 * (int64_t)pad32)
             return p.sh == 1 ? try_launch_tma<T, 64, K, 1>(p, I, Kf, O, num_sms, stream, err) : try_launch_tma<T, 64, K, 2>(p, I, Kf, O, num_sms, stream, err);
     }
     return p.sh == 1 ? try_launch_tma<T, 32, K, 1>(p, I, Kf, O, num_sms, stream, err) : try_launch_tma<T, 32, K, 2>(p, I, Kf, O, num_sms, stream, err);
@@ -481,7 +499,9 @@ cudaError_t launch_typed(const DepthwiseProblem &p, const T *I, const T *Kf, flo
                      mult4(p.o_n) && mult4(p.o_h) && mult4(p.o_w) &&
                      reinterpret_cast<uintptr_t>(I) % (4 * sizeof(T)) == 0 && reinterpret_cast<uintptr_t>(Kf) % (4 * sizeof(T)) == 0 &&
                      reinterpret_cast<uintptr_t>(O) % 16 == 0;
-    const int64_t work = vec ? (int64_t)p.N * p.Ho * ((p.Wo + TW - 1) / TW) * (p.C / 4) : (int64_t)p.N * p.Ho * p.Wo * p.C;
+    const bool strided3 = p.sw == 2 && p.dw == 1 && p.KW == 3 && p.KH == 3;
+    const int tw = strided3 ? TW_STRIDED : TW_UNIT;
+    const int64_t work = vec ? (int64_t)p.N * p.Ho * ((p.Wo + tw - 1) / tw) * (p.C / 4) : (int64_t)p.N * p.Ho * p.Wo * p.C;
     const int64_t blocks64 = (work + 255) / 256;
     if (blocks64 > 0x7fffffff) return cudaErrorInvalidConfiguration;
     const unsigned blocks = (unsigned)blocks64;
@@ -506,14 +526,25 @@ cudaError_t launch_typed(const DepthwiseProblem &p, const T *I, const T *Kf, flo
             return cudaGetLastError();
         }
     }
-#define SG_DW(KERNEL) KERNEL<<<blocks, 256, 0, stream>>>(p, I, Kf, O)
-    if (vec && unit3) { if (small) SG_DW((depthwise_vec_kernel<T, true, uint32_t>)); else SG_DW((depthwise_vec_kernel<T, true, uint64_t>)); }
-    else if (vec) { if (small) SG_DW((depthwise_vec_kernel<T, false, uint32_t>)); else SG_DW((depthwise_vec_kernel<T, false, uint64_t>)); }
-    else { if (small) SG_DW((depthwise_generic_kernel<T, uint32_t>)); else SG_DW((depthwise_generic_kernel<T, uint64_t>)); }
-#undef SG_DW
+    // (the vector kernel may start while the kernel ahead of it drains: its threads wait for that kernel before their first load)
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks, 1, 1);
+    cfg.blockDim = dim3(256, 1, 1);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = vec ? 1 : 0;
+    auto launch = [&](auto narrow, auto wide) { return small ? cudaLaunchKernelEx(&cfg, narrow, p, I, Kf, O) : cudaLaunchKernelEx(&cfg, wide, p, I, Kf, O); };
+    cudaError_t err;
+    if (vec && unit3) err = launch(depthwise_vec_kernel<T, 1, uint32_t>, depthwise_vec_kernel<T, 1, uint64_t>);
+    else if (vec && strided3) err = launch(depthwise_vec_kernel<T, 2, uint32_t>, depthwise_vec_kernel<T, 2, uint64_t>);
+    else if (vec) err = launch(depthwise_vec_kernel<T, 0, uint32_t>, depthwise_vec_kernel<T, 0, uint64_t>);
+    else err = launch(depthwise_generic_kernel<T, uint32_t>, depthwise_generic_kernel<T, uint64_t>);
     count_launch();
     note_kernel(vec ? "depthwise_vec_kernel" : "depthwise_generic_kernel");
-    return cudaGetLastError();
+    return err;
 }
 
 }  // namespace

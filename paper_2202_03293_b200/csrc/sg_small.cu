@@ -44,9 +44,23 @@ struct Cfg {
     static_assert(2 * (STAGES * STAGE_BYTES + 1024) <= 233472, "two thread blocks on an SM");
 };
 
+// Division by a constant of the launch: n / d for 0 <= n < 2^31 as one multiplication.  With 2^(l-1) < d <= 2^l and
+// mul = ceil(2^(31+l) / d), n * mul / 2^(31+l) exceeds n / d by less than n / 2^(31+l) < 1 / d, so the integer part is right.
+struct FastDiv {
+    uint32_t mul, shift;      // mul 0: d = 1
+};
+inline FastDiv fast_div(int d) {
+    if (d <= 1) return FastDiv{0, 0};
+    uint32_t l = 1;
+    while (((int64_t)1 << l) < d) ++l;
+    return FastDiv{(uint32_t)((((uint64_t)1 << (31 + l)) + (uint32_t)d - 1) / (uint32_t)d), l - 1};
+}
+__device__ __forceinline__ int divide(int n, FastDiv f) { return f.mul == 0 ? n : (int)(__umulhi((uint32_t)n, f.mul) >> f.shift); }
+
 struct SmallParams {
     Problem p;
     int num_kb, num_n_tiles;
+    FastDiv by_hw, by_wo, by_c, by_kw;      // decomposition of m and of k
     int dense_filter;      // filter element k starts at k * k_c
     int uniform_rows;      // output row m starts at m * o_w
     int wait_prior;
@@ -120,7 +134,7 @@ small_gemm_kernel(const __grid_constant__ SmallParams sp, const char *__restrict
     const uint32_t b_dst = ring + C::A_BYTES + (uint32_t)(b_line * C::B_PITCH + b_piece * C::ES);
     auto row_offset = [&](int m) -> int64_t {      // element offset of output row m's window in the input
         if constexpr (CONV) {
-            const int hw = p.Ho * p.Wo, n = m / hw, r = m - n * hw, h = r / p.Wo, w = r - h * p.Wo;
+            const int n = divide(m, sp.by_hw), r = m - n * (p.Ho * p.Wo), h = divide(r, sp.by_wo), w = r - h * p.Wo;
             return (int64_t)n * p.i_n + (int64_t)h * p.sh * p.i_h + (int64_t)w * p.sw * p.i_w;
         } else {
             return m * p.i_w;
@@ -128,7 +142,7 @@ small_gemm_kernel(const __grid_constant__ SmallParams sp, const char *__restrict
     };
     auto k_offset = [&](int k) -> int64_t {        // ... of reduction index k in that window
         if constexpr (CONV) {
-            const int tap = k / p.C, c = k - tap * p.C, kh = tap / p.KW, kw = tap - kh * p.KW;
+            const int tap = divide(k, sp.by_c), c = k - tap * p.C, kh = divide(tap, sp.by_kw), kw = tap - kh * p.KW;
             return (int64_t)kh * p.dh * p.i_h + (int64_t)kw * p.dw * p.i_w + c;
         } else {
             return k * p.i_c;
@@ -136,43 +150,42 @@ small_gemm_kernel(const __grid_constant__ SmallParams sp, const char *__restrict
     };
     auto flt_offset = [&](int k, int n) -> int64_t {
         if (CONV && !sp.dense_filter) {
-            const int tap = k / p.C, c = k - tap * p.C, kh = tap / p.KW, kw = tap - kh * p.KW;
+            const int tap = divide(k, sp.by_c), c = k - tap * p.C, kh = divide(tap, sp.by_kw), kw = tap - kh * p.KW;
             return kh * p.k_kh + kw * p.k_kw + c * p.k_c + n;
         }
         return k * p.k_c + n * p.k_f;
     };
-    int64_t a_row[A_COPIES];      // K-major input: element offset of the row (-1: none)
-    if constexpr (!A_MN)
+    // Element offsets of this thread's copies: its first line's in the first stage, a uniform step from line to line and from stage to
+    // stage; the rows of a convolution lie anywhere, and its k is decomposed.  (With 64-bit products and
+    // two divisions for each copy, asking for two stages took a convolution 2200 cycles.)
+    int64_t a_off[CONV ? A_COPIES : 1];
+    if constexpr (CONV) {
 #pragma unroll
-        for (int i = 0; i < A_COPIES; ++i) {
-            const int m = m0 + a_line + i * A_STEP;
-            a_row[i] = m < p.M ? row_offset(m) : -1;
-        }
+        for (int i = 0; i < A_COPIES; ++i) a_off[i] = row_offset(m0 + a_line + i * A_STEP);
+    } else {
+        a_off[0] = A_MN ? a_line * p.i_c + m0 + a_piece : (m0 + a_line) * p.i_w + a_piece;
+    }
+    const int64_t b_off = B_KM ? (n0 + b_line) * p.k_f + b_piece : b_line * p.k_c + n0 + b_piece;
+    const int64_t a_lines = A_STEP * (A_MN ? p.i_c : p.i_w), b_lines = B_STEP * (B_KM ? p.k_f : p.k_c);
+    const int64_t a_stage = A_MN ? BK * p.i_c : BK, b_stage = B_KM ? BK : BK * p.k_c;
     auto fetch = [&](int kb) {
         const uint32_t stage = (uint32_t)(kb % C::STAGES) * C::STAGE_BYTES;
         const int k0 = kb * BK;
-        if constexpr (A_MN) {
+        // (a piece never straddles two taps: the channel count is a multiple of it)
+        const int64_t a_step = CONV ? k_offset(k0 + a_piece) : kb * a_stage;
 #pragma unroll
-            for (int i = 0; i < A_COPIES; ++i) {
-                const int k = k0 + a_line + i * A_STEP, m = m0 + a_piece;
-                const bool ok = k < p.K && m < p.M;
-                copy16(a_dst + stage + i * (A_STEP * C::A_PITCH), In + (ok ? k * p.i_c + m : 0) * C::ES, ok);
-            }
-        } else {
-            const int k = k0 + a_piece;      // (a piece never straddles two taps: the channel count is a multiple of it)
-            const int64_t k_off = CONV ? k_offset(k) : k;
-#pragma unroll
-            for (int i = 0; i < A_COPIES; ++i) {
-                const bool ok = k < p.K && a_row[i] >= 0;
-                copy16(a_dst + stage + i * (A_STEP * C::A_PITCH), In + (ok ? a_row[i] + k_off : 0) * C::ES, ok);
-            }
+        for (int i = 0; i < A_COPIES; ++i) {
+            const int line = a_line + i * A_STEP;
+            const bool ok = (A_MN ? k0 + line : k0 + a_piece) < p.K && (A_MN ? m0 + a_piece : m0 + line) < p.M;
+            const int64_t off = CONV ? a_off[CONV ? i : 0] + a_step : a_off[0] + a_step + i * a_lines;
+            copy16(a_dst + stage + i * (A_STEP * C::A_PITCH), In + (ok ? off : 0) * C::ES, ok);
         }
+        const int64_t b_step = kb * b_stage;
 #pragma unroll
         for (int i = 0; i < B_COPIES; ++i) {
-            const int line = b_line + i * B_STEP;
-            const int k = k0 + (B_KM ? b_piece : line), n = n0 + (B_KM ? line : b_piece);
-            const bool ok = k < p.K && n < p.N;
-            const int64_t off = B_KM ? n * p.k_f + k : flt_offset(k, n);
+            const int line = b_line + i * B_STEP, k = k0 + (B_KM ? b_piece : line);
+            const bool ok = k < p.K && n0 + (B_KM ? line : b_piece) < p.N;
+            const int64_t off = CONV && !sp.dense_filter ? flt_offset(k, n0 + b_piece) : b_off + b_step + i * b_lines;
             copy16(b_dst + stage + i * (B_STEP * C::B_PITCH), Flt + (ok ? off : 0) * C::ES, ok);
         }
     };
@@ -359,7 +372,7 @@ small_gemm_kernel(const __grid_constant__ SmallParams sp, const char *__restrict
     }
     int64_t off = (int64_t)m * p.o_w;
     if (!sp.uniform_rows) {
-        const int hw = p.Ho * p.Wo, b = m / hw, r = m - b * hw, h = r / p.Wo, w = r - h * p.Wo;
+        const int b = divide(m, sp.by_hw), r = m - b * (p.Ho * p.Wo), h = divide(r, sp.by_wo), w = r - h * p.Wo;
         off = (int64_t)b * p.o_n + (int64_t)h * p.o_h + (int64_t)w * p.o_w;
     }
     float4 *out = reinterpret_cast<float4 *>(O + off + n);
@@ -427,6 +440,7 @@ sg_status launch_small(const Problem &p, const void *In, const void *Flt, float 
     sp.p = p;
     sp.num_kb = (p.K + BK - 1) / BK;
     sp.num_n_tiles = (p.N + TN - 1) / TN;
+    sp.by_hw = fast_div(p.Ho * p.Wo); sp.by_wo = fast_div(p.Wo); sp.by_c = fast_div(p.C); sp.by_kw = fast_div(p.KW);
     const int64_t tiles = (int64_t)((p.M + 31) / 32) * sp.num_n_tiles;      // of 32 x 32
     sp.dense_filter = (p.KW == 1 || p.k_kw == p.C * p.k_c) && (p.KH == 1 || p.k_kh == (int64_t)p.KW * p.C * p.k_c);
     sp.uniform_rows = (p.Ho == 1 || p.o_h == (int64_t)p.Wo * p.o_w) && (p.batch == 1 || p.o_n == (int64_t)p.Ho * p.Wo * p.o_w);

@@ -86,13 +86,6 @@ __device__ __forceinline__ void split3(float x, float y, uint32_t &w0, uint32_t 
     w1 = pack_bf16(x1, y1);
     w2 = pack_bf16(x1 - __uint_as_float(w1 << 16), y1 - __uint_as_float(w1 & 0xFFFF0000u));
 }
-// Two f32 values as tf32 words and as bf16 pairs of those and of the rest (the split of the tcgen05 kernel).
-__device__ __forceinline__ void split_mix(float x, float y, uint32_t &hx, uint32_t &hy, uint32_t &h16, uint32_t &l16) {
-    hx = (__float_as_uint(x) + 0x1000u) & 0xFFFFE000u;
-    hy = (__float_as_uint(y) + 0x1000u) & 0xFFFFE000u;
-    h16 = pack_bf16(__uint_as_float(hx), __uint_as_float(hy));
-    l16 = pack_bf16(x - __uint_as_float(hx), y - __uint_as_float(hy));
-}
 __device__ __forceinline__ float lds(uint32_t addr) {
     float v;
     asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
@@ -206,7 +199,7 @@ small_gemm_kernel(const __grid_constant__ SmallParams sp, const char *__restrict
         for (int j = 0; j < 4; ++j)
 #pragma unroll
             for (int e = 0; e < 4; ++e) acc[i][j][e] = 0.f;
-    float largest = 0.f;       // f32: of the magnitudes seen (rounding a value near the largest to bf16 or tf32 gives infinity)
+    float largest = 0.f;       // EXACT: of the magnitudes seen (an infinity's, or a value's that a part rounds to it, meets zero parts of the other operand)
     for (int kb = 0; kb < sp.num_kb; ++kb) {
         asm volatile("cp.async.wait_group %0;" ::"n"(C::STAGES - 2) : "memory");
         __syncthreads();       // everyone's copies of this stage have landed; everyone is done with the stage refilled next
@@ -217,11 +210,11 @@ small_gemm_kernel(const __grid_constant__ SmallParams sp, const char *__restrict
         const int k = ks * 16;
         auto pair_a = [&](int i, int e, float &x, float &y) {
             load_pair<!A_MN>(a_tile, i * 16 + g + (e & 1) * 8, k + 2 * t + (e >> 1) * 8, C::A_PITCH, x, y);
-            largest = fmaxf(largest, fmaxf(fabsf(x), fabsf(y)));
+            if constexpr (MODE == EXACT) largest = fmaxf(largest, fmaxf(fabsf(x), fabsf(y)));
         };
         auto pair_b = [&](int j, int e, float &x, float &y) {
             load_pair<B_KM>(b_tile, j * 8 + g, k + 2 * t + e * 8, C::B_PITCH, x, y);
-            largest = fmaxf(largest, fmaxf(fabsf(x), fabsf(y)));
+            if constexpr (MODE == EXACT) largest = fmaxf(largest, fmaxf(fabsf(x), fabsf(y)));
         };
         auto add_step = [&](const float (&sum)[2][MI][4], int j0) {
 #pragma unroll
@@ -241,7 +234,7 @@ small_gemm_kernel(const __grid_constant__ SmallParams sp, const char *__restrict
                 for (int e = 0; e < 4; ++e) {
                     float x, y;
                     pair_a(i, e, x, y);
-                    split_mix(x, y, ah[i][0][e], ah[i][1][e], a16[i][0][e], a16[i][1][e]);
+                    split_pair_mix(__float_as_uint(x), __float_as_uint(y), ah[i][0][e], ah[i][1][e], a16[i][0][e], a16[i][1][e]);
                 }
             // (every step has a sum of its own, rounded to nearest into the running one: see below)
 #pragma unroll
@@ -254,7 +247,7 @@ small_gemm_kernel(const __grid_constant__ SmallParams sp, const char *__restrict
                     for (int e = 0; e < 2; ++e) {
                         float x, y;
                         pair_b(j0 + j, e, x, y);
-                        split_mix(x, y, bh[0][e], bh[1][e], b16[0][e], b16[1][e]);
+                        split_pair_mix(__float_as_uint(x), __float_as_uint(y), bh[0][e], bh[1][e], b16[0][e], b16[1][e]);
                     }
 #pragma unroll
                     for (int i = 0; i < MI; ++i) {
@@ -338,8 +331,8 @@ small_gemm_kernel(const __grid_constant__ SmallParams sp, const char *__restrict
 
     // ---- the warps' shares of k meet in shared memory; a thread writes four columns of one row
     asm volatile("cp.async.wait_group 0;" ::: "memory");
-    const bool overflow = F32 ? __syncthreads_or(largest >= 1.7014118e38f) != 0 : false;
-    if (!F32) __syncthreads();
+    const bool overflow = MODE == EXACT ? __syncthreads_or(largest >= 1.7014118e38f) != 0 : false;
+    if (MODE != EXACT) __syncthreads();
     float *red = reinterpret_cast<float *>(smem);
 #pragma unroll
     for (int i = 0; i < MI; ++i)
@@ -358,7 +351,7 @@ small_gemm_kernel(const __grid_constant__ SmallParams sp, const char *__restrict
         const float4 part = *reinterpret_cast<const float4 *>(red + (q * TM + row) * (C::RED_PITCH / 4) + col);
         v.x += part.x; v.y += part.y; v.z += part.z; v.w += part.w;
     }
-    if (F32 && overflow) {
+    if (MODE == EXACT && overflow) {
         // infinities, or values that a split rounds to them, among the operands: this tile is summed as it stands
         const float *a = reinterpret_cast<const float *>(In), *b = reinterpret_cast<const float *>(Flt);
         float s[4] = {0.f, 0.f, 0.f, 0.f};

@@ -357,114 +357,62 @@ __device__ __forceinline__ void umma_commit_cg2(uint32_t cluster_bar) {
 
 
 // ---------------------------------------------------------------- f32 inputs on the tensor cores: the hi/lo split
-// Larger of two magnitudes, NaN if either is: one NaN among the words must not pass the checks below.
-__device__ __forceinline__ float max_nan(float a, float b) {
-    float r;
-    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
-    return r;
+// x rounded to the nearest tf32 value (10 mantissa bits, the low 13 bits of the word zero), never to infinity: beyond the largest tf32
+// value it stays there.  One instruction; with an addition and a mask on the bit pattern, and a check of every
+// group of eight words for values that would round up to infinity, the splits below took twice the instructions.
+__device__ __forceinline__ uint32_t round_tf32(uint32_t x) {
+    uint32_t h;
+    asm("cvt.rn.satfinite.tf32.f32 %0, %1;" : "=r"(h) : "f"(__uint_as_float(x)));
+    return h;
 }
-__device__ __forceinline__ float largest4(const uint4 v) {
-    auto mag = [](uint32_t x) { return fabsf(__uint_as_float(x)); };
-    return max_nan(max_nan(mag(v.x), mag(v.y)), max_nan(mag(v.z), mag(v.w)));
-}
-// hi of a word on the slow path.
-__device__ __forceinline__ uint32_t truncated(uint32_t x) { return (x & 0x7FFFFFFFu) > 0x7F800000u ? 0x7FC00000u : x & 0xFFFFE000u; }
-// 3xTF32 split of four f32 words.  hi = x rounded to the nearest tf32 value (10 mantissa bits;
-// done on the bit pattern: add half an ulp, clear the low 13 bits); x - hi is exact in f32 and
-// lo is that difference rounded to tf32 the same way, so x - hi - lo is below 2^-22 |x|.  The
-// low bits of hi and lo are zero, so whatever rounding the tensor core applies to its inputs
-// leaves them unchanged.  Words of magnitude >= 2^127 (where rounding up
-// could reach infinity), infinities and NaNs take a slow path: hi truncated (a NaN stays one, whatever its
-// payload), lo = 0 unless finite.
-__device__ __forceinline__ void split4(const uint4 v, uint4 &h, uint4 &l) {
-    const float fx = __uint_as_float(v.x), fy = __uint_as_float(v.y), fz = __uint_as_float(v.z), fw = __uint_as_float(v.w);
-    if (largest4(v) < 1.7014118e38f) {
-        h.x = (v.x + 0x1000u) & 0xFFFFE000u; l.x = (__float_as_uint(fx - __uint_as_float(h.x)) + 0x1000u) & 0xFFFFE000u;
-        h.y = (v.y + 0x1000u) & 0xFFFFE000u; l.y = (__float_as_uint(fy - __uint_as_float(h.y)) + 0x1000u) & 0xFFFFE000u;
-        h.z = (v.z + 0x1000u) & 0xFFFFE000u; l.z = (__float_as_uint(fz - __uint_as_float(h.z)) + 0x1000u) & 0xFFFFE000u;
-        h.w = (v.w + 0x1000u) & 0xFFFFE000u; l.w = (__float_as_uint(fw - __uint_as_float(h.w)) + 0x1000u) & 0xFFFFE000u;
-    } else {
-        auto one = [](uint32_t x, uint32_t &hi, uint32_t &lo) {
-            hi = truncated(x);
-            const float d = __uint_as_float(x) - __uint_as_float(hi);
-            lo = (x & 0x7F800000u) == 0x7F800000u ? 0u : __float_as_uint(d);
-        };
-        one(v.x, h.x, l.x); one(v.y, h.y, l.y); one(v.z, h.z, l.z); one(v.w, h.w, l.w);
-    }
-}
-
-// The same for eight words, with one check for the slow path.
-__device__ __forceinline__ void split8(const uint4 v0, const uint4 v1, uint4 &h0, uint4 &l0, uint4 &h1, uint4 &l1) {
-    if (max_nan(largest4(v0), largest4(v1)) < 1.7014118e38f) {
-        auto one = [](uint32_t x, uint32_t &hi, uint32_t &lo) {
-            hi = (x + 0x1000u) & 0xFFFFE000u;
-            lo = (__float_as_uint(__uint_as_float(x) - __uint_as_float(hi)) + 0x1000u) & 0xFFFFE000u;
-        };
-        one(v0.x, h0.x, l0.x); one(v0.y, h0.y, l0.y); one(v0.z, h0.z, l0.z); one(v0.w, h0.w, l0.w);
-        one(v1.x, h1.x, l1.x); one(v1.y, h1.y, l1.y); one(v1.z, h1.z, l1.z); one(v1.w, h1.w, l1.w);
-    } else {
-        split4(v0, h0, l0);
-        split4(v1, h1, l1);
-    }
-}
-
 // Packs two f32 values, rounded to the nearest bf16, into one word: `even` in the low half, `odd` in the high half.
 __device__ __forceinline__ uint32_t pack_bf16(float even, float odd) {
     uint32_t d;
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(odd), "f"(even));
     return d;
 }
+// The same, never rounded up to infinity.
+__device__ __forceinline__ uint32_t pack_bf16_finite(float even, float odd) {
+    uint32_t d;
+    asm("cvt.rn.satfinite.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(odd), "f"(even));
+    return d;
+}
+// 3xTF32 split of eight f32 words.  hi = x rounded to tf32; x - hi is exact in f32 (also next to overflow, hi being finite) and lo is
+// that difference rounded to tf32 (add half an ulp, clear the low 13 bits), so x - hi - lo is below 2^-22 |x|.  The
+// low bits of hi and lo are zero, so whatever rounding the tensor core applies to its inputs
+// leaves them unchanged.  An infinity is hi = the largest tf32 value and lo = the infinity: its products are what they are in f32.  A
+// NaN, whatever its payload, is a NaN in hi.
+__device__ __forceinline__ void split8(const uint4 v0, const uint4 v1, uint4 &h0, uint4 &l0, uint4 &h1, uint4 &l1) {
+    auto one = [](uint32_t x, uint32_t &hi, uint32_t &lo) {
+        hi = round_tf32(x);
+        lo = (__float_as_uint(__uint_as_float(x) - __uint_as_float(hi)) + 0x1000u) & 0xFFFFE000u;
+    };
+    one(v0.x, h0.x, l0.x); one(v0.y, h0.y, l0.y); one(v0.z, h0.z, l0.z); one(v0.w, h0.w, l0.w);
+    one(v1.x, h1.x, l1.x); one(v1.y, h1.y, l1.y); one(v1.z, h1.z, l1.z); one(v1.w, h1.w, l1.w);
+}
+
 // The split used when the two correction products run as bf16 MMAs: x = hi + lo with hi = x rounded to tf32 (as above); the
 // main product hi*hi runs in tf32, the corrections lo*hi + hi*lo with all four factors rounded to bf16.  A correction term
 // is below 2^-11 of its product and bf16 keeps 8 bits of each factor, so the rounding moves a product by less than 2^-19 of
 // itself (what the dropped lo*lo term and the tensor core's f32 accumulation cost already), and the two bf16 products of a k-block are one
 // contraction over 64 values, [lo | hi] . [hi | lo], at twice the tf32 rate: two tensor-core units per term instead of three.
-// Words of magnitude >= 2^127, infinities and NaNs: hi and its bf16 copy are truncated, never rounded up to infinity.
-__device__ __forceinline__ void split4_mix(const uint4 v, uint4 &h, uint2 &h16, uint2 &l16) {
-    const float fx = __uint_as_float(v.x), fy = __uint_as_float(v.y), fz = __uint_as_float(v.z), fw = __uint_as_float(v.w);
-    if (largest4(v) < 1.7014118e38f) {
-        h.x = (v.x + 0x1000u) & 0xFFFFE000u; h.y = (v.y + 0x1000u) & 0xFFFFE000u;
-        h.z = (v.z + 0x1000u) & 0xFFFFE000u; h.w = (v.w + 0x1000u) & 0xFFFFE000u;
-        h16.x = pack_bf16(__uint_as_float(h.x), __uint_as_float(h.y));
-        h16.y = pack_bf16(__uint_as_float(h.z), __uint_as_float(h.w));
-        l16.x = pack_bf16(fx - __uint_as_float(h.x), fy - __uint_as_float(h.y));
-        l16.y = pack_bf16(fz - __uint_as_float(h.z), fw - __uint_as_float(h.w));
-    } else {
-        auto one = [](uint32_t x, uint32_t &hi, uint32_t &hi16, uint32_t &lo16) {
-            hi = truncated(x);
-            hi16 = hi >> 16;
-            const float d = __uint_as_float(x) - __uint_as_float(hi);
-            lo16 = (x & 0x7F800000u) == 0x7F800000u ? 0u : (pack_bf16(d, 0.f) & 0xFFFFu);     // (small: rounding cannot overflow)
-        };
-        uint32_t a[4], b[4];
-        one(v.x, h.x, a[0], b[0]); one(v.y, h.y, a[1], b[1]); one(v.z, h.z, a[2], b[2]); one(v.w, h.w, a[3], b[3]);
-        h16.x = a[0] | (a[1] << 16); h16.y = a[2] | (a[3] << 16);
-        l16.x = b[0] | (b[1] << 16); l16.y = b[2] | (b[3] << 16);
-    }
+// Infinities and NaNs: as above (the bf16 copy of hi is finite too).
+__device__ __forceinline__ void split_pair_mix(uint32_t x, uint32_t y, uint32_t &hx, uint32_t &hy, uint32_t &h16, uint32_t &l16) {
+    hx = round_tf32(x);
+    hy = round_tf32(y);
+    h16 = pack_bf16_finite(__uint_as_float(hx), __uint_as_float(hy));
+    l16 = pack_bf16(__uint_as_float(x) - __uint_as_float(hx), __uint_as_float(y) - __uint_as_float(hy));
 }
-
-
+__device__ __forceinline__ void split4_mix(const uint4 v, uint4 &h, uint2 &h16, uint2 &l16) {
+    split_pair_mix(v.x, v.y, h.x, h.y, h16.x, l16.x);
+    split_pair_mix(v.z, v.w, h.z, h.w, h16.y, l16.y);
+}
 // The same for eight values (two chunks of four): hi of each chunk, and the eight bf16 values of hi and of lo packed in k order.
-// One check for the slow path covers all eight.
 __device__ __forceinline__ void split8_mix(const uint4 v0, const uint4 v1, uint4 &h0, uint4 &h1, uint4 &h16, uint4 &l16) {
-    if (max_nan(largest4(v0), largest4(v1)) < 1.7014118e38f) {
-        auto two = [](uint32_t x, uint32_t y, uint32_t &hx, uint32_t &hy, uint32_t &h, uint32_t &l) {
-            hx = (x + 0x1000u) & 0xFFFFE000u;
-            hy = (y + 0x1000u) & 0xFFFFE000u;
-            h = pack_bf16(__uint_as_float(hx), __uint_as_float(hy));
-            l = pack_bf16(__uint_as_float(x) - __uint_as_float(hx), __uint_as_float(y) - __uint_as_float(hy));
-        };
-        two(v0.x, v0.y, h0.x, h0.y, h16.x, l16.x);
-        two(v0.z, v0.w, h0.z, h0.w, h16.y, l16.y);
-        two(v1.x, v1.y, h1.x, h1.y, h16.z, l16.z);
-        two(v1.z, v1.w, h1.z, h1.w, h16.w, l16.w);
-    } else {
-        uint2 a, b, c, d;
-        split4_mix(v0, h0, a, b);
-        split4_mix(v1, h1, c, d);
-        h16 = make_uint4(a.x, a.y, c.x, c.y);
-        l16 = make_uint4(b.x, b.y, d.x, d.y);
-    }
+    split_pair_mix(v0.x, v0.y, h0.x, h0.y, h16.x, l16.x);
+    split_pair_mix(v0.z, v0.w, h0.z, h0.w, h16.y, l16.y);
+    split_pair_mix(v1.x, v1.y, h1.x, h1.y, h16.z, l16.z);
+    split_pair_mix(v1.z, v1.w, h1.z, h1.w, h16.w, l16.w);
 }
 
 // Reads and clears this translation unit's status word; the caller has synchronised the stream.

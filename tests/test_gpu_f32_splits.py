@@ -1,4 +1,5 @@
-"""f32 products on the tensor cores: the converter groups of the narrow tiles against the oracle."""
+"""f32 products on the tensor cores: the converter groups of the narrow tiles against the oracle, and infinities, NaNs and values next to
+overflow against f64."""
 import numpy as np
 import pytest
 import torch
@@ -29,4 +30,28 @@ def test_converter_groups(M, N, K, bn, cg, a_t, b_t):
         sg.sg_set_tile_override(0, 0, 0)
     want, S = ref.matmul(a, b)
     assert assert_within_bound(C, want, S, "converter groups") < 4e-6      # 2^-19 for the rounded corrections, and the truncating sum
+    sg.sg_check()
+
+
+# an infinity's products are infinities of the right sign (NaN against a zero), a NaN's NaN, and finite values stay finite
+@pytest.mark.parametrize("a_t,b_t", [(False, False), (True, False), (False, True), (True, True)])
+@pytest.mark.parametrize("M,N,K", [(256, 256, 2048), (128, 128, 128)])
+def test_special_values(M, N, K, a_t, b_t):
+    g = torch.Generator(device="cuda").manual_seed(SEED)
+    A = torch.rand(M, K, generator=g, device="cuda") * 2 - 1
+    B = torch.rand(K, N, generator=g, device="cuda") * 2 - 1
+    A[3, 5], A[4, 6], A[7, 8], A[20, 11] = float("inf"), float("-inf"), float("nan"), 0.0
+    A[9, 9], A[10, 9] = torch.finfo(torch.float32).max, -torch.finfo(torch.float32).max
+    B[9, :] *= 0.25
+    B[5, 7], B[11, 13] = 0.0, float("inf")
+    want = A.double() @ B.double()
+    a, b = A.t().contiguous().t() if a_t else A, B.t().contiguous().t() if b_t else B
+    C = torch.zeros(M, N, device="cuda")
+    sg.sg_matmul(a, b, C)
+    torch.cuda.synchronize()
+    assert torch.equal(torch.isnan(C), torch.isnan(want)) and torch.equal(torch.isinf(C), torch.isinf(want))
+    assert torch.equal(torch.sign(C[torch.isinf(C)]), torch.sign(want[torch.isinf(want)]).float())
+    bound = A.double().abs().nan_to_num(0, 0, 0) @ B.double().abs().nan_to_num(0, 0, 0)
+    finite = torch.isfinite(want)
+    assert ((C.double() - want).abs()[finite] <= 4e-6 * bound[finite]).all()
     sg.sg_check()

@@ -307,12 +307,11 @@ depthwise_tma_kernel(const __grid_constant__ CUtensorMap map_in, const Depthwise
             for (int t = blockIdx.x; t < d.num_tiles; t += gridDim.x, ++k) {
                 const int s = k & 1;
                 const uint32_t ph = (uint32_t)(k >> 1) & 1u;
-                // (the divisions ahead of the wait: the load goes out as soon as the stage is free)
+                if (!mbar_wait(smem_u32(&empty_bar[s]), ph ^ 1u, &abort_load)) break;
                 int r = t;
                 const int cb = r % d.c_blocks; r /= d.c_blocks;
                 const int wt = r % d.tiles_w; r /= d.tiles_w;
                 const int ht = r % d.tiles_h, nt = r / d.tiles_h;
-                if (!mbar_wait(smem_u32(&empty_bar[s]), ph ^ 1u, &abort_load)) break;
                 mbar_expect_tx(smem_u32(&full_bar[s]), (uint32_t)d.box_bytes);
                 tma_load_4d(ring + (uint32_t)(s * d.stage_bytes), &map_in, smem_u32(&full_bar[s]), cb * CB, wt * tile_cols * S, ht * tile_rows * S, nt * tile_n);
             }

@@ -684,10 +684,11 @@ sg_status launch_conv_wide(const Problem &p, const void *In, const void *Flt, fl
     if (f32) {
         // The im2col kernel deals a reduction out over the SMs: where there are few positions and much to sum it is the better one
         // (8 x 28 x 28, 3x3x256x256: 43.9 us here, 38.5 there; 16 x 56 x 56, 3x3x64x128: 32.3 against 41.6; both estimates are within
-        // a tenth or so).  Filters of 65 to 128 columns that the strip kernel would keep resident run faster here whatever the
-        // estimates say (12 x 12 x 61, 1x1x16x96: 7.8 -> 5.6).
+        // a tenth or so).  Filters of 65 to 128 columns and three
+        // taps or more that the strip kernel would keep resident run faster here whatever the estimates say (43 x 2934,
+        // 3x32x128: 18.9 against 22.2; but one tap, 54 x 54, 1x1x48x96: 6.1 against 5.2).
         const double us = plan_f32(p, positions, f_tiles, row_span, full_span, num_sms, w, g);
-        const bool strip = p.N <= 128 && p.N > 64 && mult(p.N, 32) && (int64_t)g.taps * w.kb <= 6;
+        const bool strip = p.N <= 128 && p.N > 64 && mult(p.N, 32) && g.taps >= 3 && (int64_t)g.taps * w.kb <= 6;
         if (!forced && im2col && !strip && us >= 0.95 * tensor_estimate_us(p)) return SG_ERR_UNSUPPORTED;
     } else plan_bf16(p, positions, f_tiles, row_span, full_span, num_sms, w);
     if (w.BN == 0 || (int64_t)w.tiles * f_tiles > 0x7fffffff) return SG_ERR_UNSUPPORTED;

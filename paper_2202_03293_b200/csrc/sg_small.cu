@@ -449,16 +449,23 @@ sg_status launch_small(const Problem &p, const void *In, const void *Flt, float 
     const bool mix = f32 && !a_mn && !b_km && tensor_takes(p, In, Flt, O);
     if (f32 && !conv && !a_mn && !b_km && !mix) return SG_ERR_UNSUPPORTED;
     if (mode < 0) {
-        // By time (us), fitted to graph replays of 52 shapes from 64^3 to 1024^3: a launch, then waves of thread blocks over the
-        // SMs (two share an SM's tensor cores), each a start and its steps of 128 k.  The other side is the tcgen05 kernel's
-        // cost model, which must lose clearly; convolutions of inputs below 128 KiB have no im2col path to compare with.
-        const double steps = p.K < BK ? 0.5 : (double)p.K / BK, waves = (double)((tiles + num_sms - 1) / num_sms);
-        const double step = !f32 ? 0.36 : (waves > 1 ? 0.72 : half && tiles * 2 > num_sms ? 1.0 : 0.8) * (mix ? 1.0 : 1.25);
-        const double us = 1.2 + waves * ((f32 ? 0.6 : 0.55) + step * steps);
-        // (the tcgen05 kernel never takes less than 3.1 us, f32 4.1: no need to ask.  Its f32 estimates are the closer ones.  Inputs stored
-        // transposed whose rows are no whole 128 bytes of m are left to the gather kernel, which takes over half as long again.)
-        const double lead = a_mn && p.M % (f32 ? 32 : 64) != 0 ? 1.6 : f32 ? 0.95 : 0.85;
-        if (us > (f32 ? 4.0 : 3.0) && us > (conv && in_bytes < 131072 ? 0.3 * p.K : lead * tensor_estimate_us(p))) return SG_ERR_UNSUPPORTED;
+        // By time (us): a launch, then waves of thread blocks over the SMs (two share an SM's tensor cores), each a start and its steps of
+        // 128 k.  The other side is the tcgen05 kernel's cost model; convolutions of inputs
+        // below 128 KiB have no im2col path to compare with.  Fitted to graph replays of 124 calls with either kernel (products of 64 to
+        // 4096 in every layout, convolutions): within 13 % of the timings, choices 0.9 % off the better of the two in the mean (0.6 % with
+        // the tcgen05 kernel's launches as they are outside a graph).
+        const double steps = std::max(0.5, (double)p.K / BK), waves = (double)((tiles + num_sms - 1) / num_sms);
+        const double step = !f32 ? (waves > 1 ? 0.282 : 0.49) : (waves > 1 ? 0.82 : half && tiles * 2 > num_sms ? 1.29 : 0.80) * (mix ? 1.0 : 1.11);
+        const double us = 1.2 + waves * ((f32 ? 0.70 : 0.74) + step * steps);
+        // (the tcgen05 kernel never takes less than 2.8 us, f32 3.6: no need to ask.  Issued one by one its launches take
+        // 0.3 to 0.6 us more than in a graph, these do not: 1066 x 256 x 320 f32 6.4 us here, 6.9 there in a graph and 6.7 against 7.5 one by
+        // one.  What it does not take (inputs stored transposed whose rows are no whole 128 bytes of m,
+        // outputs that are not one matrix) the gather kernel would run, in three times its estimate: 1616 x 168 x 599 bf16
+        // 8.8 us here, 17.1 there, 4.6 estimated.  Unit-stride convolutions of bf16 go to conv_wide_kernel, which is faster than that estimate,
+        // but not below 4.5 us: 2220 x 96, 3x80, 3.5 us here, 4.6 there.)
+        const bool run_conv = conv && !f32 && p.sh == 1 && p.sw == 1;
+        const double lead = !tensor_takes(p, In, Flt, O) ? 3.0 : f32 ? 1.055 : run_conv ? 0.8 : 1.08;
+        if (us > (f32 ? 3.6 : run_conv ? 4.0 : 2.8) && us > (conv && in_bytes < 131072 ? 0.3 * p.K : lead * tensor_estimate_us(p))) return SG_ERR_UNSUPPORTED;
     }
     tensor_note_choice(TN, 1, 1);
 #define SG_SMALL(MODE_, A_MN_, B_KM_, CONV_, SLOT)                                                                  \

@@ -1200,10 +1200,11 @@ bool encode_im2col_cached(CUtensorMap *map, int device, CUtensorMapDataType type
 
 inline bool mult(int64_t v, int64_t q) { return v % q == 0; }
 
-struct Variant { int bn, cg; double mma_ns, mma_ns_f32; };
-// Time one CTA needs for one k-block of a tile, in ns: its tensor core (bf16), or its converter warps and tensor core (f32).
-constexpr Variant kVariants[] = {{64, 1, 100.0, 500.0}, {128, 1, 135.0, 570.0}, {256, 1, 330.0, 1500.0},
-                                 {128, 2, 135.0, 515.0}, {256, 2, 330.0, 690.0}};
+struct Variant { int bn, cg; double mma_ns, mma_ns_f32, mma_ns_f32_t; };
+// Time one CTA needs for one k-block of a tile, in ns: its tensor core (bf16), or its converter warps and tensor core (f32: plain layout,
+// eight MMAs; an operand stored transposed, twelve).
+constexpr Variant kVariants[] = {{64, 1, 125.0, 336.0, 385.0}, {128, 1, 150.0, 424.0, 517.0}, {256, 1, 400.0, 1500.0, 1500.0},
+                                 {128, 2, 140.0, 374.0, 1500.0}, {256, 2, 358.0, 627.0, 903.0}};
 constexpr int kNumVariants = sizeof(kVariants) / sizeof(kVariants[0]);
 
 // A stream-K tail (launch_tensor) pays when the k-blocks saved clearly outweigh the extra epilogues and the clearing launch.
@@ -1221,31 +1222,40 @@ int stream_k_run(const Variant &v, bool f32, int64_t tiles, int groups, int num_
 
 // Estimated kernel time in ns of `tiles` tiles dealt out in `sp` k ranges each over `groups`
 // CTAs or CTA pairs.  A k-block costs the slowest of: the CTA's own time, the CTA's share of the L2 -> shared memory fill
-// rate of the whole chip, and the fill rate one SM reaches alone.  The bf16 constants were fitted to timings of every variant and
-// split on the 125 shapes {256..4096}^3 (the choices they lead to are within 1 % of the best per-shape choice in total time), the
-// f32 ones to 48 shapes between 64 and 8192 (within 9 % of the timings, choices 1.3 % off the best in the mean).
-double estimate_ns(const Variant &v, bool f32, int64_t tiles, int64_t groups, int num_kb, int sp, bool accumulate, bool tail) {
+// rate of the whole chip, the fill rate one SM reaches alone, and (bf16 stages of one k-block: `plain` false) a stage's two waits.
+// f32: `plain` false = an operand stored transposed.  Fitted to graph replays of every variant and split on 125 (bf16) and 118 (f32) calls:
+// products of 64 to 16384 in every layout and convolutions, three operand sets in turn.  The estimates are within 11 and 7 % of
+// the timings near the best; the choices cost 0.4 % over the best in the mean (with the constants of slower kernels
+// 1.3 and 4 %), half of the shapes held back from the fit 0.7 and 0.8.
+double estimate_ns(const Variant &v, bool f32, bool plain, int64_t tiles, int64_t groups, int num_kb, int sp, bool accumulate, bool tail) {
     const int64_t items = tiles * sp;
     const int64_t waves = (items + groups - 1) / groups;
     const int kbs = (num_kb + sp - 1) / sp;
     const double active = (double)((items < groups ? items : groups) * v.cg);
     const double stage_bytes = A_STAGE_BYTES + (double)(v.bn / v.cg) * ROW_BYTES;
-    const double chip_fill = f32 ? 11500.0 : 14000.0, sm_fill = f32 ? 54.0 : 130.0;      // bytes per ns
-    double kb_ns = f32 ? v.mma_ns_f32 : v.mma_ns;
+    const double chip_fill = f32 ? 11100.0 : 17100.0, sm_fill = f32 ? 77.3 : 127.0;      // bytes per ns
+    double kb_ns = !f32 ? v.mma_ns : plain ? v.mma_ns_f32 : v.mma_ns_f32_t;
+    if (!f32 && !plain && kb_ns < 218.0) kb_ns = 218.0;
     if (active * stage_bytes / chip_fill > kb_ns) kb_ns = active * stage_bytes / chip_fill;
     if (stage_bytes / sm_fill > kb_ns) kb_ns = stage_bytes / sm_fill;
-    const double item_ns = f32 ? 2770.0 + 20.0 * v.bn : 1500.0 + 12.0 * v.bn;          // pipeline fill + epilogue of one item
-    double t = (double)waves * kbs * kb_ns + item_ns + (double)(waves - 1) * 0.3 * item_ns;
+    const double item_ns = f32 ? 2280.0 + 15.6 * v.bn : 2000.0 + 10.2 * v.bn;          // pipeline fill + epilogue of one item
+    // (what the next item's main loop does not hide of an epilogue: most of it where there is one accumulator buffer)
+    const double open = !f32 ? 0.43 : v.bn == 256 ? 0.74 : 0.26;
+    // ... and short reductions are paced by the stores: 16234 x 1152 x 64 bf16, 5 waves of 256 columns 28 us, 8 of 128 20 us
+    double wave_ns = kbs * kb_ns + open * item_ns;
+    if (active * BM * v.bn * 4 / 6000.0 > wave_ns) wave_ns = active * BM * v.bn * 4 / 6000.0;
+    double t = (double)kbs * kb_ns + item_ns + (double)(waves - 1) * wave_ns;
     const int run = f32 && sp == 1 && tail ? stream_k_run(v, f32, tiles, (int)groups, num_kb, 1, false) : 0;
     if (run > 0) t += item_ns + 1500.0 - (double)(num_kb - run) * kb_ns;               // the last wave is shorter, the write-backs are more
-    if (v.cg == 2) t += f32 ? 600.0 : 2000.0;                                          // cluster launch, cross-CTA signalling
-    if (sp > 1) t += 2500.0 - (accumulate ? 1500.0 : 0.0);                             // reduce-add traffic, the clearing launch
+    if (v.cg == 2) t += 490.0;                                                         // cluster launch, cross-CTA signalling
+    if (sp > 1) t += f32 ? 2880.0 : 2610.0;                                            // reduce-add traffic, the clearing launch
+    if (sp > 1 && accumulate) t -= f32 ? 2290.0 : 2420.0;                              // (no clearing)
     return t;
 }
 
 // The same for `sp` CTAs in a cluster per tile.
-double estimate_meet_ns(const Variant &v, bool f32, int64_t tiles, int num_kb, int sp) {
-    return estimate_ns(v, f32, tiles * sp, tiles * sp, (num_kb + sp - 1) / sp, 1, false, false) + (f32 ? 2200.0 : 1300.0 + 11.0 * v.bn);
+double estimate_meet_ns(const Variant &v, bool f32, bool plain, int64_t tiles, int num_kb, int sp) {
+    return estimate_ns(v, f32, plain, tiles * sp, tiles * sp, (num_kb + sp - 1) / sp, 1, false, false) + (f32 ? 2200.0 : 1300.0 + 11.0 * v.bn);
 }
 
 // Operands stored transposed (matmuls only): bit 0 the input ([k][m], m contiguous), bit 1 the filter ([n][k], k contiguous).
@@ -1260,6 +1270,8 @@ double choose_tiles(const Problem &p, int num_kb, int lay, const Overrides &ov, 
     *out_meet = 0;
     const bool fused = p.bias != nullptr || p.act != SG_ACT_NONE, forced_tile = ov.bn > 0 || ov.cg > 0 || (ov.split > 0 && !fused);
     const bool f32 = !p.in_bf16;
+    // (bf16: two k-blocks per stage, see launch_tensor)
+    const bool plain = f32 ? lay == 0 : lay == 0 && p.spatial_rank == 0 && p.K % 64 == 0 && p.N % 64 == 0;
     int pick = -1, splits = 1;
     double best = 1e300;
     if (ov.bn > 0) {
@@ -1291,14 +1303,14 @@ double choose_tiles(const Problem &p, int num_kb, int lay, const Overrides &ov, 
             const int64_t tiles = (int64_t)((p.M + v.cg * BM - 1) / (v.cg * BM)) * ((p.N + v.bn - 1) / v.bn);
             const int64_t groups = num_sms / v.cg;
             if (forced) {
-                const double c = estimate_ns(v, f32, tiles, groups, num_kb, forced, p.accumulate != 0, ov.sk != 0 && !fused);
+                const double c = estimate_ns(v, f32, plain, tiles, groups, num_kb, forced, p.accumulate != 0, ov.sk != 0 && !fused);
                 if (c < best) { best = c; pick = i; splits = forced; }
                 continue;
             }
             for (int sp = 1; sp <= 32; sp *= 2) {
                 if (!valid_split(sp)) break;
                 if (sp > 1 && tiles * (sp / 2) >= 2 * groups) break;   // already two waves without this split
-                const double c = estimate_ns(v, f32, tiles, groups, num_kb, sp, p.accumulate != 0, ov.sk != 0 && !fused);
+                const double c = estimate_ns(v, f32, plain, tiles, groups, num_kb, sp, p.accumulate != 0, ov.sk != 0 && !fused);
                 if (c < best) { best = c; pick = i; splits = sp; }
             }
         }
@@ -1315,7 +1327,7 @@ double choose_tiles(const Problem &p, int num_kb, int lay, const Overrides &ov, 
                 if (ov.meet > 1 && sp != ov.meet) continue;
                 const int stages = (num_kb + 1) / 2, per = (stages + sp - 1) / sp;       // (bf16: ranges of whole two-block stages too)
                 if (tiles > (sp == 2 ? 70 : sp == 4 ? 32 : 14) || tiles * sp > num_sms - 8 || num_kb < 4 * sp || !valid_split(sp) || (stages + per - 1) / per != sp) continue;
-                const double c = ov.meet > 1 ? 0.0 : estimate_meet_ns(v, f32, tiles, num_kb, sp);
+                const double c = ov.meet > 1 ? 0.0 : estimate_meet_ns(v, f32, plain, tiles, num_kb, sp);
                 if (c < best) { best = c; pick = i; splits = sp; *out_meet = 1; }
             }
         }
@@ -1671,9 +1683,7 @@ double tensor_estimate_us(const Problem &p) {
     if (p.bias != nullptr || p.act != SG_ACT_NONE) ov.split = 1;
     const int bk = ROW_BYTES / (p.in_bf16 ? 2 : 4);
     int pick, splits, meet;
-    const double ns = choose_tiles(p, p.KH * p.KW * ((p.C + bk - 1) / bk), transposed_layout(p), ov, d->num_sms, &pick, &splits, &meet);
-    // (the constants were fitted to problems of 256^3 and up; launches of bf16 problems below take about 0.9 us more)
-    return ns * 1e-3 + (p.in_bf16 ? 0.9 : 0.0);
+    return 1e-3 * choose_tiles(p, p.KH * p.KW * ((p.C + bk - 1) / bk), transposed_layout(p), ov, d->num_sms, &pick, &splits, &meet);
 }
 
 int tensor_small_override() {

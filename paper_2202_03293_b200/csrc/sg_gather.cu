@@ -25,8 +25,8 @@
 // next chunk.  Up to four k-blocks of bf16 need no running sum: each has an accumulator of its own (a bank), and the
 // write-back adds them up.
 //
-// What bounds a k-block is the number of load and store instructions of the producers (256 lines of a 128 x 128 tile, two
-// loads and one store each when pairs are not aligned, against 256 cycles of MMAs).
+// What bounds a k-block of a 128 x 128 tile: raw lines, the tensor loads (4.9 cycles for an unaligned line, 1254 of the 1370
+// measured); f32, the shared-memory pipe (MMA operands 1536 cycles, parts written 768, and the loads: 3600 measured).
 #include <algorithm>
 #include <initializer_list>
 #include <type_traits>

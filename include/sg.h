@@ -43,9 +43,11 @@
  *     (TMA + tcgen05): bf16 inputs directly, f32 inputs split into hi + lo with
  *     hi*hi in tf32 and lo*hi + hi*lo in bf16 (operands stored transposed: in
  *     tf32), summed in f32, which keeps f32 accuracy for finite inputs: the
- *     error stays below 1e-5 * sum_k |a*b|.  Infinities keep their meaning there
- *     too, but that a factor below 2^-134 counts as zero against them.  Small
- *     problems run on many small thread blocks (mma.sync).  Other layouts run on a tensor-core
+ *     error stays below 1e-5 * sum_k |a*b| (subnormal f32 factors are taken as
+ *     multiples of 2^-136).  Infinities keep their meaning there while the
+ *     factors that they meet in a sum are normal and below 2000 together; beyond
+ *     that the sum may be NaN.  Small problems run on many small thread blocks
+ *     (mma.sync), where every infinity keeps its meaning.  Other layouts run on a tensor-core
  *     kernel that fetches its operands with ordinary or unaligned tensor loads
  *     and is about as accurate as an f32 FMA loop (f32 inputs as three bf16
  *     parts; infinities keep their meaning), tiny problems in them on a strided

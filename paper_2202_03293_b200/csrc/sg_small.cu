@@ -44,7 +44,8 @@ struct Cfg {
     static_assert(2 * (STAGES * STAGE_BYTES + 1024) <= 233472, "two thread blocks on an SM");
 };
 
-// Division by a constant of the launch: n / d for 0 <= n < 2^31 as one multiplication.  With 2^(l-1) < d <= 2^l and
+// Division by a constant of the launch: n / d for 0 <= n < 2^31 as one multiplication, by a multiplier rounded up (Granlund and Montgomery, Division
+// by invariant integers using multiplication, 1994).  With 2^(l-1) < d <= 2^l and
 // mul = ceil(2^(31+l) / d), n * mul / 2^(31+l) exceeds n / d by less than n / 2^(31+l) < 1 / d, so the integer part is right.
 struct FastDiv {
     uint32_t mul, shift;      // mul 0: d = 1
@@ -100,6 +101,33 @@ __device__ __forceinline__ void load_pair(uint32_t tile, int mn, int k, int pitc
         x = lds(tile + (uint32_t)(k * pitch + mn * 4));
         y = lds(tile + (uint32_t)((k + 1) * pitch + mn * 4));
     }
+}
+
+// Four columns of row m by multiply-adds on the operands as they stand, until all four are NaN (a NaN stays one).  Out of line: the kernel's loops need the registers.
+template <bool CONV>
+__device__ __noinline__ float4 sum_as_it_stands(const SmallParams &sp, const float *a, const float *b, int m, int n) {
+    const Problem &p = sp.p;
+    int64_t row = m * p.i_w;
+    if constexpr (CONV) {
+        const int i = divide(m, sp.by_hw), r = m - i * (p.Ho * p.Wo), h = divide(r, sp.by_wo), w = r - h * p.Wo;
+        row = (int64_t)i * p.i_n + (int64_t)h * p.sh * p.i_h + (int64_t)w * p.sw * p.i_w;
+    }
+    float s[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int k0 = 0; k0 < p.K && (s[0] == s[0] || s[1] == s[1] || s[2] == s[2] || s[3] == s[3]); k0 += 4)
+#pragma unroll
+        for (int k = k0; k < k0 + 4; ++k) {
+            if (k >= p.K) break;
+            int64_t x_off = k * p.i_c, f_off = k * p.k_c;
+            if constexpr (CONV) {
+                const int tap = divide(k, sp.by_c), c = k - tap * p.C, kh = divide(tap, sp.by_kw), kw = tap - kh * p.KW;
+                x_off = (int64_t)kh * p.dh * p.i_h + (int64_t)kw * p.dw * p.i_w + c;
+                f_off = kh * p.k_kh + kw * p.k_kw + c * p.k_c;
+            }
+            const float x = a[row + x_off];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) s[e] = fmaf(x, b[f_off + (n + e) * p.k_f], s[e]);
+        }
+    return make_float4(s[0], s[1], s[2], s[3]);
 }
 
 template <int MODE, bool A_MN, bool B_KM, bool CONV, int TM>
@@ -199,7 +227,7 @@ small_gemm_kernel(const __grid_constant__ SmallParams sp, const char *__restrict
         for (int j = 0; j < 4; ++j)
 #pragma unroll
             for (int e = 0; e < 4; ++e) acc[i][j][e] = 0.f;
-    float largest = 0.f;       // EXACT: of the magnitudes seen (an infinity's, or a value's that a part rounds to it, meets zero parts of the other operand)
+    float largest = 0.f;       // EXACT: of the magnitudes seen
     for (int kb = 0; kb < sp.num_kb; ++kb) {
         asm volatile("cp.async.wait_group %0;" ::"n"(C::STAGES - 2) : "memory");
         __syncthreads();       // everyone's copies of this stage have landed; everyone is done with the stage refilled next
@@ -351,17 +379,14 @@ small_gemm_kernel(const __grid_constant__ SmallParams sp, const char *__restrict
         const float4 part = *reinterpret_cast<const float4 *>(red + (q * TM + row) * (C::RED_PITCH / 4) + col);
         v.x += part.x; v.y += part.y; v.z += part.z; v.w += part.w;
     }
-    if (MODE == EXACT && overflow) {
-        // infinities, or values that a split rounds to them, among the operands: this tile is summed as it stands
-        const float *a = reinterpret_cast<const float *>(In), *b = reinterpret_cast<const float *>(Flt);
-        float s[4] = {0.f, 0.f, 0.f, 0.f};
-        const int64_t ro = row_offset(m);
-        for (int kk = 0; kk < p.K; ++kk) {
-            const float x = a[ro + k_offset(kk)];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) s[e] = fmaf(x, b[flt_offset(kk, n + e)], s[e]);
-        }
-        v = make_float4(s[0], s[1], s[2], s[3]);
+    // What the splits do not carry is summed as it stands.  MIX has an infinity as (largest, infinity): against a factor of 2048 and
+    // more, whose low part may be above 1/2 and of the other sign, the former's products may be an infinity of the wrong sign, and a factor below
+    // 2^-134, whose parts are zero, makes NaN of the latter.  EXACT rounds infinities, and values next to them, to infinite parts, which
+    // meet zero parts of the other operand, and either may take finite products that overflow for ones of both signs.  All of that
+    // shows in the sums: four that hold an infinity or a NaN.  (EXACT also sums tiles that have seen a value next to overflow, whose products with
+    // subnormals it would lose.  A look at the sums costs 55 x 55, stride 2, 3x3x32x64 2 %, one at every operand of MIX 5 %.)
+    if (F32 && (overflow || !(fmaf(v.x, 0.f, fmaf(v.y, 0.f, fmaf(v.z, 0.f, v.w * 0.f))) == 0.f))) {
+        v = sum_as_it_stands<CONV>(sp, reinterpret_cast<const float *>(In), reinterpret_cast<const float *>(Flt), m, n);
     }
     int64_t off = (int64_t)m * p.o_w;
     if (!sp.uniform_rows) {

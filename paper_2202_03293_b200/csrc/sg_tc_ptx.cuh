@@ -380,8 +380,9 @@ __device__ __forceinline__ uint32_t pack_bf16_finite(float even, float odd) {
 // 3xTF32 split of eight f32 words.  hi = x rounded to tf32; x - hi is exact in f32 (also next to overflow, hi being finite) and lo is
 // that difference rounded to tf32 (add half an ulp, clear the low 13 bits), so x - hi - lo is below 2^-22 |x|.  The
 // low bits of hi and lo are zero, so whatever rounding the tensor core applies to its inputs
-// leaves them unchanged.  An infinity is hi = the largest tf32 value and lo = the infinity: its products are what they are in f32.  A
-// NaN, whatever its payload, is a NaN in hi.
+// leaves them unchanged.  An infinity is hi = the largest tf32 value and lo = the infinity.  Its products are what they are in f32 while the
+// low parts of the factors that infinities meet in one sum are below 1 together (the factors, 2^11): beyond that the largest
+// value's products with them may overflow to an infinity of the other sign.  A NaN, whatever its payload, is a NaN in hi.
 __device__ __forceinline__ void split8(const uint4 v0, const uint4 v1, uint4 &h0, uint4 &l0, uint4 &h1, uint4 &l1) {
     auto one = [](uint32_t x, uint32_t &hi, uint32_t &lo) {
         hi = round_tf32(x);
@@ -396,7 +397,7 @@ __device__ __forceinline__ void split8(const uint4 v0, const uint4 v1, uint4 &h0
 // is below 2^-11 of its product and bf16 keeps 8 bits of each factor, so the rounding moves a product by less than 2^-19 of
 // itself (what the dropped lo*lo term and the tensor core's f32 accumulation cost already), and the two bf16 products of a k-block are one
 // contraction over 64 values, [lo | hi] . [hi | lo], at twice the tf32 rate: two tensor-core units per term instead of three.
-// Infinities and NaNs: as above (the bf16 copy of hi is finite too).
+// Infinities and NaNs: as above (the bf16 copy of hi is finite too); a factor below 2^-134 is zero in both bf16 parts, NaN against an infinity.
 __device__ __forceinline__ void split_pair_mix(uint32_t x, uint32_t y, uint32_t &hx, uint32_t &hy, uint32_t &h16, uint32_t &l16) {
     hx = round_tf32(x);
     hy = round_tf32(y);

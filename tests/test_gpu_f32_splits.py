@@ -55,3 +55,54 @@ def test_special_values(M, N, K, a_t, b_t):
     finite = torch.isfinite(want)
     assert ((C.double() - want).abs()[finite] <= 4e-6 * bound[finite]).all()
     sg.sg_check()
+
+
+# An infinity is (largest, infinity) here: its products are infinities of the right sign while its factors are normal and stay below 2000 together
+@pytest.mark.parametrize("bn,cg", [(64, 1), (128, 1), (256, 2)])
+@pytest.mark.parametrize("a_t,b_t", [(False, False), (True, False), (False, True), (True, True)])
+@pytest.mark.parametrize("swap", [False, True])
+def test_infinities(bn, cg, a_t, b_t, swap):
+    M, N, K = 512, 512, 96
+    g = torch.Generator(device="cuda").manual_seed(SEED)
+    A = torch.rand(M, K, generator=g, device="cuda") * 2 - 1
+    B = torch.rand(K, N, generator=g, device="cuda") * 2 - 1
+    X, Y = (B.t(), A.t()) if swap else (A, B)
+    for i, f in enumerate([1999.25, -1999.25, 1025.5, -0.75, 2.0 ** -126, -(2.0 ** -126)]):
+        X[i, 40] = f
+    Y[40, 5], Y[40, 6] = float("inf"), float("-inf")
+    want = (A.double() @ B.double()).float()
+    a, b = A.t().contiguous().t() if a_t else A, B.t().contiguous().t() if b_t else B
+    C = torch.full((M, N), float("nan"), device="cuda")
+    sg.sg_set_tile_override(bn, cg, 1)
+    try:
+        sg.sg_matmul(a, b, C)
+        torch.cuda.synchronize()
+        assert sg.sg_last_kernel_name() == "tc_gemm_kernel<f32>"
+    finally:
+        sg.sg_set_tile_override(0, 0, 0)
+    infinite = torch.isinf(want)
+    assert int(infinite.sum()) == 2 * (N if swap else M) and torch.equal(C[infinite], want[infinite])
+    assert torch.isfinite(C[~infinite]).all()
+    sg.sg_check()
+
+
+@pytest.mark.parametrize("kernel", ["CONV_STRIP", "CONV_WIDE"])
+def test_infinities_of_convolutions(kernel):
+    I = torch.zeros(2, 40, 41, 16, device="cuda")
+    K = torch.full((1, 3, 16, 96), 0.5, device="cuda")
+    I[0, 5, 6, 3], I[1, 7, 8, 4], I[1, 20, 21, 2] = float("inf"), float("-inf"), 3.0
+    K[0, 1, 3], K[0, 1, 4] = -1999.25, 2.0 ** -126
+    O = torch.full((2, 40, 39, 96), float("nan"), device="cuda")
+    sg.sg_set_kernel_override(getattr(sg, "SG_KERNEL_" + kernel))
+    try:
+        sg.sg_conv2d_nhwc_hwcf(I, K, O)
+        torch.cuda.synchronize()
+        assert sg.sg_last_kernel_name() == f"{kernel.lower()}_kernel<f32>"
+    finally:
+        sg.sg_set_kernel_override(0)
+    want = torch.nn.functional.conv2d(I.double().permute(0, 3, 1, 2), K.double().permute(3, 2, 0, 1)).permute(0, 2, 3, 1).float()
+    infinite = torch.isinf(want)
+    assert int(infinite.sum()) == 2 * 3 * 96 and torch.equal(O[infinite], want[infinite])
+    assert torch.allclose(O[~infinite], want[~infinite], rtol=1e-6, atol=0)
+    sg.sg_check()
+

@@ -53,10 +53,11 @@ __device__ __forceinline__ void fma4(float4 &acc, const float4 a, const float4 b
 // calls of a few microseconds: one memory latency is the most they can afford (with each tap loaded where it is needed a
 // stride-2 layer of 4 x 7 x 7 x 16 took nine, 9.3 us; now 2.2).  S = 0: any window, every tap loaded where it is needed; the L1 serves
 // the repeats.  IDX: the type the work index is decoded in (32-bit whenever the work fits: 64-bit divisions
-// would cost more than the op).  One work item per thread.
+// would cost more than the op).  One work item per thread.  (The operands are no __restrict__ pointers: the kernel ahead may still
+// write them when this one starts, and a load that the compiler takes for one of constant data could go ahead of the wait.)
 template <typename T, int S, typename IDX>
 __global__ void __launch_bounds__(256)
-depthwise_vec_kernel(const DepthwiseProblem p, const T *__restrict__ I, const T *__restrict__ Kf, float *__restrict__ O) {
+depthwise_vec_kernel(const DepthwiseProblem p, const T *I, const T *Kf, float *O) {
     constexpr int TW = S == 2 ? TW_STRIDED : TW_UNIT;
     asm volatile("griddepcontrol.launch_dependents;");
     const IDX c4s = (IDX)(p.C / 4);
@@ -283,7 +284,7 @@ __device__ __forceinline__ f32x2 lds2(uint32_t addr, __nv_bfloat16) {
 // thread loads its filter values once.
 template <typename T, int CB, int K, int S>
 __global__ void __launch_bounds__(DT_THREADS, 2)
-depthwise_tma_kernel(const __grid_constant__ CUtensorMap map_in, const DepthwiseProblem p, const T *__restrict__ Kf, float *__restrict__ O, const DtTiling d) {
+depthwise_tma_kernel(const __grid_constant__ CUtensorMap map_in, const DepthwiseProblem p, const T *Kf, float *O, const DtTiling d) {
     using C = DtCfg<T, CB, K, S>;
     extern __shared__ uint8_t dt_smem[];
     __shared__ uint64_t full_bar[2], empty_bar[2];

@@ -1,8 +1,10 @@
 """Small 3 x 3 depthwise layers of stride 2 (and any stride and dilation down the rows) and channel blocks of 64 against the oracle: one to a
 few output columns per thread, channel counts around a thread's four."""
 import pytest
+import torch
 
-from helpers import assert_within_bound
+from helpers import assert_within_bound, operand
+from oracle import ref
 from paper_2202_03293_b200 import binding as sg
 from test_gpu_depthwise import run2d
 
@@ -15,6 +17,7 @@ pytestmark = pytest.mark.gpu
                                               (4, 4, 9, 64, (3, 2), (1, 1)), (2, 6, 5, 16, (1, 1), (1, 1)), (1, 13, 31, 100, (2, 2), (1, 1))])
 def test_small_layers(N, Ho, Wo, C, st, dl, accumulate, dtype):
     O, want, S = run2d(N, Ho, Wo, C, 3, 3, st, dl, dtype, accumulate, extra=(1, 1))
+    assert sg.sg_last_kernel_name() == "depthwise_vec_kernel"
     assert_within_bound(O, want, S, "depthwise, small")
     sg.sg_check()
 
@@ -23,6 +26,39 @@ def test_small_layers(N, Ho, Wo, C, st, dl, accumulate, dtype):
 @pytest.mark.parametrize("C", [72, 96, 104, 136, 160, 200, 416])
 @pytest.mark.parametrize("s,K", [(1, 3), (2, 3), (2, 5)])
 def test_channel_blocks(C, s, K):
-    O, want, S = run2d(6, 21, 27, C, K, K, (s, s), (1, 1), "bf16")
+    O, want, S = run2d(30 if s == 1 else 9, 21, 27, C, K, K, (s, s), (1, 1), "bf16")       # (a tile per SM, or the kernel without tiles runs)
+    assert sg.sg_last_kernel_name() == "depthwise_tma_kernel"
     assert_within_bound(O, want, S, "depthwise, channel blocks")
+    sg.sg_check()
+
+
+# The kernel overlaps the launch ahead: its operands are the last thing that a long copy ahead writes, and a copy behind overwrites them, round after round.
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("N,W,C,s,K,kernel", [(2, 9, 24, 1, 3, "vec"), (1, 14, 200, 2, 3, "vec"), (3, 11, 36, 2, 2, "vec"), (16, 24, 64, 1, 5, "tma")])
+def test_operands_of_the_launch_ahead(N, W, C, s, K, kernel, dtype):
+    win = (W - 1) * s + K
+    n_in, n_flt, cols, rounds = N * win * win * C, K * K * C, 4096, 6
+    rows = 4096 + (n_in + n_flt + cols - 1) // cols
+    start = rows * cols - n_in - n_flt
+    buf = torch.empty(rows, cols, device="cuda", dtype=torch.float32 if dtype == "f32" else torch.bfloat16)
+    I, F = buf.view(-1)[start:start + n_in].view(N, win, win, C), buf.view(-1)[start + n_in:].view(K, K, C)
+    junk = torch.full_like(buf, 7.0)
+    sources, outs, wants = [], [], []
+    for r in range(rounds):
+        a, i = operand((N, win, win, C), 9860, 2 * r, "normal", dtype)
+        b, k = operand((K, K, C), 9860, 2 * r + 1, "normal", dtype)
+        src = torch.zeros_like(buf)
+        src.view(-1)[start:start + n_in], src.view(-1)[start + n_in:] = a.flatten(), b.flatten()
+        sources.append(src)
+        outs.append(torch.full((N, W, W, C), float("nan"), device="cuda"))
+        wants.append(ref.depthwise_conv2d_nhwc_hwc(i, k, (s, s), (1, 1), out_hw=(W, W)))
+    torch.cuda.synchronize()
+    for src, O in zip(sources, outs):
+        sg.sg_copy2d(src, buf)
+        sg.sg_depthwise_conv2d_nhwc_hwc(I, F, O, (s, s), (1, 1))
+        assert sg.sg_last_kernel_name() == f"depthwise_{kernel}_kernel"
+        sg.sg_copy2d(junk, buf)
+    torch.cuda.synchronize()
+    for O, (want, S) in zip(outs, wants):
+        assert_within_bound(O, want, S, "depthwise behind a copy")
     sg.sg_check()

@@ -721,11 +721,35 @@ bool raw_map(CUtensorMap *map, const void *ptr, Operand &op, int mn, int k, int 
                                CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
 }
 
+// Tiles, their width, and the CTAs (of one cluster) that share a tile's reduction: 2, 4 or 8 where tiles are few, at least four k-blocks each.
+struct Tiles { int bn, num_kb, splits; int64_t tiles; };
+Tiles plan_tiles(const Problem &p, int num_sms) {
+    Tiles t{p.N > 64 ? 128 : 64, (p.K + BK - 1) / BK, 1, 0};
+    t.tiles = (int64_t)((p.M + BM - 1) / BM) * ((p.N + t.bn - 1) / t.bn);
+    while (t.splits < MAX_SPLIT && t.tiles * t.splits * 2 <= num_sms - 12 && t.num_kb >= t.splits * 8) t.splits *= 2;
+    return t;
+}
+
+// Below 2^21 multiply-adds the CUDA-core kernel is as fast.
+bool too_small(const Problem &p) { return (int64_t)p.M * p.N * p.K < ((int64_t)1 << 21); }
+
 }  // namespace
 
+// A start and an end, rounds of tiles and their k-blocks, and what sharing a reduction costs.  Fitted to graph replays of 500 calls whose lines
+// are whole 16-byte pieces (those that the kernel for small problems could take): within 4 to 9 %.
+double gather_estimate_us(const Problem &p, int num_sms) {
+    if (too_small(p)) return 1e9;
+    struct Cost { double ends, kb, round, shared; };
+    constexpr Cost bf16[2][2] = {{{4.7, 0.75, 0.0, 1.0}, {6.0, 0.79, 3.0, 2.3}}, {{4.9, 1.21, 0.3, 2.1}, {6.2, 1.31, 0.0, 4.9}}};      // [convolution][128 columns]
+    constexpr Cost f32[2][2] = {{{4.7, 1.27, 0.0, 1.2}, {5.4, 1.87, 2.9, 3.8}}, {{6.0, 1.51, 2.9, 2.9}, {6.8, 2.21, 6.5, 6.9}}};
+    const Tiles t = plan_tiles(p, num_sms);
+    const Cost &c = (p.in_bf16 ? bf16 : f32)[p.spatial_rank != 0][t.bn == 128];
+    const double rounds = t.splits > 1 ? 1.0 : (double)((t.tiles + num_sms - 1) / num_sms);
+    return c.ends + (rounds - 1.0) * c.round + rounds * c.kb * (double)((t.num_kb + t.splits - 1) / t.splits) + (t.splits > 1 ? c.shared : 0.0);
+}
+
 sg_status launch_gather(const Problem &p, const void *In, const void *Flt, float *O, bool forced, cudaStream_t stream) {
-    // Below 2^21 multiply-adds the CUDA-core kernel is as fast.
-    if (!forced && (int64_t)p.M * p.N * p.K < ((int64_t)1 << 21)) return SG_ERR_UNSUPPORTED;
+    if (!forced && too_small(p)) return SG_ERR_UNSUPPORTED;
     const bool conv = p.spatial_rank != 0;
     // offsets are 32-bit
     if (reach({{p.batch, p.i_n}, {(int64_t)(p.Ho - 1) * p.sh + (int64_t)(p.KH - 1) * p.dh + 1, p.i_h},
@@ -753,19 +777,18 @@ sg_status launch_gather(const Problem &p, const void *In, const void *Flt, float
     gp.b.pair = on(Flt, 2 * es) && (gp.b.mn_major ? p.k_f == 1 && even(p.k_c) && even(p.N) && (!conv || (even(p.k_kw) && even(p.k_kh)))
                                                   : even(p.k_f) && even(p.K));
     gp.uniform_rows = (p.Ho == 1 || p.o_h == (int64_t)p.Wo * p.o_w) && (p.batch == 1 || p.o_n == (int64_t)p.Ho * p.Wo * p.o_w);
-    gp.num_kb = (p.K + BK - 1) / BK;
     gp.wait_prior = pdl == 0 ? 0 : 1;
 
-    const int bn = p.N > 64 ? 128 : 64;
+    const Tiles plan = plan_tiles(p, num_sms);
+    const int bn = plan.bn;
+    const int64_t tiles = plan.tiles;
+    gp.num_kb = plan.num_kb;
     gp.num_n_tiles = (p.N + bn - 1) / bn;
-    const int64_t tiles = (int64_t)((p.M + BM - 1) / BM) * gp.num_n_tiles;
     if (tiles > 0x7fffffff / MAX_SPLIT) return SG_ERR_UNSUPPORTED;
     // (a tile summed as it stands must end well within the waits of the next one's MMAs, 2e9 cycles)
     if (!p.in_bf16 && tiles > num_sms && p.K > 131072) return SG_ERR_UNSUPPORTED;
     gp.num_tiles = (int)tiles;
-    // few tiles: a cluster of 2, 4 or 8 CTAs shares a tile's reduction, at least four k-blocks each
-    gp.splits = 1;
-    while (gp.splits < MAX_SPLIT && tiles * gp.splits * 2 <= num_sms - 12 && gp.num_kb >= gp.splits * 8) gp.splits *= 2;
+    gp.splits = plan.splits;
     alignas(64) CUtensorMap ma = {}, mb = {};
     const bool raw = p.in_bf16 && !conv && raw_map(&ma, In, gp.a, p.M, p.K, BM) && raw_map(&mb, Flt, gp.b, p.N, p.K, bn);
     // Partial sums of bf16 products: the largest with which the error against f64 is about the CUDA-core kernel's or below it.  Relative

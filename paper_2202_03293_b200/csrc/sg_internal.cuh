@@ -77,6 +77,7 @@ void tensor_note_choice(int bn, int cg, int splits);      // what sg_last_tile_c
 // Tensor-core implicit GEMM for layouts outside the TMA rules (sg_gather.cu): any strides.  SG_ERR_UNSUPPORTED (nothing is
 // launched) when offsets do not fit 32 bits or, unless `forced`, the problem is too small to gain.
 sg_status launch_gather(const Problem &p, const void *In, const void *Flt, float *O, bool forced, cudaStream_t stream);
+double gather_estimate_us(const Problem &p, int num_sms);      // what it would take (1e9 where it leaves the problem to the CUDA cores)
 sg_status gather_read_status(cudaStream_t stream);
 void tensor_set_tile_override(int bn, int cg, int splits);
 void tensor_last_choice(int out[3]);

@@ -474,23 +474,34 @@ sg_status launch_small(const Problem &p, const void *In, const void *Flt, float 
     const bool mix = f32 && !a_mn && !b_km && tensor_takes(p, In, Flt, O);
     if (f32 && !conv && !a_mn && !b_km && !mix) return SG_ERR_UNSUPPORTED;
     if (mode < 0) {
-        // By time (us): a launch, then waves of thread blocks over the SMs (two share an SM's tensor cores), each a start and its steps of
-        // 128 k.  The other side is the tcgen05 kernel's cost model; convolutions of inputs
-        // below 128 KiB have no im2col path to compare with.  Fitted to graph replays of 124 calls with either kernel (products of 64 to
-        // 4096 in every layout, convolutions): within 13 % of the timings, choices 0.9 % off the better of the two in the mean (0.6 % with
-        // the tcgen05 kernel's launches as they are outside a graph).
+        // By time (us): a launch; where 16-row tiles do, what they take the more of the more of them there are to an SM, and steps of 128 k;
+        // else waves of 32-row tiles over the SMs, each a start and its steps.  Fitted to graph replays of 730 calls of every layout and
+        // op: within 10 % of the timings, 7 % for MIX.
         const double steps = std::max(0.5, (double)p.K / BK), waves = (double)((tiles + num_sms - 1) / num_sms);
-        const double step = !f32 ? (waves > 1 ? 0.282 : 0.49) : (waves > 1 ? 0.82 : half && tiles * 2 > num_sms ? 1.29 : 0.80) * (mix ? 1.0 : 1.11);
-        const double us = 1.2 + waves * ((f32 ? 0.70 : 0.74) + step * steps);
-        // (the tcgen05 kernel never takes less than 2.8 us, f32 3.6: no need to ask.  Issued one by one its launches take
-        // 0.3 to 0.6 us more than in a graph, these do not: 1066 x 256 x 320 f32 6.4 us here, 6.9 there in a graph and 6.7 against 7.5 one by
-        // one.  What it does not take (inputs stored transposed whose rows are no whole 128 bytes of m,
-        // outputs that are not one matrix) the gather kernel would run, in three times its estimate: 1616 x 168 x 599 bf16
-        // 8.8 us here, 17.1 there, 4.6 estimated.  Unit-stride convolutions of bf16 go to conv_wide_kernel, which is faster than that estimate,
-        // but not below 4.5 us: 2220 x 96, 3x80, 3.5 us here, 4.6 there.)
-        const bool run_conv = conv && !f32 && p.sh == 1 && p.sw == 1;
-        const double lead = !tensor_takes(p, In, Flt, O) ? 3.0 : f32 ? 1.055 : run_conv ? 0.8 : 1.08;
-        if (us > (f32 ? 3.6 : run_conv ? 4.0 : 2.8) && us > (conv && in_bytes < 131072 ? 0.3 * p.K : lead * tensor_estimate_us(p))) return SG_ERR_UNSUPPORTED;
+        const double fill = std::min(2.0, (double)((p.M + 15) / 16) * sp.num_n_tiles / num_sms);      // 16-row tiles per SM
+        struct Cost { double start, fill, step, step_fill, wave, wave_step; };
+        constexpr Cost costs[3] = {{1.35, 0.69, 0.38, 0.28, 0.65, 0.33}, {1.56, 0.44, 0.95, 0.42, 0.79, 0.98}, {1.45, 0.54, 0.73, 0.37, 0.66, 0.76}};
+        const Cost &c = costs[!f32 ? BF16 : mix ? MIX : EXACT];
+        const double us = half ? c.start + c.fill * fill + steps * (c.step + c.step_fill * std::max(0.0, fill - 0.5))
+                               : c.start + waves * (c.wave + c.wave_step * steps);
+        // The other side is what would run the call instead.  That never takes less than 2.8 us, f32 3.6 (into outputs that are not one
+        // matrix 4.2), unit-stride convolutions of bf16 4.0: no need to ask.  Where it is the tcgen05 kernel, or a convolution whose filter
+        // stays or streams past the runs of input rows, the former's cost model says what it takes; those convolutions are the faster ones in bf16.  What
+        // none of them takes (inputs stored transposed whose rows are no whole 128 bytes of m, strided convolutions into outputs that are not one matrix)
+        // the gather kernel would run, by its own model.  Of 744 calls timed both ways the choices cost 0.5 % over the better of the two
+        // in the mean; three times the tcgen05 kernel's estimate, in the gather kernel's place and where a filter
+        // stays, cost 4.8 % (27 x 24 x 24, 1x1x48x64 f32 into a padded output 5.9 us as strips, 11.7 here; 1 x 77 x 77, 3x3x64x128 bf16
+        // 4.9 and 13.5; 1048 x 32 x 3352 f32 transposed 14.2 gathered, 33.1 here).
+        const bool takes = tensor_takes(p, In, Flt, O), unit = conv && p.sh == 1 && p.sw == 1, run_conv = unit && !f32;
+        if (us > (f32 ? takes ? 3.6 : 4.2 : run_conv ? 4.0 : 2.8)) {
+            const double short_input = conv && in_bytes < 131072 ? 0.3 * p.K : 0.0;      // (inputs below 128 KiB, which no model covers)
+            if (takes || (unit && launch_conv_strip(p, In, Flt, O, true, stream) == SG_OK)) {
+                const double lead = run_conv ? 0.8 : !f32 ? 1.15 : mix ? 1.0 : 1.1;
+                if (us > (short_input > 0.0 ? short_input : lead * tensor_estimate_us(p))) return SG_ERR_UNSUPPORTED;
+            } else if (us > std::max(short_input, 0.95 * gather_estimate_us(p, num_sms))) {
+                return SG_ERR_UNSUPPORTED;
+            }
+        }
     }
     tensor_note_choice(TN, 1, 1);
 #define SG_SMALL(MODE_, A_MN_, B_KM_, CONV_, SLOT)                                                                  \

@@ -1,5 +1,5 @@
-"""Unit-stride convolutions on both sides of the rule between strips and im2col, by the automatic choice and by the strip kernel,
-against the oracle: one, three and five taps, channels that im2col pads and that it does not."""
+"""Unit-stride convolutions on both sides of the rules between strips, im2col, the filter as the M operand and the kernel for small problems, against
+the oracle: one, three and five taps, channels that im2col pads and that it does not, outputs that are one matrix and padded ones."""
 import pytest
 import torch
 
@@ -14,20 +14,47 @@ SEED = 9850
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])
 @pytest.mark.parametrize("C", [32, 40, 64])
 @pytest.mark.parametrize("KW,dl", [(1, 1), (3, 2), (5, 1)])
-def test_strip_or_im2col(C, KW, dl, dtype):
+@pytest.mark.parametrize("pad", [0, 1])
+def test_strip_or_im2col(C, KW, dl, pad, dtype):
     N, W, F = 37, 900, 32
     I, i = operand((N, W + (KW - 1) * dl, C), SEED, 1, "normal", dtype)
     K, k = operand((KW, C, F), SEED, 2, "normal", dtype)
     want, S = ref.conv1d_nwc_wcf(i, k, dilation=dl)
-    strip = dtype == "bf16" or KW * C <= 192      # (a split filter beyond that does not stay in shared memory beside a strip)
-    for kernel in (0, sg.SG_KERNEL_CONV_STRIP) if strip else (0,):
-        O = torch.full((N, W, F), float("nan"), device="cuda")
+    fits = dtype == "bf16" or KW * C <= 192      # (a split filter beyond that does not stay in shared memory beside a strip)
+    strips = pad == 1 or (dtype == "bf16" and KW >= (3 if C % 64 else 5))
+    chosen = "conv_strip_kernel" if strips and fits else "gather_gemm_kernel" if pad else "tc_gemm_kernel"
+    for kernel in (0, sg.SG_KERNEL_CONV_STRIP) if fits else (0,):
+        wide = torch.full((N, W + 2 * pad, F), float("nan"), device="cuda")
+        O = wide[:, pad:pad + W]
         sg.sg_set_kernel_override(kernel)
         try:
             sg.sg_conv1d_nwc_wcf(I, K, O, 1, dl)
             torch.cuda.synchronize()
         finally:
             sg.sg_set_kernel_override(0)
-        assert sg.sg_last_kernel_name() not in ("ffma_kernel", "")
+        assert sg.sg_last_kernel_name() == f"{'conv_strip_kernel' if kernel else chosen}<{dtype}>"
         assert_within_bound(O, want, S, "strip or im2col")
+        assert int(torch.isnan(wide).sum()) == 2 * pad * N * F
     sg.sg_check()
+
+
+# Convolutions into padded outputs, which the im2col kernel does not take.  Where a filter stays or streams past the runs of input rows, the kernel for small problems
+# has that kernel to beat; elsewhere (strides) the gather kernel.
+@pytest.mark.parametrize("N,W,C,F,KW,s,dtype,kernel", [
+    (1, 77, 64, 128, 3, 1, "bf16", "conv_wide_kernel"), (4, 32, 64, 128, 3, 1, "bf16", "conv_wide_kernel"), (27, 24, 48, 64, 1, 1, "f32", "conv_strip_kernel"),
+    (3, 10, 16, 96, 3, 1, "bf16", "small_gemm_kernel"), (14, 9, 40, 64, 1, 1, "f32", "small_gemm_kernel"), (6, 10, 64, 96, 3, 2, "f32", "small_gemm_kernel"),
+    (16, 31, 16, 64, 3, 2, "f32", "gather_gemm_kernel"), (24, 40, 64, 96, 3, 2, "bf16", "gather_gemm_kernel")])
+def test_padded_outputs(N, W, C, F, KW, s, dtype, kernel):
+    win = (W - 1) * s + KW
+    I, i = operand((N, win, win, C), SEED, 3, "normal", dtype)
+    K, k = operand((KW, KW, C, F), SEED, 4, "normal", dtype)
+    wide = torch.full((N, W + 2, W + 2, F), float("nan"), device="cuda")
+    O = wide[:, 1:-1, 1:-1]
+    sg.sg_conv2d_nhwc_hwcf(I, K, O, (s, s))
+    torch.cuda.synchronize()
+    assert sg.sg_last_kernel_name() == f"{kernel}<{dtype}>"
+    want, S = ref.conv2d_nhwc_hwcf(i, k, (s, s))
+    assert_within_bound(O, want, S, "padded output")
+    assert int(torch.isnan(wide).sum()) == wide.numel() - O.numel()
+    sg.sg_check()
+

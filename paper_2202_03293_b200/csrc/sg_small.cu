@@ -9,7 +9,9 @@
 // memory, in a fixed order.  Graph replay, us, tcgen05 kernel -> this one: 128^3 f32 6.0 -> 2.1, bf16 3.6 -> 1.7;
 // 256^3 f32 6.6 -> 3.4; a 55 x 55 stride-2 3x3x32x64 convolution f32 9.2 -> 7.1.
 //
-// bf16 inputs: mma.sync m16n8k16.  f32 inputs, in one of two forms that keep f32 accuracy:
+// bf16 inputs: mma.sync m16n8k16, a warp's share of k in one accumulator up to K = 2048 (256 products), beyond that (BF16_LONG) in chunks of 256
+// added up with rounding: the gather kernel, which would run some of these calls, holds no more in one either (relative error at K = 4096, positive
+// values, 7.1e-7 in one accumulator, 3.1e-7 there; the registers of the second sum cost short reductions a block per SM).  f32 inputs, in one of two forms that keep f32 accuracy:
 //   MIX    the split of the tcgen05 kernel: hi = x rounded to tf32, lo = x - hi; hi*hi in tf32, lo*hi + hi*lo in bf16
 //   EXACT  x = b0 + b1 + b2 with three bf16 parts of eight bits each (exact differences), six of the nine products
 // The tensor core adds by truncation, so the four or six MMAs of 16 k have a sum of their own, which is added, rounding to nearest, to
@@ -25,8 +27,10 @@ namespace {
 
 constexpr int TN = 32, BK = 128;
 constexpr int WARPS = BK / 16, THREADS = 32 * WARPS;
+constexpr int CHUNK = 16;      // BF16_LONG: stages of which a warp's accumulators, 256 products each, are added to a rounded sum
 
-enum { BF16 = 0, EXACT = 1, MIX = 2 };
+enum { BF16 = 0, EXACT = 1, MIX = 2, BF16_LONG = 3 };
+template <int MODE> constexpr bool kF32 = MODE == EXACT || MODE == MIX;
 
 // TM: rows of a tile, 16 or 32.
 template <bool F32, bool A_MN, bool B_KM, int TM>
@@ -133,7 +137,7 @@ __device__ __noinline__ float4 sum_as_it_stands(const SmallParams &sp, const flo
 template <int MODE, bool A_MN, bool B_KM, bool CONV, int TM>
 __global__ void __launch_bounds__(THREADS, 2)
 small_gemm_kernel(const __grid_constant__ SmallParams sp, const char *__restrict__ In, const char *__restrict__ Flt, float *__restrict__ O) {
-    constexpr bool F32 = MODE != BF16;
+    constexpr bool F32 = kF32<MODE>;
     using C = Cfg<F32, A_MN, B_KM, TM>;
     const Problem &p = sp.p;
     extern __shared__ __align__(16) uint8_t smem[];
@@ -227,6 +231,7 @@ small_gemm_kernel(const __grid_constant__ SmallParams sp, const char *__restrict
         for (int j = 0; j < 4; ++j)
 #pragma unroll
             for (int e = 0; e < 4; ++e) acc[i][j][e] = 0.f;
+    float done[MODE == BF16_LONG ? MI : 1][4][4] = {};      // BF16_LONG: of the finished chunks
     float largest = 0.f;       // EXACT: of the magnitudes seen
     for (int kb = 0; kb < sp.num_kb; ++kb) {
         asm volatile("cp.async.wait_group %0;" ::"n"(C::STAGES - 2) : "memory");
@@ -354,9 +359,26 @@ small_gemm_kernel(const __grid_constant__ SmallParams sp, const char *__restrict
                     const uint32_t bj[2] = {b[j >> 1][(j & 1) * 2], b[j >> 1][(j & 1) * 2 + 1]};
                     mma16816(acc[i][j], a[i], bj);
                 }
+            if constexpr (MODE == BF16_LONG)
+                if (kb % CHUNK == CHUNK - 1) {
+#pragma unroll
+                    for (int i = 0; i < MI; ++i)
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) { done[i][j][e] += acc[i][j][e]; acc[i][j][e] = 0.f; }
+                }
         }
     }
 
+    if constexpr (MODE == BF16_LONG) {
+#pragma unroll
+        for (int i = 0; i < MI; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) acc[i][j][e] += done[i][j][e];
+    }
     // ---- the warps' shares of k meet in shared memory; a thread writes four columns of one row
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     const bool overflow = MODE == EXACT ? __syncthreads_or(largest >= 1.7014118e38f) != 0 : false;
@@ -412,7 +434,7 @@ inline bool mult(int64_t v, int64_t q) { return v % q == 0; }
 
 template <int MODE, bool A_MN, bool B_KM, bool CONV, int TM>
 sg_status launch_variant(SmallParams &sp, const void *In, const void *Flt, float *O, int slot, cudaStream_t stream) {
-    using C = Cfg<MODE != BF16, A_MN, B_KM, TM>;
+    using C = Cfg<kF32<MODE>, A_MN, B_KM, TM>;
     constexpr auto kernel = small_gemm_kernel<MODE, A_MN, B_KM, CONV, TM>;
     const int smem = std::max(std::min(C::STAGES, sp.num_kb) * C::STAGE_BYTES, C::RED_BYTES);
     if (!tensor_ensure_smem_attr(slot + (TM == 16 ? 0 : 1), reinterpret_cast<const void *>(kernel), C::STAGES * C::STAGE_BYTES)) return SG_ERR_CUDA;
@@ -428,7 +450,7 @@ sg_status launch_variant(SmallParams &sp, const void *In, const void *Flt, float
     cfg.numAttrs = sp.wait_prior ? 1 : 0;
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, sp, static_cast<const char *>(In), static_cast<const char *>(Flt), O);
     count_launch();
-    note_kernel(MODE != BF16 ? "small_gemm_kernel<f32>" : "small_gemm_kernel<bf16>");
+    note_kernel(kF32<MODE> ? "small_gemm_kernel<f32>" : "small_gemm_kernel<bf16>");
     return e == cudaSuccess ? SG_OK : SG_ERR_CUDA;
 }
 
@@ -507,12 +529,16 @@ sg_status launch_small(const Problem &p, const void *In, const void *Flt, float 
 #define SG_SMALL(MODE_, A_MN_, B_KM_, CONV_, SLOT)                                                                  \
     (half ? launch_variant<MODE_, A_MN_, B_KM_, CONV_, 16>(sp, In, Flt, O, SLOT, stream)                            \
           : launch_variant<MODE_, A_MN_, B_KM_, CONV_, 32>(sp, In, Flt, O, SLOT, stream))
-    if (conv) return !f32 ? SG_SMALL(BF16, false, false, true, 160) : mix ? SG_SMALL(MIX, false, false, true, 162) : SG_SMALL(EXACT, false, false, true, 164);
+    const bool chunks = sp.num_kb > CHUNK;
+#define SG_SMALL_BF16(A_MN_, B_KM_, CONV_, SLOT, SLOT_LONG)                                                         \
+    (chunks ? SG_SMALL(BF16_LONG, A_MN_, B_KM_, CONV_, SLOT_LONG) : SG_SMALL(BF16, A_MN_, B_KM_, CONV_, SLOT))
+    if (conv) return !f32 ? SG_SMALL_BF16(false, false, true, 160, 212) : mix ? SG_SMALL(MIX, false, false, true, 162) : SG_SMALL(EXACT, false, false, true, 164);
     if (mix) return SG_SMALL(MIX, false, false, false, 166);
-    if (a_mn && b_km) return f32 ? SG_SMALL(EXACT, true, true, false, 168) : SG_SMALL(BF16, true, true, false, 170);
-    if (a_mn) return f32 ? SG_SMALL(EXACT, true, false, false, 172) : SG_SMALL(BF16, true, false, false, 174);
-    if (b_km) return f32 ? SG_SMALL(EXACT, false, true, false, 176) : SG_SMALL(BF16, false, true, false, 178);
-    return SG_SMALL(BF16, false, false, false, 180);
+    if (a_mn && b_km) return f32 ? SG_SMALL(EXACT, true, true, false, 168) : SG_SMALL_BF16(true, true, false, 170, 214);
+    if (a_mn) return f32 ? SG_SMALL(EXACT, true, false, false, 172) : SG_SMALL_BF16(true, false, false, 174, 216);
+    if (b_km) return f32 ? SG_SMALL(EXACT, false, true, false, 176) : SG_SMALL_BF16(false, true, false, 178, 218);
+    return SG_SMALL_BF16(false, false, false, 180, 220);
+#undef SG_SMALL_BF16
 #undef SG_SMALL
 }
 

@@ -2,10 +2,10 @@
 //
 // The channel iterator is parallel, only the window is reduced: KH*KW multiply-adds per output
 // element against at least one element read and one written, so the op is bound by HBM
-// bandwidth and runs on the CUDA cores.  The fast kernel gives each thread four consecutive
-// channels (one 16-byte access; consecutive threads take consecutive channel groups, so a warp
-// reads and writes whole lines) of TW consecutive output columns; for the 3 x 3 window with unit
-// stride and dilation along w the input columns the TW windows share are loaded once into
+// bandwidth and runs on the CUDA cores.  The kernel for small layers gives each thread four consecutive
+// channels (one access of 8 or 16 bytes; consecutive threads take consecutive channel groups, so a warp
+// reads and writes whole lines) of a few consecutive output columns; for the 3 x 3 window with stride 1 or 2 and
+// unit dilation along w the input columns that their windows share are loaded once into
 // registers, otherwise every tap is loaded where it is needed and the L1 serves the repeats.
 // 3 x 3 and 5 x 5 windows take a TMA-staged tile kernel (layouts that meet the TMA rules); large 3 x 3 /
 // unit-stride problems in other layouts a kernel that walks down the rows with a rolling register window.  Any other layout (channel
@@ -48,14 +48,16 @@ __device__ __forceinline__ void fma4(float4 &acc, const float4 a, const float4 b
 }
 
 // Four channels of a few output columns per thread.  S = 1, 2: a 3 x 3 window of stride S and unit dilation along w, known at compile
-// time: the columns that neighbouring windows of a filter row share are loaded once, and all of a thread's input and filter
-// loads (S = 1: 18 + 9 for four columns, S = 2: 15 + 9 for two) are issued before the first of them is needed.  These are
+// time: the columns that neighbouring windows of a filter row share are loaded once, and all of a thread's input loads (S = 1: 18
+// for four columns, S = 2: 15 for two) are issued before the first of them is needed; so are the 9 filter loads of S = 2.  These are
 // calls of a few microseconds: one memory latency is the most they can afford (with each tap loaded where it is needed a
-// stride-2 layer of 4 x 7 x 7 x 16 took nine, 9.3 us; now 2.2).  S = 0: any window, every tap loaded where it is needed; the L1 serves
+// stride-2 layer of 4 x 7 x 7 x 16 took nine, 9.3 us; now 1.8).  S = 1 loads its filter where it is used, the L1 serves it: with all 27
+// loads ahead (AHEAD) f32 is short of registers (3 x 50 x 50 x 36 3.41 us, without 2.48).  Columns wait as they lie in memory and are widened once a row
+// (bf16 widened for every use: 4 x 14 x 14 x 200 2.46 us, now 2.31).  S = 0: any window, every tap loaded where it is needed; the L1 serves
 // the repeats.  IDX: the type the work index is decoded in (32-bit whenever the work fits: 64-bit divisions
 // would cost more than the op).  One work item per thread.  (The operands are no __restrict__ pointers: the kernel ahead may still
 // write them when this one starts, and a load that the compiler takes for one of constant data could go ahead of the wait.)
-template <typename T, int S, typename IDX>
+template <typename T, int S, typename IDX, bool AHEAD = false>
 __global__ void __launch_bounds__(256)
 depthwise_vec_kernel(const DepthwiseProblem p, const T *I, const T *Kf, float *O) {
     constexpr int TW = S == 2 ? TW_STRIDED : TW_UNIT;
@@ -76,7 +78,35 @@ depthwise_vec_kernel(const DepthwiseProblem p, const T *I, const T *Kf, float *O
         const T *in_n = I + (int64_t)n * p.i_n + c;
         // the operands may be the output of the kernel ahead of this one, and the output its input
         asm volatile("griddepcontrol.wait;" ::: "memory");
-        if constexpr (S != 0) {
+        if constexpr (S == 1) {
+            Raw4<T> col[3][TW + 2], flt[3][3];
+            auto load_filter = [&](int kh, int kw) { return load_raw4(Kf + (int64_t)kh * p.k_kh + (int64_t)kw * p.k_kw + c); };
+#pragma unroll
+            for (int kh = 0; kh < 3; ++kh) {
+                const T *row = in_n + (int64_t)(h * p.sh + kh * p.dh) * p.i_h + (int64_t)w0 * p.i_w;
+#pragma unroll
+                for (int j = 0; j < TW + 2; ++j)
+                    if (w0 + j < p.Wo + 2) col[kh][j] = load_raw4(row + (int64_t)j * p.i_w);
+            }
+            if constexpr (AHEAD)
+#pragma unroll
+                for (int kh = 0; kh < 3; ++kh)
+#pragma unroll
+                    for (int kw = 0; kw < 3; ++kw) flt[kh][kw] = load_filter(kh, kw);
+#pragma unroll
+            for (int kh = 0; kh < 3; ++kh) {
+                float4 wide[TW + 2];
+#pragma unroll
+                for (int j = 0; j < TW + 2; ++j) wide[j] = widen4(col[kh][j]);
+#pragma unroll
+                for (int kw = 0; kw < 3; ++kw) {
+                    const float4 f = widen4(AHEAD ? flt[kh][kw] : load_filter(kh, kw));
+#pragma unroll
+                    for (int t = 0; t < TW; ++t)
+                        if (w0 + t < p.Wo) fma4(acc[t], wide[t + kw], f);
+                }
+            }
+        } else if constexpr (S == 2) {
             constexpr int COLS = (TW - 1) * S + 3;
             Raw4<T> col[3][COLS], flt[3][3];
 #pragma unroll
@@ -508,12 +538,13 @@ cudaError_t launch_typed(const DepthwiseProblem &p, const T *I, const T *Kf, flo
     const bool small = work < ((int64_t)1 << 32) - 256;
     const bool unit3 = p.sw == 1 && p.dw == 1 && p.KW == 3 && p.KH == 3;
     const bool win3 = p.KW == 3 && p.KH == 3 && p.dw == 1 && p.dh == 1, win5 = p.KW == 5 && p.KH == 5 && p.dw == 1 && p.dh == 1;
+    int num_sms = 0;
+    const bool ready = tensor_driver_ready(&num_sms);
     if (vec && (win3 || win5) && p.sh == p.sw && p.sh <= 2 && reinterpret_cast<uintptr_t>(I) % 16 == 0 &&
         (p.C * (int64_t)sizeof(T)) % 16 == 0) {
         // TMA-staged tiles (TMA checks the channel bound in 16-byte units, hence the condition on C)
-        int num_sms = 0;
         cudaError_t err = cudaSuccess;
-        if (p.C >= 16 && tensor_driver_ready(&num_sms) &&
+        if (p.C >= 16 && ready &&
             (win3 ? try_launch_window<T, 3>(p, I, Kf, O, num_sms, stream, &err) : try_launch_window<T, 5>(p, I, Kf, O, num_sms, stream, &err))) return err;
     }
     if (vec && unit3 && p.sh == 1 && p.dh == 1) {
@@ -526,7 +557,7 @@ cudaError_t launch_typed(const DepthwiseProblem &p, const T *I, const T *Kf, flo
             return cudaGetLastError();
         }
     }
-    // (the vector kernel may start while the kernel ahead of it drains: its threads wait for that kernel before their first load)
+    // The vector kernel may start while the kernel ahead of it drains: its threads wait for that kernel before their first load.
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(blocks, 1, 1);
     cfg.blockDim = dim3(256, 1, 1);
@@ -536,12 +567,26 @@ cudaError_t launch_typed(const DepthwiseProblem &p, const T *I, const T *Kf, flo
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = vec ? 1 : 0;
-    auto launch = [&](auto narrow, auto wide) { return small ? cudaLaunchKernelEx(&cfg, narrow, p, I, Kf, O) : cudaLaunchKernelEx(&cfg, wide, p, I, Kf, O); };
+    // Behind a kernel that leaves some SMs free its blocks would all be dealt out to those, two, three and four to one, and take that much longer: shared memory
+    // that nobody uses keeps an SM to its even share of them.  bf16, us, without overlap / with it / with that: 1 x 59 x 59 x 144, 125 blocks,
+    // 2.8 / 3.5 / 2.3; 2 x 31 x 31 x 476, 231, 3.5 / 4.0 / 3.0; at stride 2 4 x 14 x 14 x 416, 160, - / 3.2 / 2.4.
+    const int64_t share = num_sms > 0 ? (blocks64 + num_sms - 1) / num_sms : 4;
+    auto launch = [&](int slot, auto narrow, auto wide) {
+        if (!small) return cudaLaunchKernelEx(&cfg, wide, p, I, Kf, O);
+        if (slot != 0 && share <= 3 && tensor_ensure_smem_attr(slot, reinterpret_cast<const void *>(narrow), 115 * 1024))
+            cfg.dynamicSmemBytes = (share == 1 ? 115 : share == 2 ? 77 : 58) * 1024;
+        return cudaLaunchKernelEx(&cfg, narrow, p, I, Kf, O);
+    };
     cudaError_t err;
-    if (vec && unit3) err = launch(depthwise_vec_kernel<T, 1, uint32_t>, depthwise_vec_kernel<T, 1, uint64_t>);
-    else if (vec && strided3) err = launch(depthwise_vec_kernel<T, 2, uint32_t>, depthwise_vec_kernel<T, 2, uint64_t>);
-    else if (vec) err = launch(depthwise_vec_kernel<T, 0, uint32_t>, depthwise_vec_kernel<T, 0, uint64_t>);
-    else err = launch(depthwise_generic_kernel<T, uint32_t>, depthwise_generic_kernel<T, uint64_t>);
+    // (f32 filters ahead of the multiplications where that matters more than the registers: a lone block, 2 x 6 x 6 x 4, 1.5 us against 1.6, and more blocks than
+    // SMs, 7 x 24 x 24 x 184, 182, 3.2 and 3.9; but 3 x 50 x 50 x 36, 69, 3.4 and 2.5)
+    const bool ahead = sizeof(T) == 4 && (blocks64 == 1 || blocks64 > num_sms);
+    constexpr int slots = sizeof(T) == 2 ? 222 : 224;
+    if (vec && unit3 && ahead) err = launch(0, depthwise_vec_kernel<T, 1, uint32_t, sizeof(T) == 4>, depthwise_vec_kernel<T, 1, uint64_t, sizeof(T) == 4>);
+    else if (vec && unit3) err = launch(slots, depthwise_vec_kernel<T, 1, uint32_t>, depthwise_vec_kernel<T, 1, uint64_t>);
+    else if (vec && strided3) err = launch(slots + 1, depthwise_vec_kernel<T, 2, uint32_t>, depthwise_vec_kernel<T, 2, uint64_t>);
+    else if (vec) err = launch(0, depthwise_vec_kernel<T, 0, uint32_t>, depthwise_vec_kernel<T, 0, uint64_t>);
+    else err = launch(0, depthwise_generic_kernel<T, uint32_t>, depthwise_generic_kernel<T, uint64_t>);
     count_launch();
     note_kernel(vec ? "depthwise_vec_kernel" : "depthwise_generic_kernel");
     return err;

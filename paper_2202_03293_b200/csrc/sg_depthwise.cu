@@ -13,6 +13,7 @@
 // pitches) takes a one-output-per-thread kernel with full stride arithmetic.
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -445,13 +446,11 @@ depthwise_generic_kernel(const DepthwiseProblem p, const T *__restrict__ I, cons
     }
 }
 
+// Groups of a tile: the fewest rounds of thread blocks, weighed with what a tile fetches (a round costs at least what its 256 threads
+// compute, about 16 KB worth).  Returns that cost.
 template <typename T, int CB, int K, int S>
-bool try_launch_tma(const DepthwiseProblem &p, const T *I, const T *Kf, float *O, int num_sms, cudaStream_t stream, cudaError_t *err) {
+double plan_tma(const DepthwiseProblem &p, int num_sms, DtTiling &d) {
     using C = DtCfg<T, CB, K, S>;
-    const int64_t es = sizeof(T);
-    // ---- groups of a tile: the fewest rounds of thread blocks, weighed with what a tile fetches (a round costs at least what
-    // its 256 threads compute, about 16 KB worth)
-    DtTiling d{};
     double best = 1e300;
     for (int cg = C::GROUPS; cg >= 1; cg >>= 1)       // (wide first: longer runs of memory)
         for (int stack = 0; stack < 2; ++stack) {
@@ -471,6 +470,12 @@ bool try_launch_tma(const DepthwiseProblem &p, const T *I, const T *Kf, float *O
                 d = DtTiling{cg, rg, stack, in_w, in_h, bytes, (bytes + 127) / 128 * 128, (int)tw, (int)th, (int)tn, (int)cbs, (int)tiles};
             }
         }
+    return best;
+}
+
+template <typename T, int CB, int K, int S>
+bool try_launch_tma(const DepthwiseProblem &p, const DtTiling &d, const T *I, const T *Kf, float *O, int num_sms, cudaStream_t stream, cudaError_t *err) {
+    const int64_t es = sizeof(T);
     if (d.num_tiles == 0 || d.c_blocks > num_sms) return false;
     // 3 x 3 problems too small for a tile per SM are left to the kernel without tiles (2.9 us a launch against 3.5)
     if (K == 3 && d.num_tiles < num_sms) return false;
@@ -507,17 +512,31 @@ bool try_launch_tma(const DepthwiseProblem &p, const T *I, const T *Kf, float *O
     return true;
 }
 
-template <typename T, int K>
-bool try_launch_window(const DepthwiseProblem &p, const T *I, const T *Kf, float *O, int num_sms, cudaStream_t stream, cudaError_t *err) {
+template <typename T, int K, int S>
+bool try_launch_window(const DepthwiseProblem &p, const T *I, const T *Kf, float *O, int num_sms, int64_t vec_blocks, cudaStream_t stream, cudaError_t *err) {
     // Blocks of 64 channels; 32 where (bf16) those cover the channels with a fifth less padding, and for 5 x 5 f32 tiles, which would
     // not fit twice.  (Groups of 16 lanes keep two columns open instead of four, and a pixel's 64 bytes of bf16 cost a tensor load what
     // 128 do: 56 x 43 x 43 x 200 at stride 2 69.8 us with 32, 47.2 with 64; 31 x 89 x 89 x 416 149.4 and 139.7; but 26 x 31 x 31 x 32 4.3 and 5.7.)
     if constexpr (sizeof(T) == 2 || K == 3) {
         const int pad64 = (p.C + 63) / 64 * 64, pad32 = (p.C + 31) / 32 * 32;
-        if (sizeof(T) == 4 ? pad64 == pad32 || p.C > 64 : 4 * (int64_t)pad64 <= 5 * (int64_t)pad32)
-            return p.sh == 1 ? try_launch_tma<T, 64, K, 1>(p, I, Kf, O, num_sms, stream, err) : try_launch_tma<T, 64, K, 2>(p, I, Kf, O, num_sms, stream, err);
+        bool wide = sizeof(T) == 4 ? pad64 == pad32 || p.C > 64 : 4 * (int64_t)pad64 <= 5 * (int64_t)pad32;
+        DtTiling d64{};
+        const double cost = wide ? plan_tma<T, 64, K, S>(p, num_sms, d64) : 0.0;
+        if (sizeof(T) == 2 && wide && pad64 != pad32) {
+            // The last block is half empty, and tiles twice as large fill whole rounds less well: 32 where that costs a fifth more.  us, 32
+            // and 64: 8 x 28 x 28 x 288 4.6 and 5.2 (cost 1.56), 24 x 14 x 14 x 224 at stride 2 4.6 and 5.6 (1.42), 5 x 5 windows 8 x 28 x 28 x 152
+            // 5.5 and 7.3 (1.53), 32 x 28 x 28 x 160 8.1 and 8.9 (1.23); but 32 x 28 x 28 x 288 14.8 and 13.5 (1.17), 5 x 5 24 x 14 x 14 x 416 10.4 and 9.7 (1.13).
+            // 3 x 3 layers with less than a tile of 64 per SM belong to the kernel without tiles as long as that has no more than about 7/3 blocks per SM
+            // (307, 8 x 28 x 28 x 200, 4.1 and 4.8 with tiles of 32; 347, 24 x 14 x 14 x 264, 4.2 and 4.0; at stride 2 160, 4 x 14 x 14 x 416, 2.4 and 2.8).
+            DtTiling d32{};
+            if (K == 3 && d64.num_tiles < num_sms) wide = 3 * vec_blocks <= 7 * (int64_t)num_sms;
+            else wide = cost <= 1.2 * plan_tma<T, 32, K, S>(p, num_sms, d32);
+        }
+        if (wide) return try_launch_tma<T, 64, K, S>(p, d64, I, Kf, O, num_sms, stream, err);
     }
-    return p.sh == 1 ? try_launch_tma<T, 32, K, 1>(p, I, Kf, O, num_sms, stream, err) : try_launch_tma<T, 32, K, 2>(p, I, Kf, O, num_sms, stream, err);
+    DtTiling d{};
+    plan_tma<T, 32, K, S>(p, num_sms, d);
+    return try_launch_tma<T, 32, K, S>(p, d, I, Kf, O, num_sms, stream, err);
 }
 
 inline bool mult4(int64_t v) { return v % 4 == 0; }
@@ -544,8 +563,13 @@ cudaError_t launch_typed(const DepthwiseProblem &p, const T *I, const T *Kf, flo
         (p.C * (int64_t)sizeof(T)) % 16 == 0) {
         // TMA-staged tiles (TMA checks the channel bound in 16-byte units, hence the condition on C)
         cudaError_t err = cudaSuccess;
+        auto tiles = [&](auto window, auto stride) {
+            return try_launch_window<T, decltype(window)::value, decltype(stride)::value>(p, I, Kf, O, num_sms, blocks64, stream, &err);
+        };
+        using std::integral_constant;
         if (p.C >= 16 && ready &&
-            (win3 ? try_launch_window<T, 3>(p, I, Kf, O, num_sms, stream, &err) : try_launch_window<T, 5>(p, I, Kf, O, num_sms, stream, &err))) return err;
+            (win3 ? p.sh == 1 ? tiles(integral_constant<int, 3>{}, integral_constant<int, 1>{}) : tiles(integral_constant<int, 3>{}, integral_constant<int, 2>{})
+                  : p.sh == 1 ? tiles(integral_constant<int, 5>{}, integral_constant<int, 1>{}) : tiles(integral_constant<int, 5>{}, integral_constant<int, 2>{}))) return err;
     }
     if (vec && unit3 && p.sh == 1 && p.dh == 1) {
         // enough row segments to give every SM several thread blocks: walk down the rows with a rolling window

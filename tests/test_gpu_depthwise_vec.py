@@ -32,6 +32,27 @@ def test_channel_blocks(C, s, K):
     sg.sg_check()
 
 
+# bf16: numbers of thread blocks around one and two to an SM (shared memory keeps an SM to its share of them), tiles in their place from 7/3 on, and
+# where tiles of 64 channels fill the rounds badly
+@pytest.mark.parametrize("N,W,C,s,kernel", [(4, 14, 400, 1, "vec"), (4, 14, 408, 1, "vec"), (23, 14, 152, 1, "vec"), (24, 14, 152, 1, "vec"), (8, 28, 224, 1, "vec"),
+                                            (24, 14, 264, 1, "tma"), (4, 14, 352, 2, "vec"), (4, 14, 416, 2, "vec"), (8, 28, 288, 1, "tma"), (24, 14, 224, 2, "tma")])
+def test_lines(N, W, C, s, kernel):
+    O, want, S = run2d(N, W, W, C, 3, 3, (s, s), (1, 1), "bf16")
+    assert sg.sg_last_kernel_name() == f"depthwise_{kernel}_kernel"
+    assert_within_bound(O, want, S, "depthwise, lines")
+    sg.sg_check()
+
+
+# f32: a lone block, a block more, one to an SM and one more (filters ahead of the multiplications on the outer sides)
+@pytest.mark.parametrize("N,W,C", [(1, 7, 64), (2, 7, 64), (1, 30, 320), (1, 30, 628), (1, 30, 632), (7, 24, 184)])
+@pytest.mark.parametrize("accumulate", [False, True])
+def test_filters_ahead(N, W, C, accumulate):
+    O, want, S = run2d(N, W, W, C, 3, 3, (1, 1), (1, 1), "f32", accumulate)
+    assert sg.sg_last_kernel_name() == "depthwise_vec_kernel"
+    assert_within_bound(O, want, S, "depthwise, filters ahead")
+    sg.sg_check()
+
+
 # The kernel overlaps the launch ahead: its operands are the last thing that a long copy ahead writes, and a copy behind overwrites them, round after round.
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("N,W,C,s,K,kernel", [(2, 9, 24, 1, 3, "vec"), (1, 14, 200, 2, 3, "vec"), (3, 11, 36, 2, 2, "vec"), (16, 24, 64, 1, 5, "tma")])

@@ -588,7 +588,8 @@ void plan_bf16(const Problem &p, int64_t positions, int f_tiles, int row_span, i
 // A block is paced by the slowest of its MMAs (N / 2 cycles each), what it fetches (19.4 bytes a cycle with all SMs fetching the
 // same filter) and its converters (685 cycles a step with four groups, 9.1 a row of a run); one accumulator instead of two
 // leaves the write-back in the open.  (Constants fitted to 400 timings of 17 shapes and 32 to 256 positions, within 8 %; the choices
-// are the best of each sweep but for two, 5 and 12 % off.)
+// are the best of each sweep but for two, 5 and 12 % off.  The converters have become faster since, which filters that stream feel: 170 timings of the
+// tiles chosen are within 10 % of the estimate where the filter stays, and of 0.86 of it where it streams.)
 double plan_f32(const Problem &p, int64_t positions, int f_tiles, int row_span, int64_t full_span, int num_sms, WideParams &w, F32Filter &g) {
     const int kb = (p.C + 31) / 32;
     g.taps = p.KH * p.KW;
@@ -638,7 +639,7 @@ double plan_f32(const Problem &p, int64_t positions, int f_tiles, int row_span, 
             g.stages = stages; g.run_rows = (int)rows; g.tiles = flt_tiles; g.groups = groups;
         }
     }
-    return best * (1.0 / 1900.0);
+    return best * (1.0 / 1900.0) * (w.resident ? 1.0 : 0.86);
 }
 
 }  // namespace
@@ -683,8 +684,8 @@ sg_status launch_conv_wide(const Problem &p, const void *In, const void *Flt, fl
     F32Filter g{};
     if (f32) {
         // The im2col kernel deals a reduction out over the SMs: where there are few positions and much to sum it is the better one
-        // (8 x 28 x 28, 3x3x256x256: 43.9 us here, 38.5 there; 16 x 56 x 56, 3x3x64x128: 32.3 against 41.6; both estimates are within
-        // a tenth or so).  Filters of 65 to 128 columns and three
+        // (8 x 28 x 28, 3x3x256x256: 43.9 us here, 38.5 there; 16 x 56 x 56, 3x3x64x128: 32.3 against 41.6; 5 x 80 x 80, 3x3x16x128: 10.3 and 13.3; both
+        // estimates are within a tenth or so).  Filters of 65 to 128 columns and three
         // taps or more that the strip kernel would keep resident run faster here whatever the estimates say (43 x 2934,
         // 3x32x128: 18.9 against 22.2; but one tap, 54 x 54, 1x1x48x96: 6.1 against 5.2).
         const double us = plan_f32(p, positions, f_tiles, row_span, full_span, num_sms, w, g);

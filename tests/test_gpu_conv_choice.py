@@ -58,3 +58,17 @@ def test_padded_outputs(N, W, C, F, KW, s, dtype, kernel):
     assert int(torch.isnan(wide).sum()) == wide.numel() - O.numel()
     sg.sg_check()
 
+
+# f32, im2col or the filter as the M operand: a long reduction over few positions, filters that stream past many, filters that stay
+@pytest.mark.parametrize("N,W,C,F,KW,kernel", [(8, 28, 256, 256, 3, "tc_gemm_kernel"), (10, 57, 16, 128, 3, "conv_wide_kernel"), (5, 80, 16, 128, 3, "conv_wide_kernel"),
+                                               (18, 47, 16, 64, 3, "tc_gemm_kernel")])
+def test_wide_or_im2col(N, W, C, F, KW, kernel):
+    I, i = operand((N, W + KW - 1, W + KW - 1, C), SEED, 5, "normal", "f32")
+    K, k = operand((KW, KW, C, F), SEED, 6, "normal", "f32")
+    O = torch.full((N, W, W, F), float("nan"), device="cuda")
+    sg.sg_conv2d_nhwc_hwcf(I, K, O)
+    torch.cuda.synchronize()
+    assert sg.sg_last_kernel_name() == f"{kernel}<f32>"
+    want, S = ref.conv2d_nhwc_hwcf(i, k)
+    assert assert_within_bound(O, want, S, "wide or im2col") < 4e-6
+    sg.sg_check()

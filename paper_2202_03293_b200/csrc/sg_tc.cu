@@ -1207,15 +1207,18 @@ constexpr Variant kVariants[] = {{64, 1, 125.0, 336.0, 385.0}, {128, 1, 150.0, 4
                                  {128, 2, 140.0, 374.0, 1500.0}, {256, 2, 358.0, 627.0, 903.0}};
 constexpr int kNumVariants = sizeof(kVariants) / sizeof(kVariants[0]);
 
+inline double kb_own_ns(const Variant &v, bool f32, bool plain) { return !f32 ? v.mma_ns : plain ? v.mma_ns_f32 : v.mma_ns_f32_t; }
+
 // A stream-K tail (launch_tensor) pays when the k-blocks saved clearly outweigh the extra epilogues and the clearing launch.
-// Returns the k-blocks of a group's run, 0: no tail.
-int stream_k_run(const Variant &v, bool f32, int64_t tiles, int groups, int num_kb, int kps, bool whenever) {
+// Returns the k-blocks of a group's run, 0: no tail.  (`plain` as in estimate_ns: k-blocks of transposed operands at the plain layout's price
+// forwent tails that pay, f32 A.B^T 7936 x 1536 x 2528 219 us with one, 245 without, A^T.B 1984 x 7552 x 1536 179 and 213.)
+int stream_k_run(const Variant &v, bool f32, bool plain, int64_t tiles, int groups, int num_kb, int kps, bool whenever) {
     const int left = (int)(tiles % groups);
     if (tiles <= groups || left == 0 || num_kb % kps != 0) return 0;
     const int64_t units = (int64_t)left * num_kb;
     int run = (int)((units + groups - 1) / groups);
     run = (run + kps - 1) / kps * kps;
-    const double saved = (double)(num_kb - run) * (f32 ? v.mma_ns_f32 : v.mma_ns);
+    const double saved = (double)(num_kb - run) * kb_own_ns(v, f32, plain);
     const double extra = 2.0 * (1500.0 + (double)v.bn * (f32 ? 24.0 : 12.0)) + 2500.0;
     return run >= 4 * kps && (saved > (f32 ? 1.4 : 2.0) * extra || whenever) ? run : 0;
 }
@@ -1234,7 +1237,7 @@ double estimate_ns(const Variant &v, bool f32, bool plain, int64_t tiles, int64_
     const double active = (double)((items < groups ? items : groups) * v.cg);
     const double stage_bytes = A_STAGE_BYTES + (double)(v.bn / v.cg) * ROW_BYTES;
     const double chip_fill = f32 ? 11100.0 : 17100.0, sm_fill = f32 ? 77.3 : 127.0;      // bytes per ns
-    double kb_ns = !f32 ? v.mma_ns : plain ? v.mma_ns_f32 : v.mma_ns_f32_t;
+    double kb_ns = kb_own_ns(v, f32, plain);
     if (!f32 && !plain && kb_ns < 218.0) kb_ns = 218.0;
     if (active * stage_bytes / chip_fill > kb_ns) kb_ns = active * stage_bytes / chip_fill;
     if (stage_bytes / sm_fill > kb_ns) kb_ns = stage_bytes / sm_fill;
@@ -1245,7 +1248,7 @@ double estimate_ns(const Variant &v, bool f32, bool plain, int64_t tiles, int64_
     double wave_ns = kbs * kb_ns + open * item_ns;
     if (active * BM * v.bn * 4 / 6000.0 > wave_ns) wave_ns = active * BM * v.bn * 4 / 6000.0;
     double t = (double)kbs * kb_ns + item_ns + (double)(waves - 1) * wave_ns;
-    const int run = f32 && sp == 1 && tail ? stream_k_run(v, f32, tiles, (int)groups, num_kb, 1, false) : 0;
+    const int run = f32 && sp == 1 && tail ? stream_k_run(v, f32, plain, tiles, (int)groups, num_kb, 1, false) : 0;
     if (run > 0) t += item_ns + 1500.0 - (double)(num_kb - run) * kb_ns;               // the last wave is shorter, the write-backs are more
     if (v.cg == 2) t += 490.0;                                                         // cluster launch, cross-CTA signalling
     if (sp > 1) t += f32 ? 2880.0 : 2610.0;                                            // reduce-add traffic, the clearing launch
@@ -1594,7 +1597,7 @@ sg_status launch_tensor(const Problem &p, const void *In, const void *Flt, float
         const int64_t tiles = (int64_t)num_m_tiles * num_n_tiles;
         const int left = (int)(tiles % groups);
         if (ov.sk != 0 && splits == 1) {
-            const int run = stream_k_run(var, f32, tiles, groups, tp.num_kb, kps, ov.sk == 2);
+            const int run = stream_k_run(var, f32, lay == 0, tiles, groups, tp.num_kb, kps, ov.sk == 2);
             if (run > 0) {
                 tp.sk_first_tile = (int)(tiles - left);
                 tp.sk_units = run;

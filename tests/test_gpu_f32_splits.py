@@ -106,3 +106,19 @@ def test_infinities_of_convolutions(kernel):
     assert torch.allclose(O[~infinite], want[~infinite], rtol=1e-6, atol=0)
     sg.sg_check()
 
+
+# transposed operands whose last wave is partly filled: their own k-blocks' price decides on the stream-K tail
+@pytest.mark.parametrize("M,N,K,a_t,b_t,accumulate", [(1792, 1664, 1472, False, True, False), (1856, 1792, 2048, True, False, False), (1952, 1184, 1248, True, True, True)])
+def test_tail_of_transposed_operands(M, N, K, a_t, b_t, accumulate):
+    g = torch.Generator(device="cuda").manual_seed(SEED)
+    A = torch.rand((K, M) if a_t else (M, K), generator=g, device="cuda") * 2 - 1
+    B = torch.rand((N, K) if b_t else (K, N), generator=g, device="cuda") * 2 - 1
+    A, B = A.t() if a_t else A, B.t() if b_t else B
+    C = torch.full((M, N), 1.0 if accumulate else float("nan"), device="cuda")
+    sg.sg_matmul(A, B, C, sg.SG_ACCUMULATE if accumulate else sg.SG_OVERWRITE)
+    torch.cuda.synchronize()
+    assert sg.sg_last_stream_k()[1] > 0, "these shapes were meant to take the stream-K tail"
+    start = 1.0 if accumulate else 0.0
+    err = (C.double() - start - A.double() @ B.double()).abs()
+    assert (err <= 4e-6 * (A.double().abs() @ B.double().abs() + start)).all()
+    sg.sg_check()

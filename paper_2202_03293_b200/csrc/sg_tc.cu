@@ -23,7 +23,7 @@
 //                          an MN-major operand instead of being transposed.
 //
 // f32 inputs run on the same pipeline with every element split as x = hi + lo, hi = x rounded to tf32: the TMA
-// writes the raw f32 tiles into its ring, sixteen converter warps split them and write a second ring of two slots
+// writes the raw f32 tiles into its ring, sixteen converter warps split them and write a second ring of two or four slots
 // (transposing the filter tile to K-major on the way, which kind::tf32 needs; the split input tile goes to tensor
 // memory), and the MMA thread accumulates lo*hi + hi*lo + hi*hi in f32: the dropped term is below 2^-21 |a*b|, so
 // f32 accuracy is kept.  In the plain layout hi*hi runs in tf32 and the two corrections as one bf16 contraction over
@@ -94,13 +94,11 @@ struct Cfg {
     static constexpr int B_COLS = BN / CG;                    // filter columns staged by this CTA
     static constexpr int B_STAGE_BYTES = B_COLS * ROW_BYTES;  // = BK * B_COLS * ELT
     // KPS k-blocks travel together in one stage: [input tile of each k-block | filter tile: sub-tiles of
-    // KPS*BK k-rows], fetched by ONE load per operand (a TMA instruction costs the same whatever its size)
+    // KPS*BK k-rows], fetched by ONE load per operand
     static constexpr int STAGE_BYTES = KPS * (A_STAGE_BYTES + B_STAGE_BYTES);   // written by TMA per stage
     // bf16: one ring of stages, TMA -> MMA.  f32: the TMA ring holds raw tiles; a second ring of
-    // two slots holds what the converter warps make of them, [input hi | input lo | filter hi |
+    // a slot per converter group holds what the converter warps make of them, [input hi | input lo | filter hi |
     // filter lo], the filter transposed to K-major on the way (kind::tf32 takes no N-major operand).
-    // (two slots are enough: with three the kernel is no faster - a k-block is bound by shared-memory bandwidth: the raw tiles
-    // written by TMA and read by the converters, the split filter written, and the MMAs' filter reads)
     // The converter warps work in groups that take the k-blocks in turn, each with a slot of its own: a k-block is a chain of about 900
     // cycles of latencies (two barriers, loads, stores, fences) plus its share of the instructions, longer than its
     // MMAs.  Where a CTA stages 64 filter columns there is room for four slots, and four groups of four warps have twice as many
@@ -114,10 +112,10 @@ struct Cfg {
     static constexpr int RING_BUDGET = 196608 - SPLIT_SLOTS * SPLIT_BYTES;
     static constexpr int MOST_STAGES = (RING_BUDGET / STAGE_BYTES) > 8 ? 8 : (RING_BUDGET / STAGE_BYTES);
     static constexpr int STAGES = F32 ? MOST_STAGES / GROUPS * GROUPS : MOST_STAGES;
-    // warps: input producer, MMA, 4 epilogue (, 8 converter), filter producer
+    // warps: input producer, MMA, 4 epilogue (, 16 converter), filter producer
     static constexpr int THREADS = 192 + (F32 ? CONVERTER_THREADS : 0) + 32;
     static constexpr int FLT_WARP = THREADS / 32 - 1;
-    // two accumulator buffers (one when the split input's 2 slots x 64 columns would not fit beside two)
+    // two accumulator buffers (one when the split input's slots of 64 columns would not fit beside two)
     static constexpr int A_TMEM_COLS = TA ? SPLIT_SLOTS * 64 : 0;
     static constexpr int ACC_BUFS = 2 * BN + A_TMEM_COLS > 512 ? 1 : 2;
     static constexpr int USED_COLS = ACC_BUFS * BN + A_TMEM_COLS;
@@ -519,7 +517,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant
             // MIX: this thread's fixed share of a k-block.  Input: row (warp & 3) * 32 + lane (the TMEM lane quarter this warp
             // may touch), k columns 16 * (cw >> 2) ..: four 16-byte chunks of the swizzled raw row.  Filter: units cw and cw + 8
             // (sub-tile of 32 columns, quarter of its 32 k): lane = column f reads 8 k down its column and owns chunks of row f.
-            constexpr int UNITS = C::B_COLS / 64;                         // 4 * B_COLS / 32 units on 8 warps (64 columns: one each)
+            constexpr int UNITS = C::B_COLS / 64;                         // 4 * B_COLS / 32 units on 8 warps
             uint32_t mx_a_off[4] = {0, 0, 0, 0}, mx_hi_off[2] = {0, 0}, mx_b_src = 0, mx_h16_off = 0, mx_l16_off = 0, mx_tmem = 0;
             if constexpr (MIX && C::GROUPS == 2) {
                 const int row = (warp & 3) * 32 + lane;

@@ -29,7 +29,7 @@ constexpr int TN = 32, BK = 128;
 constexpr int WARPS = BK / 16, THREADS = 32 * WARPS;
 constexpr int CHUNK = 16;      // BF16_LONG: stages of which a warp's accumulators, 256 products each, are added to a rounded sum
 
-enum { BF16 = 0, EXACT = 1, MIX = 2, BF16_LONG = 3 };
+enum { BF16 = 0, EXACT = 1, MIX = 2, BF16_LONG = 3, BF16_THREE = 4 };
 template <int MODE> constexpr bool kF32 = MODE == EXACT || MODE == MIX;
 
 // TM: rows of a tile, 16 or 32.
@@ -134,8 +134,9 @@ __device__ __noinline__ float4 sum_as_it_stands(const SmallParams &sp, const flo
     return make_float4(s[0], s[1], s[2], s[3]);
 }
 
+// BF16_THREE: BF16 in the 80 registers that three thread blocks on an SM have.
 template <int MODE, bool A_MN, bool B_KM, bool CONV, int TM>
-__global__ void __launch_bounds__(THREADS, 2)
+__global__ void __launch_bounds__(THREADS, MODE == BF16_THREE ? 3 : 2)
 small_gemm_kernel(const __grid_constant__ SmallParams sp, const char *__restrict__ In, const char *__restrict__ Flt, float *__restrict__ O) {
     constexpr bool F32 = kF32<MODE>;
     using C = Cfg<F32, A_MN, B_KM, TM>;
@@ -529,9 +530,14 @@ sg_status launch_small(const Problem &p, const void *In, const void *Flt, float 
 #define SG_SMALL(MODE_, A_MN_, B_KM_, CONV_, SLOT)                                                                  \
     (half ? launch_variant<MODE_, A_MN_, B_KM_, CONV_, 16>(sp, In, Flt, O, SLOT, stream)                            \
           : launch_variant<MODE_, A_MN_, B_KM_, CONV_, 32>(sp, In, Flt, O, SLOT, stream))
-    const bool chunks = sp.num_kb > CHUNK;
+    // bf16: three thread blocks to an SM where shared memory has room for them (three stages) and there are more than two to each (368 tiles, 2 x 727, 3x32x256,
+    // 4.3 us with two and 3.6 with three); with fewer, blocks behind an overlapped launch would be dealt out three to one (232 tiles, K = 288, 4.1 and 5.2), and
+    // longer reductions are the slower for the fewer registers (930 tiles, K = 1280, 28.3 and 29.3)
+    const bool chunks = sp.num_kb > CHUNK, three = sp.num_kb <= 3 && tiles > 2 * (int64_t)num_sms;
 #define SG_SMALL_BF16(A_MN_, B_KM_, CONV_, SLOT, SLOT_LONG)                                                         \
-    (chunks ? SG_SMALL(BF16_LONG, A_MN_, B_KM_, CONV_, SLOT_LONG) : SG_SMALL(BF16, A_MN_, B_KM_, CONV_, SLOT))
+    (chunks  ? SG_SMALL(BF16_LONG, A_MN_, B_KM_, CONV_, SLOT_LONG)                                                  \
+     : three ? launch_variant<BF16_THREE, A_MN_, B_KM_, CONV_, 32>(sp, In, Flt, O, SLOT_LONG + 13, stream)          \
+             : SG_SMALL(BF16, A_MN_, B_KM_, CONV_, SLOT))
     if (conv) return !f32 ? SG_SMALL_BF16(false, false, true, 160, 212) : mix ? SG_SMALL(MIX, false, false, true, 162) : SG_SMALL(EXACT, false, false, true, 164);
     if (mix) return SG_SMALL(MIX, false, false, false, 166);
     if (a_mn && b_km) return f32 ? SG_SMALL(EXACT, true, true, false, 168) : SG_SMALL_BF16(true, true, false, 170, 214);

@@ -1005,7 +1005,7 @@ typedef CUresult (*EncodeIm2colFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_
 // g_mu guards the driver entry points, the per-device records and the overrides; it is held for a few loads and stores,
 // never across a tensor-map encode or a launch.  The tensor-map cache has a lock of its own.
 constexpr int kMaxDevices = 64;
-constexpr int kAttrSlots = 226;
+constexpr int kAttrSlots = 236;
 struct DeviceState {
     bool ready = false;
     int num_sms = 0;

@@ -518,6 +518,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant
             // may touch), k columns 16 * (cw >> 2) ..: four 16-byte chunks of the swizzled raw row.  Filter: units cw and cw + 8
             // (sub-tile of 32 columns, quarter of its 32 k): lane = column f reads 8 k down its column and owns chunks of row f.
             constexpr int UNITS = C::B_COLS / 64;                         // 4 * B_COLS / 32 units on 8 warps
+            const uint32_t never = (uint32_t)p.splits >> 16;              // 0, which the compiler cannot know
             uint32_t mx_a_off[4] = {0, 0, 0, 0}, mx_hi_off[2] = {0, 0}, mx_b_src = 0, mx_h16_off = 0, mx_l16_off = 0, mx_tmem = 0;
             if constexpr (MIX && C::GROUPS == 2) {
                 const int row = (warp & 3) * 32 + lane;
@@ -554,7 +555,9 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant
                         // A warp has all 32 k of the 32 rows of its TMEM lane quarter (two halves of 16 k, lane = row), and of either
                         // sub-tile of 32 filter columns a quarter of the k (lane = column).  The raw stage is handed back once
                         // everything has been read, half-way through the splits: there is one stage per group, and its refill takes
-                        // as long as the rest of the chain.
+                        // as long as the rest of the chain.  Read means that the values are in registers: a load that is only issued
+                        // may be served after the refill (10560 x 1792 x 512 came out with eight rows of one k-block wrong about once in a
+                        // hundred calls), so the barrier's address depends on a word of every load that nothing has used by then.
                         const int quarter = warp & 3, row = quarter * 32 + lane;
                         auto load_a = [&](int half, uint4 (&a)[4]) {
                             if constexpr (A_MN) {      // four [32 k][32 rows] sub-tiles: 16 values down a column
@@ -632,8 +635,13 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant
                         split_a(0, a);
                         load_a(1, a);
                         split_b(0, x0);
+                        uint32_t loaded = a[0].x | a[1].x | a[2].x | a[3].x | x1[0].x | x1[1].x;
+                        if constexpr (A_MN)
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) loaded |= a[i].y | a[i].z | a[i].w;
+                        if constexpr (!B_KM) loaded |= x1[0].y | x1[0].z | x1[0].w | x1[1].y | x1[1].z | x1[1].w;
                         __syncwarp();
-                        if (lane == 0) mbar_arrive(empty_bar(r));      // the raw stage may be refilled
+                        if (lane == 0) mbar_arrive(empty_bar(r) + (loaded & never));      // the raw stage may be refilled
                         split_a(1, a);
                         split_b(1, x1);
                     } else if constexpr (MIX) {

@@ -1,0 +1,37 @@
+"""f32 products whose converter warps hand a raw stage back while they still split it: the tile loads behind it must not reach
+the values of this k-block.  A sum's order is fixed where a tile has one work item, so every call gives the same bits."""
+import pytest
+import torch
+
+from paper_2202_03293_b200 import binding as sg
+
+pytestmark = pytest.mark.gpu
+
+
+# both tiles of 64 filter columns to a CTA, several tiles to a CTA or pair, every layout of the operands that is built for them
+@pytest.mark.parametrize("bn,cg,a_t,b_t", [(128, 2, False, False), (64, 1, False, False), (64, 1, True, False), (64, 1, False, True), (64, 1, True, True)])
+@pytest.mark.parametrize("M,N,K", [(10560, 1792, 512), (4736, 1280, 1056)])
+def test_same_bits_every_time(M, N, K, bn, cg, a_t, b_t):
+    g = torch.Generator(device="cuda").manual_seed(M)
+    A = torch.rand(M, K, generator=g, device="cuda") * 2 - 1
+    B = torch.rand(K, N, generator=g, device="cuda") * 2 - 1
+    want = A.double() @ B.double()
+    bound = A.double().abs() @ B.double().abs()
+    a, b = A.t().contiguous().t() if a_t else A, B.t().contiguous().t() if b_t else B
+    sg.sg_set_tile_override(bn, cg, 1)
+    try:
+        first = torch.zeros(M, N, device="cuda")
+        sg.sg_matmul(a, b, first)
+        # one k-block of a row's four values amiss is 1e-2 of the bound
+        assert ((first.double() - want).abs() <= 4e-6 * bound).all()
+        if sg.sg_last_stream_k()[0] >= 0:
+            pytest.skip("a stream-K tail adds partial sums in any order")
+        C = torch.zeros(M, N, device="cuda")
+        wrong = torch.zeros((), dtype=torch.int64, device="cuda")
+        for _ in range(200):
+            sg.sg_matmul(a, b, C)
+            wrong += (C != first).any()
+        assert wrong.item() == 0
+    finally:
+        sg.sg_set_tile_override(0, 0, 0)
+    sg.sg_check()

@@ -1215,18 +1215,22 @@ constexpr int kNumVariants = sizeof(kVariants) / sizeof(kVariants[0]);
 
 inline double kb_own_ns(const Variant &v, bool f32, bool plain) { return !f32 ? v.mma_ns : plain ? v.mma_ns_f32 : v.mma_ns_f32_t; }
 
-// A stream-K tail (launch_tensor) pays when the k-blocks saved clearly outweigh the extra epilogues and the clearing launch.
-// Returns the k-blocks of a group's run, 0: no tail.  (`plain` as in estimate_ns: k-blocks of transposed operands at the plain layout's price
-// forwent tails that pay, f32 A.B^T 7936 x 1536 x 2528 219 us with one, 245 without, A^T.B 1984 x 7552 x 1536 179 and 213.)
-int stream_k_run(const Variant &v, bool f32, bool plain, int64_t tiles, int groups, int num_kb, int kps, bool whenever) {
+// What a stream-K tail (launch_tensor) costs in ns: the write-backs of its runs, which are open, and the launch that clears its tiles (which an
+// accumulating call does not need).  Measured with and without a tail on 170 calls (products in every layout, tiles of 64 to 256 columns): f32
+// 3.7 us for tiles of 64 columns, 4.8 for 128, 6.5 for pairs of 128, 10.2 for 256; accumulating 1.2, 2.0, 3.0 and 4.5; bf16 the same within 1 us.
+inline double tail_ns(const Variant &v, bool accumulate) { return (1500.0 + 33.0 * v.bn + (v.cg == 2 ? 500.0 : 0.0)) * (accumulate ? 0.45 : 1.0); }
+
+// Returns the k-blocks of a group's run in a stream-K tail that pays, 0: none does.  (`plain` as in estimate_ns: k-blocks at another layout's price
+// forwent tails that pay, f32 A.B^T 7936 x 1536 x 2528 219 us with one, 245 without, A^T.B 1984 x 7552 x 1536 179 and 213.)  The margin is for the
+// price of a k-block, which is known to 20 %: with twice it 6720 x 296 x 1328 f32 had no tail (31.3 us, 28.1 with it).
+int stream_k_run(const Variant &v, bool f32, bool plain, int64_t tiles, int groups, int num_kb, int kps, bool accumulate, bool whenever) {
     const int left = (int)(tiles % groups);
     if (tiles <= groups || left == 0 || num_kb % kps != 0) return 0;
     const int64_t units = (int64_t)left * num_kb;
     int run = (int)((units + groups - 1) / groups);
     run = (run + kps - 1) / kps * kps;
     const double saved = (double)(num_kb - run) * kb_own_ns(v, f32, plain);
-    const double extra = 2.0 * (1500.0 + (double)v.bn * (f32 ? 24.0 : 12.0)) + 2500.0;
-    return run >= 4 * kps && (saved > (f32 ? 1.4 : 2.0) * extra || whenever) ? run : 0;
+    return run >= 4 * kps && (saved > 1.2 * tail_ns(v, accumulate) || whenever) ? run : 0;
 }
 
 // Estimated kernel time in ns of `tiles` tiles dealt out in `sp` k ranges each over `groups`
@@ -1254,7 +1258,7 @@ double estimate_ns(const Variant &v, bool f32, bool plain, int64_t tiles, int64_
     double wave_ns = kbs * kb_ns + open * item_ns;
     if (active * BM * v.bn * 4 / 6000.0 > wave_ns) wave_ns = active * BM * v.bn * 4 / 6000.0;
     double t = (double)kbs * kb_ns + item_ns + (double)(waves - 1) * wave_ns;
-    const int run = f32 && sp == 1 && tail ? stream_k_run(v, f32, plain, tiles, (int)groups, num_kb, 1, false) : 0;
+    const int run = f32 && sp == 1 && tail ? stream_k_run(v, f32, plain, tiles, (int)groups, num_kb, 1, accumulate, false) : 0;
     if (run > 0) t += item_ns + 1500.0 - (double)(num_kb - run) * kb_ns;               // the last wave is shorter, the write-backs are more
     if (v.cg == 2) t += 490.0;                                                         // cluster launch, cross-CTA signalling
     if (sp > 1) t += f32 ? 2880.0 : 2610.0;                                            // reduce-add traffic, the clearing launch
@@ -1603,7 +1607,7 @@ sg_status launch_tensor(const Problem &p, const void *In, const void *Flt, float
         const int64_t tiles = (int64_t)num_m_tiles * num_n_tiles;
         const int left = (int)(tiles % groups);
         if (ov.sk != 0 && splits == 1) {
-            const int run = stream_k_run(var, f32, lay == 0, tiles, groups, tp.num_kb, kps, ov.sk == 2);
+            const int run = stream_k_run(var, f32, lay == 0, tiles, groups, tp.num_kb, kps, p.accumulate != 0, ov.sk == 2);
             if (run > 0) {
                 tp.sk_first_tile = (int)(tiles - left);
                 tp.sk_units = run;

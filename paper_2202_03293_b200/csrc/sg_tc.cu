@@ -26,8 +26,8 @@
 // writes the raw f32 tiles into its ring, sixteen converter warps split them and write a second ring of two or four slots
 // (transposing the filter tile to K-major on the way, which kind::tf32 needs; the split input tile goes to tensor
 // memory), and the MMA thread accumulates lo*hi + hi*lo + hi*hi in f32: the dropped term is below 2^-21 |a*b|, so
-// f32 accuracy is kept.  In the plain layout hi*hi runs in tf32 and the two corrections as one bf16 contraction over
-// [lo | hi] . [hi | lo] (8 MMAs per k-block); the transposed layouts run three tf32 products (12).  Raw tiles are
+// f32 accuracy is kept.  hi*hi runs in tf32 and the two corrections as one bf16 contraction over
+// [lo | hi] . [hi | lo] (8 MMAs per k-block); short reductions of transposed operands run three tf32 products (12; see bf16_corrections).  Raw tiles are
 // 128 rows x 32 f32 (input) and 32 k-rows x 32 f32 sub-tiles (filter), again 128 bytes per row.
 //
 // Every wait in this file is bounded: a wait that expires sets an abort flag in shared
@@ -161,17 +161,17 @@ __global__ void __launch_bounds__(256) zero_tiles_kernel(float *__restrict__ O, 
 
 // LAY: bit 0 = the input operand is stored transposed ([k][m], m contiguous: A^T B of Section 4.6.1; bf16: consumed as an M-major
 // operand); bit 1 = the filter operand is stored transposed ([n][k], k contiguous: A B^T; bf16: consumed K-major); bit 2 (f32) = the
-// split input tile goes to tensor memory; bit 3 (f32, plain layout) = the correction products run as bf16 MMAs.
+// split input tile goes to tensor memory; bit 3 (f32) = the correction products run as bf16 MMAs.
 template <int BN, int CG, bool F32, int KPS, int LAY>
 __global__ void __launch_bounds__(Cfg<BN, CG, F32, KPS, (LAY & 4) != 0>::THREADS, 1)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant__ CUtensorMap map_flt,
                const __grid_constant__ CUtensorMap map_out, const TcParams p) {
     constexpr bool A_MN = (LAY & 1) != 0, B_KM = (LAY & 2) != 0, TA = (LAY & 4) != 0;
-    // MIX (f32, plain layout, split input in tensor memory): the correction products lo*hi + hi*lo run as bf16 MMAs
+    // MIX (f32, split input in tensor memory): the correction products lo*hi + hi*lo run as bf16 MMAs
     constexpr bool MIX = (LAY & 8) != 0;
     using C = Cfg<BN, CG, F32, KPS, TA>;
     static_assert(!TA || F32, "tensor-memory input operand: f32 path only");
-    static_assert(!MIX || LAY == 12, "bf16 corrections: plain layout with the split input in tensor memory");
+    static_assert(!MIX || TA, "bf16 corrections: with the split input in tensor memory");
     static_assert(LAY == 0 || KPS == 1, "transposed layouts: one k-block per stage");
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -523,6 +523,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant
             if constexpr (MIX && C::GROUPS == 2) {
                 const int row = (warp & 3) * 32 + lane;
                 for (int i = 0; i < 4; ++i) mx_a_off[i] = (uint32_t)(row * 128 + ((((cw >> 2) * 4 + i) ^ (row & 7)) << 4));
+                if (A_MN) mx_a_off[0] = (uint32_t)((warp & 3) * C::SUB_BYTES + ((cw >> 2) * 16 * 32 + lane) * 4);
                 const int uj = cw >> 2, uq = cw & 3, f = uj * 32 + lane;
                 mx_b_src = (uint32_t)(A_STAGE_BYTES + uj * C::SUB_BYTES + (uq * 8 * 32 + lane) * 4);
                 const uint32_t rowoff = (uint32_t)((f >> 3) * 1024 + (f & 7) * 128);
@@ -645,14 +646,29 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant
                         split_a(1, a);
                         split_b(1, x1);
                     } else if constexpr (MIX) {
-                        // Plain layout, corrections as bf16 MMAs.  Every address below is fixed per thread (set up ahead of
+                        // Corrections as bf16 MMAs.  Every address below is fixed per thread (set up ahead of
                         // the loops); the loads go out first, input rows then filter columns.
                         uint4 a[4];
+                        if constexpr (A_MN) {       // stored transposed: 16 values down a column of a [32 k][32 rows] sub-tile
+                            const uint32_t *col = reinterpret_cast<const uint32_t *>(raw + mx_a_off[0]);
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) a[i] = *reinterpret_cast<const uint4 *>(raw + mx_a_off[i]);
+                            for (int i = 0; i < 4; ++i) a[i] = make_uint4(col[i * 128], col[i * 128 + 32], col[i * 128 + 64], col[i * 128 + 96]);
+                        } else {
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) a[i] = *reinterpret_cast<const uint4 *>(raw + mx_a_off[i]);
+                        }
                         uint32_t x[UNITS][8];
 #pragma unroll
                         for (int u = 0; u < UNITS; ++u) {
+                            if constexpr (B_KM) {   // stored transposed: two chunks of the column's row, swizzled as the hi tile is
+                                const uint8_t *tile_b = raw + A_STAGE_BYTES + u * 8192;
+#pragma unroll
+                                for (int h = 0; h < 2; ++h) {
+                                    const uint4 v = *reinterpret_cast<const uint4 *>(tile_b + mx_hi_off[h]);
+                                    x[u][4 * h] = v.x; x[u][4 * h + 1] = v.y; x[u][4 * h + 2] = v.z; x[u][4 * h + 3] = v.w;
+                                }
+                                continue;
+                            }
                             const uint32_t *col = reinterpret_cast<const uint32_t *>(raw + mx_b_src + u * 2 * C::SUB_BYTES);
 #pragma unroll
                             for (int k = 0; k < 8; ++k) x[u][k] = col[k * 32];
@@ -1013,7 +1029,8 @@ typedef CUresult (*EncodeIm2colFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_
 // g_mu guards the driver entry points, the per-device records and the overrides; it is held for a few loads and stores,
 // never across a tensor-map encode or a launch.  The tensor-map cache has a lock of its own.
 constexpr int kMaxDevices = 64;
-constexpr int kAttrSlots = 236;
+constexpr int kMixSlots = 236;                   // transposed f32 operands with bf16 corrections: three layouts of five variants
+constexpr int kAttrSlots = kMixSlots + 15;
 struct DeviceState {
     bool ready = false;
     int num_sms = 0;
@@ -1206,49 +1223,52 @@ bool encode_im2col_cached(CUtensorMap *map, int device, CUtensorMapDataType type
 
 inline bool mult(int64_t v, int64_t q) { return v % q == 0; }
 
-struct Variant { int bn, cg; double mma_ns, mma_ns_f32, mma_ns_f32_t; };
-// Time one CTA needs for one k-block of a tile, in ns: its tensor core (bf16), or its converter warps and tensor core (f32: plain layout,
-// eight MMAs; an operand stored transposed, twelve).
-constexpr Variant kVariants[] = {{64, 1, 125.0, 336.0, 385.0}, {128, 1, 150.0, 424.0, 517.0}, {256, 1, 400.0, 1500.0, 1500.0},
-                                 {128, 2, 140.0, 374.0, 1500.0}, {256, 2, 358.0, 627.0, 903.0}};
+// What a k-block is: f32 one of the first three (an operand stored transposed: twelve MMAs, or eight; the plain layout, eight), bf16 one of the
+// last two (stages of one k-block or of two).
+enum KbKind { F32_TRANSPOSED_TF32, F32_TRANSPOSED, F32_PLAIN, BF16_ONE, BF16_TWO };
+struct Variant { int bn, cg; double mma_ns, f32_ns[3]; };
+// Time one CTA needs for one k-block of a tile, in ns: its tensor core (bf16), or its converter warps and tensor core (f32, by KbKind).
+constexpr Variant kVariants[] = {{64, 1, 125.0, {385.0, 336.0, 336.0}}, {128, 1, 150.0, {517.0, 424.0, 424.0}}, {256, 1, 400.0, {1500.0, 1500.0, 1500.0}},
+                                 {128, 2, 140.0, {1500.0, 352.0, 374.0}}, {256, 2, 358.0, {903.0, 627.0, 627.0}}};
 constexpr int kNumVariants = sizeof(kVariants) / sizeof(kVariants[0]);
 
-inline double kb_own_ns(const Variant &v, bool f32, bool plain) { return !f32 ? v.mma_ns : plain ? v.mma_ns_f32 : v.mma_ns_f32_t; }
+inline double kb_own_ns(const Variant &v, KbKind kind) { return kind >= BF16_ONE ? v.mma_ns : v.f32_ns[kind]; }
 
 // What a stream-K tail (launch_tensor) costs in ns: the write-backs of its runs, which are open, and the launch that clears its tiles (which an
 // accumulating call does not need).  Measured with and without a tail on 170 calls (products in every layout, tiles of 64 to 256 columns): f32
 // 3.7 us for tiles of 64 columns, 4.8 for 128, 6.5 for pairs of 128, 10.2 for 256; accumulating 1.2, 2.0, 3.0 and 4.5; bf16 the same within 1 us.
 inline double tail_ns(const Variant &v, bool accumulate) { return (1500.0 + 33.0 * v.bn + (v.cg == 2 ? 500.0 : 0.0)) * (accumulate ? 0.45 : 1.0); }
 
-// Returns the k-blocks of a group's run in a stream-K tail that pays, 0: none does.  (`plain` as in estimate_ns: k-blocks at another layout's price
+// Returns the k-blocks of a group's run in a stream-K tail that pays, 0: none does.  (k-blocks at another layout's price
 // forwent tails that pay, f32 A.B^T 7936 x 1536 x 2528 219 us with one, 245 without, A^T.B 1984 x 7552 x 1536 179 and 213.)  The margin is for the
 // price of a k-block, which is known to 20 %: with twice it 6720 x 296 x 1328 f32 had no tail (31.3 us, 28.1 with it).
-int stream_k_run(const Variant &v, bool f32, bool plain, int64_t tiles, int groups, int num_kb, int kps, bool accumulate, bool whenever) {
+int stream_k_run(const Variant &v, KbKind kind, int64_t tiles, int groups, int num_kb, int kps, bool accumulate, bool whenever) {
     const int left = (int)(tiles % groups);
     if (tiles <= groups || left == 0 || num_kb % kps != 0) return 0;
     const int64_t units = (int64_t)left * num_kb;
     int run = (int)((units + groups - 1) / groups);
     run = (run + kps - 1) / kps * kps;
-    const double saved = (double)(num_kb - run) * kb_own_ns(v, f32, plain);
+    const double saved = (double)(num_kb - run) * kb_own_ns(v, kind);
     return run >= 4 * kps && (saved > 1.2 * tail_ns(v, accumulate) || whenever) ? run : 0;
 }
 
 // Estimated kernel time in ns of `tiles` tiles dealt out in `sp` k ranges each over `groups`
 // CTAs or CTA pairs.  A k-block costs the slowest of: the CTA's own time, the CTA's share of the L2 -> shared memory fill
-// rate of the whole chip, the fill rate one SM reaches alone, and (bf16 stages of one k-block: `plain` false) a stage's two waits.
-// f32: `plain` false = an operand stored transposed.  Fitted to graph replays of every variant and split on 125 (bf16) and 118 (f32) calls:
+// rate of the whole chip, the fill rate one SM reaches alone, and (bf16 stages of one k-block) a stage's two waits.
+// Fitted to graph replays of every variant and split on 125 (bf16) and 118 (f32) calls:
 // products of 64 to 16384 in every layout and convolutions, three operand sets in turn.  The estimates are within 11 and 7 % of
 // the timings near the best; the choices cost 0.4 % over the best in the mean (with the constants of slower kernels
 // 1.3 and 4 %), half of the shapes held back from the fit 0.7 and 0.8.
-double estimate_ns(const Variant &v, bool f32, bool plain, int64_t tiles, int64_t groups, int num_kb, int sp, bool accumulate, bool tail) {
+double estimate_ns(const Variant &v, KbKind kind, int64_t tiles, int64_t groups, int num_kb, int sp, bool accumulate, bool tail) {
+    const bool f32 = kind < BF16_ONE;
     const int64_t items = tiles * sp;
     const int64_t waves = (items + groups - 1) / groups;
     const int kbs = (num_kb + sp - 1) / sp;
     const double active = (double)((items < groups ? items : groups) * v.cg);
     const double stage_bytes = A_STAGE_BYTES + (double)(v.bn / v.cg) * ROW_BYTES;
     const double chip_fill = f32 ? 11100.0 : 17100.0, sm_fill = f32 ? 77.3 : 127.0;      // bytes per ns
-    double kb_ns = kb_own_ns(v, f32, plain);
-    if (!f32 && !plain && kb_ns < 218.0) kb_ns = 218.0;
+    double kb_ns = kb_own_ns(v, kind);
+    if (kind == BF16_ONE && kb_ns < 218.0) kb_ns = 218.0;
     if (active * stage_bytes / chip_fill > kb_ns) kb_ns = active * stage_bytes / chip_fill;
     if (stage_bytes / sm_fill > kb_ns) kb_ns = stage_bytes / sm_fill;
     const double item_ns = f32 ? 2280.0 + 15.6 * v.bn : 2000.0 + 10.2 * v.bn;          // pipeline fill + epilogue of one item
@@ -1258,17 +1278,17 @@ double estimate_ns(const Variant &v, bool f32, bool plain, int64_t tiles, int64_
     double wave_ns = kbs * kb_ns + open * item_ns;
     if (active * BM * v.bn * 4 / 6000.0 > wave_ns) wave_ns = active * BM * v.bn * 4 / 6000.0;
     double t = (double)kbs * kb_ns + item_ns + (double)(waves - 1) * wave_ns;
-    const int run = f32 && sp == 1 && tail ? stream_k_run(v, f32, plain, tiles, (int)groups, num_kb, 1, accumulate, false) : 0;
+    const int run = f32 && sp == 1 && tail ? stream_k_run(v, kind, tiles, (int)groups, num_kb, 1, accumulate, false) : 0;
     if (run > 0) t += item_ns + 1500.0 - (double)(num_kb - run) * kb_ns;               // the last wave is shorter, the write-backs are more
-    if (v.cg == 2) t += 490.0;                                                         // cluster launch, cross-CTA signalling
+    if (v.cg == 2) t += kind == F32_TRANSPOSED && v.bn == 128 ? 700.0 : 490.0;         // cluster launch, cross-CTA signalling
     if (sp > 1) t += f32 ? 2880.0 : 2610.0;                                            // reduce-add traffic, the clearing launch
     if (sp > 1 && accumulate) t -= f32 ? 2290.0 : 2420.0;                              // (no clearing)
     return t;
 }
 
 // The same for `sp` CTAs in a cluster per tile.
-double estimate_meet_ns(const Variant &v, bool f32, bool plain, int64_t tiles, int num_kb, int sp) {
-    return estimate_ns(v, f32, plain, tiles * sp, tiles * sp, (num_kb + sp - 1) / sp, 1, false, false) + (f32 ? 2200.0 : 1300.0 + 11.0 * v.bn);
+double estimate_meet_ns(const Variant &v, KbKind kind, int64_t tiles, int num_kb, int sp) {
+    return estimate_ns(v, kind, tiles * sp, tiles * sp, (num_kb + sp - 1) / sp, 1, false, false) + (kind < BF16_ONE ? 2200.0 : 1300.0 + 11.0 * v.bn);
 }
 
 // Operands stored transposed (matmuls only): bit 0 the input ([k][m], m contiguous), bit 1 the filter ([n][k], k contiguous).
@@ -1277,21 +1297,49 @@ inline int transposed_layout(const Problem &p) {
     return (a_mn ? 1 : 0) | (b_km ? 2 : 0);
 }
 
+// f32: whether the correction products of an item of `kbs` k-blocks run as bf16 MMAs (eight MMAs a k-block) or all three products in
+// tf32 (twelve).  A product is 2^-22 of itself off in tf32 and up to 2^-19 with bf16 corrections, but every MMA also truncates the sum that it
+// adds to, which is most of the error of a longer sum and less with fewer MMAs.  Relative error (2-norm) of 2048 x K x 1024, uniform / normal
+// operands, three tf32 products and bf16 corrections: K = 64 4.6e-7 / 4.6e-7 and 6.2e-7 / 7.2e-7, 96 6.8e-7 / 6.9e-7 and 7.0e-7 / 7.9e-7, 128 9.1e-7 / 9.1e-7 and
+// 8.1e-7 / 8.8e-7, 256 1.8e-6 and 1.3e-6, 1024 7.2e-6 and 4.8e-6.  So from 128 values of k on; 2048^3 A.B^T 67 -> 51 us.  (The plain layout has
+// always had them.)
+constexpr int kMixKb = 4;
+bool bf16_corrections(const Overrides &ov, int lay, int kbs) {
+    return ov.ta != 0 && ov.mix != 0 && (lay == 0 || kbs >= kMixKb);
+}
+
 // Tile variant and k split of lowest estimated time, which is returned (unless the variant is forced); *out_pick = -1: none.
 // *out_meet: the split's partial sums meet in a cluster.
-double choose_tiles(const Problem &p, int num_kb, int lay, const Overrides &ov, int num_sms, int *out_pick, int *out_splits, int *out_meet) {
+// `longest`: the most k-blocks of a range that runs with bf16 corrections (transposed f32 operands).
+double choose_tiles(const Problem &p, int num_kb, int lay, const Overrides &ov, int num_sms, int *out_pick, int *out_splits, int *out_meet, int longest = 1 << 30) {
     *out_meet = 0;
+    if (!p.in_bf16 && lay != 0 && num_kb >= kMixKb && ov.mix != 0 && ov.bn == 0 && ov.split == 0 && longest == 1 << 30) {
+        // A cheaper k-block asks for longer ranges, and the error grows with them: a range gets at most half as long again as three tf32
+        // products would have had, which is as accurate (256 x 4096 x 256 A.B^T: 32 ranges 9.2e-7, 16 with bf16 corrections 1.3e-6).
+        Overrides tf32 = ov;
+        tf32.mix = 0;
+        choose_tiles(p, num_kb, lay, tf32, num_sms, out_pick, out_splits, out_meet);
+        longest = (num_kb + *out_splits - 1) / *out_splits * 3 / 2;
+        return choose_tiles(p, num_kb, lay, ov, num_sms, out_pick, out_splits, out_meet, longest);
+    }
     const bool fused = p.bias != nullptr || p.act != SG_ACT_NONE, forced_tile = ov.bn > 0 || ov.cg > 0 || (ov.split > 0 && !fused);
     const bool f32 = !p.in_bf16;
-    // (bf16: two k-blocks per stage, see launch_tensor)
-    const bool plain = f32 ? lay == 0 : lay == 0 && p.spatial_rank == 0 && p.K % 64 == 0 && p.N % 64 == 0;
+    auto kind = [&](int sp) {
+        if (f32) return lay == 0 ? F32_PLAIN : bf16_corrections(ov, lay, (num_kb + sp - 1) / sp) ? F32_TRANSPOSED : F32_TRANSPOSED_TF32;
+        return lay == 0 && p.spatial_rank == 0 && p.K % 64 == 0 && p.N % 64 == 0 ? BF16_TWO : BF16_ONE;      // (see launch_tensor)
+    };
+    // variants that are not built (or that would sum too long a range): f32 tiles of 256 columns to a CTA (shared memory), and for transposed
+    // operands a few more
+    auto built = [&](const Variant &v, int sp) {
+        if (kind(sp) == F32_TRANSPOSED && (num_kb + sp - 1) / sp > longest) return false;
+        if (v.bn == 256 && v.cg == 1) return !f32 && lay == 0;
+        return lay == 0 || v.bn != 128 || v.cg != 2 || kind(sp) == F32_TRANSPOSED;
+    };
     int pick = -1, splits = 1;
     double best = 1e300;
     if (ov.bn > 0) {
         for (int i = 0; i < kNumVariants; ++i)
-            if (kVariants[i].bn == ov.bn && kVariants[i].cg == (ov.cg > 0 ? ov.cg : 1) &&
-                !(f32 && kVariants[i].bn == 256 && kVariants[i].cg == 1) &&
-                !(lay != 0 && ((kVariants[i].bn == 256 && kVariants[i].cg == 1) || (kVariants[i].bn == 128 && kVariants[i].cg == 2)))) pick = i;
+            if (kVariants[i].bn == ov.bn && kVariants[i].cg == (ov.cg > 0 ? ov.cg : 1) && built(kVariants[i], ov.split > 0 ? ov.split : 1)) pick = i;
     }
     auto valid_split = [&](int s) {      // every range of ceil(num_kb / s) k-blocks must be non-empty
         const int per = (num_kb + s - 1) / s;
@@ -1309,21 +1357,21 @@ double choose_tiles(const Problem &p, int num_kb, int lay, const Overrides &ov, 
             // (forced == 1 for a fused consumer: one work item per tile)
             const Variant &v = kVariants[i];
             if (pass == 0 && ov.cg > 0 && v.cg != ov.cg && !(v.cg == 1 && p.M <= BM)) continue;
-            if (f32 && v.bn == 256 && v.cg == 1) continue;       // not built (shared-memory budget)
-            if (lay != 0 && ((v.bn == 256 && v.cg == 1) || (v.bn == 128 && v.cg == 2))) continue;   // not built for transposed operands
             if (v.bn > 64 && v.bn / 2 >= p.N) continue;          // at most half of the tile would be used
             if (v.cg == 2 && p.M <= BM) continue;                // the second CTA would have no rows
             const int64_t tiles = (int64_t)((p.M + v.cg * BM - 1) / (v.cg * BM)) * ((p.N + v.bn - 1) / v.bn);
             const int64_t groups = num_sms / v.cg;
             if (forced) {
-                const double c = estimate_ns(v, f32, plain, tiles, groups, num_kb, forced, p.accumulate != 0, ov.sk != 0 && !fused);
+                if (!built(v, forced)) continue;
+                const double c = estimate_ns(v, kind(forced), tiles, groups, num_kb, forced, p.accumulate != 0, ov.sk != 0 && !fused);
                 if (c < best) { best = c; pick = i; splits = forced; }
                 continue;
             }
             for (int sp = 1; sp <= 32; sp *= 2) {
                 if (!valid_split(sp)) break;
                 if (sp > 1 && tiles * (sp / 2) >= 2 * groups) break;   // already two waves without this split
-                const double c = estimate_ns(v, f32, plain, tiles, groups, num_kb, sp, p.accumulate != 0, ov.sk != 0 && !fused);
+                if (!built(v, sp)) continue;
+                const double c = estimate_ns(v, kind(sp), tiles, groups, num_kb, sp, p.accumulate != 0, ov.sk != 0 && !fused);
                 if (c < best) { best = c; pick = i; splits = sp; }
             }
         }
@@ -1339,8 +1387,9 @@ double choose_tiles(const Problem &p, int num_kb, int lay, const Overrides &ov, 
             for (int sp = 2; sp <= MAX_MEET; sp *= 2) {
                 if (ov.meet > 1 && sp != ov.meet) continue;
                 const int stages = (num_kb + 1) / 2, per = (stages + sp - 1) / sp;       // (bf16: ranges of whole two-block stages too)
+                if (kind(sp) == F32_TRANSPOSED && (num_kb + sp - 1) / sp > longest) continue;
                 if (tiles > (sp == 2 ? 70 : sp == 4 ? 32 : 14) || tiles * sp > num_sms - 8 || num_kb < 4 * sp || !valid_split(sp) || (stages + per - 1) / per != sp) continue;
-                const double c = ov.meet > 1 ? 0.0 : estimate_meet_ns(v, f32, plain, tiles, num_kb, sp);
+                const double c = ov.meet > 1 ? 0.0 : estimate_meet_ns(v, kind(sp), tiles, num_kb, sp);
                 if (c < best) { best = c; pick = i; splits = sp; *out_meet = 1; }
             }
         }
@@ -1359,12 +1408,12 @@ template <int BN, int CG, bool F32, int KPS, int LAY = 0>
 sg_status launch_variant(const CUtensorMap &mi, const CUtensorMap &mf, const CUtensorMap &mo, TcParams tp, int M, int N,
                          int slot, const LaunchCtx &ctx) {
   if constexpr ((F32 && BN == 256 && CG == 1) || (KPS == 2 && (F32 || (BN == 256 && CG == 1))) ||
-                ((LAY & 3) != 0 && (KPS != 1 || (BN == 256 && CG == 1) || (BN == 128 && CG == 2))) ||
+                ((LAY & 3) != 0 && (KPS != 1 || (BN == 256 && CG == 1) || (BN == 128 && CG == 2 && (LAY & 8) == 0))) ||
                 ((LAY & 4) != 0 && !F32)) {
     return SG_ERR_INTERNAL;   // the split slots of a 128 x 256 f32 tile do not fit beside a TMA ring
   } else {
     using C = Cfg<BN, CG, F32, KPS, (LAY & 4) != 0>;
-    static_assert(5 * 3 * 8 <= kAttrSlots, "attribute slots");
+    static_assert(5 * 3 * 9 <= 144 && 3 * kNumVariants <= kAttrSlots - kMixSlots, "attribute slots");
     if (!ensure_smem_attr(ctx.device, slot, tc_gemm_kernel<BN, CG, F32, KPS, LAY>, C::SMEM_BYTES)) return SG_ERR_CUDA;
     tp.num_m_tiles = (M + CG * BM - 1) / (CG * BM);
     tp.num_n_tiles = (N + BN - 1) / BN;
@@ -1607,7 +1656,7 @@ sg_status launch_tensor(const Problem &p, const void *In, const void *Flt, float
         const int64_t tiles = (int64_t)num_m_tiles * num_n_tiles;
         const int left = (int)(tiles % groups);
         if (ov.sk != 0 && splits == 1) {
-            const int run = stream_k_run(var, f32, lay == 0, tiles, groups, tp.num_kb, kps, p.accumulate != 0, ov.sk == 2);
+            const int run = stream_k_run(var, !f32 ? BF16_ONE : lay == 0 ? F32_PLAIN : bf16_corrections(ov, lay, per) ? F32_TRANSPOSED : F32_TRANSPOSED_TF32, tiles, groups, tp.num_kb, kps, p.accumulate != 0, ov.sk == 2);
             if (run > 0) {
                 tp.sk_first_tile = (int)(tiles - left);
                 tp.sk_units = run;
@@ -1626,12 +1675,16 @@ sg_status launch_tensor(const Problem &p, const void *In, const void *Flt, float
     // 256-column tiles that costs the second accumulator buffer, which short reductions used to feel; since the
     // converters stopped being the bottleneck the sweep is no slower with it everywhere (5.72 to 5.79 ms per step
     // either way), so there is one rule.
-    // In the plain layout the two correction products of the split run as bf16 MMAs (see split4_mix).
+    // The two correction products of the split run as bf16 MMAs (see split4_mix and bf16_corrections).
     int lay_k = (f32 && ov.ta != 0) ? (lay | 4) : lay;
-    if (lay_k == 4 && ov.mix != 0) lay_k = 12;
-    const int slot = pick + (f32 ? kNumVariants : 0) + (kps == 2 ? 2 * kNumVariants : 0) + (lay_k == 12 ? 8 : lay_k) * 3 * kNumVariants;
+    if (f32 && bf16_corrections(ov, lay, per)) lay_k |= 8;
+    const int slot = lay_k > 12 ? kMixSlots + (lay_k - 13) * kNumVariants + pick
+                                : pick + (f32 ? kNumVariants : 0) + (kps == 2 ? 2 * kNumVariants : 0) + (lay_k == 12 ? 8 : lay_k) * 3 * kNumVariants;
 #define SG_LAUNCH(BN_, CG_)                                                                                \
     (f32 ? (lay_k == 12 ? launch_variant<BN_, CG_, true, 1, 12>(map_in, map_flt, map_out, tp, p.M, p.N, slot, ctx)   \
+            : lay_k == 13 ? launch_variant<BN_, CG_, true, 1, 13>(map_in, map_flt, map_out, tp, p.M, p.N, slot, ctx) \
+            : lay_k == 14 ? launch_variant<BN_, CG_, true, 1, 14>(map_in, map_flt, map_out, tp, p.M, p.N, slot, ctx) \
+            : lay_k == 15 ? launch_variant<BN_, CG_, true, 1, 15>(map_in, map_flt, map_out, tp, p.M, p.N, slot, ctx) \
             : lay_k == 4 ? launch_variant<BN_, CG_, true, 1, 4>(map_in, map_flt, map_out, tp, p.M, p.N, slot, ctx)     \
             : lay_k == 6 ? launch_variant<BN_, CG_, true, 1, 6>(map_in, map_flt, map_out, tp, p.M, p.N, slot, ctx)   \
             : lay_k == 5 ? launch_variant<BN_, CG_, true, 1, 5>(map_in, map_flt, map_out, tp, p.M, p.N, slot, ctx)   \
@@ -1694,6 +1747,8 @@ double tensor_estimate_us(const Problem &p) {
     const DeviceState *d = device_state(nullptr, &ov);
     if (!d) return 0.0;
     if (p.bias != nullptr || p.act != SG_ACT_NONE) ov.split = 1;
+    // (its caller keeps what is more accurate than either form of transposed f32 operands, at the price that they had with three tf32 products)
+    if (transposed_layout(p) != 0) ov.mix = 0;
     const int bk = ROW_BYTES / (p.in_bf16 ? 2 : 4);
     int pick, splits, meet;
     return 1e-3 * choose_tiles(p, p.KH * p.KW * ((p.C + bk - 1) / bk), transposed_layout(p), ov, d->num_sms, &pick, &splits, &meet);

@@ -1,0 +1,40 @@
+"""Operands stored transposed: every tile that is built for them, and (f32) the reductions on either side of the line from which
+the correction products run in bf16."""
+import numpy as np
+import pytest
+import torch
+
+from helpers import assert_within_bound, operand
+from oracle import ref
+from paper_2202_03293_b200 import binding as sg
+
+pytestmark = pytest.mark.gpu
+SEED = 9750
+
+
+# a k-block is 32 values (f32) or 64 (bf16): one, the last with three tf32 products, the first with bf16 corrections, a remainder;
+# one ragged tile, and more tiles than SMs
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("a_t,b_t", [(True, False), (False, True), (True, True)])
+@pytest.mark.parametrize("bn,cg", [(64, 1), (128, 1), (128, 2), (256, 2)])
+@pytest.mark.parametrize("M,N,K", [(320, 264, 32), (320, 264, 96), (320, 264, 128), (320, 264, 168), (5120, 1096, 136)])
+def test_transposed_tiles(M, N, K, bn, cg, a_t, b_t, dtype):
+    A, a = operand((K, M) if a_t else (M, K), SEED, 1, "uniform", dtype)
+    B, b = operand((N, K) if b_t else (K, N), SEED, 2, "uniform", dtype)
+    A, a = (A.t(), np.ascontiguousarray(a.T)) if a_t else (A, a)
+    B, b = (B.t(), np.ascontiguousarray(b.T)) if b_t else (B, b)
+    C = torch.full((M, N), float("nan"), device="cuda")
+    sg.sg_set_tile_override(bn, cg, 1)
+    try:
+        sg.sg_matmul(A, B, C)
+        torch.cuda.synchronize()
+        name, choice = sg.sg_last_kernel_name(), tuple(sg.sg_last_tile_choice())
+    finally:
+        sg.sg_set_tile_override(0, 0, 0)
+    assert name == f"tc_gemm_kernel<{dtype}>"
+    if (bn, cg) != (128, 2) or (dtype == "f32" and K >= 128):      # (else not built)
+        assert choice == (bn, cg, 1)
+    rows = np.unique(np.r_[0:M:max(1, M // 40), M - 1])
+    want, S = ref.matmul(np.ascontiguousarray(a[rows]), b)
+    assert assert_within_bound(C[torch.from_numpy(rows).cuda()], want, S, "transposed tiles") < 4e-6      # 2^-19 for the rounded corrections, and the truncating sum
+    sg.sg_check()

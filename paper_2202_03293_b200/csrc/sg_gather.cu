@@ -721,13 +721,31 @@ bool raw_map(CUtensorMap *map, const void *ptr, Operand &op, int mn, int k, int 
                                CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
 }
 
-// Tiles, their width, and the CTAs (of one cluster) that share a tile's reduction: 2, 4 or 8 where tiles are few, at least four k-blocks each.
-struct Tiles { int bn, num_kb, splits; int64_t tiles; };
+// Tiles, their width, and the CTAs (of one cluster) that share a tile's reduction.
+struct Tiles { int bn, num_kb, splits; int64_t tiles; double us; };
+// By time (us): a start and an end, a k-block of every round of tiles, what a further round adds, and for shared reductions what sharing costs;
+// 148 SMs hold 74, 33 and 15 clusters of 2, 4 and 8 CTAs at once.  Fitted to graph replays of 200 calls whose lines start anywhere, each in both widths and with
+// 1 to 8 CTAs a tile: the estimates are within 5 % in the mean, the choices cost 0.6 % over the best.  (With 128 columns wherever there are
+// more than 64, and only as many CTAs as fit beside one another, products took 22 % (f32) and 12 % (bf16) longer, convolutions 7 and 17:
+// 3181 x 682 x 868 f32 is 150 tiles of 128 columns, two rounds, 62 us, and 275 of 64, 42 us; 155 x 172 x 1369 19.7 and 10.5.)
 Tiles plan_tiles(const Problem &p, int num_sms) {
-    Tiles t{p.N > 64 ? 128 : 64, (p.K + BK - 1) / BK, 1, 0};
-    t.tiles = (int64_t)((p.M + BM - 1) / BM) * ((p.N + t.bn - 1) / t.bn);
-    while (t.splits < MAX_SPLIT && t.tiles * t.splits * 2 <= num_sms - 12 && t.num_kb >= t.splits * 8) t.splits *= 2;
-    return t;
+    struct Cost { double ends, round, kb, shared, shared_round; };
+    constexpr Cost costs[2][2][2] = {{{{6.3, 1.2, 0.66, 1.1, 7.0}, {6.9, 3.6, 0.79, 2.1, 8.4}}, {{5.7, 1.3, 1.12, 1.1, 7.0}, {6.3, 2.1, 1.40, 2.1, 8.4}}},
+                                     {{{5.5, 1.3, 1.35, 1.9, 7.2}, {5.5, 2.0, 1.98, 3.4, 7.8}}, {{6.3, 1.3, 1.48, 1.9, 7.2}, {7.3, 2.2, 2.06, 3.4, 7.8}}}};      // [f32][convolution][128 columns]
+    const int num_kb = (p.K + BK - 1) / BK;
+    Tiles best{};
+    best.us = 1e300;
+    for (int bn = 64; bn <= (p.N > 64 ? 128 : 64); bn *= 2) {
+        const Cost &c = costs[!p.in_bf16][p.spatial_rank != 0][bn == 128];
+        const int64_t tiles = (int64_t)((p.M + BM - 1) / BM) * ((p.N + bn - 1) / bn);
+        for (int splits = 1; splits == 1 || (splits <= MAX_SPLIT && num_kb > 2 * splits); splits *= 2) {
+            const int at_once = splits == 1 ? num_sms : splits == 2 ? num_sms / 2 : splits == 4 ? num_sms / 4 - 4 : num_sms / 8 - 3;
+            const double rounds = (double)((tiles + at_once - 1) / at_once);
+            const double us = c.ends + rounds * c.kb * ((num_kb + splits - 1) / splits) + (splits == 1 ? (rounds - 1.0) * c.round : c.shared + (rounds - 1.0) * c.shared_round);
+            if (us < best.us) { best = Tiles{bn, num_kb, splits, tiles, us}; }
+        }
+    }
+    return best;
 }
 
 // Below 2^21 multiply-adds the CUDA-core kernel is as fast.
@@ -735,21 +753,24 @@ bool too_small(const Problem &p) { return (int64_t)p.M * p.N * p.K < ((int64_t)1
 
 }  // namespace
 
-// A start and an end, rounds of tiles and their k-blocks, and what sharing a reduction costs.  Fitted to graph replays of 500 calls whose lines
-// are whole 16-byte pieces (those that the kernel for small problems could take): within 4 to 9 %.
+// What the kernel for small problems competes with: the time of tiles of 128 columns wherever there are more than 64, shared by as many CTAs as fit beside one
+// another.  A start and an end, rounds of tiles and their k-blocks, and what sharing a reduction costs, fitted to graph replays of 500 calls whose lines are whole
+// 16-byte pieces (those that the kernel for small problems could take): within 4 to 9 %.  (Better tiles would take some of them from that kernel, which is the
+// more accurate one: bf16, K = 1024, 1.1e-7 and 1.9e-7.)
 double gather_estimate_us(const Problem &p, int num_sms) {
     if (too_small(p)) return 1e9;
     struct Cost { double ends, kb, round, shared; };
     constexpr Cost bf16[2][2] = {{{4.7, 0.75, 0.0, 1.0}, {6.0, 0.79, 3.0, 2.3}}, {{4.9, 1.21, 0.3, 2.1}, {6.2, 1.31, 0.0, 4.9}}};      // [convolution][128 columns]
     constexpr Cost f32[2][2] = {{{4.7, 1.27, 0.0, 1.2}, {5.4, 1.87, 2.9, 3.8}}, {{6.0, 1.51, 2.9, 2.9}, {6.8, 2.21, 6.5, 6.9}}};
-    const Tiles t = plan_tiles(p, num_sms);
+    Tiles t{p.N > 64 ? 128 : 64, (p.K + BK - 1) / BK, 1, 0, 0.0};
+    t.tiles = (int64_t)((p.M + BM - 1) / BM) * ((p.N + t.bn - 1) / t.bn);
+    while (t.splits < MAX_SPLIT && t.tiles * t.splits * 2 <= num_sms - 12 && t.num_kb >= t.splits * 8) t.splits *= 2;
     const Cost &c = (p.in_bf16 ? bf16 : f32)[p.spatial_rank != 0][t.bn == 128];
     const double rounds = t.splits > 1 ? 1.0 : (double)((t.tiles + num_sms - 1) / num_sms);
     return c.ends + (rounds - 1.0) * c.round + rounds * c.kb * (double)((t.num_kb + t.splits - 1) / t.splits) + (t.splits > 1 ? c.shared : 0.0);
 }
 
 sg_status launch_gather(const Problem &p, const void *In, const void *Flt, float *O, bool forced, cudaStream_t stream) {
-    if (!forced && too_small(p)) return SG_ERR_UNSUPPORTED;
     const bool conv = p.spatial_rank != 0;
     // offsets are 32-bit
     if (reach({{p.batch, p.i_n}, {(int64_t)(p.Ho - 1) * p.sh + (int64_t)(p.KH - 1) * p.dh + 1, p.i_h},
@@ -761,6 +782,8 @@ sg_status launch_gather(const Problem &p, const void *In, const void *Flt, float
     int dev = 0, num_sms = 0, pdl = -1, unused = 0;
     if (!tensor_device_info(&dev, &num_sms, &pdl, &unused)) return SG_ERR_CUDA;
 
+    const Tiles plan = plan_tiles(p, num_sms);
+    if (!forced && too_small(p)) return SG_ERR_UNSUPPORTED;
     GatherParams gp{};
     gp.p = p;
     const int es = p.in_bf16 ? 2 : 4;
@@ -779,7 +802,6 @@ sg_status launch_gather(const Problem &p, const void *In, const void *Flt, float
     gp.uniform_rows = (p.Ho == 1 || p.o_h == (int64_t)p.Wo * p.o_w) && (p.batch == 1 || p.o_n == (int64_t)p.Ho * p.Wo * p.o_w);
     gp.wait_prior = pdl == 0 ? 0 : 1;
 
-    const Tiles plan = plan_tiles(p, num_sms);
     const int bn = plan.bn;
     const int64_t tiles = plan.tiles;
     gp.num_kb = plan.num_kb;

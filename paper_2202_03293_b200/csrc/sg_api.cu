@@ -21,7 +21,7 @@ sg_status run(const Problem &p, const void *In, const void *Flt, float *O, cudaS
     if (p.M == 0 || p.N == 0) return SG_OK;                       // nothing to write
     if (p.K == 0 && (p.bias != nullptr || p.act != SG_ACT_NONE)) {
         // empty reduction under a fused consumer: act(bias), written by the CUDA-core kernel's write-back
-        if (launch_ffma(p, In, Flt, O, stream) != cudaSuccess) return SG_ERR_CUDA;
+        if (launch_ffma(p, In, Flt, O, true, stream) != cudaSuccess) return SG_ERR_CUDA;
         t_last_kernel = SG_KERNEL_FFMA;
         return SG_OK;
     }
@@ -58,7 +58,7 @@ sg_status run(const Problem &p, const void *In, const void *Flt, float *O, cudaS
         if (st == SG_OK) { t_last_kernel = SG_KERNEL_TENSOR; return SG_OK; }
         if (st != SG_ERR_UNSUPPORTED || force == SG_KERNEL_TENSOR) return st;
     }
-    if (launch_ffma(p, In, Flt, O, stream) != cudaSuccess) return SG_ERR_CUDA;
+    if (launch_ffma(p, In, Flt, O, force == SG_KERNEL_FFMA, stream) != cudaSuccess) return SG_ERR_CUDA;
     t_last_kernel = SG_KERNEL_FFMA;
     return SG_OK;
 }

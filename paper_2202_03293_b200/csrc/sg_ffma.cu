@@ -10,6 +10,8 @@
 // additive neutral 0 on load and predicated on store (Section 3.2).  The operand subset
 // of a tile is the image of the tile under the operand's indexing map, which for these
 // ops separates into a per-row offset plus a per-k offset (see Problem).
+#include <algorithm>
+
 #include "sg_internal.cuh"
 
 namespace sg {
@@ -222,6 +224,97 @@ ffma_kernel(Problem p, const T *__restrict__ In, const T *__restrict__ Flt, floa
     }
 }
 
+// The same contraction in 32 x 32 tiles, for outputs of few tiles of 128 x 128, where those leave most SMs idle and walk along k for long (16
+// values a microsecond).  A thread block fetches up to 128 values of k at once, every load in flight together, from tables of its rows' and its k's offsets;
+// four groups of 64 threads take every fourth k, four rows by four columns a thread, and their sums are added at the end (four
+// short sums are also more accurate than a long one).  Bound by the launch and two latencies (the tables and the loads); us here and in 128 x 128 tiles,
+// which reach along k at 16 values a microsecond: 127^3 f32 5.5 and 36.5, 55 x 97 x 81 4.9 and 24.9, 333 x 7 x 327 12 and 83, 1 x 29 x 29, 3x3x3x64 with stride 2 3.0 and
+// 11, 100 x 100 x 200 bf16 8.6 and 36.
+constexpr int ST = 32, SK = 128, SPITCH = ST + 4, RPITCH = ST + 8;      // tile, k of a fetch, floats between staged lines and between rows of partial sums
+
+// (plain pointers: a load of data that is declared constant may move ahead of griddepcontrol.wait)
+template <typename T>
+__global__ void __launch_bounds__(THREADS)
+ffma_small_kernel(Problem p, const T *In, const T *Flt, float *O, int a_along_k, int b_along_k, int wait_prior) {
+    __shared__ __align__(16) float tiles[2 * SK * SPITCH];      // As[k][m], Bs[k][f]; at the end the groups' sums
+    __shared__ int64_t row_in[ST], k_in[SK], k_flt[SK];
+    static_assert(4 * ST * RPITCH <= 2 * SK * SPITCH, "the groups' sums fit");
+    float *As = tiles, *Bs = tiles + SK * SPITCH;
+    asm volatile("griddepcontrol.launch_dependents;");
+    const int t = threadIdx.x, m0 = blockIdx.x * ST, n0 = blockIdx.y * ST;
+    if (t < ST) {
+        int64_t unused;
+        row_in[t] = 0;
+        if (m0 + t < p.M) row_offsets(p, m0 + t, row_in[t], unused);
+    }
+    const int group = t >> 6, ty = (t >> 3) & 7, tx = t & 7;
+    // (up to eight products are one sum: nothing to gain from four)
+    const int first_k = p.K > 8 ? group : group == 0 ? 0 : SK, step_k = p.K > 8 ? 4 : 1;
+    float acc[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+    if (wait_prior) asm volatile("griddepcontrol.wait;" ::: "memory");
+    for (int k0 = 0; k0 < p.K; k0 += SK) {
+        const int len = min(SK, p.K - k0);
+        const int shift = len > 64 ? 7 : len > 32 ? 6 : 5;      // threads along k: 128, 64 or 32
+        if (t < len) k_offsets(p, k0 + t, k_in[t], k_flt[t]);
+        __syncthreads();
+        // thread t fetches (k, x) pairs; x is a row of the tile, or a column
+        auto fetch = [&](const T *base, float *dst, int along_k, auto offset, int limit) {
+            const int ka = along_k ? t & ((1 << shift) - 1) : t >> 5, xa = along_k ? t >> shift : t & 31;
+            const int k_step = along_k ? 0 : THREADS / 32, x_step = along_k ? THREADS >> shift : 0;
+#pragma unroll 1
+            for (int i0 = 0; i0 < 1 << (shift - 3); i0 += 4) {
+                float v[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int k = ka + (i0 + i) * k_step, x = xa + (i0 + i) * x_step;
+                    v[i] = k < len && x < limit ? to_f32(base[offset(k, x)]) : 0.f;
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) dst[(ka + (i0 + i) * k_step) * SPITCH + xa + (i0 + i) * x_step] = v[i];
+            }
+        };
+        fetch(In, As, a_along_k, [&](int k, int m) { return row_in[m] + k_in[k]; }, min(ST, p.M - m0));
+        fetch(Flt, Bs, b_along_k, [&](int k, int f) { return k_flt[k] + (int64_t)(n0 + f) * p.k_f; }, min(ST, p.N - n0));
+        __syncthreads();
+#pragma unroll 4
+        for (int k = first_k; k < len; k += step_k) {
+            float a[4], b[4];
+            load4(As + k * SPITCH + ty * 4, a);
+            load4(Bs + k * SPITCH + tx * 4, b);
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        *reinterpret_cast<float4 *>(tiles + (group * ST + ty * 4 + i) * RPITCH + tx * 4) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+    __syncthreads();
+    const int row = t >> 3, m = m0 + row;
+    if (m >= p.M) return;
+    int64_t unused, out_off;
+    row_offsets(p, m, unused, out_off);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int col = (t & 7) + 8 * j, n = n0 + col;
+        if (n >= p.N) break;
+        float part[4];
+#pragma unroll
+        for (int g = 0; g < 4; ++g) part[g] = tiles[(g * ST + row) * RPITCH + col];
+        float v = (part[0] + part[1]) + (part[2] + part[3]);
+        if (p.bias != nullptr) v += p.bias[(int64_t)n * p.bias_f];
+        if (p.act == SG_ACT_RELU && v < 0.f) v = 0.f;
+        float *d = O + out_off + (int64_t)n * p.o_f;
+        *d = p.accumulate ? *d + v : v;
+    }
+}
+
 __global__ void zero_fill_kernel(Problem p, float *__restrict__ O) {
     asm volatile("griddepcontrol.launch_dependents;");   // a dependent launch waits for this grid's end where it needs the zeros
     int64_t total = (int64_t)p.M * p.N;
@@ -247,8 +340,20 @@ __global__ void zero_fill_rows_kernel(float *__restrict__ O, int M, int n4, int6
 
 inline bool mult_of(int64_t v, int64_t q) { return v % q == 0; }
 
+// Time in us of the two kernels, within 20 % of the timings of 40 calls: latencies of a fetch of 128 k and rounds of blocks; and rounds of tiles, 16 k at a time
+// (`vec`: both operands in 8- or 16-byte loads).  32 x 32 and 128 x 128: 511^3 f32 29 and 125, 1023^3 121 and 244, 333 x 4001 x 9 9.2 and 10.2, 1500 x 1500 x 100 34 and (vec) 20.
+double small_tiles_us(const Problem &p) {
+    const int rest = p.K % SK, k = p.K - rest + (rest > 64 ? 128 : rest > 32 ? 64 : rest > 0 ? 32 : 0);
+    const double blocks = (double)((p.M + ST - 1) / ST) * ((p.N + ST - 1) / ST);
+    return 1.9 + 0.027 * k + blocks * (0.0015 + 0.0001 * k);
+}
+double large_tiles_us(const Problem &p, bool vec) {
+    const int64_t tiles = (int64_t)((p.M + BM - 1) / BM) * ((p.N + BN - 1) / BN);
+    return 5.0 + (double)((tiles + 147) / 148) * ((p.K + BK - 1) / BK) * (vec ? 2.1 : 3.9);
+}
+
 template <typename T>
-cudaError_t launch_typed(const Problem &p, const T *In, const T *Flt, float *O, cudaStream_t stream) {
+cudaError_t launch_typed(const Problem &p, const T *In, const T *Flt, float *O, bool forced, cudaStream_t stream) {
     // 4 consecutive k (resp. f) may be fetched as one 8- or 16-byte load when they are
     // contiguous in memory and every address involved is a multiple of 4 elements.
     const uintptr_t vec_bytes = 4 * sizeof(T);
@@ -258,6 +363,26 @@ cudaError_t launch_typed(const Problem &p, const T *In, const T *Flt, float *O, 
                  mult_of(p.k_c, 4) && (reinterpret_cast<uintptr_t>(Flt) % vec_bytes == 0);
     int vec_c = p.o_f == 1 && mult_of(p.o_n, 4) && mult_of(p.o_h, 4) && mult_of(p.o_w, 4) &&
                 (reinterpret_cast<uintptr_t>(O) % 16 == 0);
+    // A caller who asks for this kernel by name gets 128 x 128 and one sum along k: the accuracy that the tensor-core kernels of these layouts are held against.
+    if (!forced && (p.N + ST - 1) / ST <= 65535 && small_tiles_us(p) < large_tiles_us(p, vec_a && vec_b)) {
+        int device, num_sms, pdl = 0, unused;
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute attr[1];
+        const int wait_prior = tensor_device_info(&device, &num_sms, &pdl, &unused) && pdl != 0;
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.gridDim = dim3((p.M + ST - 1) / ST, (p.N + ST - 1) / ST);
+        cfg.blockDim = dim3(THREADS);
+        cfg.stream = stream;
+        cfg.attrs = attr;
+        cfg.numAttrs = wait_prior ? 1 : 0;
+        // (a lane to each k, or to each row or column, whichever is contiguous in memory)
+        const int a_along_k = p.spatial_rank != 0 || p.i_c == 1 || p.i_w != 1, b_along_k = p.k_f != 1 && p.k_c == 1;
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, ffma_small_kernel<T>, p, In, Flt, O, a_along_k, b_along_k, wait_prior);
+        count_launch();
+        note_kernel("ffma_kernel");
+        return e;
+    }
     dim3 grid((p.M + BM - 1) / BM, (p.N + BN - 1) / BN);
     if (grid.y > 65535) return cudaErrorInvalidConfiguration;
     if (vec_a && vec_b) ffma_kernel<T, true, true><<<grid, THREADS, 0, stream>>>(p, In, Flt, O, vec_c);
@@ -271,10 +396,12 @@ cudaError_t launch_typed(const Problem &p, const T *In, const T *Flt, float *O, 
 
 }  // namespace
 
-cudaError_t launch_ffma(const Problem &p, const void *In, const void *Flt, float *O, cudaStream_t stream) {
+double ffma_estimate_us(const Problem &p) { return std::min(small_tiles_us(p), large_tiles_us(p, false)); }
+
+cudaError_t launch_ffma(const Problem &p, const void *In, const void *Flt, float *O, bool forced, cudaStream_t stream) {
     if (p.in_bf16)
-        return launch_typed(p, static_cast<const unsigned short *>(In), static_cast<const unsigned short *>(Flt), O, stream);
-    return launch_typed(p, static_cast<const float *>(In), static_cast<const float *>(Flt), O, stream);
+        return launch_typed(p, static_cast<const unsigned short *>(In), static_cast<const unsigned short *>(Flt), O, forced, stream);
+    return launch_typed(p, static_cast<const float *>(In), static_cast<const float *>(Flt), O, forced, stream);
 }
 
 cudaError_t launch_zero_fill(const Problem &p, float *O, cudaStream_t stream) {

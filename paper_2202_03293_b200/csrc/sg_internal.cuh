@@ -36,8 +36,10 @@ struct Problem {
 };
 
 // Launchers (each returns the cudaError_t of its launch).
-cudaError_t launch_ffma(const Problem &p, const void *In, const void *Flt, float *O,
+// `forced`: the caller asks for this kernel, which then runs in 128 x 128 tiles whatever the size.
+cudaError_t launch_ffma(const Problem &p, const void *In, const void *Flt, float *O, bool forced,
                         cudaStream_t stream);
+double ffma_estimate_us(const Problem &p);      // what it would take
 cudaError_t launch_zero_fill(const Problem &p, float *O, cudaStream_t stream);
 
 // Tensor-core path: returns SG_ERR_UNSUPPORTED (and launches nothing) when the layout

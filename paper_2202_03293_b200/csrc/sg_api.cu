@@ -27,7 +27,7 @@ sg_status run(const Problem &p, const void *In, const void *Flt, float *O, cudaS
     }
     if (p.K == 0) {                                               // empty reduction: the sum is 0
         if (p.accumulate) return SG_OK;
-        return launch_zero_fill(p, O, stream) == cudaSuccess ? SG_OK : SG_ERR_CUDA;
+        return launch_zero_fill(p, O, true, stream) == cudaSuccess ? SG_OK : SG_ERR_CUDA;
     }
     const int force = g_override.load();
     if (force == SG_KERNEL_AUTO) {

@@ -315,8 +315,15 @@ ffma_small_kernel(Problem p, const T *In, const T *Flt, float *O, int a_along_k,
     }
 }
 
-__global__ void zero_fill_kernel(Problem p, float *__restrict__ O) {
-    asm volatile("griddepcontrol.launch_dependents;");   // a dependent launch waits for this grid's end where it needs the zeros
+// The clearing kernels start while the kernel ahead drains, wait for its end (the output may be in its use), and let a dependent launch start at
+// once, which then knows that everything ahead has finished and waits for this grid's end where it needs the zeros.  (Launched behind the end of the kernel ahead,
+// they cost a split product 1.2 to 2 us more: 192 x 256 x 1920 f32 10.3, so 8.6, call by call.)
+__device__ __forceinline__ void clear_after_prior(int wait_prior) {
+    if (wait_prior) asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
+}
+__global__ void zero_fill_kernel(Problem p, float *__restrict__ O, int wait_prior) {
+    clear_after_prior(wait_prior);
     int64_t total = (int64_t)p.M * p.N;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
          i += (int64_t)gridDim.x * blockDim.x) {
@@ -329,8 +336,8 @@ __global__ void zero_fill_kernel(Problem p, float *__restrict__ O) {
 
 // The output as one M x N matrix of contiguous, 16-byte aligned rows `pitch` floats apart
 // (what the tensor-core path requires of it): four columns per thread.
-__global__ void zero_fill_rows_kernel(float *__restrict__ O, int M, int n4, int64_t pitch) {
-    asm volatile("griddepcontrol.launch_dependents;");
+__global__ void zero_fill_rows_kernel(float *__restrict__ O, int M, int n4, int64_t pitch, int wait_prior) {
+    clear_after_prior(wait_prior);
     const int64_t total = (int64_t)M * n4;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
         const int m = (int)(i / n4), c = (int)(i - (int64_t)m * n4);
@@ -339,6 +346,24 @@ __global__ void zero_fill_rows_kernel(float *__restrict__ O, int M, int n4, int6
 }
 
 inline bool mult_of(int64_t v, int64_t q) { return v % q == 0; }
+
+// Launches a kernel that (`overlap`) may start while the kernel ahead of it drains; its last argument says whether it then has to wait for that one.
+template <typename Kernel, typename... Args>
+cudaError_t launch_after(bool overlap, Kernel *kernel, dim3 grid, int block, cudaStream_t stream, Args... args) {
+    int device, num_sms, pdl = 0, unused;
+    const int wait_prior = overlap && tensor_device_info(&device, &num_sms, &pdl, &unused) && pdl != 0;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.stream = stream;
+    cfg.attrs = attr;
+    cfg.numAttrs = wait_prior ? 1 : 0;
+    count_launch();
+    return cudaLaunchKernelEx(&cfg, kernel, args..., wait_prior);
+}
 
 // Time in us of the two kernels, within 20 % of the timings of 40 calls: latencies of a fetch of 128 k and rounds of blocks; and rounds of tiles, 16 k at a time
 // (`vec`: both operands in 8- or 16-byte loads).  32 x 32 and 128 x 128: 511^3 f32 29 and 125, 1023^3 121 and 244, 333 x 4001 x 9 9.2 and 10.2, 1500 x 1500 x 100 34 and (vec) 20.
@@ -365,23 +390,10 @@ cudaError_t launch_typed(const Problem &p, const T *In, const T *Flt, float *O, 
                 (reinterpret_cast<uintptr_t>(O) % 16 == 0);
     // A caller who asks for this kernel by name gets 128 x 128 and one sum along k: the accuracy that the tensor-core kernels of these layouts are held against.
     if (!forced && (p.N + ST - 1) / ST <= 65535 && small_tiles_us(p) < large_tiles_us(p, vec_a && vec_b)) {
-        int device, num_sms, pdl = 0, unused;
-        cudaLaunchConfig_t cfg = {};
-        cudaLaunchAttribute attr[1];
-        const int wait_prior = tensor_device_info(&device, &num_sms, &pdl, &unused) && pdl != 0;
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.gridDim = dim3((p.M + ST - 1) / ST, (p.N + ST - 1) / ST);
-        cfg.blockDim = dim3(THREADS);
-        cfg.stream = stream;
-        cfg.attrs = attr;
-        cfg.numAttrs = wait_prior ? 1 : 0;
         // (a lane to each k, or to each row or column, whichever is contiguous in memory)
         const int a_along_k = p.spatial_rank != 0 || p.i_c == 1 || p.i_w != 1, b_along_k = p.k_f != 1 && p.k_c == 1;
-        const cudaError_t e = cudaLaunchKernelEx(&cfg, ffma_small_kernel<T>, p, In, Flt, O, a_along_k, b_along_k, wait_prior);
-        count_launch();
         note_kernel("ffma_kernel");
-        return e;
+        return launch_after(true, ffma_small_kernel<T>, dim3((p.M + ST - 1) / ST, (p.N + ST - 1) / ST), THREADS, stream, p, In, Flt, O, a_along_k, b_along_k);
     }
     dim3 grid((p.M + BM - 1) / BM, (p.N + BN - 1) / BN);
     if (grid.y > 65535) return cudaErrorInvalidConfiguration;
@@ -404,21 +416,17 @@ cudaError_t launch_ffma(const Problem &p, const void *In, const void *Flt, float
     return launch_typed(p, static_cast<const float *>(In), static_cast<const float *>(Flt), O, forced, stream);
 }
 
-cudaError_t launch_zero_fill(const Problem &p, float *O, cudaStream_t stream) {
+cudaError_t launch_zero_fill(const Problem &p, float *O, bool overlap, cudaStream_t stream) {
     const bool uniform_rows = p.o_f == 1 && (p.Ho == 1 || p.o_h == (int64_t)p.Wo * p.o_w) &&
                               (p.batch == 1 || p.o_n == (int64_t)p.Ho * p.Wo * p.o_w);
     if (uniform_rows && p.N % 4 == 0 && p.o_w % 4 == 0 && reinterpret_cast<uintptr_t>(O) % 16 == 0) {
         const int64_t work = (int64_t)p.M * (p.N / 4);
         const int blocks = (int)((work + 255) / 256 < 148 * 8 ? (work + 255) / 256 : 148 * 8);
-        zero_fill_rows_kernel<<<blocks, 256, 0, stream>>>(O, p.M, p.N / 4, p.o_w);
-        count_launch();
-        return cudaGetLastError();
+        return launch_after(overlap, zero_fill_rows_kernel, dim3(blocks), 256, stream, O, p.M, p.N / 4, p.o_w);
     }
     int64_t total = (int64_t)p.M * p.N;
     int blocks = (int)((total + 255) / 256 < 148 * 8 ? (total + 255) / 256 : 148 * 8);
-    zero_fill_kernel<<<blocks, 256, 0, stream>>>(p, O);
-    count_launch();
-    return cudaGetLastError();
+    return launch_after(overlap, zero_fill_kernel, dim3(blocks), 256, stream, p, O);
 }
 
 }  // namespace sg

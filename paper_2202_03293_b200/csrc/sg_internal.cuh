@@ -40,7 +40,8 @@ struct Problem {
 cudaError_t launch_ffma(const Problem &p, const void *In, const void *Flt, float *O, bool forced,
                         cudaStream_t stream);
 double ffma_estimate_us(const Problem &p);      // what it would take
-cudaError_t launch_zero_fill(const Problem &p, float *O, cudaStream_t stream);
+// `overlap`: the clearing may start while the kernel ahead drains.
+cudaError_t launch_zero_fill(const Problem &p, float *O, bool overlap, cudaStream_t stream);
 
 // Tensor-core path: returns SG_ERR_UNSUPPORTED (and launches nothing) when the layout
 // does not satisfy the TMA rules.

@@ -1558,7 +1558,7 @@ sg_status launch_tensor(const Problem &p, const void *In, const void *Flt, float
 
     // ---- tile variant and k split: lowest estimated time ----
     int pick, splits, meet;
-    choose_tiles(p, tp.num_kb, lay, ov, num_sms, &pick, &splits, &meet);
+    const double estimate = choose_tiles(p, tp.num_kb, lay, ov, num_sms, &pick, &splits, &meet);
     if (pick < 0) return SG_ERR_INTERNAL;
     const Variant &var = kVariants[pick];
     // bf16 matmuls with whole k-blocks move two k-blocks per stage and per TMA load
@@ -1637,9 +1637,10 @@ sg_status launch_tensor(const Problem &p, const void *In, const void *Flt, float
     // before its first global read or write.
     tp.wait_prior = ov.pdl == 0 ? 0 : 2;
     if (splits > 1 && !tp.meet) {
-        // partial sums meet in the output by TMA reduce-add: an overwriting call clears it first
+        // Partial sums meet in the output by TMA reduce-add: an overwriting call clears it first.  The clearing overlaps the kernel ahead in calls of up to
+        // 40 us; in longer ones, of pairs above all, its blocks are in the way when pairs are placed (832 x 2240 x 6208 f32 79 us, 82 so).
         if (!p.accumulate) {
-            if (launch_zero_fill(p, O, stream) != cudaSuccess) return SG_ERR_CUDA;
+            if (launch_zero_fill(p, O, estimate < 40e3, stream) != cudaSuccess) return SG_ERR_CUDA;
             tp.wait_prior = 1;      // the clearing kernel lets its dependents start at once: only the stores wait for it
         }
         tp.accumulate = 1;

@@ -46,7 +46,7 @@ sg_status run(const Problem &p, const void *In, const void *Flt, float *O, cudaS
     // Stride-1 convolutions whose filter fits in shared memory, where the im2col kernel does not take them, or bf16 with five taps and more, or
     // three of channels that it pads to 64.  Elsewhere that kernel is the better one (us, strip / im2col: bf16 5 taps of 40 channels
     // 4.3 / 5.1 and of 80 5.3 / 5.3, 3 of 40 6.7 / 8.8 and of 128 4.4 / 4.1, 1 of 48 24.3 / 21.2; f32 7 of 32 6.9 / 5.7, 1 of 256 84 / 46 and 10.7 / 5.9).
-    if (force == SG_KERNEL_CONV_STRIP || (force == SG_KERNEL_AUTO && (!tensor_takes(p, In, Flt, O) || (p.in_bf16 && p.KH * p.KW >= (p.C % 64 != 0 ? 3 : 5))))) {
+    if (force == SG_KERNEL_CONV_STRIP || (force == SG_KERNEL_AUTO && (!tensor_takes(p, In, Flt, O) || conv_strip_preferred(p)))) {
         const sg_status st = launch_conv_strip(p, In, Flt, O, false, stream);
         if (st == SG_OK) { t_last_kernel = SG_KERNEL_CONV_STRIP; return SG_OK; }
         if (st != SG_ERR_UNSUPPORTED || force == SG_KERNEL_CONV_STRIP) return st;

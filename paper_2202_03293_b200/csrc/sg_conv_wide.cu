@@ -554,11 +554,13 @@ inline bool plan_run(int bn, int KH, int row_span, int64_t full_span, Run *r) {
 // outputs go out at the block's share of the HBM rate; between the first run and the last write-back the slowest of run, MMAs and
 // write-back paces the rounds.  (Fitted to sweeps of 32 to 256 positions on nine shapes; the choices are within 4 % of the best
 // but for one 9 %.)
-void plan_bf16(const Problem &p, int64_t positions, int f_tiles, int row_span, int64_t full_span, int num_sms, WideParams &w) {
+// Returns the estimated time in microseconds of the tiles chosen, in which the write-back counts as well: 20 cycles a position, since only the two warps of a
+// quarter of the lanes write a filter (337 timings: within 9 % in the mean).
+double plan_bf16(const Problem &p, int64_t positions, int f_tiles, int row_span, int64_t full_span, int num_sms, WideParams &w) {
     const int kb = (p.C + 63) / 64, total_slots = kb * p.KH;
     const int flt_rows = kb > 1 ? 64 : (p.C + 15) / 16 * 16;           // channels of a filter block
     const int slot_bytes = p.KW * BF * 2 * flt_rows;
-    double best = 1e300;
+    double best = 1e300, us = 1e300;
     const int ksteps = (kb - 1) * 4 + ((p.C - (kb - 1) * 64) + 15) / 16;
     for (int bn = 32; bn <= 256; bn += 16) {
         Run r;
@@ -576,12 +578,15 @@ void plan_bf16(const Problem &p, int64_t positions, int f_tiles, int row_span, i
         const double cost = load + mma + (double)(rounds - 1) * std::max(mma, std::max(load, store)) + store + 300.0 * (double)rounds;
         if (cost >= best) continue;
         best = cost;
+        const double write = std::max(store, 20.0 * bn), further = (double)(rounds - 1);
+        us = 3.5 + 0.87 / 1900.0 * (load + mma + further * std::max(std::max(mma, load), write) + write + 300.0 * (double)rounds) + 0.38 * further;
         w.BN = bn; w.tiles = (int)tiles; w.run_boxes = r.boxes; w.box_rows = r.box_rows; w.run_bytes = (int)r.bytes; w.run_tx = (int)r.tx;
         w.slots = slots; w.resident = resident; w.per_row = r.per_row; w.bufs = 2;
     }
     w.kb = kb;
     w.slot_bytes = slot_bytes;
     w.last_ksteps = (p.C - (kb - 1) * 64 + 15) / 16;
+    return us;
 }
 
 // The same for the f32 kernel, whose slots share tensor memory with the accumulators.  Returns the estimated time in microseconds.
@@ -691,7 +696,14 @@ sg_status launch_conv_wide(const Problem &p, const void *In, const void *Flt, fl
         const double us = plan_f32(p, positions, f_tiles, row_span, full_span, num_sms, w, g);
         const bool strip = p.N <= 128 && p.N > 64 && mult(p.N, 32) && g.taps >= 3 && (int64_t)g.taps * w.kb <= 6;
         if (!forced && im2col && !strip && us >= 0.95 * tensor_estimate_us(p)) return SG_ERR_UNSUPPORTED;
-    } else plan_bf16(p, positions, f_tiles, row_span, full_span, num_sms, w);
+    } else {
+        // bf16: the im2col kernel where its estimate (5 % and 0.6 us low for convolutions) is clearly the lower one: 4 x 105 x 105, 5x5x64x96 24 us, here 48; 5 x 15 x 15,
+        // 5x5x128x96 7.5 and 11.7.  With this margin 35 of 243 convolutions that this kernel took for their shape alone are more than 5 % faster, and one slower.
+        // (Where the strip kernel would take over instead it is the slower one; single taps, which both kernels read once, and accumulating calls stay.)
+        const double us = plan_bf16(p, positions, f_tiles, row_span, full_span, num_sms, w);
+        if (!forced && im2col && !p.accumulate && p.KH * p.KW > 1 && us >= 1.15 * (0.63 + 1.05 * tensor_estimate_us(p)) &&
+            (!conv_strip_preferred(p) || launch_conv_strip(p, In, Flt, O, true, stream) != SG_OK)) return SG_ERR_UNSUPPORTED;
+    }
     if (w.BN == 0 || (int64_t)w.tiles * f_tiles > 0x7fffffff) return SG_ERR_UNSUPPORTED;
     w.row_step = w.per_row ? w.box_rows : (int)shift;
 

@@ -66,6 +66,8 @@ bool tensor_encode_tiled(CUtensorMap *map, CUtensorMapDataType type, int rank, v
 // Stride-1 convolutions with a resident filter (sg_conv.cu): SG_ERR_UNSUPPORTED when the
 // shape or layout does not qualify (nothing is launched then).  `ask`: only says whether it does.
 sg_status launch_conv_strip(const Problem &p, const void *In, const void *Flt, float *O, bool ask, cudaStream_t stream);
+// Whether the strip kernel goes ahead of the im2col kernel where both take a call.
+inline bool conv_strip_preferred(const Problem &p) { return p.in_bf16 && p.KH * p.KW >= (p.C % 64 != 0 ? 3 : 5); }
 sg_status conv_read_status(cudaStream_t stream);
 // Stride-1 convolutions with the filter as the M operand (sg_conv_wide.cu); same contract.
 // `forced`: also where other kernels are the better ones; *resident_filter reports whether the filter stays on the SM.

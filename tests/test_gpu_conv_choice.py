@@ -72,3 +72,18 @@ def test_wide_or_im2col(N, W, C, F, KW, kernel):
     want, S = ref.conv2d_nhwc_hwcf(i, k)
     assert assert_within_bound(O, want, S, "wide or im2col") < 4e-6
     sg.sg_check()
+
+
+# few positions and a long reduction: the im2col kernel deals it out over the SMs; many positions, or few filters that stay: the filter as the M operand
+@pytest.mark.parametrize("N,H,C,KH,F,kernel", [(5, 15, 128, 5, 96, "tc_gemm_kernel<bf16>"), (1, 31, 256, 3, 64, "tc_gemm_kernel<bf16>"), (16, 56, 64, 3, 128, "conv_wide_kernel<bf16>"), (29, 37, 32, 5, 32, "conv_wide_kernel<bf16>")])
+def test_im2col_or_filter_as_the_m_operand(N, H, C, KH, F, kernel):
+    I, i = operand((N, H + KH - 1, H + KH - 1, C), SEED, 31, "normal", "bf16")
+    K, k = operand((KH, KH, C, F), SEED, 32, "normal", "bf16")
+    O = torch.full((N, H, H, F), float("nan"), device="cuda")
+    sg.sg_conv2d_nhwc_hwcf(I, K, O)
+    torch.cuda.synchronize()
+    assert sg.sg_last_kernel_name() == kernel
+    want = torch.nn.functional.conv2d(I[:2].double().permute(0, 3, 1, 2), K.double().permute(3, 2, 0, 1)).permute(0, 2, 3, 1)
+    S = torch.nn.functional.conv2d(I[:2].double().abs().permute(0, 3, 1, 2), K.double().abs().permute(3, 2, 0, 1)).permute(0, 2, 3, 1)
+    assert ((O[:2].double() - want).abs() <= 4e-6 * S).all()      # the truncating sum of up to 3200 products
+    sg.sg_check()

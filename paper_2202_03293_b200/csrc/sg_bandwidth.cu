@@ -7,9 +7,12 @@
 //
 // All four are bound by HBM traffic; the kernels differ in how they keep enough bytes in flight.
 //   - Copy2D and Transpose2D, when the layout meets the TMA rules (unit column stride, 16-byte
-//     aligned bases and row pitches), move tiles with TMA only: a persistent CTA per SM slot runs
-//     a shared-memory ring that one thread fills with tensor loads and another drains with tensor
-//     stores.  The copy never touches the data with an ordinary instruction; the transpose has
+//     aligned bases and row pitches), move tiles with TMA only, one tile per thread block, and as many
+//     blocks as there are tiles.  Blocks start in order as others end, so what is in flight is one
+//     window that advances through both tensors; persistent blocks, each with a ring of tiles, drift
+//     apart, and the two streams then meet in the same DRAM pages less often (16384 x 12288 bf16:
+//     copy 133 us with a ring per SM, so 117; transpose 143, so 123).
+//     The copy never touches the data with an ordinary instruction; the transpose has
 //     four warps turn each 128-row tile around in shared memory between the load and the store
 //     (4-byte elements: 16-byte reads of the 128-byte swizzled input tile, a register transpose
 //     of a 4 x 4 block, 16-byte writes into the swizzled output tile; 2-byte elements: 8 x 8
@@ -47,88 +50,56 @@ __device__ __forceinline__ void start_dependents() { asm volatile("griddepcontro
 __device__ __forceinline__ void wait_for_prior() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // ------------------------------------------------------------------------------ Copy2D (TMA)
-#ifndef SG_CP_STAGES
-#define SG_CP_STAGES 6
-#endif
-#ifndef SG_CP_STORES_IN_FLIGHT
-#define SG_CP_STORES_IN_FLIGHT 2
-#endif
-#ifndef SG_CP_STAGE_BYTES
-#define SG_CP_STAGE_BYTES 32768
-#endif
-#ifndef SG_CP_CTAS_PER_SM
-#define SG_CP_CTAS_PER_SM 1
-#endif
-#ifndef SG_CP_BOX_X
-#define SG_CP_BOX_X 256
-#endif
-constexpr int CP_STAGES = SG_CP_STAGES;                         // ring depth
-constexpr int CP_STORES_IN_FLIGHT = SG_CP_STORES_IN_FLIGHT;     // stores whose shared-memory reads may be pending
-constexpr int CP_STAGE_BYTES = SG_CP_STAGE_BYTES;
-constexpr int CP_CTAS_PER_SM = SG_CP_CTAS_PER_SM;
-static_assert(CP_STAGES > CP_STORES_IN_FLIGHT + 1, "the ring must leave room for loads");
+constexpr int CP_BOX_X = 256;             // elements of a row in a box
+// Bytes of a box and thread blocks of one box each that an SM holds: 64 KB in flight per SM.  Fewer leave the memory idle, more of
+// them only widen the window (16384 x 12288 bf16 / 2112 x 5952 bf16 / 640 x 15360 bf16: 5 blocks 125.6 / 9.8 / 7.7 us, 8 blocks 116.6 /
+// 8.75 / 6.9, 16 blocks 118.4 / 8.7 / 6.9, 24 blocks 119.0 / 9.2 / 7.9; a ring of 32 KB stages per SM 133.4 / 9.6 / 7.7); 250 x 960 f32
+// 2.3 -> 1.8.  4 and 16 KB boxes in blocks of several: 1 to 10 % slower.
+constexpr int CP_BOX_BYTES = 8192;
+constexpr int CP_CTAS_PER_SM = 8;
 
-// Tiles are dealt round-robin to the CTAs; warp 0 loads, warp 1 stores, one lane each.
-__global__ void __launch_bounds__(64) copy_tma_kernel(const __grid_constant__ CUtensorMap map_src,
-                                                       const __grid_constant__ CUtensorMap map_dst, int tiles_x, int num_tiles,
-                                                       int box_x, int box_y, uint32_t box_bytes) {
+// One box per thread block: bound by HBM (16384 x 12288: 6.9 TB/s).
+__global__ void __launch_bounds__(32) copy_tma_kernel(const __grid_constant__ CUtensorMap map_src, const __grid_constant__ CUtensorMap map_dst,
+                                                       int tiles_x, int box_x, int box_y, uint32_t box_bytes) {
     extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t full_bar[CP_STAGES], empty_bar[CP_STAGES];
-    __shared__ int abort_load, abort_store;
+    __shared__ uint64_t full_bar;
+    __shared__ int abort_load;
     start_dependents();
-    const uint32_t ring = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < CP_STAGES; ++s) { mbar_init(smem_u32(&full_bar[s]), 1); mbar_init(smem_u32(&empty_bar[s]), 1); }
-        abort_load = 0; abort_store = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    if (threadIdx.x != 0) return;
+    const uint32_t box = (smem_u32(smem_raw) + 127u) & ~127u, bar = smem_u32(&full_bar);
+    const int ty = (int)blockIdx.x / tiles_x, x = ((int)blockIdx.x - ty * tiles_x) * box_x, y = ty * box_y;
+    mbar_init(bar, 1);
+    abort_load = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    prefetch_tensormap(&map_src);
+    prefetch_tensormap(&map_dst);
+    wait_for_prior();
+    mbar_expect_tx(bar, box_bytes);
+    tma_load_2d(box, &map_src, bar, x, y);
+    if (!mbar_wait(bar, 0, &abort_load)) {
+        mbar_drain(bar, 0);        // gave up: let the load land
+        return;
     }
-    __syncthreads();
-    if (warp == 0 && lane == 0) {
-        prefetch_tensormap(&map_src);
-        wait_for_prior();
-        int k = 0;
-        for (int t = blockIdx.x; t < num_tiles; t += gridDim.x, ++k) {
-            const int s = k % CP_STAGES;
-            const uint32_t ph = (uint32_t)(k / CP_STAGES) & 1u;
-            if (!mbar_wait(smem_u32(&empty_bar[s]), ph ^ 1u, &abort_load)) break;
-            mbar_expect_tx(smem_u32(&full_bar[s]), box_bytes);
-            tma_load_2d(ring + (uint32_t)s * CP_STAGE_BYTES, &map_src, smem_u32(&full_bar[s]), (t % tiles_x) * box_x, (t / tiles_x) * box_y);
-        }
-        if (abort_load)   // gave up: let the loads already issued land
-            for (int j = (k > CP_STAGES ? k - CP_STAGES : 0); j < k; ++j) mbar_drain(smem_u32(&full_bar[j % CP_STAGES]), (uint32_t)(j / CP_STAGES) & 1u);
-    } else if (warp == 1 && lane == 0) {
-        prefetch_tensormap(&map_dst);
-        wait_for_prior();
-        int k = 0;
-        for (int t = blockIdx.x; t < num_tiles; t += gridDim.x, ++k) {
-            const int s = k % CP_STAGES;
-            const uint32_t ph = (uint32_t)(k / CP_STAGES) & 1u;
-            if (!mbar_wait(smem_u32(&full_bar[s]), ph, &abort_store)) break;
-            tma_store_2d(&map_dst, ring + (uint32_t)s * CP_STAGE_BYTES, (t % tiles_x) * box_x, (t / tiles_x) * box_y);
-            bulk_commit();
-            if (k >= CP_STORES_IN_FLIGHT) {   // the store issued CP_STORES_IN_FLIGHT tiles ago has read its stage
-                bulk_wait_read<CP_STORES_IN_FLIGHT>();
-                mbar_arrive(smem_u32(&empty_bar[(k - CP_STORES_IN_FLIGHT) % CP_STAGES]));
-            }
-        }
-        bulk_wait_read<0>();      // the ring must stay until the last stores have read it; the grid's end completes the writes
-    }
-    __syncthreads();
+    tma_store_2d(&map_dst, box, x, y);
+    bulk_commit();
+    bulk_wait_read<0>();           // the box must stay until the store has read it; the grid's end completes the write
 }
 
 // ------------------------------------------------------------------------- Transpose2D (TMA)
-// One tile = 128 input rows x 128 bytes (W = 128/ES columns).  Input stage: the tile as TMA wrote
-// it with the 128-byte swizzle (16-byte chunk index XOR row mod 8).  Output staging: the W x 128
-// transposed tile as 128/W blocks of [W rows][128 bytes], same swizzle, stored by four tensor
-// stores of 32 rows each (one per transposer warp, which also produces exactly those rows).
-#ifndef SG_TR_PANEL
-#define SG_TR_PANEL 8
-#endif
-constexpr int TR_PANEL = SG_TR_PANEL;     // tile columns per panel of the tile order
-constexpr int TR_IN_STAGES = 4;
+// One tile = 128 input rows x 128 bytes (W = 128/ES columns), one tile per thread block.  The tile arrives as TMA writes it with
+// the 128-byte swizzle (16-byte chunk index XOR row mod 8) and is turned around in place: the W x 128 transposed tile as 128/W
+// blocks of [W rows][128 bytes], same swizzle, stored by four tensor stores of 32 rows each (one per warp, which also produces
+// exactly those rows).  Bound by HBM and by the 128-byte rows of the requests (16384 x 12288: 6.5 TB/s).
+constexpr int TR_PANEL = 8;               // tile columns per panel of the tile order (2: 126.0, 4: 125.3, 8: 123.4, 16: 124.8 us)
 constexpr int TR_TILE_BYTES = 16384;
-constexpr int TR_THREADS = 32 + 128;
+constexpr int TR_THREADS = 128;
+// Thread blocks that an SM holds.  A tensor far beyond the caches wants a narrow window, one that the L2 absorbs as many tiles in flight
+// as help (4 / 5 / 6 / 8 / 12 blocks: 16384 x 12288 bf16 135 / 123.4 / 125.3 / 127.5 / 129.1 us, 4736 x 3456 f32 25.1 / 23.0 / 22.9 / 23.1 / 23.3,
+// 12288 x 512 f32 11.5 / 10.7 / 10.0 / 9.4 / 9.3, 640 x 15360 bf16 8.8 / 8.3 / 7.9 / 7.5 / 7.7; rings of four tiles, two per SM: 143 / 25.0 /
+// 10.1 / 8.0).
+inline int transpose_ctas_per_sm(int64_t bytes) { return bytes >= ((int64_t)64 << 20) ? 5 : 8; }
+// dynamic shared memory of a block that needs `least` bytes, so that an SM holds `ctas` of them (228 KB, 1 KB of it taken per block)
+inline int smem_for(int ctas, int least) { return std::max(least, (228 * 1024 / ctas - 1200) & ~127); }
 
 // 4 x 4 block of 4-byte elements held as four 16-byte rows: the transpose is a renaming of registers.
 __device__ __forceinline__ void transpose_block(const uint4 (&v)[4], uint4 (&o)[4]) {
@@ -153,117 +124,94 @@ template <int ES>
 __global__ void __launch_bounds__(TR_THREADS) transpose_tma_kernel(const __grid_constant__ CUtensorMap map_src,
                                                                     const __grid_constant__ CUtensorMap map_dst, int tiles_c,
                                                                     int tiles_r, int panel, int dst_cols, int dst_rows) {
-    const int num_tiles = tiles_c * tiles_r;
-    constexpr int E = 16 / ES;       // elements per 16-byte chunk = side of the register block
     constexpr int W = 128 / ES;      // input columns per tile = output rows per tile
-    constexpr int P = 128 / E;       // row groups per tile
     extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t full_bar[TR_IN_STAGES], empty_bar[TR_IN_STAGES];
-    __shared__ int abort_load, abort_turn;
+    __shared__ uint64_t full_bar;
+    __shared__ int abort_turn;
     start_dependents();
-    const uint32_t in_ring = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    const uint32_t out_ring = in_ring + TR_IN_STAGES * TR_TILE_BYTES;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t tile = (smem_u32(smem_raw) + 1023u) & ~1023u, bar = smem_u32(&full_bar);
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    int tr, tc;
+    tile_coords(blockIdx.x, tiles_c, tiles_r, panel, tr, tc);
     if (threadIdx.x == 0) {
-        for (int s = 0; s < TR_IN_STAGES; ++s) { mbar_init(smem_u32(&full_bar[s]), 1); mbar_init(smem_u32(&empty_bar[s]), 4); }
-        abort_load = 0; abort_turn = 0;
+        mbar_init(bar, 1);
+        abort_turn = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        prefetch_tensormap(&map_src);
+        wait_for_prior();
+        mbar_expect_tx(bar, TR_TILE_BYTES);
+        tma_load_2d(tile, &map_src, bar, tc * W, tr * 128);
+        prefetch_tensormap(&map_dst);
     }
     __syncthreads();
-    if (warp == 0) {
-        if (lane == 0) {
-            prefetch_tensormap(&map_src);
-            wait_for_prior();
-            int k = 0;
-            for (int t = blockIdx.x; t < num_tiles; t += gridDim.x, ++k) {
-                const int s = k % TR_IN_STAGES;
-                const uint32_t ph = (uint32_t)(k / TR_IN_STAGES) & 1u;
-                if (!mbar_wait(smem_u32(&empty_bar[s]), ph ^ 1u, &abort_load)) break;
-                mbar_expect_tx(smem_u32(&full_bar[s]), TR_TILE_BYTES);
-                int tr, tc;
-                tile_coords(t, tiles_c, tiles_r, panel, tr, tc);
-                tma_load_2d(in_ring + (uint32_t)s * TR_TILE_BYTES, &map_src, smem_u32(&full_bar[s]), tc * W, tr * 128);
-            }
-            if (abort_load)
-                for (int j = (k > TR_IN_STAGES ? k - TR_IN_STAGES : 0); j < k; ++j)
-                    mbar_drain(smem_u32(&full_bar[j % TR_IN_STAGES]), (uint32_t)(j / TR_IN_STAGES) & 1u);
+    wait_for_prior();
+    const bool ok = mbar_wait(bar, 0, &abort_turn);
+    if (!__syncthreads_and(ok)) {
+        mbar_drain(bar, 0);          // gave up: let the load land
+        return;
+    }
+    // Warp w owns store w of the tile: the 32 output rows x 128 bytes at offset w * 4 KB, which it makes of input rows 32w .. 32w+31,
+    // all 32 columns (4-byte elements), or of rows 64(w/2) .. +63, columns 32(w%2) .. +31 (2-byte elements).
+    const int b = w / (W / 32), h = w % (W / 32);
+    if constexpr (ES == 2) {
+        // 2-byte elements: the matrix load/store instructions do the turn.  Instruction i handles input rows
+        // 8p .. 8p+7 (p = 8b + i) of the warp's four chunks: ldmatrix.trans hands every lane two consecutive
+        // elements of a transposed 8 x 8 block per chunk, stmatrix writes those blocks as 16-byte rows.  In both,
+        // the eight row addresses of a block fall on eight different swizzled chunks: no bank conflicts.
+        const int m = lane >> 3, rr = lane & 7;           // this lane addresses row rr of block m
+        const int qm = 4 * h + m;                         // chunk of block m
+        const int c = 8 * qm + rr;                        // output row this lane addresses
+        uint32_t r[8][4];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int row = 8 * (8 * b + i) + rr;
+            const uint32_t src_addr = tile + (uint32_t)row * 128u + (uint32_t)((qm ^ rr) << 4);
+            asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                         : "=r"(r[i][0]), "=r"(r[i][1]), "=r"(r[i][2]), "=r"(r[i][3]) : "r"(src_addr) : "memory");
+        }
+        __syncthreads();             // the two warps of a half read what each of them overwrites
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const uint32_t dst_addr = tile + (uint32_t)b * (uint32_t)(W * 128) + (uint32_t)c * 128u + (uint32_t)((i ^ (c & 7)) << 4);
+            asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};"
+                         ::"r"(dst_addr), "r"(r[i][0]), "r"(r[i][1]), "r"(r[i][2]), "r"(r[i][3]) : "memory");
         }
     } else {
-        // Warp w owns store w of every tile: the 32 output rows x 128 bytes that sit at staging offset w * 4 KB.  What it
-        // reads for them (f32: input rows 32w .. 32w+31, all 32 columns; 2-byte elements: rows 64(w/2) .. +63, columns
-        // 32(w%2) .. +31) nobody else reads, so the four warps never wait for one another.
-        const int w = warp - 1;
-        if (lane == 0) prefetch_tensormap(&map_dst);
-        wait_for_prior();
-        // each lane turns E x E blocks (row group p, 16-byte chunk q); a quarter-warp covers two row groups x four chunks
-        const int q = ES == 4 ? ((lane & 3) | ((lane >> 1) & 4)) : (4 * (w & 1) + (lane & 3));
-        const int p0 = ES == 4 ? (8 * w + ((lane >> 2) & 1) + 2 * ((lane >> 4) & 1)) : (8 * (w >> 1) + (lane >> 2));
-        constexpr int BLOCKS_PER_LANE = ES == 4 ? 2 : 1;
-        const int b = w / (W / 32), h = w % (W / 32);
-        int k = 0;
-        for (int t = blockIdx.x; t < num_tiles; t += gridDim.x, ++k) {
-            const int s = k % TR_IN_STAGES;
-            const uint32_t ph = (uint32_t)(k / TR_IN_STAGES) & 1u;
-            const bool ok = mbar_wait(smem_u32(&full_bar[s]), ph, &abort_turn);
-            if (!__all_sync(0xffffffffu, ok)) break;
-            if (lane == 0) bulk_wait_read<1>();                        // this warp's store from two tiles ago has read its staging
-            __syncwarp();
-            const uint32_t in_tile = in_ring + (uint32_t)s * TR_TILE_BYTES;
-            const uint32_t out_tile = out_ring + (uint32_t)(k & 1) * TR_TILE_BYTES;
-            if constexpr (ES == 2) {
-                // 2-byte elements: the matrix load/store instructions do the turn.  Instruction i handles input rows
-                // 8p .. 8p+7 (p = 8b + i) of the warp's four chunks: ldmatrix.trans hands every lane two consecutive
-                // elements of a transposed 8 x 8 block per chunk, stmatrix writes those blocks as 16-byte rows.  In both,
-                // the eight row addresses of a block fall on eight different swizzled chunks: no bank conflicts.
-                const int m = lane >> 3, rr = lane & 7;           // this lane addresses row rr of block m
-                const int qm = 4 * h + m;                         // chunk of block m
-                const int c = 8 * qm + rr;                        // output row this lane addresses
+        // each lane turns two 4 x 4 blocks (row group p, 16-byte chunk q); a quarter-warp covers two row groups x four chunks
+        const int q = (lane & 3) | ((lane >> 1) & 4);
+        const int p0 = 8 * w + ((lane >> 2) & 1) + 2 * ((lane >> 4) & 1);
+        uint4 v[2][4];
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const int row = 8 * (8 * b + i) + rr;
-                    const uint32_t src_addr = in_tile + (uint32_t)row * 128u + (uint32_t)((qm ^ rr) << 4);
-                    uint32_t r0, r1, r2, r3;
-                    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
-                                 : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3) : "r"(src_addr));
-                    const uint32_t dst_addr = out_tile + (uint32_t)b * (uint32_t)(W * 128) + (uint32_t)c * 128u + (uint32_t)((i ^ (c & 7)) << 4);
-                    asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};"
-                                 ::"r"(dst_addr), "r"(r0), "r"(r1), "r"(r2), "r"(r3) : "memory");
-                }
-            } else {
+        for (int i = 0; i < 2; ++i)
 #pragma unroll
-                for (int i = 0; i < BLOCKS_PER_LANE; ++i) {
-                    const int p = p0 + 4 * i;
-                    uint4 v[E], o[E];
-#pragma unroll
-                    for (int kk = 0; kk < E; ++kk) {
-                        const int row = E * p + kk;
-                        const uint32_t addr = in_tile + (uint32_t)row * 128u + (uint32_t)((q ^ (row & 7)) << 4);
-                        asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v[kk].x), "=r"(v[kk].y), "=r"(v[kk].z), "=r"(v[kk].w) : "r"(addr));
-                    }
-                    transpose_block(v, o);
-#pragma unroll
-                    for (int j = 0; j < E; ++j) {
-                        const int c = E * q + j;                       // output row within the tile
-                        const uint32_t addr = out_tile + (uint32_t)(p >> 3) * (uint32_t)(W * 128) + (uint32_t)c * 128u +
-                                              (uint32_t)(((p & 7) ^ (c & 7)) << 4);
-                        asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(o[j].x), "r"(o[j].y), "r"(o[j].z), "r"(o[j].w) : "memory");
-                    }
-                }
+            for (int kk = 0; kk < 4; ++kk) {
+                const int row = 4 * (p0 + 4 * i) + kk;
+                const uint32_t addr = tile + (uint32_t)row * 128u + (uint32_t)((q ^ (row & 7)) << 4);
+                asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                             : "=r"(v[i][kk].x), "=r"(v[i][kk].y), "=r"(v[i][kk].z), "=r"(v[i][kk].w) : "r"(addr) : "memory");
             }
-            fence_async_smem();                                        // staging writes -> visible to the tensor store
-            __syncwarp();
-            if (lane == 0) {
-                mbar_arrive(smem_u32(&empty_bar[s]));                  // this warp is done with the input stage
-                int tr, tc;
-                tile_coords(t, tiles_c, tiles_r, panel, tr, tc);
-                const int x = tr * 128 + b * W, y = tc * W + h * 32;
-                if (x < dst_cols && y < dst_rows) tma_store_2d(&map_dst, out_tile + (uint32_t)w * 4096u, x, y);
-                bulk_commit();
+        __syncwarp();                // (what this warp overwrites nobody else reads)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const int p = p0 + 4 * i;
+            uint4 o[4];
+            transpose_block(v[i], o);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int c = 4 * q + j;                   // output row within the tile
+                const uint32_t addr = tile + (uint32_t)(p >> 3) * (uint32_t)(W * 128) + (uint32_t)c * 128u + (uint32_t)(((p & 7) ^ (c & 7)) << 4);
+                asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(o[j].x), "r"(o[j].y), "r"(o[j].z), "r"(o[j].w) : "memory");
             }
         }
-        if (lane == 0) bulk_wait_read<0>();
     }
-    __syncthreads();
+    fence_async_smem();              // tile writes -> visible to the tensor store
+    __syncwarp();
+    if (lane == 0) {
+        const int x = tr * 128 + b * W, y = tc * W + h * 32;
+        if (x < dst_cols && y < dst_rows) tma_store_2d(&map_dst, tile + (uint32_t)w * 4096u, x, y);
+        bulk_commit();
+        bulk_wait_read<0>();
+    }
 }
 
 // ------------------------------------------------------------------------- strided mover
@@ -811,10 +759,6 @@ cudaError_t launch_tile_move(const U *src, int64_t s_i, int64_t s_j, U *dst, int
     return launch_straight(src, s_i, s_j, dst, d_i, d_j, R, C, num_sms, stream, nullptr, nullptr, 0);
 }
 
-// device on which each kernel's shared-memory limit was last raised (the attribute is per device)
-int g_attr_copy = -1, g_attr_tr4 = -1, g_attr_tr2 = -1;
-inline int current_device() { int d = 0; cudaGetDevice(&d); return d; }
-
 }  // namespace
 
 sg_status launch_move2d(bool transpose, int64_t R, int64_t C, const void *src, int64_t s_r, int64_t s_c, void *dst, int64_t d_r,
@@ -833,15 +777,21 @@ sg_status launch_move2d(bool transpose, int64_t R, int64_t C, const void *src, i
     const int64_t inner = transpose ? R : C;             // extent of the destination's contiguous dimension
     const int64_t body = inner - inner % vec, tail = inner - body;
     if (tma_ok && body > 0 && (tail == 0 || force != 2)) {
-        const int64_t Rb = transpose ? body : R, Cb = transpose ? C : body;      // the source part the TMA kernel moves
+        int64_t Rb = transpose ? body : R, Cb = transpose ? C : body;      // the source part the TMA kernel moves
         bool launched = false;
         CUtensorMap map_src, map_dst;
         cuuint64_t st_src[1] = {(cuuint64_t)(s_r * esize)}, st_dst[1] = {(cuuint64_t)(d_r * esize)};
         if (!transpose) {
-            // box: up to 256 elements wide, as many rows as fit a 32 KB stage
-            const int box_x = (int)std::min<int64_t>(SG_CP_BOX_X, Cb);
-            int box_y = (int)std::min<int64_t>(std::min<int64_t>(256, CP_STAGE_BYTES / (box_x * esize)), Rb);
-            // (a small tensor: rather a box per SM than whole stages; 250 x 960 f32 2.75 -> 2.1 us)
+            // dense on both sides: one run of memory, in rows of 256 elements
+            if ((R == 1 || (s_r == C && d_r == C)) && (R * C) % CP_BOX_X == 0 && R * C / CP_BOX_X < 0x7fffffff) {
+                Rb = R * C / CP_BOX_X;
+                Cb = CP_BOX_X;
+                st_src[0] = st_dst[0] = (cuuint64_t)(CP_BOX_X * esize);
+            }
+            // box: up to 256 elements wide, as many rows as CP_BOX_BYTES hold
+            const int box_x = (int)std::min<int64_t>(CP_BOX_X, Cb);
+            int box_y = (int)std::min<int64_t>(std::min<int64_t>(256, CP_BOX_BYTES / (box_x * esize)), Rb);
+            // (a small tensor: rather a box per SM than whole boxes)
             while (box_y > 4 && ((Cb + box_x - 1) / box_x) * ((Rb + box_y - 1) / box_y) < num_sms) box_y = (box_y + 1) / 2;
             cuuint64_t dims[2] = {(cuuint64_t)Cb, (cuuint64_t)Rb};
             cuuint32_t box[2] = {(cuuint32_t)box_x, (cuuint32_t)box_y};
@@ -851,15 +801,9 @@ sg_status launch_move2d(bool transpose, int64_t R, int64_t C, const void *src, i
                                     CU_TENSOR_MAP_L2_PROMOTION_L2_256B) &&
                 tensor_encode_tiled(&map_dst, type, 2, dst, dims, st_dst, box, CU_TENSOR_MAP_SWIZZLE_NONE,
                                     CU_TENSOR_MAP_L2_PROMOTION_L2_256B)) {
-                const int smem = CP_STAGES * CP_STAGE_BYTES + 1024;
-                const int dev = current_device();
-                if (g_attr_copy != dev) {
-                    if (cudaFuncSetAttribute(copy_tma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return SG_ERR_CUDA;
-                    g_attr_copy = dev;
-                }
-                const int num_tiles = (int)(tiles_x * tiles_y);
-                if (launch_overlapped(copy_tma_kernel, dim3(std::min(num_tiles, CP_CTAS_PER_SM * num_sms)), 64, smem, 1, stream, map_src, map_dst, (int)tiles_x,
-                                      num_tiles, box_x, box_y, (uint32_t)(box_x * box_y * esize)) != cudaSuccess) return SG_ERR_CUDA;
+                const uint32_t box_bytes = (uint32_t)(box_x * box_y * esize);
+                if (launch_overlapped(copy_tma_kernel, dim3((unsigned)(tiles_x * tiles_y)), 32, smem_for(CP_CTAS_PER_SM, CP_BOX_BYTES + 128), 1, stream,
+                                      map_src, map_dst, (int)tiles_x, box_x, box_y, box_bytes) != cudaSuccess) return SG_ERR_CUDA;
                 launched = true;
             }
         } else {
@@ -872,20 +816,9 @@ sg_status launch_move2d(bool transpose, int64_t R, int64_t C, const void *src, i
                                     CU_TENSOR_MAP_L2_PROMOTION_L2_128B) &&
                 tensor_encode_tiled(&map_dst, type, 2, dst, dims_d, st_dst, box_d, CU_TENSOR_MAP_SWIZZLE_128B,
                                     CU_TENSOR_MAP_L2_PROMOTION_L2_128B)) {
-                const int smem = (TR_IN_STAGES + 2) * TR_TILE_BYTES + 1024;
-                int &attr = esize == 4 ? g_attr_tr4 : g_attr_tr2;
-                const int dev = current_device();
-                if (attr != dev) {
-                    const cudaError_t e = esize == 4
-                        ? cudaFuncSetAttribute(transpose_tma_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)
-                        : cudaFuncSetAttribute(transpose_tma_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-                    if (e != cudaSuccess) return SG_ERR_CUDA;
-                    attr = dev;
-                }
-                const int num_tiles = (int)(tiles_c * tiles_r);
-                const int grid = std::min(num_tiles, 2 * num_sms);
+                const int smem = smem_for(transpose_ctas_per_sm(R * C * esize), TR_TILE_BYTES + 1024);
                 const int panel = (int)std::min<int64_t>(tiles_c, TR_PANEL);
-                if (launch_overlapped(esize == 4 ? transpose_tma_kernel<4> : transpose_tma_kernel<2>, dim3(grid), TR_THREADS, smem, 1, stream, map_src, map_dst,
+                if (launch_overlapped(esize == 4 ? transpose_tma_kernel<4> : transpose_tma_kernel<2>, dim3((unsigned)(tiles_c * tiles_r)), TR_THREADS, smem, 1, stream, map_src, map_dst,
                                       (int)tiles_c, (int)tiles_r, panel, (int)Rb, (int)Cb) != cudaSuccess) return SG_ERR_CUDA;
                 launched = true;
             }

@@ -1,0 +1,40 @@
+"""Copies of dense tensors, which move as rows of 256 elements, and transposes on both sides of the size from which fewer tiles
+are in flight: bit patterns come out unchanged and nothing around the destination is written."""
+import pytest
+import torch
+
+from paper_2202_03293_b200 import binding as sg
+
+pytestmark = pytest.mark.gpu
+FILL = -7
+
+
+def run(op, R, C, dtype, src_pitch, dst_pitch):
+    bits = torch.int16 if dtype == torch.bfloat16 else torch.int32
+    n_r, n_c = (C, R) if op == "transpose" else (R, C)
+    g = torch.Generator(device="cuda").manual_seed(R * 31 + C)
+    src = torch.randint(-30000, 30000, (R, src_pitch), dtype=bits, device="cuda", generator=g)
+    dst = torch.full((n_r + 1, dst_pitch), FILL, dtype=bits, device="cuda")
+    (sg.sg_transpose2d if op == "transpose" else sg.sg_copy2d)(src.view(dtype)[:, :C], dst.view(dtype)[:n_r, :n_c])
+    torch.cuda.synchronize()
+    sg.sg_check()
+    assert sg.sg_last_kernel() == sg.SG_KERNEL_TMA_MOVE
+    want = src[:, :C].t() if op == "transpose" else src[:, :C]
+    assert torch.equal(dst[:n_r, :n_c], want)
+    assert bool((dst[n_r:] == FILL).all()) and bool((dst[:, n_c:] == FILL).all())
+
+
+# one row; rows shorter than 256; totals that are and are not multiples of 256; the last box cut off; a pitch on either side
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("R,C,src_pad,dst_pad", [(1, 256, 0, 0), (1, 256 * 37, 0, 0), (1, 264, 0, 0), (32, 24, 0, 0), (33, 24, 0, 0),
+                                                 (256 * 9, 8, 0, 0), (250, 1024, 0, 0), (1031, 512, 0, 0), (1031, 512, 8, 0), (1031, 512, 0, 8),
+                                                 (3000, 1016, 0, 0), (2, 65536, 0, 0)])
+def test_dense_copies(R, C, src_pad, dst_pad, dtype):
+    run("copy", R, C, dtype, C + src_pad, C + dst_pad)
+
+
+# 64 MB in elements of 4 and of 2 bytes, less one row of tiles and exactly; tiles cut off on both sides
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("R,C", [(4096, 4096), (4088, 4104), (8192, 4096), (8184, 4088), (128, 64), (136, 72), (8, 2048)])
+def test_transposes_around_the_window_rule(R, C, dtype):
+    run("transpose", R, C, dtype, C, R)

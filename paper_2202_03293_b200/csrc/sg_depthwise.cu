@@ -493,8 +493,19 @@ bool try_launch_tma(const DepthwiseProblem &p, const DtTiling &d, const T *I, co
         return false;
     constexpr int slot = 184 + (sizeof(T) == 4 ? 8 : 0) + (CB == 64 ? 0 : 4) + (K == 5 ? 2 : 0) + (S - 1);
     if (!tensor_ensure_smem_attr(slot, reinterpret_cast<const void *>(depthwise_tma_kernel<T, CB, K, S>), 2 * 56 * 1024 + 128)) return false;
-    // two CTAs per SM, rounded down to a multiple of the channel blocks: tile t has block t % c_blocks, so every CTA keeps one
+    // two CTAs per SM at a time, rounded down to a multiple of the channel blocks: tile t has block t % c_blocks, so every CTA keeps one
     int64_t grid = std::min<int64_t>(d.num_tiles, 2 * (int64_t)num_sms);
+    // Calls that HBM bounds: several times as many CTAs, of 2.6 tiles or more each, that start in order as others end: persistent ones
+    // drift apart, and reads and writes then come from all over the two tensors.  us, two per SM and so: bf16 32 x 112 x 112 x 64 28.8
+    // and 26.7, x 192 88 and 73, 96 x 150 x 150 x 64 150 and 126, f32 31 x 150 x 157 x 256 278 and 226, bf16 64 x 97 x 97 x 72 72 and 55.
+    // Not for 5 x 5 windows (arithmetic), f32 at stride 2 (61 and 73) or blocks that miss channels of 64 (f32 40 x 106 x 106 x 48 30.7 and
+    // 34.9, bf16 8 x 104 x 104 x 536 48.1 and 51.3); nor where the uneven shares take an eighth more rounds (32 x 112 x 119 x 64 28.6 and 29.6).
+    if (K == 3 && (S == 1 || sizeof(T) == 2) && (CB == 32 || p.C % 64 == 0)) {
+        const int64_t slots = grid, once = (d.num_tiles + slots - 1) / slots;
+        int64_t m = d.num_tiles * (int64_t)10 / (26 * slots);
+        while (m > 1 && 100 * m * ((d.num_tiles + m * slots - 1) / (m * slots)) > 113 * once) --m;
+        if (m > 1) grid = m * slots;
+    }
     grid -= grid % d.c_blocks;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid, 1, 1);

@@ -238,33 +238,29 @@ __global__ void __launch_bounds__(256) tile_move_kernel(const U *__restrict__ sr
         constexpr int H = MV / 32, K = MV / 8;
         __shared__ U tile[MV][MV + (sizeof(U) == 2 ? 2 : 1)];
         const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-        const int num_tiles = tiles_i * tiles_j;
-        for (int t = blockIdx.x; t < num_tiles; t += gridDim.x) {
-            int ti, tj;
-            tile_coords(t, tiles_j, tiles_i, panel, ti, tj);
-            const int i0 = ti * MV, j0 = tj * MV;
-            U v[H * K];
+        int ti, tj;
+        tile_coords(blockIdx.x, tiles_j, tiles_i, panel, ti, tj);
+        const int i0 = ti * MV, j0 = tj * MV;
+        U v[H * K];
 #pragma unroll
-            for (int k = 0; k < K; ++k)
+        for (int k = 0; k < K; ++k)
 #pragma unroll
-                for (int h = 0; h < H; ++h) {
-                    const int i = i0 + ty + 8 * k, j = j0 + tx + 32 * h;
-                    if (i < R && j < C) v[H * k + h] = src[(int64_t)i * s_i + (int64_t)j * s_j];
-                }
+            for (int h = 0; h < H; ++h) {
+                const int i = i0 + ty + 8 * k, j = j0 + tx + 32 * h;
+                if (i < R && j < C) v[H * k + h] = src[(int64_t)i * s_i + (int64_t)j * s_j];
+            }
 #pragma unroll
-            for (int k = 0; k < K; ++k)
+        for (int k = 0; k < K; ++k)
 #pragma unroll
-                for (int h = 0; h < H; ++h) tile[ty + 8 * k][tx + 32 * h] = v[H * k + h];
-            __syncthreads();
+            for (int h = 0; h < H; ++h) tile[ty + 8 * k][tx + 32 * h] = v[H * k + h];
+        __syncthreads();
 #pragma unroll
-            for (int k = 0; k < K; ++k)
+        for (int k = 0; k < K; ++k)
 #pragma unroll
-                for (int h = 0; h < H; ++h) {
-                    const int i = i0 + tx + 32 * h, j = j0 + ty + 8 * k;
-                    if (i < R && j < C) dst[(int64_t)i * d_i + (int64_t)j * d_j] = tile[tx + 32 * h][ty + 8 * k];
-                }
-            __syncthreads();
-        }
+            for (int h = 0; h < H; ++h) {
+                const int i = i0 + tx + 32 * h, j = j0 + ty + 8 * k;
+                if (i < R && j < C) dst[(int64_t)i * d_i + (int64_t)j * d_j] = tile[tx + 32 * h][ty + 8 * k];
+            }
     } else {
         constexpr int KR = 8 / KC;
         const int cw_log = KC > 1 ? 8 : shape.cw_log, cw = 1 << cw_log, rows_log = 8 - cw_log, rows = 1 << rows_log;
@@ -695,13 +691,16 @@ cudaError_t launch_reduce_typed(bool colred, const T *A, int64_t ld, int64_t sc,
                              rows_per_split, meet);
 }
 
-// Runs along j on both sides.  Narrow rows: a power of two of threads covers one; wide rows: up to four elements of one per thread (eight
-// of the 16-byte units), of up to eight in all.  Fewer elements a thread where that leaves SMs idle.  Up to four waves of thread blocks: in
-// one wave all blocks load, then store, together (every other column of 12288 x 16384 f32: one wave 217 us, four 185).
+// Runs along j on both sides.  Narrow rows: a power of two of threads covers one; wide rows: up to four elements of one per thread, of
+// up to eight in all.  Fewer elements a thread where that leaves SMs idle.  Wide rows of 4 bytes or more: a thread block for every
+// piece; they start in order as others end, and reads and writes each advance in one window (dense 16383 x 12287 bf16 / f32 16383 x 6001:
+// four waves of blocks that walk on 125.0 / 121.5 us, so 117.6 / 114.8; every other column of 12288 x 16384 f32 185 and 174, in one
+// wave 217).  Pieces of 4 KB, or of narrow rows, are too little for a block of their own: four waves (8192 x 8192 bf16 of odd pitch 85 us,
+// a block each 89.2; 4M x 3 f32 of pitch 4 24.8 and 26.1).
 template <typename U>
 cudaError_t launch_straight(const U *src, int64_t s_i, int64_t s_j, U *dst, int64_t d_i, int64_t d_j, int R, int C, int num_sms, cudaStream_t stream,
                             const uint8_t *tail_src, uint8_t *tail_dst, int tail_bytes) {
-    constexpr int MOST = sizeof(U) == 16 ? 8 : 4;
+    constexpr int MOST = 4;
     Straight t{0, 1};
     int kc = 1;
     while (t.cw_log < 8 && (1 << t.cw_log) < C) ++t.cw_log;
@@ -717,20 +716,12 @@ cudaError_t launch_straight(const U *src, int64_t s_i, int64_t s_j, U *dst, int6
         else kc /= 2;
     }
     using Kernel = void (*)(const U *, int64_t, int64_t, U *, int64_t, int64_t, int, int, int, int, int, Straight, const uint8_t *, uint8_t *, int);
-    static constexpr Kernel kernels[4] = {tile_move_kernel<U, 0, 1>, tile_move_kernel<U, 0, 2>, tile_move_kernel<U, 0, 4>, tile_move_kernel<U, 0, MOST>};
-    struct Resident {
-        int n[4];
-        Resident() {
-            for (int i = 0; i < 4; ++i)
-                if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n[i], kernels[i], 256, 0) != cudaSuccess || n[i] < 1) n[i] = 4;
-        }
-    };
-    static const Resident resident;
-    const int which = kc == 1 ? 0 : kc == 2 ? 1 : kc == 4 ? 2 : 3;
-    const Kernel kernel = kernels[which];
-    const int64_t most = (int64_t)num_sms * resident.n[which] * 4, grid_i = std::min(units_i, std::max<int64_t>(1, most / std::min<int64_t>(units_j, 32)));
-    return launch_overlapped(kernel, dim3((unsigned)std::min(units_j, most / grid_i), (unsigned)grid_i), 256, 0, 1, stream, src, s_i, s_j, dst, d_i, d_j, R, C,
-                             0, 0, 0, t, tail_src, tail_dst, tail_bytes);
+    const Kernel kernel = kc == 1 ? tile_move_kernel<U, 0, 1> : kc == 2 ? tile_move_kernel<U, 0, 2> : tile_move_kernel<U, 0, MOST>;
+    const bool all = sizeof(U) >= 4 && t.cw_log == 8;
+    const int64_t most = (int64_t)num_sms * 8 * 4;
+    const int64_t grid_i = std::min<int64_t>({units_i, 65535, all ? 65535 : std::max<int64_t>(1, most / std::min<int64_t>(units_j, 32))});
+    return launch_overlapped(kernel, dim3((unsigned)(all ? units_j : std::min(units_j, most / grid_i)), (unsigned)grid_i), 256, 0, 1, stream, src, s_i, s_j, dst, d_i,
+                             d_j, R, C, 0, 0, 0, t, tail_src, tail_dst, tail_bytes);
 }
 
 template <typename U>
@@ -745,8 +736,8 @@ cudaError_t launch_tile_move(const U *src, int64_t s_i, int64_t s_j, U *dst, int
         const int mv = (int64_t)((R + 63) / 64) * ((C + 63) / 64) < 2 * num_sms ? 32 : 64;
         const int tiles_i = (R + mv - 1) / mv, tiles_j = (C + mv - 1) / mv;
         if ((int64_t)tiles_i * tiles_j > 0x7fffffff) return cudaErrorInvalidConfiguration;
-        const int grid = std::min(tiles_i * tiles_j, num_sms * 8);
-        return launch_overlapped(mv == 32 ? tile_move_kernel<U, 32, 0> : tile_move_kernel<U, 64, 0>, dim3(grid), 256, 0, 1, stream, src, s_i, s_j, dst, d_i, d_j, R, C,
+        // a thread block per tile (eight per SM that walk on: 16383 x 6001 f32 201 us, so 150; 4737 x 3457 33.0 and 27.9; 16383 x 12287 bf16 315 and 293)
+        return launch_overlapped(mv == 32 ? tile_move_kernel<U, 32, 0> : tile_move_kernel<U, 64, 0>, dim3((unsigned)(tiles_i * tiles_j)), 256, 0, 1, stream, src, s_i, s_j, dst, d_i, d_j, R, C,
                                  tiles_i, tiles_j, std::min(tiles_j, TR_PANEL), Straight{}, (const uint8_t *)nullptr, (uint8_t *)nullptr, 0);
     }
     const int64_t bytes = (int64_t)R * C * (int64_t)sizeof(U);

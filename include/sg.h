@@ -42,7 +42,8 @@
  *     16-byte aligned bases and row pitches) run on the tensor-core path
  *     (TMA + tcgen05): bf16 inputs directly, f32 inputs split into hi + lo with
  *     hi*hi in tf32 and lo*hi + hi*lo in bf16 (operands stored transposed, less
- *     than 128 values of k: in tf32), summed in f32, which keeps f32 accuracy for finite inputs: the
+ *     than 128 values of k: in tf32), summed in f32, which keeps f32 accuracy for
+ *     finite inputs: the
  *     error stays below 1e-5 * sum_k |a*b| (subnormal f32 factors are taken as
  *     multiples of 2^-136).  Infinities keep their meaning there while the
  *     factors that they meet in a sum are normal and below 2000 together; beyond

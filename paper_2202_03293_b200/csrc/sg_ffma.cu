@@ -11,6 +11,7 @@
 // of a tile is the image of the tile under the operand's indexing map, which for these
 // ops separates into a per-row offset plus a per-k offset (see Problem).
 #include <algorithm>
+#include <limits>
 
 #include "sg_internal.cuh"
 
@@ -345,6 +346,8 @@ __global__ void zero_fill_rows_kernel(float *__restrict__ O, int M, int n4, int6
     }
 }
 
+constexpr unsigned MAX_GRID_Y = 65535;
+
 inline bool mult_of(int64_t v, int64_t q) { return v % q == 0; }
 
 // Launches a kernel that (`overlap`) may start while the kernel ahead of it drains; its last argument says whether it then has to wait for that one.
@@ -372,31 +375,50 @@ double small_tiles_us(const Problem &p) {
     const double blocks = (double)((p.M + ST - 1) / ST) * ((p.N + ST - 1) / ST);
     return 1.9 + 0.027 * k + blocks * (0.0015 + 0.0001 * k);
 }
-double large_tiles_us(const Problem &p, bool vec) {
+double large_tiles_us(const Problem &p, bool vec, int num_sms) {
     const int64_t tiles = (int64_t)((p.M + BM - 1) / BM) * ((p.N + BN - 1) / BN);
-    return 5.0 + (double)((tiles + 147) / 148) * ((p.K + BK - 1) / BK) * (vec ? 2.1 : 3.9);
+    return 5.0 + (double)((tiles + num_sms - 1) / num_sms) * ((p.K + BK - 1) / BK) * (vec ? 2.1 : 3.9);
+}
+
+// What a call that names no kernel gets here: which operands go in 8- or 16-byte loads, which tiles, and what those take.  A grid has up to 65535 tiles along
+// the columns: beyond that 32 x 32 tiles are out, then 128 x 128 ones too (`us` is infinite).  (Priced without that limit, 1 x 8388481 x 1 bf16 was refused,
+// and 2 x 2097129 x 32 took 1.64 ms in 128 x 128 tiles; the gather kernel takes 1.0.)
+struct Plan { bool vec_a, vec_b, small; double us; };
+template <typename T>
+Plan plan_call(const Problem &p, const T *In, const T *Flt) {
+    int device = 0, num_sms = 148, pdl = 0, unused = 0;
+    tensor_device_info(&device, &num_sms, &pdl, &unused);
+    Plan r{};
+    // 4 consecutive k (resp. f) may be fetched as one 8- or 16-byte load when they are
+    // contiguous in memory and every address involved is a multiple of 4 elements.
+    const uintptr_t vec_bytes = 4 * sizeof(T);
+    r.vec_a = p.i_c == 1 && mult_of(p.C, 4) && mult_of(p.i_n, 4) && mult_of(p.i_h, 4) &&
+              mult_of(p.i_w, 4) && (reinterpret_cast<uintptr_t>(In) % vec_bytes == 0);
+    r.vec_b = p.k_f == 1 && mult_of(p.N, 4) && mult_of(p.k_kh, 4) && mult_of(p.k_kw, 4) &&
+              mult_of(p.k_c, 4) && (reinterpret_cast<uintptr_t>(Flt) % vec_bytes == 0);
+    const double none = std::numeric_limits<double>::infinity();
+    const double small = ((int64_t)p.N + ST - 1) / ST <= MAX_GRID_Y ? small_tiles_us(p) : none;
+    const double large = ((int64_t)p.N + BN - 1) / BN <= MAX_GRID_Y ? large_tiles_us(p, r.vec_a && r.vec_b, num_sms) : none;
+    r.small = small < large;
+    r.us = std::min(small, large);
+    return r;
 }
 
 template <typename T>
 cudaError_t launch_typed(const Problem &p, const T *In, const T *Flt, float *O, bool forced, cudaStream_t stream) {
-    // 4 consecutive k (resp. f) may be fetched as one 8- or 16-byte load when they are
-    // contiguous in memory and every address involved is a multiple of 4 elements.
-    const uintptr_t vec_bytes = 4 * sizeof(T);
-    bool vec_a = p.i_c == 1 && mult_of(p.C, 4) && mult_of(p.i_n, 4) && mult_of(p.i_h, 4) &&
-                 mult_of(p.i_w, 4) && (reinterpret_cast<uintptr_t>(In) % vec_bytes == 0);
-    bool vec_b = p.k_f == 1 && mult_of(p.N, 4) && mult_of(p.k_kh, 4) && mult_of(p.k_kw, 4) &&
-                 mult_of(p.k_c, 4) && (reinterpret_cast<uintptr_t>(Flt) % vec_bytes == 0);
+    const Plan plan = plan_call(p, In, Flt);
+    const bool vec_a = plan.vec_a, vec_b = plan.vec_b;
     int vec_c = p.o_f == 1 && mult_of(p.o_n, 4) && mult_of(p.o_h, 4) && mult_of(p.o_w, 4) &&
                 (reinterpret_cast<uintptr_t>(O) % 16 == 0);
     // A caller who asks for this kernel by name gets 128 x 128 and one sum along k: the accuracy that the tensor-core kernels of these layouts are held against.
-    if (!forced && (p.N + ST - 1) / ST <= 65535 && small_tiles_us(p) < large_tiles_us(p, vec_a && vec_b)) {
+    if (!forced && plan.small) {
         // (a lane to each k, or to each row or column, whichever is contiguous in memory)
         const int a_along_k = p.spatial_rank != 0 || p.i_c == 1 || p.i_w != 1, b_along_k = p.k_f != 1 && p.k_c == 1;
         note_kernel("ffma_kernel");
         return launch_after(true, ffma_small_kernel<T>, dim3((p.M + ST - 1) / ST, (p.N + ST - 1) / ST), THREADS, stream, p, In, Flt, O, a_along_k, b_along_k);
     }
     dim3 grid((p.M + BM - 1) / BM, (p.N + BN - 1) / BN);
-    if (grid.y > 65535) return cudaErrorInvalidConfiguration;
+    if (grid.y > MAX_GRID_Y) return cudaErrorInvalidConfiguration;
     if (vec_a && vec_b) ffma_kernel<T, true, true><<<grid, THREADS, 0, stream>>>(p, In, Flt, O, vec_c);
     else if (vec_a) ffma_kernel<T, true, false><<<grid, THREADS, 0, stream>>>(p, In, Flt, O, vec_c);
     else if (vec_b) ffma_kernel<T, false, true><<<grid, THREADS, 0, stream>>>(p, In, Flt, O, vec_c);
@@ -408,7 +430,10 @@ cudaError_t launch_typed(const Problem &p, const T *In, const T *Flt, float *O, 
 
 }  // namespace
 
-double ffma_estimate_us(const Problem &p) { return std::min(small_tiles_us(p), large_tiles_us(p, false)); }
+double ffma_estimate_us(const Problem &p, const void *In, const void *Flt) {
+    return p.in_bf16 ? plan_call(p, static_cast<const unsigned short *>(In), static_cast<const unsigned short *>(Flt)).us
+                     : plan_call(p, static_cast<const float *>(In), static_cast<const float *>(Flt)).us;
+}
 
 cudaError_t launch_ffma(const Problem &p, const void *In, const void *Flt, float *O, bool forced, cudaStream_t stream) {
     if (p.in_bf16)

@@ -754,10 +754,10 @@ bool too_small(const Problem &p) { return (int64_t)p.M * p.N * p.K < ((int64_t)1
 // The CUDA-core kernel by time where its sums are as accurate: below that line all of f32's (longer ones are the more accurate here too), and bf16's of up to
 // 256 values (relative error of sums of either sign, K = 27, 127 and 255: 2.8e-8, 5.1e-8 and 6.7e-8, here 3.1e-8, 6.0e-8 and 6.8e-8).  Below the line those of up to
 // 160 values, f32 8, stay there whatever the time.  6 x 35 x 35, 3x3x3x32 bf16 takes 3.7 us there and 6.6 here, 39 x 7 x 267 f32 10 and 9.
-bool better_on_cuda_cores(const Problem &p, double us) {
+bool better_on_cuda_cores(const Problem &p, const void *In, const void *Flt, double us) {
     const bool small = too_small(p);
     if (p.in_bf16 ? p.K > 256 && !small : !small) return false;
-    return (small && p.K <= (p.in_bf16 ? 160 : 8)) || ffma_estimate_us(p) <= us;
+    return (small && p.K <= (p.in_bf16 ? 160 : 8)) || ffma_estimate_us(p, In, Flt) <= us;
 }
 
 }  // namespace
@@ -792,7 +792,7 @@ sg_status launch_gather(const Problem &p, const void *In, const void *Flt, float
     if (!tensor_device_info(&dev, &num_sms, &pdl, &unused)) return SG_ERR_CUDA;
 
     const Tiles plan = plan_tiles(p, num_sms);
-    if (!forced && better_on_cuda_cores(p, plan.us)) return SG_ERR_UNSUPPORTED;
+    if (!forced && better_on_cuda_cores(p, In, Flt, plan.us)) return SG_ERR_UNSUPPORTED;
     GatherParams gp{};
     gp.p = p;
     const int es = p.in_bf16 ? 2 : 4;

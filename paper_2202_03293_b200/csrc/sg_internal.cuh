@@ -39,7 +39,7 @@ struct Problem {
 // `forced`: the caller asks for this kernel, which then runs in 128 x 128 tiles whatever the size.
 cudaError_t launch_ffma(const Problem &p, const void *In, const void *Flt, float *O, bool forced,
                         cudaStream_t stream);
-double ffma_estimate_us(const Problem &p);      // what it would take
+double ffma_estimate_us(const Problem &p, const void *In, const void *Flt);      // what a call that names no kernel would take (infinity: it cannot run)
 // `overlap`: the clearing may start while the kernel ahead drains.
 cudaError_t launch_zero_fill(const Problem &p, float *O, bool overlap, cudaStream_t stream);
 

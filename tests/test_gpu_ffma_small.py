@@ -85,3 +85,16 @@ def test_values_that_are_not_finite():
     fine = torch.isfinite(want)
     assert torch.equal(torch.isnan(C), torch.isnan(want)) and torch.equal(torch.isinf(C), torch.isinf(want))
     assert torch.allclose(C[fine].double(), want[fine], rtol=1e-6)
+
+
+# a grid has up to 65535 tiles along the columns: 32 x 32 tiles end at 2097120 of them, 128 x 128 tiles at 8388480
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("M,N,K", [(1, 2097121, 1), (2, 2097129, 9), (1, 8388479, 1), (1, 8388481, 1), (3, 8388481, 5)])
+def test_columns_at_the_limits_of_a_grid(M, N, K, dtype):
+    g = torch.Generator(device="cuda").manual_seed(SEED)
+    t = torch.bfloat16 if dtype == "bf16" else torch.float32
+    A, B = (torch.randint(-4, 5, shape, generator=g, device="cuda").to(t) for shape in ((M, K), (K, N)))
+    C = torch.full((M, N), float("nan"), device="cuda")
+    sg.sg_matmul(A, B, C)
+    assert torch.equal(C, (A.double() @ B.double()).float())
+    sg.sg_check()

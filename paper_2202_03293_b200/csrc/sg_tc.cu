@@ -35,6 +35,7 @@
 // drains its copies, frees its TMEM and returns.
 #include <cuda.h>
 
+#include <algorithm>
 #include <atomic>
 #include <cstdlib>
 #include <cstring>
@@ -1298,14 +1299,16 @@ inline int transposed_layout(const Problem &p) {
 }
 
 // f32: whether the correction products of an item of `kbs` k-blocks run as bf16 MMAs (eight MMAs a k-block) or all three products in
-// tf32 (twelve).  A product is 2^-22 of itself off in tf32 and up to 2^-19 with bf16 corrections, but every MMA also truncates the sum that it
-// adds to, which is most of the error of a longer sum and less with fewer MMAs.  Relative error (2-norm) of 2048 x K x 1024, uniform / normal
+// tf32 (twelve).  Every MMA truncates the sum that it adds to, which is most of the error of a longer dense sum and less with fewer MMAs.
+// Relative error (2-norm) of 2048 x K x 1024, uniform / normal
 // operands, three tf32 products and bf16 corrections: K = 64 4.6e-7 / 4.6e-7 and 6.2e-7 / 7.2e-7, 96 6.8e-7 / 6.9e-7 and 7.0e-7 / 7.9e-7, 128 9.1e-7 / 9.1e-7 and
-// 8.1e-7 / 8.8e-7, 256 1.8e-6 and 1.3e-6, 1024 7.2e-6 and 4.8e-6.  So from 128 values of k on; 2048^3 A.B^T 67 -> 51 us.  (The plain layout has
-// always had them.)
-constexpr int kMixKb = 4;
-bool bf16_corrections(const Overrides &ov, int lay, int kbs) {
-    return ov.ta != 0 && ov.mix != 0 && (lay == 0 || kbs >= kMixKb);
+// 8.1e-7 / 8.8e-7, 256 1.8e-6 and 1.3e-6, 1024 7.2e-6 and 4.8e-6.  So from 128 values of k on (values, not begun k-blocks: with 97 there are four of those);
+// 2048^3 A.B^T 67 -> 51 us.  (The plain layout has always had them.)
+// A single product is the less exact for it: 7e-8 of itself off (root mean square; 8e-7 at most) in tf32, 6e-7 (6e-6) with bf16 corrections, and so is a
+// sum that one product rules.
+constexpr int kMixValues = 128;
+bool bf16_corrections(const Overrides &ov, int lay, const Problem &p, int kbs) {
+    return ov.ta != 0 && ov.mix != 0 && (lay == 0 || std::min<int64_t>(p.K, (int64_t)kbs * (ROW_BYTES / 4)) >= kMixValues);
 }
 
 // Tile variant and k split of lowest estimated time, which is returned (unless the variant is forced); *out_pick = -1: none.
@@ -1313,7 +1316,7 @@ bool bf16_corrections(const Overrides &ov, int lay, int kbs) {
 // `longest`: the most k-blocks of a range that runs with bf16 corrections (transposed f32 operands).
 double choose_tiles(const Problem &p, int num_kb, int lay, const Overrides &ov, int num_sms, int *out_pick, int *out_splits, int *out_meet, int longest = 1 << 30) {
     *out_meet = 0;
-    if (!p.in_bf16 && lay != 0 && num_kb >= kMixKb && ov.mix != 0 && ov.bn == 0 && ov.split == 0 && longest == 1 << 30) {
+    if (!p.in_bf16 && lay != 0 && p.K >= kMixValues && ov.mix != 0 && ov.bn == 0 && ov.split == 0 && longest == 1 << 30) {
         // A cheaper k-block asks for longer ranges, and the error grows with them: a range gets at most half as long again as three tf32
         // products would have had, which is as accurate (256 x 4096 x 256 A.B^T: 32 ranges 9.2e-7, 16 with bf16 corrections 1.3e-6).
         Overrides tf32 = ov;
@@ -1325,7 +1328,7 @@ double choose_tiles(const Problem &p, int num_kb, int lay, const Overrides &ov, 
     const bool fused = p.bias != nullptr || p.act != SG_ACT_NONE, forced_tile = ov.bn > 0 || ov.cg > 0 || (ov.split > 0 && !fused);
     const bool f32 = !p.in_bf16;
     auto kind = [&](int sp) {
-        if (f32) return lay == 0 ? F32_PLAIN : bf16_corrections(ov, lay, (num_kb + sp - 1) / sp) ? F32_TRANSPOSED : F32_TRANSPOSED_TF32;
+        if (f32) return lay == 0 ? F32_PLAIN : bf16_corrections(ov, lay, p, (num_kb + sp - 1) / sp) ? F32_TRANSPOSED : F32_TRANSPOSED_TF32;
         return lay == 0 && p.spatial_rank == 0 && p.K % 64 == 0 && p.N % 64 == 0 ? BF16_TWO : BF16_ONE;      // (see launch_tensor)
     };
     // variants that are not built (or that would sum too long a range): f32 tiles of 256 columns to a CTA (shared memory), and for transposed
@@ -1657,7 +1660,7 @@ sg_status launch_tensor(const Problem &p, const void *In, const void *Flt, float
         const int64_t tiles = (int64_t)num_m_tiles * num_n_tiles;
         const int left = (int)(tiles % groups);
         if (ov.sk != 0 && splits == 1) {
-            const int run = stream_k_run(var, !f32 ? BF16_ONE : lay == 0 ? F32_PLAIN : bf16_corrections(ov, lay, per) ? F32_TRANSPOSED : F32_TRANSPOSED_TF32, tiles, groups, tp.num_kb, kps, p.accumulate != 0, ov.sk == 2);
+            const int run = stream_k_run(var, !f32 ? BF16_ONE : lay == 0 ? F32_PLAIN : bf16_corrections(ov, lay, p, per) ? F32_TRANSPOSED : F32_TRANSPOSED_TF32, tiles, groups, tp.num_kb, kps, p.accumulate != 0, ov.sk == 2);
             if (run > 0) {
                 tp.sk_first_tile = (int)(tiles - left);
                 tp.sk_units = run;
@@ -1678,7 +1681,7 @@ sg_status launch_tensor(const Problem &p, const void *In, const void *Flt, float
     // either way), so there is one rule.
     // The two correction products of the split run as bf16 MMAs (see split4_mix and bf16_corrections).
     int lay_k = (f32 && ov.ta != 0) ? (lay | 4) : lay;
-    if (f32 && bf16_corrections(ov, lay, per)) lay_k |= 8;
+    if (f32 && bf16_corrections(ov, lay, p, per)) lay_k |= 8;
     const int slot = lay_k > 12 ? kMixSlots + (lay_k - 13) * kNumVariants + pick
                                 : pick + (f32 ? kNumVariants : 0) + (kps == 2 ? 2 * kNumVariants : 0) + (lay_k == 12 ? 8 : lay_k) * 3 * kNumVariants;
 #define SG_LAUNCH(BN_, CG_)                                                                                \

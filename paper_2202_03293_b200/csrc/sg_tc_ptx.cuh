@@ -394,8 +394,8 @@ __device__ __forceinline__ void split8(const uint4 v0, const uint4 v1, uint4 &h0
 
 // The split used when the two correction products run as bf16 MMAs: x = hi + lo with hi = x rounded to tf32 (as above); the
 // main product hi*hi runs in tf32, the corrections lo*hi + hi*lo with all four factors rounded to bf16.  A correction term
-// is below 2^-11 of its product and bf16 keeps 8 bits of each factor, so the rounding moves a product by less than 2^-19 of
-// itself (what the dropped lo*lo term and the tensor core's f32 accumulation cost already), and the two bf16 products of a k-block are one
+// is up to 2^-11 of its product, and bf16 rounds lo by up to 2^-9 and hi by up to 2^-8 of itself: the rounding moves a product by up to
+// 2 (2^-20 + 2^-19) = 5.8e-6 of itself, 6e-7 in the root mean square, and the two bf16 products of a k-block are one
 // contraction over 64 values, [lo | hi] . [hi | lo], at twice the tf32 rate: two tensor-core units per term instead of three.
 // Infinities and NaNs: as above (the bf16 copy of hi is finite too); a factor below 2^-134 is zero in both bf16 parts, NaN against an infinity.
 __device__ __forceinline__ void split_pair_mix(uint32_t x, uint32_t y, uint32_t &hx, uint32_t &hy, uint32_t &h16, uint32_t &l16) {

@@ -38,3 +38,31 @@ def test_transposed_tiles(M, N, K, bn, cg, a_t, b_t, dtype):
     want, S = ref.matmul(np.ascontiguousarray(a[rows]), b)
     assert assert_within_bound(C[torch.from_numpy(rows).cuda()], want, S, "transposed tiles") < 4e-6      # 2^-19 for the rounded corrections, and the truncating sum
     sg.sg_check()
+
+
+# One product a sum, so that nothing hides its own error: three tf32 products below 128 values of k, bf16 corrections from there on.  A factor is hi + lo,
+# lo up to 2^-11 of it; rounding lo to tf32 moves it by 2^-12, to bf16 by 2^-9, hi to bf16 by 2^-8; lo * lo is dropped, up to 2^-22, and three
+# truncating additions take up to 2^-23 each (the first adds to zero).
+@pytest.mark.parametrize("K", [97, 100, 124, 127, 128, 160])
+@pytest.mark.parametrize("a_t,b_t", [(True, False), (False, True), (True, True)])
+@pytest.mark.parametrize("bn", [64, 128])
+def test_single_products(K, a_t, b_t, bn):
+    if (b_t or not a_t) and K % 4:
+        pytest.skip("rows of K values do not start on 16-byte boundaries")
+    M, N = 512, 512
+    g = torch.Generator(device="cuda").manual_seed(K)
+    A, B = torch.zeros(M, K, device="cuda"), torch.rand(K, N, generator=g, device="cuda") + 1
+    A[torch.arange(M), torch.randint(0, K, (M,), generator=g, device="cuda")] = torch.rand(M, generator=g, device="cuda") + 1
+    a, b = A.t().contiguous().t() if a_t else A, B.t().contiguous().t() if b_t else B
+    C = torch.full((M, N), float("nan"), device="cuda")
+    sg.sg_set_tile_override(bn, 1, 1)
+    try:
+        sg.sg_matmul(a, b, C)
+        torch.cuda.synchronize()
+        assert sg.sg_last_kernel_name() == "tc_gemm_kernel<f32>" and tuple(sg.sg_last_tile_choice()) == (bn, 1, 1)
+    finally:
+        sg.sg_set_tile_override(0, 0, 0)
+    want = A.double() @ B.double()
+    factor = 2.0 ** -23 if K < 128 else 2.0 ** -20 + 2.0 ** -19
+    assert ((C.double() - want).abs() <= (2 * factor + 2.0 ** -22 + 2 * 2.0 ** -23) * want).all()
+    sg.sg_check()

@@ -1316,16 +1316,18 @@ bool bf16_corrections(const Overrides &ov, int lay, const Problem &p, int kbs) {
 // `longest`: the most k-blocks of a range that runs with bf16 corrections (transposed f32 operands).
 double choose_tiles(const Problem &p, int num_kb, int lay, const Overrides &ov, int num_sms, int *out_pick, int *out_splits, int *out_meet, int longest = 1 << 30) {
     *out_meet = 0;
-    if (!p.in_bf16 && lay != 0 && p.K >= kMixValues && ov.mix != 0 && ov.bn == 0 && ov.split == 0 && longest == 1 << 30) {
+    const bool fused = p.bias != nullptr || p.act != SG_ACT_NONE;
+    if (!p.in_bf16 && lay != 0 && p.K >= kMixValues && ov.mix != 0 && ov.bn == 0 && (ov.split == 0 || fused) && longest == 1 << 30) {
         // A cheaper k-block asks for longer ranges, and the error grows with them: a range gets at most half as long again as three tf32
-        // products would have had, which is as accurate (256 x 4096 x 256 A.B^T: 32 ranges 9.2e-7, 16 with bf16 corrections 1.3e-6).
+        // products would have had, which is as accurate (256 x 4096 x 256 A.B^T: 32 ranges 9.2e-7, 16 with bf16 corrections 1.3e-6; with a consumer,
+        // 512 x 512 x 384: two CTAs a tile 1.35e-6, one with bf16 corrections 1.86e-6, two of those 1.04e-6).
         Overrides tf32 = ov;
         tf32.mix = 0;
         choose_tiles(p, num_kb, lay, tf32, num_sms, out_pick, out_splits, out_meet);
         longest = (num_kb + *out_splits - 1) / *out_splits * 3 / 2;
         return choose_tiles(p, num_kb, lay, ov, num_sms, out_pick, out_splits, out_meet, longest);
     }
-    const bool fused = p.bias != nullptr || p.act != SG_ACT_NONE, forced_tile = ov.bn > 0 || ov.cg > 0 || (ov.split > 0 && !fused);
+    const bool forced_tile = ov.bn > 0 || ov.cg > 0 || (ov.split > 0 && !fused);
     const bool f32 = !p.in_bf16;
     auto kind = [&](int sp) {
         if (f32) return lay == 0 ? F32_PLAIN : bf16_corrections(ov, lay, p, (num_kb + sp - 1) / sp) ? F32_TRANSPOSED : F32_TRANSPOSED_TF32;

@@ -1,5 +1,10 @@
 """Operands stored transposed: every tile that is built for them, and (f32) the reductions on either side of the line from which
 the correction products run in bf16."""
+import json
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -66,3 +71,39 @@ def test_single_products(K, a_t, b_t, bn):
     factor = 2.0 ** -23 if K < 128 else 2.0 ** -20 + 2.0 ** -19
     assert ((C.double() - want).abs() <= (2 * factor + 2.0 ** -22 + 2 * 2.0 ** -23) * want).all()
     sg.sg_check()
+
+
+_CHOICES = """
+import json, sys, torch
+from paper_2202_03293_b200 import binding as sg
+out = []
+for M, N, K, fused in json.loads(sys.argv[1]):
+    for a_t, b_t in ((True, False), (False, True), (True, True)):
+        A, B = torch.zeros((K, M) if a_t else (M, K), device="cuda"), torch.zeros((N, K) if b_t else (K, N), device="cuda")
+        A, B, C = A.t() if a_t else A, B.t() if b_t else B, torch.empty(M, N, device="cuda")
+        if fused:
+            sg.sg_matmul_bias_act(A, B, torch.zeros(N, device="cuda"), C, sg.SG_ACT_RELU)
+        else:
+            sg.sg_matmul(A, B, C)
+        out.append([sg.sg_last_kernel_name(), sg.sg_last_tile_choice()[2]])
+sg.sg_check()
+print(json.dumps(out))
+"""
+
+
+def test_ranges_are_as_short_as_their_error_asks():
+    """A range of k gets at most half as long again as three tf32 products would have had, also where a consumer takes the sum."""
+    shapes = [[512, 512, 384], [512, 512, 416], [512, 1024, 512], [256, 512, 1024], [256, 256, 1024], [512, 512, 2048], [1024, 1024, 512], [256, 256, 4096]]
+    shapes = [s + [f] for s in shapes for f in (0, 1)]
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    found = []
+    for mix in ("1", "0"):
+        r = subprocess.run([sys.executable, "-c", _CHOICES, json.dumps(shapes)], cwd=root, env={**os.environ, "SG_TC_MIX": mix}, capture_output=True,
+                           text=True, timeout=300)
+        assert r.returncode == 0, r.stderr
+        found.append(json.loads(r.stdout))
+    for i, ((name, shares), (name0, shares0)) in enumerate(zip(*found)):
+        M, N, K, fused = shapes[i // 3]
+        assert name == name0 == "tc_gemm_kernel<f32>"
+        kb = K // 32
+        assert -(-kb // shares) <= -(-kb // shares0) * 3 // 2, (M, N, K, fused, shares, shares0)

@@ -495,16 +495,24 @@ bool try_launch_tma(const DepthwiseProblem &p, const DtTiling &d, const T *I, co
     if (!tensor_ensure_smem_attr(slot, reinterpret_cast<const void *>(depthwise_tma_kernel<T, CB, K, S>), 2 * 56 * 1024 + 128)) return false;
     // two CTAs per SM at a time, rounded down to a multiple of the channel blocks: tile t has block t % c_blocks, so every CTA keeps one
     int64_t grid = std::min<int64_t>(d.num_tiles, 2 * (int64_t)num_sms);
-    // Calls that HBM bounds: several times as many CTAs, of 2.6 tiles or more each, that start in order as others end: persistent ones
+    // Calls that HBM bounds: m times as many CTAs, of 2.6 tiles or more each, that start in order as others end: persistent ones
     // drift apart, and reads and writes then come from all over the two tensors.  us, two per SM and so: bf16 32 x 112 x 112 x 64 28.8
-    // and 26.7, x 192 88 and 73, 96 x 150 x 150 x 64 150 and 126, f32 31 x 150 x 157 x 256 278 and 226, bf16 64 x 97 x 97 x 72 72 and 55.
+    // and 26.9, x 192 88 and 73, 96 x 150 x 150 x 64 150 and 126, f32 31 x 150 x 157 x 256 278 and 226, bf16 64 x 97 x 97 x 72 72 and 55.
+    // A CTA's start and end cost about 1 us for every further one in a place.  f32 tiles make up for that only where most of what they compute is output: below 90 %
+    // with 5 tiles each (with 2.6, 66 x 17 x 17 x 512 19.7 and 21.8, 12 x 74 x 81 x 384 38.5 and 41.6), below 78 % not at all (37 x 66 x 66 x 192 42 and 47).
+    // bf16 at stride 2 needs three CTAs to a place to gain at all (two: 2 to 7 % slower), and wide tiles of one image (narrow ones and stacks of images fetch
+    // shorter runs: 67 x 49 x 49 x 576 180 and 200, 25 x 26 x 26 x 960 35.0 and 40.7, 34 x 81 x 81 x 256 106 and 120).
     // Not for 5 x 5 windows (arithmetic), f32 at stride 2 (61 and 73) or blocks that miss channels of 64 (f32 40 x 106 x 106 x 48 30.7 and
     // 34.9, bf16 8 x 104 x 104 x 536 48.1 and 51.3); nor where the uneven shares take an eighth more rounds (32 x 112 x 119 x 64 28.6 and 29.6).
-    if (K == 3 && (S == 1 || sizeof(T) == 2) && (CB == 32 || p.C % 64 == 0)) {
+    constexpr bool F32 = sizeof(T) == 4;
+    using C = DtCfg<T, CB, K, S>;
+    const double used = (double)p.N * p.Ho * p.Wo * p.C / ((double)d.num_tiles * (CB * C::GROUPS * C::WC * C::ROWS));
+    const bool gains = F32 ? S == 1 && used >= 0.78 : S == 1 || (d.cg > 1 && !d.stack);
+    if (K == 3 && gains && (CB == 32 || p.C % 64 == 0)) {
         const int64_t slots = grid, once = (d.num_tiles + slots - 1) / slots;
-        int64_t m = d.num_tiles * (int64_t)10 / (26 * slots);
+        int64_t m = d.num_tiles * (int64_t)10 / ((F32 && used < 0.9 ? 50 : 26) * slots);
         while (m > 1 && 100 * m * ((d.num_tiles + m * slots - 1) / (m * slots)) > 113 * once) --m;
-        if (m > 1) grid = m * slots;
+        if (m >= (S == 1 ? 2 : 3)) grid = m * slots;
     }
     grid -= grid % d.c_blocks;
     cudaLaunchConfig_t cfg = {};

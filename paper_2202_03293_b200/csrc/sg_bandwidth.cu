@@ -223,11 +223,20 @@ __global__ void __launch_bounds__(TR_THREADS) transpose_tma_kernel(const __grid_
 // Every thread has sixteen or up to eight loads in flight: with four, and 32 x 32 tiles, an unaligned 16383 x 12287 transpose
 // ran at 2.4 TB/s.
 // Without a turn: cw = 2^cw_log threads side by side along j, 256 / cw rows of them; a thread moves kr x KC elements, KC of them
-// 256 columns apart (1, 2, 4 or 8; more than one only where cw is 256), kr <= 8 / KC of them 256 / cw rows apart.  (Narrow rows are
+// 256 columns apart (1, 2 or 4; more than one only where cw is 256), kr <= 8 / KC of them 256 / cw rows apart.  (Narrow rows are
 // why: with 2048 columns of one row as the only shape 1M x 3 f32 of pitch 4 took 1.8 ms; now 7 us.)
 struct Straight {
     int cw_log, kr;
 };
+// Loads one element (2 or 4 bytes) if it exists, else 0.  Such loads go out back to back, whatever the compiler makes of the registers (behind branches 16383 x 6001 f32 took
+// 149 us, so 139).
+template <typename U>
+__device__ __forceinline__ void load_if(bool exists, const U *p, uint32_t &v) {
+    if constexpr (sizeof(U) == 4)
+        asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\tmov.u32 %0, 0;\n\t@q ld.global.u32 %0, [%1];\n\t}" : "=&r"(v) : "l"(p), "r"((uint32_t)exists) : "memory");
+    else
+        asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\tmov.u32 %0, 0;\n\t@q ld.global.u16 %0, [%1];\n\t}" : "=&r"(v) : "l"(p), "r"((uint32_t)exists) : "memory");
+}
 template <typename U, int MV, int KC>
 __global__ void __launch_bounds__(256) tile_move_kernel(const U *__restrict__ src, int64_t s_i, int64_t s_j, U *__restrict__ dst,
                                                          int64_t d_i, int64_t d_j, int R, int C, int tiles_i, int tiles_j, int panel,
@@ -241,18 +250,18 @@ __global__ void __launch_bounds__(256) tile_move_kernel(const U *__restrict__ sr
         int ti, tj;
         tile_coords(blockIdx.x, tiles_j, tiles_i, panel, ti, tj);
         const int i0 = ti * MV, j0 = tj * MV;
-        U v[H * K];
+        uint32_t v[H * K];
 #pragma unroll
         for (int k = 0; k < K; ++k)
 #pragma unroll
             for (int h = 0; h < H; ++h) {
                 const int i = i0 + ty + 8 * k, j = j0 + tx + 32 * h;
-                if (i < R && j < C) v[H * k + h] = src[(int64_t)i * s_i + (int64_t)j * s_j];
+                load_if(i < R && j < C, src + (int64_t)i * s_i + (int64_t)j * s_j, v[H * k + h]);
             }
 #pragma unroll
         for (int k = 0; k < K; ++k)
 #pragma unroll
-            for (int h = 0; h < H; ++h) tile[ty + 8 * k][tx + 32 * h] = v[H * k + h];
+            for (int h = 0; h < H; ++h) tile[ty + 8 * k][tx + 32 * h] = (U)v[H * k + h];
         __syncthreads();
 #pragma unroll
         for (int k = 0; k < K; ++k)
@@ -736,9 +745,16 @@ cudaError_t launch_tile_move(const U *src, int64_t s_i, int64_t s_j, U *dst, int
         const int mv = (int64_t)((R + 63) / 64) * ((C + 63) / 64) < 2 * num_sms ? 32 : 64;
         const int tiles_i = (R + mv - 1) / mv, tiles_j = (C + mv - 1) / mv;
         if ((int64_t)tiles_i * tiles_j > 0x7fffffff) return cudaErrorInvalidConfiguration;
-        // a thread block per tile (eight per SM that walk on: 16383 x 6001 f32 201 us, so 150; 4737 x 3457 33.0 and 27.9; 16383 x 12287 bf16 315 and 293)
-        return launch_overlapped(mv == 32 ? tile_move_kernel<U, 32, 0> : tile_move_kernel<U, 64, 0>, dim3((unsigned)(tiles_i * tiles_j)), 256, 0, 1, stream, src, s_i, s_j, dst, d_i, d_j, R, C,
-                                 tiles_i, tiles_j, std::min(tiles_j, TR_PANEL), Straight{}, (const uint8_t *)nullptr, (uint8_t *)nullptr, 0);
+        // a thread block per tile (eight per SM that walk on: 16383 x 6001 f32 201 us, so 139; 4737 x 3457 33.0 and 25.1; 16383 x 12287 bf16 315 and 242).
+        // Few of them: shared memory that nobody uses keeps an SM to its share of the blocks (four at least), which would otherwise go where the launch ahead left
+        // room (301 x 603 bf16 2.08 us, so 1.53; 512 x 4001 6.8 and 4.7; f32 801 x 603 3.06 and 2.46).  Not where SMs have none or one, nor for larger tiles of 4 bytes beyond
+        // five to an SM: what the spare memory takes from the L1 costs those more (3001 x 1201 f32 8.1, with six 9.0).
+        const int64_t tiles = (int64_t)tiles_i * tiles_j;
+        const int share = (int)std::max<int64_t>(4, (tiles + num_sms - 1) / num_sms), taken = mv * (mv + (sizeof(U) == 2 ? 2 : 1)) * (int)sizeof(U);
+        const bool even = tiles > num_sms && share < (mv == 64 && sizeof(U) == 4 ? 6 : 8);
+        const int spare = even ? std::min(smem_for(share, 0), 48 * 1024) - taken : 0;
+        return launch_overlapped(mv == 32 ? tile_move_kernel<U, 32, 0> : tile_move_kernel<U, 64, 0>, dim3((unsigned)tiles), 256, spare, 1, stream, src, s_i, s_j, dst, d_i,
+                                 d_j, R, C, tiles_i, tiles_j, std::min(tiles_j, TR_PANEL), Straight{}, (const uint8_t *)nullptr, (uint8_t *)nullptr, 0);
     }
     const int64_t bytes = (int64_t)R * C * (int64_t)sizeof(U);
     if (s_j == 1 && d_j == 1 && (R == 1 || (s_i == C && d_i == C)) && aligned16(src) && aligned16(dst) && bytes >= 16 && bytes / 16 < 0x7fffffff) {

@@ -368,16 +368,18 @@ cudaError_t launch_after(bool overlap, Kernel *kernel, dim3 grid, int block, cud
     return cudaLaunchKernelEx(&cfg, kernel, args..., wait_prior);
 }
 
-// Time in us of the two kernels, within 20 % of the timings of 40 calls: latencies of a fetch of 128 k and rounds of blocks; and rounds of tiles, 16 k at a time
-// (`vec`: both operands in 8- or 16-byte loads).  32 x 32 and 128 x 128: 511^3 f32 29 and 125, 1023^3 121 and 244, 333 x 4001 x 9 9.2 and 10.2, 1500 x 1500 x 100 34 and (vec) 20.
+// Time in us of the two kernels: a start, fetches of 128 k, k and blocks; and rounds of tiles, each with a start and its steps of 16 k (`vec`: both operands in 8- or 16-byte loads).
+// Fitted to graph replays of 640 and 630 calls, products and convolutions: within 7 % in the mean, and 11 (`vec` 2).  32 x 32 and 128 x 128: 511^3 f32 29 and 125, 1023^3 121 and
+// 244, 333 x 4001 x 9 9.2 and 10.2, 1500 x 1500 x 100 34 and (vec) 20, 3252 x 848 x 4 bf16 15.2 and (vec) 12.5.
 double small_tiles_us(const Problem &p) {
-    const int rest = p.K % SK, k = p.K - rest + (rest > 64 ? 128 : rest > 32 ? 64 : rest > 0 ? 32 : 0);
+    const int rest = p.K % SK, k = p.K - rest + (rest > 64 ? 128 : rest > 32 ? 64 : rest > 0 ? 32 : 0), fetches = (p.K + SK - 1) / SK;
     const double blocks = (double)((p.M + ST - 1) / ST) * ((p.N + ST - 1) / ST);
-    return 1.9 + 0.027 * k + blocks * (0.0015 + 0.0001 * k);
+    return p.spatial_rank == 0 ? 1.1 + 0.9 * fetches + 0.0206 * k + blocks * (0.00164 + 0.0001 * k) : 1.1 + 0.95 * fetches + 0.021 * k + blocks * (0.0024 + 0.00009 * k);
 }
 double large_tiles_us(const Problem &p, bool vec, int num_sms) {
     const int64_t tiles = (int64_t)((p.M + BM - 1) / BM) * ((p.N + BN - 1) / BN);
-    return 5.0 + (double)((tiles + num_sms - 1) / num_sms) * ((p.K + BK - 1) / BK) * (vec ? 2.1 : 3.9);
+    const double rounds = (double)((tiles + num_sms - 1) / num_sms), steps = (double)((p.K + BK - 1) / BK);
+    return vec ? 1.3 + rounds * (3.6 + 2.2 * steps) : 1.0 + rounds * (4.9 + (p.spatial_rank == 0 ? 3.8 : 2.7) * steps);
 }
 
 // What a call that names no kernel gets here: which operands go in 8- or 16-byte loads, which tiles, and what those take.  A grid has up to 65535 tiles along

@@ -723,25 +723,31 @@ bool raw_map(CUtensorMap *map, const void *ptr, Operand &op, int mn, int k, int 
 
 // Tiles, their width, and the CTAs (of one cluster) that share a tile's reduction.
 struct Tiles { int bn, num_kb, splits; int64_t tiles; double us; };
-// By time (us): a start and an end, a k-block of every round of tiles, what a further round adds, and for shared reductions what sharing costs;
-// 148 SMs hold 74, 33 and 15 clusters of 2, 4 and 8 CTAs at once.  Fitted to graph replays of 200 calls whose lines start anywhere, each in both widths and with
-// 1 to 8 CTAs a tile: the estimates are within 5 % in the mean, the choices cost 0.6 % over the best.  (With 128 columns wherever there are
+// By time (us): a start and an end, a k-block of every round of tiles, what a further round adds (its write-back paces it where the reduction is short), and what
+// sharing a reduction costs, the less of the tile a CTA sums up and writes the less;
+// 148 SMs hold 74, 33 and 15 clusters of 2, 4 and 8 CTAs at once.  Fitted to graph replays of 700 calls whose lines start anywhere, each in both widths and with
+// 1 to 8 CTAs a tile: the estimates are within 6 % in the mean, the choices cost 0.1 % over the best; with one cost of sharing for all numbers of CTAs 5 %
+// (9 x 11 x 11, 3x3x33x64 bf16 11.8 us by one CTA, 14.3 by two, 10.7 by four; two were taken), and without a least round 2970 x 12 x 3782 bf16 took tiles of 64 columns,
+// 30.9 and 26.2.  (With 128 columns wherever there are
 // more than 64, and only as many CTAs as fit beside one another, products took 22 % (f32) and 12 % (bf16) longer, convolutions 7 and 17:
 // 3181 x 682 x 868 f32 is 150 tiles of 128 columns, two rounds, 62 us, and 275 of 64, 42 us; 155 x 172 x 1369 19.7 and 10.5.)
 Tiles plan_tiles(const Problem &p, int num_sms) {
-    struct Cost { double ends, round, kb, shared, shared_round; };
-    constexpr Cost costs[2][2][2] = {{{{6.3, 1.2, 0.66, 1.1, 7.0}, {6.9, 3.6, 0.79, 2.1, 8.4}}, {{5.7, 1.3, 1.12, 1.1, 7.0}, {6.3, 2.1, 1.40, 2.1, 8.4}}},
-                                     {{{5.5, 1.3, 1.35, 1.9, 7.2}, {5.5, 2.0, 1.98, 3.4, 7.8}}, {{6.3, 1.3, 1.48, 1.9, 7.2}, {7.3, 2.2, 2.06, 3.4, 7.8}}}};      // [f32][convolution][128 columns]
+    struct Cost { double ends, round, kb, shared[3], shared_round, least_round; };
+    constexpr Cost costs[2][2][2] = {      // [f32][convolution][128 columns]
+        {{{5.7, 1.4, 0.64, {1.3, 0.5, 0.25}, 6.6, 2.7}, {6.5, 2.6, 0.79, {2.4, 1.1, 0.6}, 7.6, 4.6}},
+         {{5.5, 1.0, 1.09, {5.0, 2.3, 1.7}, 8.5, 2.4}, {6.2, 2.2, 1.29, {8.2, 3.5, 2.6}, 14.5, 1.6}}},
+        {{{5.4, 1.3, 1.20, {1.8, 0.9, 0.5}, 7.6, 2.3}, {6.0, 2.4, 1.79, {3.9, 1.4, 0.8}, 9.1, 2.5}},
+         {{5.9, 1.3, 1.57, {5.0, 2.7, 1.5}, 9.6, 2.5}, {6.6, 2.1, 2.29, {8.0, 4.0, 3.0}, 12.9, 2.7}}}};
     const int num_kb = (p.K + BK - 1) / BK;
     Tiles best{};
     best.us = 1e300;
     for (int bn = 64; bn <= (p.N > 64 ? 128 : 64); bn *= 2) {
         const Cost &c = costs[!p.in_bf16][p.spatial_rank != 0][bn == 128];
         const int64_t tiles = (int64_t)((p.M + BM - 1) / BM) * ((p.N + bn - 1) / bn);
-        for (int splits = 1; splits == 1 || (splits <= MAX_SPLIT && num_kb > 2 * splits); splits *= 2) {
+        for (int splits = 1, log = 0; splits == 1 || (splits <= MAX_SPLIT && num_kb > 2 * splits); splits *= 2, ++log) {
             const int at_once = splits == 1 ? num_sms : splits == 2 ? num_sms / 2 : splits == 4 ? num_sms / 4 - 4 : num_sms / 8 - 3;
-            const double rounds = (double)((tiles + at_once - 1) / at_once);
-            const double us = c.ends + rounds * c.kb * ((num_kb + splits - 1) / splits) + (splits == 1 ? (rounds - 1.0) * c.round : c.shared + (rounds - 1.0) * c.shared_round);
+            const double rounds = (double)((tiles + at_once - 1) / at_once), k = c.kb * ((num_kb + splits - 1) / splits);
+            const double us = c.ends + k + (splits == 1 ? 0.0 : c.shared[log - 1]) + (rounds - 1.0) * std::max(c.least_round, k + (splits == 1 ? c.round : c.shared_round));
             if (us < best.us) { best = Tiles{bn, num_kb, splits, tiles, us}; }
         }
     }
@@ -751,9 +757,11 @@ Tiles plan_tiles(const Problem &p, int num_sms) {
 // Below 2^21 multiply-adds the CUDA-core kernel may be the better one.
 bool too_small(const Problem &p) { return (int64_t)p.M * p.N * p.K < ((int64_t)1 << 21); }
 
-// The CUDA-core kernel by time where its sums are as accurate: below that line all of f32's (longer ones are the more accurate here too), and bf16's of up to
+// The CUDA-core kernel by time, where its sums are accurate enough: f32's below that line (the choice makes them no less exact than one chain of products: from some 190 values of k on
+// it is this kernel, 0.9e-7 for 2.7e-7 and more), and bf16's of up to
 // 256 values (relative error of sums of either sign, K = 27, 127 and 255: 2.8e-8, 5.1e-8 and 6.7e-8, here 3.1e-8, 6.0e-8 and 6.8e-8).  Below the line those of up to
-// 160 values, f32 8, stay there whatever the time.  6 x 35 x 35, 3x3x3x32 bf16 takes 3.7 us there and 6.6 here, 39 x 7 x 267 f32 10 and 9.
+// 160 values, f32 8, stay there whatever the time.  6 x 35 x 35, 3x3x3x32 bf16 takes 3.7 us there and 6.6 here, 39 x 7 x 267 f32 10 and 9.  Above the line f32 stays here for its
+// accuracy, not for the time: 163 x 166 x 125 8.2 us and 7.6e-8, in 32 x 32 tiles there 5.8 and 1.1e-7; 74 x 662 x 57 6.7 and 6.8e-8, 4.3 and 7.9e-8.
 bool better_on_cuda_cores(const Problem &p, const void *In, const void *Flt, double us) {
     const bool small = too_small(p);
     if (p.in_bf16 ? p.K > 256 && !small : !small) return false;
@@ -765,7 +773,8 @@ bool better_on_cuda_cores(const Problem &p, const void *In, const void *Flt, dou
 // What the kernel for small problems competes with: the time of tiles of 128 columns wherever there are more than 64, shared by as many CTAs as fit beside one
 // another.  A start and an end, rounds of tiles and their k-blocks, and what sharing a reduction costs, fitted to graph replays of 500 calls whose lines are whole
 // 16-byte pieces (those that the kernel for small problems could take): within 4 to 9 %.  (Better tiles would take some of them from that kernel, which is the
-// more accurate one: bf16, K = 1024, 1.1e-7 and 1.9e-7.)
+// more accurate one: bf16, K = 1024, 1.1e-7 and 1.9e-7.  That costs little: of 250 products of transposed operands that the small kernel could take, the present plan's estimate
+// moves four, 200 x 112 x 1520 bf16 12.5 -> 10.1 us, 328 x 480 x 1816 12.4 -> 10.8, two by 2 to 4 %.)
 double gather_estimate_us(const Problem &p, int num_sms) {
     if (too_small(p)) return 1e9;
     struct Cost { double ends, kb, round, shared; };

@@ -50,6 +50,41 @@ def test_products(M, N, K, orders, dtype):
     sg.sg_check()
 
 
+# Two and three fetches of 128 k, the last by 32 and 64 threads along k.  One chain of additions along k would give another sum: every k but the first adds 1 to
+# 2^24, which a chain loses each time, while the three of the four groups that do not hold 2^24 count theirs.
+@pytest.mark.parametrize("orders", [("n", "n"), ("t", "t"), ("gaps", "n"), ("t", "gaps")])
+@pytest.mark.parametrize("M,N,K", [(5, 33, 257), (33, 31, 287), (1, 7, 299), (7, 5, 129)])
+def test_four_short_sums_over_several_fetches(M, N, K, orders):
+    A, B = torch.ones(M, K, device="cuda"), torch.ones(K, N, device="cuda")
+    A[:, 0] = 2.0 ** 24
+    A, B = strided(A, orders[0]), strided(B, orders[1])
+    C = torch.full((M, N), float("nan"), device="cuda")
+    sg.sg_matmul(A, B, C)
+    torch.cuda.synchronize()
+    assert sg.sg_last_kernel_name() == "ffma_kernel"
+    groups = [len(range(i, K, 4)) for i in range(4)]
+    f = np.float32
+    want = (f(2 ** 24) + f(groups[1])) + (f(groups[2]) + f(groups[3]))
+    assert want > 2 ** 24 + K / 2 and (C == float(want)).all()
+    sg.sg_check()
+
+
+@pytest.mark.parametrize("orders", [("n", "n"), ("t", "t"), ("gaps", "n"), ("t", "gaps")])
+@pytest.mark.parametrize("M,N,K", [(5, 33, 257), (33, 31, 287), (1, 7, 299)])
+def test_products_of_several_fetches(M, N, K, orders):
+    A, a = operand((M, K), SEED, 6, "uniform", "f32")
+    B, b = operand((K, N), SEED, 7, "uniform", "f32")
+    A, B = strided(A, orders[0]), strided(B, orders[1])
+    want, S = ref.matmul(a, b)
+    C = torch.full((M, N), float("nan"), device="cuda")
+    sg.sg_matmul(A, B, C)
+    assert sg.sg_last_kernel_name() == "ffma_kernel"
+    assert assert_within_bound(C, want, S, "overwrite") <= (K / 4 + 4) * 2.0 ** -24
+    sg.sg_matmul(A, B, C, sg.SG_ACCUMULATE)
+    assert_within_bound(C, 2 * want, 2 * S, "accumulate")
+    sg.sg_check()
+
+
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("N,H,W,C,F,KH,KW,s,d", [(1, 29, 29, 3, 64, 3, 3, 2, 1), (1, 7, 5, 5, 33, 5, 3, 1, 1), (2, 9, 11, 3, 32, 3, 3, 1, 2), (3, 1, 2, 1, 1, 1, 1, 1, 1), (1, 6, 6, 9, 31, 5, 5, 1, 1)])
 def test_convolutions(N, H, W, C, F, KH, KW, s, d, dtype):

@@ -35,3 +35,30 @@ def test_same_bits_every_time(M, N, K, bn, cg, a_t, b_t):
     finally:
         sg.sg_set_tile_override(0, 0, 0)
     sg.sg_check()
+
+
+# pairs of 128 columns for transposed operands: 64 filter columns to a CTA as well
+@pytest.mark.parametrize("a_t,b_t", [(True, False), (False, True), (True, True)])
+@pytest.mark.parametrize("M,N,K", [(10560, 1792, 512), (4736, 1280, 1056)])
+def test_same_bits_every_time_pairs_of_transposed_operands(M, N, K, a_t, b_t):
+    g = torch.Generator(device="cuda").manual_seed(M)
+    A = torch.rand(M, K, generator=g, device="cuda") * 2 - 1
+    B = torch.rand(K, N, generator=g, device="cuda") * 2 - 1
+    want = A.double() @ B.double()
+    bound = A.double().abs() @ B.double().abs()
+    a, b = A.t().contiguous().t() if a_t else A, B.t().contiguous().t() if b_t else B
+    sg.sg_set_tile_override(128, 2, 1)
+    try:
+        first = torch.zeros(M, N, device="cuda")
+        sg.sg_matmul(a, b, first)
+        assert tuple(sg.sg_last_tile_choice()) == (128, 2, 1) and sg.sg_last_stream_k()[0] < 0
+        assert ((first.double() - want).abs() <= 4e-6 * bound).all()
+        C = torch.zeros(M, N, device="cuda")
+        wrong = torch.zeros((), dtype=torch.int64, device="cuda")
+        for _ in range(200):
+            sg.sg_matmul(a, b, C)
+            wrong += (C != first).any()
+        assert wrong.item() == 0
+    finally:
+        sg.sg_set_tile_override(0, 0, 0)
+    sg.sg_check()

@@ -86,6 +86,35 @@ def test_infinities(bn, cg, a_t, b_t, swap):
     sg.sg_check()
 
 
+# transposed operands from 128 values of k on: there the correction products are bf16 ones
+@pytest.mark.parametrize("bn,cg", [(64, 1), (128, 1), (128, 2), (256, 2)])
+@pytest.mark.parametrize("a_t,b_t", [(True, False), (False, True), (True, True)])
+@pytest.mark.parametrize("swap", [False, True])
+def test_infinities_and_bf16_corrections(bn, cg, a_t, b_t, swap):
+    M, N, K = 512, 512, 128
+    g = torch.Generator(device="cuda").manual_seed(SEED)
+    A = torch.rand(M, K, generator=g, device="cuda") * 2 - 1
+    B = torch.rand(K, N, generator=g, device="cuda") * 2 - 1
+    X, Y = (B.t(), A.t()) if swap else (A, B)
+    for i, f in enumerate([1999.25, -1999.25, 1025.5, -0.75, 2.0 ** -126, -(2.0 ** -126)]):
+        X[i, 40] = f
+    Y[40, 5], Y[40, 6] = float("inf"), float("-inf")
+    want = (A.double() @ B.double()).float()
+    a, b = A.t().contiguous().t() if a_t else A, B.t().contiguous().t() if b_t else B
+    C = torch.full((M, N), float("nan"), device="cuda")
+    sg.sg_set_tile_override(bn, cg, 1)
+    try:
+        sg.sg_matmul(a, b, C)
+        torch.cuda.synchronize()
+        assert sg.sg_last_kernel_name() == "tc_gemm_kernel<f32>" and tuple(sg.sg_last_tile_choice()) == (bn, cg, 1)
+    finally:
+        sg.sg_set_tile_override(0, 0, 0)
+    infinite = torch.isinf(want)
+    assert int(infinite.sum()) == 2 * (N if swap else M) and torch.equal(C[infinite], want[infinite])
+    assert torch.isfinite(C[~infinite]).all()
+    sg.sg_check()
+
+
 @pytest.mark.parametrize("kernel", ["CONV_STRIP", "CONV_WIDE"])
 def test_infinities_of_convolutions(kernel):
     I = torch.zeros(2, 40, 41, 16, device="cuda")

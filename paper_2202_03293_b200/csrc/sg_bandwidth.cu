@@ -96,8 +96,14 @@ constexpr int TR_THREADS = 128;
 // Thread blocks that an SM holds.  A tensor far beyond the caches wants a narrow window, one that the L2 absorbs as many tiles in flight
 // as help (4 / 5 / 6 / 8 / 12 blocks: 16384 x 12288 bf16 135 / 123.4 / 125.3 / 127.5 / 129.1 us, 4736 x 3456 f32 25.1 / 23.0 / 22.9 / 23.1 / 23.3,
 // 12288 x 512 f32 11.5 / 10.7 / 10.0 / 9.4 / 9.3, 640 x 15360 bf16 8.8 / 8.3 / 7.9 / 7.5 / 7.7; rings of four tiles, two per SM: 143 / 25.0 /
-// 10.1 / 8.0).
-inline int transpose_ctas_per_sm(int64_t bytes) { return bytes >= ((int64_t)64 << 20) ? 5 : 8; }
+// 10.1 / 8.0).  Few tiles: no more than an SM's share of them, two at least, or launches that overlap deal them out unevenly (f32 2512 x 800, 500 tiles: 5.6 us with room
+// for eight, 4.9 for four; 10552 x 200, 581: 6.4 and 5.9; a tile to an SM or less needs no such care).
+inline int transpose_ctas_per_sm(int64_t bytes, int64_t tiles, int num_sms) {
+    if (bytes >= ((int64_t)64 << 20)) return 5;
+    return tiles <= num_sms ? 8 : (int)std::min<int64_t>(8, std::max<int64_t>(2, (tiles + num_sms - 1) / num_sms));
+}
+constexpr int ATTR_SLOT = 251;            // of tensor_ensure_smem_attr: transpose_tma_kernel<4>, <2>, tile_move_kernel<uint32_t, 32, 0>, <uint16_t, 32, 0>
+constexpr int SMEM_MOST = 115 * 1024;     // two blocks to an SM
 // dynamic shared memory of a block that needs `least` bytes, so that an SM holds `ctas` of them (228 KB, 1 KB of it taken per block)
 inline int smem_for(int ctas, int least) { return std::max(least, (228 * 1024 / ctas - 1200) & ~127); }
 
@@ -823,7 +829,10 @@ sg_status launch_move2d(bool transpose, int64_t R, int64_t C, const void *src, i
                                     CU_TENSOR_MAP_L2_PROMOTION_L2_128B) &&
                 tensor_encode_tiled(&map_dst, type, 2, dst, dims_d, st_dst, box_d, CU_TENSOR_MAP_SWIZZLE_128B,
                                     CU_TENSOR_MAP_L2_PROMOTION_L2_128B)) {
-                const int smem = smem_for(transpose_ctas_per_sm(R * C * esize), TR_TILE_BYTES + 1024);
+                const int smem = smem_for(transpose_ctas_per_sm(R * C * esize, tiles_c * tiles_r, num_sms), TR_TILE_BYTES + 1024);
+                if (smem > 48 * 1024 && !tensor_ensure_smem_attr(ATTR_SLOT + (esize == 4 ? 0 : 1), esize == 4 ? reinterpret_cast<const void *>(transpose_tma_kernel<4>)
+                                                                                                              : reinterpret_cast<const void *>(transpose_tma_kernel<2>), SMEM_MOST))
+                    return SG_ERR_CUDA;
                 const int panel = (int)std::min<int64_t>(tiles_c, TR_PANEL);
                 if (launch_overlapped(esize == 4 ? transpose_tma_kernel<4> : transpose_tma_kernel<2>, dim3((unsigned)(tiles_c * tiles_r)), TR_THREADS, smem, 1, stream, map_src, map_dst,
                                       (int)tiles_c, (int)tiles_r, panel, (int)Rb, (int)Cb) != cudaSuccess) return SG_ERR_CUDA;

@@ -1031,7 +1031,7 @@ typedef CUresult (*EncodeIm2colFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_
 // never across a tensor-map encode or a launch.  The tensor-map cache has a lock of its own.
 constexpr int kMaxDevices = 64;
 constexpr int kMixSlots = 236;                   // transposed f32 operands with bf16 corrections: three layouts of five variants
-constexpr int kAttrSlots = kMixSlots + 15;
+constexpr int kAttrSlots = kMixSlots + 15 + 4;   // ... and four kernels of sg_bandwidth.cu
 struct DeviceState {
     bool ready = false;
     int num_sms = 0;
@@ -1418,7 +1418,7 @@ sg_status launch_variant(const CUtensorMap &mi, const CUtensorMap &mf, const CUt
     return SG_ERR_INTERNAL;   // the split slots of a 128 x 256 f32 tile do not fit beside a TMA ring
   } else {
     using C = Cfg<BN, CG, F32, KPS, (LAY & 4) != 0>;
-    static_assert(5 * 3 * 9 <= 144 && 3 * kNumVariants <= kAttrSlots - kMixSlots, "attribute slots");
+    static_assert(5 * 3 * 9 <= 144 && 3 * kNumVariants <= 15, "attribute slots");
     if (!ensure_smem_attr(ctx.device, slot, tc_gemm_kernel<BN, CG, F32, KPS, LAY>, C::SMEM_BYTES)) return SG_ERR_CUDA;
     tp.num_m_tiles = (M + CG * BM - 1) / (CG * BM);
     tp.num_n_tiles = (N + BN - 1) / BN;

@@ -38,3 +38,21 @@ def test_dense_copies(R, C, src_pad, dst_pad, dtype):
 @pytest.mark.parametrize("R,C", [(4096, 4096), (4088, 4104), (8192, 4096), (8184, 4088), (128, 64), (136, 72), (8, 2048)])
 def test_transposes_around_the_window_rule(R, C, dtype):
     run("transpose", R, C, dtype, C, R)
+
+
+# Few tiles: the number of thread blocks that an SM may hold goes by the tiles (148 SMs), on either side of each line: 128 rows by 128 bytes where TMA
+# moves them, 32 x 32 where a row does not start on 16 bytes
+@pytest.mark.parametrize("dtype,es", [(torch.float32, 4), (torch.bfloat16, 2)])
+@pytest.mark.parametrize("tiles", [148, 149, 185, 186, 296, 297, 444, 445, 740, 889, 1184, 1190])
+@pytest.mark.parametrize("aligned", [True, False])
+def test_transposes_of_few_tiles(tiles, aligned, dtype, es):
+    a = max(d for d in range(1, 21) if tiles % d == 0)
+    R, C = (128 * a, 128 // es * (tiles // a)) if aligned else (32 * a - 5, 32 * (tiles // a) - 3)
+    src = torch.randint(-2 ** 15, 2 ** 15, (R, C * es // 2), device="cuda", dtype=torch.int16).view(dtype)
+    dst = torch.zeros(C, R, device="cuda", dtype=dtype)
+    for _ in range(3):
+        sg.sg_transpose2d(src, dst)
+    assert sg.sg_last_kernel_name() == ("transpose_tma_kernel" if aligned else "tile_move_kernel")
+    bits = torch.int32 if es == 4 else torch.int16
+    assert torch.equal(dst.view(bits), src.view(bits).t())
+    sg.sg_check()

@@ -752,13 +752,18 @@ cudaError_t launch_tile_move(const U *src, int64_t s_i, int64_t s_j, U *dst, int
         const int tiles_i = (R + mv - 1) / mv, tiles_j = (C + mv - 1) / mv;
         if ((int64_t)tiles_i * tiles_j > 0x7fffffff) return cudaErrorInvalidConfiguration;
         // a thread block per tile (eight per SM that walk on: 16383 x 6001 f32 201 us, so 139; 4737 x 3457 33.0 and 25.1; 16383 x 12287 bf16 315 and 242).
-        // Few of them: shared memory that nobody uses keeps an SM to its share of the blocks (four at least), which would otherwise go where the launch ahead left
-        // room (301 x 603 bf16 2.08 us, so 1.53; 512 x 4001 6.8 and 4.7; f32 801 x 603 3.06 and 2.46).  Not where SMs have none or one, nor for larger tiles of 4 bytes beyond
-        // five to an SM: what the spare memory takes from the L1 costs those more (3001 x 1201 f32 8.1, with six 9.0).
+        // Few of them: shared memory that nobody uses keeps an SM to its share of the blocks, which would otherwise go where the launch ahead left
+        // room (512 x 4001 bf16 6.8 us, so 4.7; f32 801 x 603 3.06 and 2.46).  Two of the smaller tiles to an SM from a quarter more of them than SMs on (tiles of f32 for each SM,
+        // without / for two / for four: 1.1 0.91 / 0.97 / 1.05 of eight blocks that walk on, 1.4 0.94 / 0.88 / 0.96, 1.6 0.91 / 0.83 / 0.99, 1.9 0.90 / 0.82 / 0.89), else four at
+        // least.  Not for larger tiles of 4 bytes beyond five to an SM (3001 x 1201 f32 8.1, with six 9.0).
         const int64_t tiles = (int64_t)tiles_i * tiles_j;
-        const int share = (int)std::max<int64_t>(4, (tiles + num_sms - 1) / num_sms), taken = mv * (mv + (sizeof(U) == 2 ? 2 : 1)) * (int)sizeof(U);
-        const bool even = tiles > num_sms && share < (mv == 64 && sizeof(U) == 4 ? 6 : 8);
-        const int spare = even ? std::min(smem_for(share, 0), 48 * 1024) - taken : 0;
+        const int taken = mv * (mv + (sizeof(U) == 2 ? 2 : 1)) * (int)sizeof(U);
+        const bool two = mv == 32 && 4 * tiles > 5 * num_sms && tiles <= 2 * num_sms;
+        const int share = (int)std::max<int64_t>(two ? 2 : 4, (tiles + num_sms - 1) / num_sms);
+        const bool even = two || (tiles > 2 * num_sms && share < (mv == 64 && sizeof(U) == 4 ? 6 : 8));
+        const int spare = even ? std::min(smem_for(share, 0), two ? SMEM_MOST : 48 * 1024) - taken : 0;
+        if (two && !tensor_ensure_smem_attr(ATTR_SLOT + (sizeof(U) == 4 ? 2 : 3), reinterpret_cast<const void *>(tile_move_kernel<U, 32, 0>), SMEM_MOST - taken))
+            return cudaErrorInvalidConfiguration;
         return launch_overlapped(mv == 32 ? tile_move_kernel<U, 32, 0> : tile_move_kernel<U, 64, 0>, dim3((unsigned)tiles), 256, spare, 1, stream, src, s_i, s_j, dst, d_i,
                                  d_j, R, C, tiles_i, tiles_j, std::min(tiles_j, TR_PANEL), Straight{}, (const uint8_t *)nullptr, (uint8_t *)nullptr, 0);
     }

@@ -225,7 +225,7 @@ __global__ void __launch_bounds__(TR_THREADS) transpose_tma_kernel(const __grid_
 // strides exchanged.  MV > 0: the destination is contiguous along i, the source along j: square tiles of MV elements go through
 // shared memory, a warp reads runs along j and writes runs along i.  Otherwise runs along j on both sides, straight from registers
 // (dense operands arrive here flattened, in units of 16 bytes, with up to 15 bytes left over that block 0 moves).  MV: side of a
-// tile, 64, or 32 while those are too few; 0: no turn.
+// tile, 64, or 32 while those are too few; 0: no turn.  (With a turn KC says how tiles are loaded, see launch_tile_move.)
 // Every thread has sixteen or up to eight loads in flight: with four, and 32 x 32 tiles, an unaligned 16383 x 12287 transpose
 // ran at 2.4 TB/s.
 // Without a turn: cw = 2^cw_log threads side by side along j, 256 / cw rows of them; a thread moves kr x KC elements, KC of them
@@ -262,7 +262,11 @@ __global__ void __launch_bounds__(256) tile_move_kernel(const U *__restrict__ sr
 #pragma unroll
             for (int h = 0; h < H; ++h) {
                 const int i = i0 + ty + 8 * k, j = j0 + tx + 32 * h;
-                load_if(i < R && j < C, src + (int64_t)i * s_i + (int64_t)j * s_j, v[H * k + h]);
+                if constexpr (KC == 1) {
+                    if (i < R && j < C) v[H * k + h] = src[(int64_t)i * s_i + (int64_t)j * s_j];
+                } else {
+                    load_if(i < R && j < C, src + (int64_t)i * s_i + (int64_t)j * s_j, v[H * k + h]);
+                }
             }
 #pragma unroll
         for (int k = 0; k < K; ++k)
@@ -755,7 +759,8 @@ cudaError_t launch_tile_move(const U *src, int64_t s_i, int64_t s_j, U *dst, int
         // Few of them: shared memory that nobody uses keeps an SM to its share of the blocks, which would otherwise go where the launch ahead left
         // room (512 x 4001 bf16 6.8 us, so 4.7; f32 801 x 603 3.06 and 2.46).  Two of the smaller tiles to an SM from a quarter more of them than SMs on (tiles of f32 for each SM,
         // without / for two / for four: 1.1 0.91 / 0.97 / 1.05 of eight blocks that walk on, 1.4 0.94 / 0.88 / 0.96, 1.6 0.91 / 0.83 / 0.99, 1.9 0.90 / 0.82 / 0.89), else four at
-        // least.  Not for larger tiles of 4 bytes beyond five to an SM (3001 x 1201 f32 8.1, with six 9.0).
+        // least.  Not for larger tiles of 4 bytes beyond five to an SM (3001 x 1201 f32 8.1, with six 9.0).  Those with five to six to an SM load behind branches, which takes
+        // 40 registers: an SM then has room for six of them and as much L1 as before (760 x 4168 8.0 us, so 7.3; outside that range 1 to 15 % slower).
         const int64_t tiles = (int64_t)tiles_i * tiles_j;
         const int taken = mv * (mv + (sizeof(U) == 2 ? 2 : 1)) * (int)sizeof(U);
         const bool two = mv == 32 && 4 * tiles > 5 * num_sms && tiles <= 2 * num_sms;
@@ -764,7 +769,9 @@ cudaError_t launch_tile_move(const U *src, int64_t s_i, int64_t s_j, U *dst, int
         const int spare = even ? std::min(smem_for(share, 0), two ? SMEM_MOST : 48 * 1024) - taken : 0;
         if (two && !tensor_ensure_smem_attr(ATTR_SLOT + (sizeof(U) == 4 ? 2 : 3), reinterpret_cast<const void *>(tile_move_kernel<U, 32, 0>), SMEM_MOST - taken))
             return cudaErrorInvalidConfiguration;
-        return launch_overlapped(mv == 32 ? tile_move_kernel<U, 32, 0> : tile_move_kernel<U, 64, 0>, dim3((unsigned)tiles), 256, spare, 1, stream, src, s_i, s_j, dst, d_i,
+        constexpr int BRANCHES = sizeof(U) == 4 ? 1 : 0;
+        const bool branches = mv == 64 && tiles > 5 * num_sms && tiles <= 6 * num_sms;
+        return launch_overlapped(mv == 32 ? tile_move_kernel<U, 32, 0> : branches ? tile_move_kernel<U, 64, BRANCHES> : tile_move_kernel<U, 64, 0>, dim3((unsigned)tiles), 256, spare, 1, stream, src, s_i, s_j, dst, d_i,
                                  d_j, R, C, tiles_i, tiles_j, std::min(tiles_j, TR_PANEL), Straight{}, (const uint8_t *)nullptr, (uint8_t *)nullptr, 0);
     }
     const int64_t bytes = (int64_t)R * C * (int64_t)sizeof(U);

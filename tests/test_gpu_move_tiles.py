@@ -56,3 +56,18 @@ def test_transposes_of_few_tiles(tiles, aligned, dtype, es):
     bits = torch.int32 if es == 4 else torch.int16
     assert torch.equal(dst.view(bits), src.view(bits).t())
     sg.sg_check()
+
+
+# 64 x 64 tiles, on either side of five and six to an SM (148 SMs), where tiles of 4 bytes are loaded another way; the last ones cut off
+@pytest.mark.parametrize("dtype,bits", [(torch.float32, torch.int32), (torch.bfloat16, torch.int16)])
+@pytest.mark.parametrize("a,b", [(20, 37), (19, 39), (24, 37), (7, 127), (1, 741)])
+@pytest.mark.parametrize("cut", [0, 1, 31, 63])
+def test_unaligned_transposes_of_five_and_six_tiles_to_an_sm(a, b, cut, dtype, bits):
+    R, C = 64 * a - cut, 64 * b - cut
+    src = torch.randint(-30000, 30000, (R, C + 1 + C % 2), dtype=bits, device="cuda")       # odd pitches
+    dst = torch.full((C + 1, R + 1 + R % 2), FILL, dtype=bits, device="cuda")
+    sg.sg_transpose2d(src.view(dtype)[:, :C], dst.view(dtype)[:C, :R])
+    assert sg.sg_last_kernel_name() == "tile_move_kernel"
+    assert torch.equal(dst[:C, :R], src[:, :C].t())
+    assert bool((dst[C:] == FILL).all()) and bool((dst[:, R:] == FILL).all())
+    sg.sg_check()

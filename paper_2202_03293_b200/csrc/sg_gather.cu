@@ -728,7 +728,8 @@ struct Tiles { int bn, num_kb, splits; int64_t tiles; double us; };
 // 148 SMs hold 74, 33 and 15 clusters of 2, 4 and 8 CTAs at once.  Fitted to graph replays of 700 calls whose lines start anywhere, each in both widths and with
 // 1 to 8 CTAs a tile: the estimates are within 6 % in the mean, the choices cost 0.1 % over the best; with one cost of sharing for all numbers of CTAs 5 %
 // (9 x 11 x 11, 3x3x33x64 bf16 11.8 us by one CTA, 14.3 by two, 10.7 by four; two were taken), and without a least round 2970 x 12 x 3782 bf16 took tiles of 64 columns,
-// 30.9 and 26.2.  (With 128 columns wherever there are
+// 30.9 and 26.2.  Five k-blocks of bf16 by one CTA are five partial sums (see launch_gather), each met with the running one: 0.4 us more, with 128 columns 1.4
+// (200 products of 257 to 320 values, in every width and by 1 and 2 CTAs; without it 1 x 68 x 267 was left to one CTA, 9.3 us, 7.4 by two).  (With 128 columns wherever there are
 // more than 64, and only as many CTAs as fit beside one another, products took 22 % (f32) and 12 % (bf16) longer, convolutions 7 and 17:
 // 3181 x 682 x 868 f32 is 150 tiles of 128 columns, two rounds, 62 us, and 275 of 64, 42 us; 155 x 172 x 1369 19.7 and 10.5.)
 Tiles plan_tiles(const Problem &p, int num_sms) {
@@ -739,6 +740,7 @@ Tiles plan_tiles(const Problem &p, int num_sms) {
         {{{5.4, 1.3, 1.20, {1.8, 0.9, 0.5}, 7.6, 2.3}, {6.0, 2.4, 1.79, {3.9, 1.4, 0.8}, 9.1, 2.5}},
          {{5.9, 1.3, 1.57, {5.0, 2.7, 1.5}, 9.6, 2.5}, {6.6, 2.1, 2.29, {8.0, 4.0, 3.0}, 12.9, 2.7}}}};
     const int num_kb = (p.K + BK - 1) / BK;
+    const bool five = p.in_bf16 && p.spatial_rank == 0 && num_kb == 5;
     Tiles best{};
     best.us = 1e300;
     for (int bn = 64; bn <= (p.N > 64 ? 128 : 64); bn *= 2) {
@@ -746,7 +748,8 @@ Tiles plan_tiles(const Problem &p, int num_sms) {
         const int64_t tiles = (int64_t)((p.M + BM - 1) / BM) * ((p.N + bn - 1) / bn);
         for (int splits = 1, log = 0; splits == 1 || (splits <= MAX_SPLIT && num_kb > 2 * splits); splits *= 2, ++log) {
             const int at_once = splits == 1 ? num_sms : splits == 2 ? num_sms / 2 : splits == 4 ? num_sms / 4 - 4 : num_sms / 8 - 3;
-            const double rounds = (double)((tiles + at_once - 1) / at_once), k = c.kb * ((num_kb + splits - 1) / splits);
+            const double rounds = (double)((tiles + at_once - 1) / at_once);
+            const double k = c.kb * ((num_kb + splits - 1) / splits) + (five && splits == 1 ? (bn == 64 ? 0.4 : 1.4) : 0.0);
             const double us = c.ends + k + (splits == 1 ? 0.0 : c.shared[log - 1]) + (rounds - 1.0) * std::max(c.least_round, k + (splits == 1 ? c.round : c.shared_round));
             if (us < best.us) { best = Tiles{bn, num_kb, splits, tiles, us}; }
         }

@@ -41,18 +41,27 @@
  *   - Shapes whose layout allows it (unit stride on the contiguous dimension,
  *     16-byte aligned bases and row pitches) run on the tensor-core path
  *     (TMA + tcgen05): bf16 inputs directly, f32 inputs split into hi + lo with
- *     hi*hi in tf32 and lo*hi + hi*lo in bf16 (operands stored transposed, less
- *     than 128 values of k: in tf32), summed in f32, which keeps f32 accuracy for
+ *     hi*hi in tf32 and lo*hi + hi*lo in bf16 (operands stored transposed, sums or ranges
+ *     of them of less than 128 values of k: in tf32), summed in f32, which keeps f32 accuracy for
  *     finite inputs: the
  *     error stays below 1e-5 * sum_k |a*b| (subnormal f32 factors are taken as
- *     multiples of 2^-136).  Infinities keep their meaning there while the
+ *     multiples of 2^-136).  A product by itself is up to 6.3e-6 of itself off (with
+ *     the corrections in tf32: 8e-7), so sums that one product rules, of sparse or
+ *     one-hot operands, are less exact than dense ones, whose error is mostly that of
+ *     the summing and smaller with the bf16 corrections.  Infinities keep their meaning there while the
  *     factors that they meet in a sum are normal and below 2000 together; beyond
  *     that the sum may be NaN.  Small problems run on many small thread blocks
  *     (mma.sync), where every infinity keeps its meaning.  Other layouts run on a tensor-core
  *     kernel that fetches its operands with ordinary or unaligned tensor loads
  *     and is about as accurate as an f32 FMA loop (f32 inputs as three bf16
- *     parts; infinities keep their meaning), tiny problems in them on a strided
- *     CUDA-core FFMA kernel.  There is no CPU fallback.
+ *     parts; infinities keep their meaning), or, where that is estimated to be the
+ *     faster one, on a strided CUDA-core FFMA kernel (bf16: sums of up to 256 products and all of less
+ *     than 2^21 multiply-adds; f32: less than 2^21).  There is no CPU fallback.
+ *   - Where the tensor-core path deals out a sum in ranges of k (few tiles and a long
+ *     reduction, or the last, partly filled wave of tiles), the ranges' sums meet in the output by
+ *     f32 additions in the order in which they arrive: the rounding of the last
+ *     bits may differ from call to call.  Which calls do so is chosen by
+ *     estimated time (sg_last_tile_choice and sg_last_stream_k tell).
  */
 #ifndef SG_H_
 #define SG_H_
@@ -270,7 +279,7 @@ int sg_last_kernel(void);
  * kernels launched ahead of it are not named): "tc_gemm_kernel<bf16>", "tc_gemm_kernel<f32>",
  * "gather_gemm_kernel<bf16>", "gather_gemm_kernel<f32>" (layouts outside the TMA rules), "small_gemm_kernel<bf16>",
  * "small_gemm_kernel<f32>", "conv_strip_kernel<bf16>", "conv_strip_kernel<f32>", "conv_wide_kernel<bf16>",
- * "conv_wide_kernel<f32>", "ffma_kernel", "depthwise_tma_kernel",
+ * "conv_wide_kernel<f32>", "ffma_kernel" (in tiles of 128 x 128 or 32 x 32), "depthwise_tma_kernel",
  * "depthwise_roll_kernel", "depthwise_vec_kernel", "depthwise_generic_kernel", "copy_tma_kernel",
  * "transpose_tma_kernel", "tile_move_kernel", "colred_kernel<vec>", "colred_kernel<scalar>",
  * "rowred_kernel<vec>", "rowred_kernel<scalar>", "rowred_short_kernel<vec>", "rowred_short_kernel<scalar>".  (Row sums

@@ -498,6 +498,7 @@ bool try_launch_tma(const DepthwiseProblem &p, const DtTiling &d, const T *I, co
     // Calls that HBM bounds: m times as many CTAs, of 2.6 tiles or more each, that start in order as others end: persistent ones
     // drift apart, and reads and writes then come from all over the two tensors.  us, two per SM and so: bf16 32 x 112 x 112 x 64 28.8
     // and 26.9, x 192 88 and 73, 96 x 150 x 150 x 64 150 and 126, f32 31 x 150 x 157 x 256 278 and 226, bf16 64 x 97 x 97 x 72 72 and 55.
+    // (2.0 to 2.4 tiles at least: of 350 layers of 4 to 64 images 16 of bf16 change, 11 of them 2 to 6 % slower and five up to 3 % faster, and nine to twelve of f32, 2 to 8 % slower.)
     // A CTA's start and end cost about 1 us for every further one in a place.  f32 tiles make up for that only where most of what they compute is output: below 90 %
     // with 5 tiles each (with 2.6, 66 x 17 x 17 x 512 19.7 and 21.8, 12 x 74 x 81 x 384 38.5 and 41.6), below 78 % not at all (37 x 66 x 66 x 192 42 and 47).
     // bf16 at stride 2 needs three CTAs to a place to gain at all (two: 2 to 7 % slower), and wide tiles of one image (narrow ones and stacks of images fetch
